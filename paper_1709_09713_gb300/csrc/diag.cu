@@ -10,6 +10,12 @@ namespace sbli {
 template <typename T>
 Coef<T> make_coef(const int n[3], const sbli_params& p) {
   Coef<T> c;
+  double e0s = 0.0;
+  for (int a = 0; a < 3; ++a) {
+    const double h = 2.0 * M_PI * p.L / (double)n[a];
+    e0s += -5.0 / (2.0 * h * h);
+  }
+  c.e0s = T(e0s);
   for (int a = 0; a < 3; ++a) {
     const double h = 2.0 * M_PI * p.L / (double)n[a];
     c.c1[a] = T(2.0 / (3.0 * h));
@@ -17,6 +23,13 @@ Coef<T> make_coef(const int n[3], const sbli_params& p) {
     c.e0[a] = T(-5.0 / (2.0 * h * h));
     c.e1[a] = T(4.0 / (3.0 * h * h));
     c.e2[a] = T(-1.0 / (12.0 * h * h));
+    c.hc1[a] = T(-1.0 / (3.0 * h));
+    c.hc2[a] = T(-1.0 / (24.0 * h));
+    c.t1[a] = T(2.0 / (9.0 * h));
+    c.t2[a] = T(1.0 / (36.0 * h));
+    c.f1[a] = T(16.0 / (9.0 * h * h));
+    c.f2[a] = T(-1.0 / (9.0 * h * h));
+    c.v0[a] = T(e0s - 5.0 / (6.0 * h * h));
   }
   const double inv_re = isinf(p.Re) ? 0.0 : 1.0 / p.Re;
   c.gm1 = T(p.gamma - 1.0);

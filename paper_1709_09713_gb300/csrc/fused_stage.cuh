@@ -79,7 +79,7 @@ constexpr int NSLOT = 5;
 // pressure enters Eqs. 2-3 only as 2 D_i p and 2 D_j(p u_j) in the combined
 // skew form, so the factor 2 is applied once per point instead of once per
 // stencil neighbour; scaling by 2 is exact)
-enum { V_RHO, V_M0, V_M1, V_M2, V_E, V_U0, V_U1, V_U2, V_P, V_T, NV };
+enum { V_RHO, V_M0, V_M1, V_M2, V_H, V_E = V_H, V_U0, V_U1, V_U2, V_P, V_T, NV };
 static_assert(V_U2 == V_U1 + 1 && V_U1 % 2 == 0, "u1, u2 form one 8-byte pair of a binary32 record");
 
 // ZT (binary32 with the TMEM z queue): the x2 neighbours of a thread's own
@@ -97,6 +97,12 @@ constexpr int full_slots() {
 template <typename T>
 constexpr bool mixz() {
   return std::is_same<T, float>::value || std::is_same<T, f32x2>::value;
+}
+// The hardware FMA types keep H = E' + 2p' in the record (see StreamTerms),
+// double-float E' itself.
+template <typename T>
+constexpr bool hrec() {
+  return !std::is_same<T, dfloat>::value;
 }
 template <typename T, int TY, bool ZT = false>
 struct FusedSmem {
@@ -552,7 +558,7 @@ struct Terms {
 
 // All derivatives along axis A at one point.  ldrec(k, r) loads the record of
 // the neighbour k = 0..3 (offsets -2, -1, +1, +2 along A); uc are the centre
-// velocities; sfun(k, record) gives the mixed-term helper s_A at neighbour k.
+// velocities; sfun(k) gives the mixed-term helper s_A at neighbour k.
 template <int A, typename T, typename LD, typename SF>
 __device__ __forceinline__ void axis_terms(const LD& ldrec, const SF& sfun, const Coef<T>& c, const T (&uc)[3],
                                            Terms<T>& t) {
@@ -565,7 +571,7 @@ __device__ __forceinline__ void axis_terms(const LD& ldrec, const SF& sfun, cons
   for (int k = 0; k < 4; ++k) ldrec(k, r[k]);
   T s[4];
 #pragma unroll
-  for (int k = 0; k < 4; ++k) s[k] = sfun(k, r[k]);
+  for (int k = 0; k < 4; ++k) s[k] = sfun(k);
 #define SBLI_D1(V) d1(r[0][V], r[1][V], r[2][V], r[3][V])
   const T ua = uc[A];
   // stencil weights times (u_A + u_A^c):  D1(f w) = f+1 W1 - f-1 V1 - f+2 W2 + f-2 V2
@@ -597,21 +603,48 @@ __device__ __forceinline__ void axis_terms(const LD& ldrec, const SF& sfun, cons
 #undef SBLI_D1
 }
 
-// The same terms with the four neighbours streamed through registers one at
-// a time: each neighbour's record is folded into the accumulators with its
-// stencil weights (Eq. 6: +c2, -c1, +c1, -c2; Eq. 7 off-centre: e2, e1, e1,
-// e2 for offsets -2, -1, +1, +2), so only one record is live.  Fewer
-// operations than the difference-first form for hardware FMA types; the
-// double-float type keeps the difference-first form (its products cost more
-// than its sums).
-// a + b, never contracted with the product that formed b (so its rounding
-// does not depend on how the compiler schedules that product)
-__device__ __forceinline__ float add_nc(float a, float b) { return __fadd_rn(a, b); }
-__device__ __forceinline__ f32x2 add_nc(f32x2 a, f32x2 b) { return a + b; }
+// a * b + c with one rounding in every scalar type (and lane): the streamed
+// terms below never leave a contraction to the compiler, so that every
+// instantiation of the kernel rounds alike.
+__device__ __forceinline__ double fmadd(double a, double b, double c) { return ::fma(a, b, c); }
+__device__ __forceinline__ float fmadd(float a, float b, float c) { return ::fmaf(a, b, c); }
+__device__ __forceinline__ f32x2 fmadd(f32x2 a, f32x2 b, f32x2 c) { return fma(a, b, c); }
+
+// Accumulated terms of the residual at one point for the hardware FMA types.
+// The centre values u_j^c, m_i^c are constant over a stencil, so the
+// convective terms of Eqs. 2-3 share the weight w = c (u_j + u_j^c) and
+//   E' (u_j + u_j^c) + 2 p' u_j = (E' + 2p')(u_j + u_j^c) - u_j^c 2p'
+// makes those of Eq. 3 one multiply-add a neighbour with H = E' + 2p' (the
+// record keeps H) and u_j^c times the pressure derivative that Eq. 2 needs
+// anyway.  (The like for Eq. 1, m_j + u_j^c rho' = u_j + rho' (u_j + u_j^c), would
+// take the rounding of u_j = m_j / rho into the mass balance: 1.45 times its
+// error, so Eq. 1 keeps two.)  The viscous terms of Eq. 2 are accumulated as
+// their sum (Laplacian + G/3), the symmetric off-diagonal gradients as their
+// sum: 15 multiply-adds a neighbour instead of the 17 of one accumulator per
+// derivative.  The number of instructions is what bounds these kernels
+// (binary64: of binary64 ones, at 0.92 of the pipe's measured peak): a 256^3
+// stage of binary64 went from 10.25 to 9.25 ms, the 512^3 binary32 one (binary64
+// accumulator) from 3.73 to 3.63 ms.
+// Binary64 also takes the factors -1/2 (convective terms) and 1/3, 4/3
+// (viscous terms) in its weights, 1.5 % fewer instructions; in binary32 the
+// 24 constants of that are too many for the uniform registers (479 -> 504 us),
+// and the factors are applied to the sums of an axis.
 template <typename T>
-__device__ __forceinline__ T add_nc(T a, T b) {
-  return a + b;
+constexpr bool scaled_weights() {
+  return std::is_same<T, double>::value;
 }
+template <typename T>
+struct StreamTerms {
+  // with scaled_weights times -1/2:
+  T rrho;     // sum_j D_j(m_j + u_j^c rho')                      (Eq. 1)
+  T rM[3];    // sum_j D_j(m_i (u_j + u_j^c)) + 2 D_i p'          (Eq. 2)
+  T rE;       // sum_j D_j(E' (u_j + u_j^c)) + 2 D_j(p' u_j)      (Eq. 3)
+  T v[3];     // sum_j D2_j u_i + 1/3 sum_j d2 u_j / dx_i dx_j
+  T lapT;     // sum_j D2_j T'
+  T a[3];     // D1_j u_i + D1_i u_j for (i, j) = (0, 1), (0, 2), (1, 2)
+  T lo[3];    // the first of the two alone (vorticity; diagnostics only)
+  T gd[3];    // D1_j u_j
+};
 
 // No x2-regrouped mixed terms (every axis but the binary32 x2 axis).
 struct NoXTerms {
@@ -619,66 +652,98 @@ struct NoXTerms {
   __device__ void operator()(int, T&, T&) const {}
 };
 
-// ZX (binary32, A = 2): the mixed derivatives that involve x2 are taken with
-// the x2 derivative last, D1_z(D1_x u2) and D1_z(D1_y u2) from xfun(k, ...)
-// (the neighbours' in-plane gradients of u2), added to G_0 and G_1; the
-// stream also forms D1_z u2 at the centre (g_22).
-template <int A, bool ZX = false, typename T, typename LD, typename SF, typename XF = NoXTerms>
+// All derivatives along axis A, the four neighbours streamed through
+// registers one at a time, so only one record is live.  ldrec(k, r) loads the
+// record of the neighbour k = 0..3 (offsets -2, -1, +1, +2 along A; Eq. 6
+// weights +c2, -c1, +c1, -c2, Eq. 7 e2, e1, e1, e2); sfun(k) gives the
+// mixed-term helper s_A there.  ZX (binary32, A = 2): the mixed derivatives
+// that involve x2 are taken with the x2 derivative last, D1_z(D1_x u2) and
+// D1_z(D1_y u2) from xfun(k, ...) (the neighbours' in-plane gradients of u2);
+// the stream also forms D1_z u2 at the centre.  WITH_KE: also lo[].
+template <int A, bool ZX, bool WITH_KE, typename T, typename LD, typename SF, typename XF = NoXTerms>
 __device__ __forceinline__ void axis_terms_stream(const LD& ldrec, const SF& sfun, const Coef<T>& c,
-                                                  const T (&uc)[3], Terms<T>& t, const XF& xfun = XF()) {
+                                                  const T (&uc)[3], StreamTerms<T>& t, const XF& xfun = XF()) {
   static_assert(!ZX || A == 2, "x2-last mixed terms belong to the x2 axis");
-  const T c1 = c.c1[A], c2 = c.c2[A], e1 = c.e1[A], e2 = c.e2[A];
+  constexpr bool SW = scaled_weights<T>();
   const T ua = uc[A];
-  T gz0 = T(0), gz1 = T(0), g22 = T(0);  // ZX only
-  T lAA = T(0);                       // sum_k e_k u_A,k: D2_A u_A without its centre term
-  T gA = T(0);                        // sum_k c_k s_k = D1_A s_A
-  T gI[3] = {T(0), T(0), T(0)};      // D1_A u_i, i != A
-  // the per-axis products c u_A^c once, so that each neighbour's two
-  // weights are one multiply and one fused multiply-add
-  const T cu1 = c1 * ua, cu2 = c2 * ua;
+  T dp = T(0);                            // D1_A 2p' (times -1/2)
+  T lA = T(0), gA = T(0);                 // !SW: D2_A u_A off-centre, D1_A s_A
+  T gz0 = T(0), gz1 = T(0);               // !SW, ZX: the x2 parts of G_0, G_1
+  auto sgn = [](int k, T inner, T outer) {  // the antisymmetric weight of neighbour k
+    return k == 0 ? outer : k == 1 ? -inner : k == 2 ? inner : -outer;
+  };
+  const T* w1 = SW ? c.hc1 : c.c1;
+  const T* w2 = SW ? c.hc2 : c.c2;
+  // the per-axis products c u_A^c once, so that each neighbour's weight is one multiply-add
+  const T cu1 = w1[A] * ua, cu2 = w2[A] * ua;
 #pragma unroll
   for (int k = 0; k < 4; ++k) {
-    const T cd = (k == 0) ? c2 : (k == 1) ? -c1 : (k == 2) ? c1 : -c2;
-    const T ed = (k == 0 || k == 3) ? e2 : e1;
-    const T cdu = (k == 0) ? cu2 : (k == 1) ? -cu1 : (k == 2) ? cu1 : -cu2;
+    const T cd = sgn(k, c.c1[A], c.c2[A]);
+    const T hd = sgn(k, w1[A], w2[A]);
+    const T ed = (k == 0 || k == 3) ? c.e2[A] : c.e1[A];
     T r[NV];
     ldrec(k, r);
-    const T sk = sfun(k, r);
-    const T w = fma(cd, r[V_U0 + A], cdu);  // D1(f (u_A + u_A^c)) weight
-    const T x = cd * r[V_U0 + A];          // D1(f u_A) weight (times 2 p' below)
+    const T w = fmadd(hd, r[V_U0 + A], sgn(k, cu1, cu2));
 #pragma unroll
-    for (int i = 0; i < 3; ++i) t.rM[i] = mad(w, r[V_M0 + i], t.rM[i]);
-    t.rM[A] = mad(cd, r[V_P], t.rM[A]);
-    t.rE = mad(w, r[V_E], mad(x, r[V_P], t.rE));
-    t.rrho = mad(cd, fma(ua, r[V_RHO], r[V_M0 + A]), t.rrho);
+    for (int i = 0; i < 3; ++i) t.rM[i] = fmadd(w, r[V_M0 + i], t.rM[i]);
+    t.rE = fmadd(w, r[V_H], t.rE);
+    t.rrho = fmadd(hd, fmadd(ua, r[V_RHO], r[V_M0 + A]), t.rrho);
+    dp = fmadd(hd, r[V_P], dp);
 #pragma unroll
     for (int i = 0; i < 3; ++i) {
       if (i != A) {
-        t.lap[i] = mad(ed, r[V_U0 + i], t.lap[i]);
-        gI[i] = mad(cd, r[V_U0 + i], gI[i]);
+        t.v[i] = fmadd(ed, r[V_U0 + i], t.v[i]);
+        const int pair = i + A - 1;  // (0,1) -> 0, (0,2) -> 1, (1,2) -> 2
+        t.a[pair] = fmadd(cd, r[V_U0 + i], t.a[pair]);
+        if (WITH_KE && i < A) t.lo[pair] = fmadd(cd, r[V_U0 + i], t.lo[pair]);
       }
     }
-    lAA = mad(ed, r[V_U0 + A], lAA);  // shared by the Laplacian of u_A and G_A
-    gA = mad(cd, sk, gA);
-    t.lapT = mad(ed, r[V_T], t.lapT);
+    // the Laplacian and one third of Eq. 7 on j = A, one third of D1_A s_A
+    if constexpr (SW) {
+      t.v[A] = fmadd((k == 0 || k == 3) ? c.f2[A] : c.f1[A], r[V_U0 + A], t.v[A]);
+      t.v[A] = fmadd(sgn(k, c.t1[A], c.t2[A]), sfun(k), t.v[A]);
+    } else {
+      lA = fmadd(ed, r[V_U0 + A], lA);
+      gA = fmadd(cd, sfun(k), gA);
+    }
+    t.lapT = fmadd(ed, r[V_T], t.lapT);
     if constexpr (ZX) {
+      static_assert(!SW, "binary32 only");
       T x02, x12;
       xfun(k, x02, x12);
-      gz0 = mad(cd, x02, gz0);
-      gz1 = mad(cd, x12, gz1);
-      g22 = add_nc(g22, x);  // x = cd u_2 (above): an add the compiler may not contract
+      gz0 = fmadd(cd, x02, gz0);
+      gz1 = fmadd(cd, x12, gz1);
+      t.gd[2] = fmadd(cd, r[V_U2], t.gd[2]);
     }
   }
-#pragma unroll
-  for (int i = 0; i < 3; ++i)
-    if (i != A) t.g[i][A] = gI[i];
-  t.lap[A] += lAA;
-  t.G[A] = fma(c.e0[A], uc[A], lAA + gA);  // D2_A u_A + D1_A s_A (Eq. 7 on j = A, D1 o D1 otherwise)
+  t.rM[A] = t.rM[A] + dp;
+  t.rE = fmadd(-ua, dp, t.rE);
+  if constexpr (!SW) t.v[A] = fmadd(T(4.0 / 3.0), lA, fmadd(T(1.0 / 3.0), gA, t.v[A]));
   if constexpr (ZX) {
-    t.G[0] = t.G[0] + gz0;
-    t.G[1] = t.G[1] + gz1;
-    t.g[2][2] = g22;
+    t.v[0] = fmadd(T(1.0 / 3.0), gz0, t.v[0]);
+    t.v[1] = fmadd(T(1.0 / 3.0), gz1, t.v[1]);
   }
+}
+
+// Eqs. 1-3 at one point from the streamed terms and the centre values.
+template <typename T>
+__device__ __forceinline__ void assemble_streamed(const StreamTerms<T>& t, T rho_p, const T (&mc)[3], T Ec,
+                                                  const T (&uc)[3], const Coef<T>& c, T (&R)[5]) {
+  constexpr bool SW = scaled_weights<T>();
+  const T div = t.gd[0] + t.gd[1] + t.gd[2];
+  const T hdiv = SW ? T(-0.5) * div : div;
+  auto half = [](T x) { return SW ? x : T(-0.5) * x; };
+  R[0] = half(fmadd(T(1) + rho_p, hdiv, t.rrho));
+#pragma unroll
+  for (int i = 0; i < 3; ++i) R[1 + i] = fmadd(c.inv_re, t.v[i], half(fmadd(mc[i], hdiv, t.rM[i])));
+  // viscous dissipation du_i/dx_j (du_i/dx_j + du_j/dx_i - 2/3 div delta_ij) and the work of the viscous force
+  T d = t.gd[0] * t.gd[0];
+  d = fmadd(t.gd[2], t.gd[2], fmadd(t.gd[1], t.gd[1], d));
+  T q = (T(-2.0 / 3.0) * div) * div;
+  q = fmadd(t.a[2], t.a[2], fmadd(t.a[1], t.a[1], fmadd(t.a[0], t.a[0], q)));
+  q = fmadd(T(2), d, q);
+  q = fmadd(uc[2], t.v[2], fmadd(uc[1], t.v[1], fmadd(uc[0], t.v[0], q)));
+  R[4] = fmadd(c.kappa, t.lapT, fmadd(c.inv_re, q, fmadd(-c.H0, div, half(fmadd(Ec, hdiv, t.rE)))));
 }
 
 // Eqs. 1-3 at one point from the accumulated derivative terms and the
@@ -704,17 +769,6 @@ __device__ __forceinline__ void assemble_residual(const Terms<T>& t, T rho_p, co
   const T diss = mad(T(2), sq, mad(a12, a12, mad(a02, a02, mad(a01, a01, T(-2.0 / 3.0) * div * div))));
   const T lapT = fma(e0sum, Tc, t.lapT);
   R[4] = mad(c.kappa, lapT, mad(c.inv_re, uvisc + diss, mad(-c.H0, div, T(-0.5) * mad(Ec, div, t.rE))));
-}
-
-template <int A, bool ZX = false, typename T, typename LD, typename SF, typename XF = NoXTerms>
-__device__ __forceinline__ void axis_terms_any(const LD& ldrec, const SF& sfun, const Coef<T>& c, const T (&uc)[3],
-                                               Terms<T>& t, const XF& xfun = XF()) {
-  if constexpr (std::is_same<T, dfloat>::value) {
-    static_assert(!ZX, "double-float keeps the s_i helpers");
-    axis_terms<A>(ldrec, sfun, c, uc, t);
-  } else {
-    axis_terms_stream<A, ZX>(ldrec, sfun, c, uc, t, xfun);
-  }
 }
 
 // TIN: type of the stage input in HBM; TOUT: type of the stage output.
@@ -925,7 +979,7 @@ __device__ __forceinline__ void fused_march(const StageArgs& a, const Coef<T>& c
           rec[V_M0] = m0;
           rec[V_M1] = m1;
           rec[V_M2] = m2;
-          rec[V_E] = E_p;
+          rec[V_H] = hrec<T>() ? E_p + p2 : E_p;
           rec[V_U0] = u0;
           rec[V_U1] = u1;
           rec[V_U2] = u2;
@@ -1042,6 +1096,7 @@ __device__ __forceinline__ void fused_march(const StageArgs& a, const Coef<T>& c
     // halo; binary32 has its helpers already (phase 2a of the plane's entry)
     // and needs only the centre's in-plane gradients.
     if constexpr (MIXZ) {
+      d22 = T(0);
       if constexpr (ZT) {
         tmem_load_diag(twin, scen, g00c, g11c);
       } else {
@@ -1097,69 +1152,94 @@ __device__ __forceinline__ void fused_march(const StageArgs& a, const Coef<T>& c
         load_rec(&C[sy][sx][0], cen);
       const T rho_p = cen[V_RHO];
       const T mc[3] = {cen[V_M0], cen[V_M1], cen[V_M2]};
-      const T Ec = cen[V_E];
+      const T Ec = hrec<T>() ? cen[V_H] - cen[V_P] : cen[V_E];
       const T uc[3] = {cen[V_U0], cen[V_U1], cen[V_U2]};
       const T Tc = cen[V_T];
 
-      Terms<T> t;
-      t.rrho = t.rE = t.lapT = T(0);
-#pragma unroll
-      for (int i = 0; i < 3; ++i) {
-        t.rM[i] = T(0);
-        t.lap[i] = T(0);
-      }
-      t.g[0][0] = g00c;
-      t.g[1][1] = g11c;
-      t.g[2][2] = d22;
-
-      // x0 group first (SN2 ordering), then x1, x2
+      // neighbours k = 0..3 (offsets -2, -1, +1, +2): records and mixed-term helpers
       const int sbc = MIXZ ? rb[0] : 0;  // helper buffers of the centre plane
-      {
-        const int off[4] = {-2, -1, 1, 2};
-        auto ld = [&](int k, T(&r)[NV]) { load_rec(&C[sy][sx + off[k]][0], r); };
-        auto sf = [&](int k, const T(&)[NV]) { return sm.s0buf[sbc][ty][sx + off[k]]; };
-        axis_terms_any<0>(ld, sf, c, uc, t);
-      }
-      {
-        const int off[4] = {-2, -1, 1, 2};
-        auto ld = [&](int k, T(&r)[NV]) { load_rec(&C[sy + off[k]][sx][0], r); };
-        auto sf = [&](int k, const T(&)[NV]) { return sm.s1buf[sbc][sy + off[k]][tx]; };
-        axis_terms_any<1>(ld, sf, c, uc, t);
-      }
-      {
-        const int zs[4] = {sl[0], sl[1], sl[3], sl[4]};
-        auto ld = [&](int k, T(&r)[NV]) {
-          if constexpr (ZT)
-            tmem_load_rec(twin, zs[k], r);
-          else
-            load_rec(&sm.ring[zs[k]][sy][sx][0], r);
-        };
-        auto sf = [&](int k, const T(&)[NV]) {
+      const int off[4] = {-2, -1, 1, 2};
+      const int zs[4] = {sl[0], sl[1], sl[3], sl[4]};
+      auto ld0 = [&](int k, T(&r)[NV]) { load_rec(&C[sy][sx + off[k]][0], r); };
+      auto sf0 = [&](int k) { return sm.s0buf[sbc][ty][sx + off[k]]; };
+      auto ld1 = [&](int k, T(&r)[NV]) { load_rec(&C[sy + off[k]][sx][0], r); };
+      auto sf1 = [&](int k) { return sm.s1buf[sbc][sy + off[k]][tx]; };
+      auto ld2 = [&](int k, T(&r)[NV]) {
+        if constexpr (ZT)
+          tmem_load_rec(twin, zs[k], r);
+        else
+          load_rec(&sm.ring[zs[k]][sy][sx][0], r);
+      };
+      auto sf2 = [&](int k) {
+        if constexpr (ZT) {
+          T a, b;
+          tmem_load_diag(twin, zs[k], a, b);
+          return a + b;
+        } else {
+          return sm.dring[zs[k]][0][ty][tx] + sm.dring[zs[k]][1][ty][tx];
+        }
+      };
+      // binary32: D1_x u2 and D1_y u2 of the x2 neighbours
+      auto xf = [&](int k, T& d02, T& d12) {
+        if constexpr (MIXZ) {
           if constexpr (ZT) {
-            T a, b;
-            tmem_load_diag(twin, zs[k], a, b);
-            return a + b;
+            tmem_load_xdiag(twin2, zs[k], d02, d12);
           } else {
-            return sm.dring[zs[k]][0][ty][tx] + sm.dring[zs[k]][1][ty][tx];
+            d02 = sm.dring[zs[k]][2][ty][tx];
+            d12 = sm.dring[zs[k]][3][ty][tx];
           }
-        };
-        // binary32: D1_x u2 and D1_y u2 of the x2 neighbours
-        auto xf = [&](int k, T& d02, T& d12) {
-          if constexpr (MIXZ) {
-            if constexpr (ZT) {
-              tmem_load_xdiag(twin2, zs[k], d02, d12);
-            } else {
-              d02 = sm.dring[zs[k]][2][ty][tx];
-              d12 = sm.dring[zs[k]][3][ty][tx];
-            }
-          }
-        };
-        axis_terms_any<2, MIXZ>(ld, sf, c, uc, t, xf);
-      }
+        }
+      };
 
-      const T rho = T(1) + rho_p;
       T R[5];
-      assemble_residual(t, rho_p, mc, Ec, uc, Tc, c, R);
+      T w0 = T(0), w1 = T(0), w2 = T(0);  // vorticity (WITH_KE)
+      // x0 group first (SN2 ordering), then x1, x2
+      if constexpr (std::is_same<T, dfloat>::value) {
+        Terms<T> t;
+        t.rrho = t.rE = t.lapT = T(0);
+#pragma unroll
+        for (int i = 0; i < 3; ++i) {
+          t.rM[i] = T(0);
+          t.lap[i] = T(0);
+        }
+        t.g[0][0] = g00c;
+        t.g[1][1] = g11c;
+        t.g[2][2] = d22;
+        axis_terms<0>(ld0, sf0, c, uc, t);
+        axis_terms<1>(ld1, sf1, c, uc, t);
+        axis_terms<2>(ld2, sf2, c, uc, t);
+        assemble_residual(t, rho_p, mc, Ec, uc, Tc, c, R);
+        if (WITH_KE) {
+          w0 = t.g[2][1] - t.g[1][2];
+          w1 = t.g[0][2] - t.g[2][0];
+          w2 = t.g[1][0] - t.g[0][1];
+        }
+      } else {
+        StreamTerms<T> t;
+        t.rrho = t.rE = T(0);
+        t.lapT = c.e0s * Tc;
+#pragma unroll
+        for (int i = 0; i < 3; ++i) {
+          t.rM[i] = t.a[i] = t.lo[i] = T(0);
+          t.v[i] = c.v0[i] * uc[i];
+        }
+        t.gd[0] = g00c;
+        t.gd[1] = g11c;
+        t.gd[2] = d22;
+        axis_terms_stream<0, false, WITH_KE>(ld0, sf0, c, uc, t);
+        // shared-memory loads of one axis at a time: hoisted over the axes they spill at the binary32 ring
+        // kernel's 128 registers (256^3: 674 us a stage without these two, 651 with)
+        if constexpr (!ZT && sizeof(T) == 4) asm volatile("" ::: "memory");
+        axis_terms_stream<1, false, WITH_KE>(ld1, sf1, c, uc, t);
+        if constexpr (!ZT && sizeof(T) == 4) asm volatile("" ::: "memory");
+        axis_terms_stream<2, MIXZ, WITH_KE>(ld2, sf2, c, uc, t, xf);
+        assemble_streamed(t, rho_p, mc, Ec, uc, c, R);
+        if (WITH_KE) {  // D1_j u_i - D1_i u_j = 2 D1_j u_i - (their sum), lo = D1_j u_i with i < j
+          w2 = fmadd(T(-2), t.lo[0], t.a[0]);
+          w1 = fmadd(T(2), t.lo[1], -t.a[1]);
+          w0 = fmadd(T(-2), t.lo[2], t.a[2]);
+        }
+      }
 
 #pragma unroll
       for (int j = 0; j < PP; ++j) {
@@ -1261,9 +1341,8 @@ __device__ __forceinline__ void fused_march(const StageArgs& a, const Coef<T>& c
           }
         }
         if (WITH_KE) {
-          const T w0 = t.g[2][1] - t.g[1][2], w1 = t.g[0][2] - t.g[2][0], w2 = t.g[1][0] - t.g[0][1];
           const T ke_t = T(0.5) * (mc[0] * uc[0] + mc[1] * uc[1] + mc[2] * uc[2]);
-          const T ens_t = T(0.5) * rho * (w0 * w0 + w1 * w1 + w2 * w2);
+          const T ens_t = T(0.5) * (T(1) + rho_p) * (w0 * w0 + w1 * w1 + w2 * w2);
           ke_acc += double(lane(ke_t, j));
           ens_acc += double(lane(ens_t, j));
         }
