@@ -211,7 +211,8 @@ SBLI_API int sbli_kinetic_energy_noalloc(const double* q_dev, int n0, int n1, in
 /* Launch configuration of the fused kernel: in-plane tile height (the tile
  * is 32 x tile_y points per column a thread owns; binary64-register grids
  * (SBLI_FP64, SBLI_DF64) use 8, binary32 grids 8 or 16), planes per CTA
- * along x2 (>= 4), where each thread keeps its column's records of the five
+ * along x2 (>= 4; binary64-register grids split all planes evenly over the SMs
+ * instead where that leaves the longest CTA fewer of them), where each thread keeps its column's records of the five
  * x2 planes (z_queue = 0: the shared-memory ring; 1: a per-thread queue in
  * Blackwell tensor memory, with only three full-record planes in shared
  * memory -- four for binary32 tile_y 16, which saves one barrier per plane)
@@ -265,7 +266,8 @@ SBLI_API int sbli_batch_work_items(const sbli_batch* b, long long* items);
  * a CTA marches through; >= 4, clamped to the member's n2).  A batch starts
  * with the TMEM queue for binary32 precisions and the ring otherwise, and
  * min(n2, 32) planes per item.  Every schedule gives bitwise the same
- * results.  set_schedule (between steps; SBLI_EINVAL for z_queue outside 0..1
+ * results.  Members of the binary64-register precisions are split evenly over
+ * the CTAs whatever their planes per item.  set_schedule (between steps; SBLI_EINVAL for z_queue outside 0..1
  * or fewer than 4 planes) drops the captured step graphs; planes_per_item may
  * be NULL in both calls (keep, or do not return, the per-member values). */
 SBLI_API int sbli_batch_get_schedule(const sbli_batch* b, int* z_queue, int* planes_per_item);

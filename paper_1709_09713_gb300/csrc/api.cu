@@ -62,6 +62,9 @@ bool valid_sizes(int n0, int n1, int n2) {
 
 FusedConfig default_config(const Geom& g, int precision);
 
+// most CTAs (one per SM) the even split of a binary64-register grid may use
+constexpr int MAX_EVEN_CTAS = 512;
+
 // binary64 state, accumulator and stage registers (three-register rotation)
 bool f64_registers(int precision) { return precision == SBLI_FP64 || precision == SBLI_DF64; }
 
@@ -76,7 +79,7 @@ Layout layout_for(int n0, int n1, int n2, int precision, int variant) {
   // use (the smallest zc gives the most CTAs), or the KE kernel's blocks
   const long long tiles = (long long)((n0 + 31) / 32) * ((n1 + 3) / 4);
   const long long max_ctas = tiles * ((n2 + 3) / 4);
-  const long long np = std::max<long long>(max_ctas, ke_num_partials(g));
+  const long long np = std::max<long long>(std::max<long long>(max_ctas, ke_num_partials(g)), MAX_EVEN_CTAS);
   L.partials = align_up((size_t)(2 * np + 2) * sizeof(double));
   L.storeall = variant == SBLI_STORE_ALL
                    ? align_up(storeall_scratch_doubles(g, precision == SBLI_FP64 ? 8 : 4) * sizeof(double))
@@ -109,6 +112,8 @@ struct sbli_grid {
   int next_stage;  // 0, 1, 2
   long long stages_done;
   FusedConfig cfg;
+  int sms;      // SMs of the device
+  Split split;  // binary64-register grids: the work split of cfg
   Coef<double> cd;
   Coef<float> cf;
   Coef<dfloat> cw;
@@ -173,6 +178,11 @@ void rank_zc(const Geom& g, int precision, int ty, int* best, int nbest, int px 
   }
   for (int i = 0; i < nbest; ++i)
     if (best[i] == 0) best[i] = best[0] ? best[0] : std::min(4, g.n2);
+}
+
+void use_config(sbli_grid* g, const FusedConfig& cfg) {
+  g->cfg = cfg;
+  if (f64_registers(g->precision)) g->split = plan_split(g->geom, cfg.zc, g->sms, g->precision == SBLI_DF64);
 }
 
 FusedConfig default_config(const Geom& g, int precision) {
@@ -285,6 +295,8 @@ cudaError_t enqueue_stage(sbli_grid* g, int k, int state, double dt, double* ke_
     StageArgs a{};
     a.g = g->geom;
     a.zc = g->cfg.zc;
+    a.ctas = g->split.ctas;
+    a.even = g->split.even;
     a.q_in = p.q_in;
     a.acc_in = p.acc_in;
     a.acc_out = p.acc_out;
@@ -430,7 +442,10 @@ int sbli_create_grid(sbli_grid** out, int n0, int n1, int n2, int precision, int
   g->state = initial_state(precision);
   g->next_stage = 0;
   g->stages_done = 0;
-  g->cfg = default_config(g->geom, precision);
+  int dev = 0, sms = 152;
+  if (cudaGetDevice(&dev) == cudaSuccess) cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+  g->sms = std::min(sms, MAX_EVEN_CTAS);
+  use_config(g, default_config(g->geom, precision));
   g->cd = make_coef<double>(g->n, p);
   g->cf = make_coef<float>(g->n, p);
   g->cw = make_coef<dfloat>(g->n, p);
@@ -597,6 +612,8 @@ int sbli_rhs(sbli_grid* g, double* r_dev) {
     StageArgs a{};
     a.g = g->geom;
     a.zc = g->cfg.zc;
+    a.ctas = g->split.ctas;
+    a.even = g->split.even;
     a.q_in = q;
     a.r_out = r_dev;
     cudaError_t e = g->precision == SBLI_FP64      ? launch_fused_fp64(a, g->cd, g->cfg, true, g->stream)
@@ -664,7 +681,7 @@ int sbli_step_n_history(sbli_grid* g, int nsteps, double dt, double* ke_hist_dev
   if (!(dt > 0) || !isfinite(dt)) return fail(SBLI_EINVAL, "dt must be finite and > 0");
   if (g->next_stage != 0) return fail(SBLI_EINVAL, "step_n_history must start at a step boundary");
   if (g->variant != SBLI_FUSED) return fail(SBLI_EUNSUPPORTED, "history needs the fused variant");
-  const int nctas = fused_num_ctas(g->geom, g->cfg);
+  const int nctas = f64_registers(g->precision) ? g->split.ctas : fused_num_ctas(g->geom, g->cfg);
   for (int s = 0; s < nsteps; ++s) {
     SBLI_TRY(enqueue_stage(g, 0, g->state, dt, g->partials, g->stream), "stage launch");
     SBLI_TRY(launch_finalize_ke(g->partials, nctas, 1.0 / (double)g->geom.P, ke_hist_dev + 2 * s, g->stream),
@@ -727,7 +744,7 @@ int sbli_set_config(sbli_grid* g, int tile_y, int planes_per_cta, int z_queue, i
   cfg.zq = z_queue;
   cfg.px = columns_per_thread;
   if (cfg.ty != g->cfg.ty || cfg.zc != g->cfg.zc || cfg.zq != g->cfg.zq || cfg.px != g->cfg.px) {
-    g->cfg = cfg;
+    use_config(g, cfg);
     drop_graphs(g);
   }
   return SBLI_OK;
@@ -769,7 +786,7 @@ int sbli_autotune(sbli_grid* g, int reps, int* tile_y, int* planes_per_cta, int*
   float best_ms = 1e30f;
   cudaError_t err = cudaSuccess;
   for (int i = 0; i < nc && err == cudaSuccess; ++i) {
-    g->cfg = cand[i];
+    use_config(g, cand[i]);
     // stage 0 with dt = 0: the accumulator it writes equals the state it
     // reads (acc + 0 * R), so a double-float grid's state, updated in place,
     // keeps its value; the stage field goes to a free register
@@ -789,10 +806,10 @@ int sbli_autotune(sbli_grid* g, int reps, int* tile_y, int* planes_per_cta, int*
   cudaEventDestroy(e0);
   cudaEventDestroy(e1);
   if (err != cudaSuccess) {
-    g->cfg = saved;
+    use_config(g, saved);
     return cuda_fail(err, "autotune launch");
   }
-  g->cfg = cand[best];
+  use_config(g, cand[best]);
   if (g->cfg.ty != saved.ty || g->cfg.zc != saved.zc || g->cfg.zq != saved.zq || g->cfg.px != saved.px)
     drop_graphs(g);
   if (tile_y) *tile_y = g->cfg.ty;

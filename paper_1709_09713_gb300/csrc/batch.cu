@@ -33,36 +33,62 @@ __global__ void __launch_bounds__(TX* TY, fused_min_blocks<T, TY, ZT>())
   constexpr int NCOL2 = tmem_columns2<TY, T>();
   uint32_t tbase = 0, tbase2 = 0;
   if (ZT) tmem_acquire<NCOL, NCOL2>(sm.tmem_base, tbase, tbase2);
-  for (long long item = blockIdx.x; item < p.total_items; item += gridDim.x) {
-    // member owning this item (binary search over item_begin)
+  // member owning item or unit u (binary search over item_begin)
+  auto member_of = [&](long long u) {
     int lo = 0, hi = p.count - 1;
     while (lo < hi) {
       const int mid = (lo + hi + 1) >> 1;
-      if (p.item_begin[mid] <= item) lo = mid;
+      if (p.item_begin[mid] <= u) lo = mid;
       else hi = mid - 1;
     }
-    const StageArgs& a = p.a[lo];
-    const long long local = item - p.item_begin[lo];
-    const int ntile = p.tiles_x[lo] * p.tiles_y[lo];
-    const int chunk = (int)(local / ntile);
-    const int tile = (int)(local - (long long)chunk * ntile);
-    const int bx = tile % p.tiles_x[lo], by = tile / p.tiles_x[lo];
-    const int zbeg = chunk * a.zc;
+    return lo;
+  };
+  if constexpr (even_split<T>()) {
+    long long u = p.total_items * blockIdx.x / gridDim.x;
+    const long long end = p.total_items * (blockIdx.x + 1) / gridDim.x;
     double ke = 0.0, ens = 0.0;
-    fused_march<T, TIN, TOUT, TY, false, WITH_KE, DF, ZT>(a, p.c[lo], bx, by, zbeg, zbeg + a.zc, sm, ke, ens,
+    while (u < end) {
+      const int m = member_of(u);
+      const StageArgs& a = p.a[m];
+      const long long local = u - p.item_begin[m];
+      const int n2 = a.g.n2;
+      const int tile = (int)(local / n2), z = (int)(local - (long long)tile * n2);
+      const int len = (int)min((long long)(n2 - z), end - u);
+      fused_march<T, TIN, TOUT, TY, false, WITH_KE, DF, ZT>(a, p.c[m], tile % p.tiles_x[m], tile / p.tiles_x[m], z,
+                                                            z + len, sm, ke, ens, tbase, tbase2);
+      u += len;
+      // the CTA's part of this member ends: CTA + member numbers its partial sum
+      if (WITH_KE && (u == end || u == p.item_begin[m + 1])) {
+        block_reduce_pair<TX * TY>(sm.red, ke, ens, p.ke_items + 2 * ((long long)blockIdx.x + m));
+        ke = ens = 0.0;
+      }
+    }
+  } else {
+    for (long long item = blockIdx.x; item < p.total_items; item += gridDim.x) {
+      const int lo = member_of(item);
+      const StageArgs& a = p.a[lo];
+      const long long local = item - p.item_begin[lo];
+      const int ntile = p.tiles_x[lo] * p.tiles_y[lo];
+      const int chunk = (int)(local / ntile);
+      const int tile = (int)(local - (long long)chunk * ntile);
+      const int bx = tile % p.tiles_x[lo], by = tile / p.tiles_x[lo];
+      const int zbeg = chunk * a.zc;
+      double ke = 0.0, ens = 0.0;
+      fused_march<T, TIN, TOUT, TY, false, WITH_KE, DF, ZT>(a, p.c[lo], bx, by, zbeg, zbeg + a.zc, sm, ke, ens,
                                                             tbase, tbase2);
-    if (WITH_KE) block_reduce_pair<TX * TY>(sm.red, ke, ens, p.ke_items + 2 * item);
+      if (WITH_KE) block_reduce_pair<TX * TY>(sm.red, ke, ens, p.ke_items + 2 * item);
+    }
   }
   if (ZT) tmem_release<NCOL, NCOL2>(tbase, tbase2);
 }
 
-// Per member: fixed-order sum of its items' partials, scaled by 1/P.
+// Per member: fixed-order sum of its partials, scaled by 1/P.
 __global__ void __launch_bounds__(256) batch_ke_finalize(const double* __restrict__ items,
-                                                         const long long* __restrict__ begin,
+                                                         const long long* __restrict__ range,
                                                          const double* __restrict__ inv_p, double* __restrict__ out) {
   const int m = blockIdx.x;
   double a = 0.0, b = 0.0;
-  for (long long i = begin[m] + threadIdx.x; i < begin[m + 1]; i += 256) {
+  for (long long i = range[2 * m] + threadIdx.x; i < range[2 * m + 1]; i += 256) {
     a += items[2 * i];
     b += items[2 * i + 1];
   }
@@ -82,6 +108,7 @@ static cudaError_t launch_batch_k(const BatchParams<T>& p, int grid, cudaStream_
   const size_t smem = sizeof(FusedSmem<T, 8, ZT>);
   static std::atomic<unsigned long long> done{0};
   if (cudaError_t e = ensure_smem_limit(k, smem, done)) return e;
+  if (even_split<T>()) grid = (int)std::min<long long>(grid, p.total_items);
   k<<<grid, TX * 8, smem, s>>>(p);
   return cudaGetLastError();
 }
@@ -117,9 +144,9 @@ cudaError_t launch_batch_t<double>(const BatchParams<double>& p, bool, int grid,
   return launch_batch_zq<double, double, double, false>(p, grid, s, zq);
 }
 
-cudaError_t launch_batch_ke_finalize(const double* items, const long long* begin, const double* inv_p, double* out,
+cudaError_t launch_batch_ke_finalize(const double* items, const long long* range, const double* inv_p, double* out,
                                      int count, cudaStream_t s) {
-  batch_ke_finalize<<<count, 256, 0, s>>>(items, begin, inv_p, out);
+  batch_ke_finalize<<<count, 256, 0, s>>>(items, range, inv_p, out);
   return cudaGetLastError();
 }
 
@@ -191,12 +218,13 @@ BatchLayout batch_layout(int count, const int* n, int precision) {
   L.reg32 = batch_f64_registers(precision) ? 0 : o32;
   L.n64 = batch_f64_registers(precision) ? 3 : 2;
   L.n32 = batch_f64_registers(precision) ? 0 : 2;
-  L.items_bytes = balign((size_t)(2 * L.total_items + 2) * sizeof(double));
+  // partials: one per work item, or (even split) one per CTA and member
+  L.items_bytes = balign((size_t)(2 * std::max<long long>(L.total_items, BATCH_MAX_EVEN_CTAS + count) + 2) * sizeof(double));
   L.total_items = 0;
   for (const MemberLayout& M : L.m) L.total_items += member_items(M.n, M.zc);
-  // per member: KE result pair, 1/P, item begin; plus the KE kernel partials
+  // per member: KE result pair, 1/P, range of partials; plus the KE kernel partials
   L.misc_bytes = balign((size_t)count * 2 * sizeof(double)) + balign((size_t)count * sizeof(double)) +
-                 balign((size_t)(count + 1) * sizeof(long long)) + balign(2 * 1024 * sizeof(double));
+                 balign((size_t)(2 * count) * sizeof(long long)) + balign(2 * 1024 * sizeof(double));
   L.total = L.reg64 * L.n64 + L.reg32 * L.n32 + L.items_bytes + L.misc_bytes;
   return L;
 }
@@ -213,7 +241,7 @@ struct sbli_batch {
   double* ke_items;
   double* ke_out;     // count pairs
   double* inv_p;      // count
-  long long* begin;   // count + 1 (device copy of item_begin)
+  long long* range;   // 2 count: first and past-the-last partial sum of each member
   double* ke_scratch; // partials of the single-member KE kernel
   int state;
   long long steps_done;
@@ -311,7 +339,7 @@ cudaError_t enqueue_batch_stage_t(sbli_batch* b, int k, int state, double dt, do
     p.item_begin[m] = acc;
     p.tiles_x[m] = (M.n[0] + TX - 1) / TX;
     p.tiles_y[m] = (M.n[1] + 7) / 8;
-    acc += member_items(M.n, M.zc);
+    acc += batch_f64_registers(b->precision) ? member_planes(M.n) : member_items(M.n, M.zc);
     p.a[m] = member_stage(b, m, k, state, dt, &in64);
     p.c[m] = make_coef<T>(M.n, b->params[m]);
   }
@@ -362,20 +390,37 @@ int batch_build_graph(sbli_batch* b, int state, double dt) {
   return SBLI_OK;
 }
 
-// Item ranges of the members under the current schedule, for the KE
+// Ranges of the members' partial sums under the current schedule, for the KE
 // finalisation (device copy, written on the batch's stream).
-cudaError_t upload_item_begin(sbli_batch* b) {
-  std::vector<long long> beg(b->count + 1);
-  long long acc = 0;
+cudaError_t upload_ranges(sbli_batch* b) {
+  std::vector<long long> range(2 * b->count);
+  long long items = 0, units = 0;
+  for (const MemberLayout& M : b->L.m) units += member_planes(M.n);
+  const long long ctas = std::min<long long>(b->grid_ctas, units);
+  // the CTA whose run [units c / ctas, units (c + 1) / ctas) holds unit u
+  auto cta_of = [&](long long u) {
+    long long c = u * ctas / units;
+    while (units * (c + 1) / ctas <= u) ++c;
+    while (units * c / ctas > u) --c;
+    return c;
+  };
+  long long at = 0;
   for (int m = 0; m < b->count; ++m) {
-    beg[m] = acc;
-    acc += member_items(b->L.m[m].n, b->L.m[m].zc);
+    const MemberLayout& M = b->L.m[m];
+    if (batch_f64_registers(b->precision)) {
+      range[2 * m] = cta_of(at) + m;
+      at += member_planes(M.n);
+      range[2 * m + 1] = cta_of(at - 1) + m + 1;
+    } else {
+      range[2 * m] = items;
+      range[2 * m + 1] = items + member_items(M.n, M.zc);
+    }
+    items += member_items(M.n, M.zc);
   }
-  beg[b->count] = acc;
-  b->L.total_items = acc;
-  cudaError_t e = cudaMemcpyAsync(b->begin, beg.data(), (b->count + 1) * sizeof(long long), cudaMemcpyHostToDevice,
+  b->L.total_items = items;
+  cudaError_t e = cudaMemcpyAsync(b->range, range.data(), range.size() * sizeof(long long), cudaMemcpyHostToDevice,
                                   b->stream);
-  if (e == cudaSuccess) e = cudaStreamSynchronize(b->stream);  // beg is a host temporary
+  if (e == cudaSuccess) e = cudaStreamSynchronize(b->stream);  // range is a host temporary
   return e;
 }
 
@@ -385,10 +430,10 @@ cudaError_t apply_schedule(sbli_batch* b, int zq, const std::vector<int>& zc) {
   int dev = 0, sms = 152;
   if (cudaGetDevice(&dev) == cudaSuccess) cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
   b->zq = zq;
-  b->grid_ctas = sms * batch_ctas_per_sm(b->precision, zq);
+  b->grid_ctas = batch_grid_ctas(sms, b->precision, zq);
   for (int m = 0; m < b->count; ++m) b->L.m[m].zc = zc[m];
   batch_drop_graphs(b);
-  return upload_item_begin(b);
+  return upload_ranges(b);
 }
 
 int check_batch(const sbli_batch* b, int member) {
@@ -451,8 +496,8 @@ int sbli_batch_create(sbli_batch** out, int count, const int* n, const sbli_para
   w += balign((size_t)count * 2 * sizeof(double));
   b->inv_p = reinterpret_cast<double*>(w);
   w += balign((size_t)count * sizeof(double));
-  b->begin = reinterpret_cast<long long*>(w);
-  w += balign((size_t)(count + 1) * sizeof(long long));
+  b->range = reinterpret_cast<long long*>(w);
+  w += balign((size_t)(2 * count) * sizeof(long long));
   b->ke_scratch = reinterpret_cast<double*>(w);
   b->state = batch_initial_state(b->precision);
   b->steps_done = 0;
@@ -460,13 +505,13 @@ int sbli_batch_create(sbli_batch** out, int count, const int* n, const sbli_para
   cudaGetDevice(&dev);
   cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
   b->zq = batch_default_zq(precision);
-  b->grid_ctas = sms * batch_ctas_per_sm(precision, b->zq);
+  b->grid_ctas = batch_grid_ctas(sms, precision, b->zq);
   // per-member constants for the KE finalisation
   std::vector<double> inv(count);
   for (int m = 0; m < count; ++m) inv[m] = 1.0 / (double)b->L.m[m].P;
   cudaError_t e = cudaStreamCreateWithFlags(&b->cap_stream, cudaStreamNonBlocking);
   if (e == cudaSuccess) e = cudaMemcpyAsync(b->inv_p, inv.data(), count * sizeof(double), cudaMemcpyHostToDevice, b->stream);
-  if (e == cudaSuccess) e = upload_item_begin(b);
+  if (e == cudaSuccess) e = upload_ranges(b);
   if (e == cudaSuccess) e = cudaStreamSynchronize(b->stream);
   if (e != cudaSuccess) {
     delete b;
@@ -593,7 +638,7 @@ int sbli_batch_step_n_history(sbli_batch* b, int nsteps, double dt, double* ke_h
   if (!(dt > 0) || !isfinite(dt)) return bfail(SBLI_EINVAL, "dt must be finite and > 0");
   for (int s = 0; s < nsteps; ++s) {
     SBLI_BTRY(enqueue_batch_stage(b, 0, b->state, dt, b->ke_items, b->stream), "batch stage");
-    SBLI_BTRY(launch_batch_ke_finalize(b->ke_items, b->begin, b->inv_p, ke_hist_dev + (size_t)2 * b->count * s,
+    SBLI_BTRY(launch_batch_ke_finalize(b->ke_items, b->range, b->inv_p, ke_hist_dev + (size_t)2 * b->count * s,
                                        b->count, b->stream),
               "ke finalize");
     for (int k = 1; k < 3; ++k) SBLI_BTRY(enqueue_batch_stage(b, k, b->state, dt, nullptr, b->stream), "batch stage");

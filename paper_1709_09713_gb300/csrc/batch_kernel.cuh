@@ -11,13 +11,15 @@ constexpr int BATCH_MAX_MEMBERS = 64;  // members per launch (parameter space bo
 template <typename T>
 struct BatchParams {
   int count;                                  // members in this launch
+  // binary32 members: work items (z chunk x tile); binary64-register members:
+  // planes of tiles, split evenly over the CTAs
   long long total_items;                      // sum of the members' items
   long long item_begin[BATCH_MAX_MEMBERS + 1];
   int tiles_x[BATCH_MAX_MEMBERS];
   int tiles_y[BATCH_MAX_MEMBERS];
   StageArgs a[BATCH_MAX_MEMBERS];             // geometry, zc, stage pointers, a_k dt, b_k dt
   Coef<T> c[BATCH_MAX_MEMBERS];
-  double* ke_items;                           // per-item (ke, ens) partials, or nullptr
+  double* ke_items;                           // (ke, ens) partials per item (even split: CTA + member), or nullptr
 };
 
 // One persistent launch of stage work for p.count members (grid = CTAs).
@@ -43,6 +45,15 @@ inline int batch_ctas_per_sm(int precision, int zq) {
   return 1;
 }
 
+// CTAs of a launch: persistent ones that fill the SMs.  The even split keeps
+// a partial sum per CTA and member, which bounds them.
+constexpr int BATCH_MAX_EVEN_CTAS = 512;
+inline int batch_grid_ctas(int sms, int precision, int zq) {
+  const int ctas = sms * batch_ctas_per_sm(precision, zq);
+  const bool even = precision == SBLI_FP64 || precision == SBLI_DF64;
+  return even && ctas > BATCH_MAX_EVEN_CTAS ? BATCH_MAX_EVEN_CTAS : ctas;
+}
+
 // Work items (z chunk of zc planes x 32 x 8 tile) of one member; batch_zc is
 // the planes per item a member starts with.
 inline int batch_zc(int n2) { return n2 < 32 ? n2 : 32; }
@@ -50,9 +61,11 @@ inline long long member_items(const int n[3], int zc) {
   return (long long)((n[0] + 31) / 32) * ((n[1] + 7) / 8) * ((n[2] + zc - 1) / zc);
 }
 inline long long member_items(const int n[3]) { return member_items(n, batch_zc(n[2])); }
+// Planes of all tiles of one member: the units of the even split.
+inline long long member_planes(const int n[3]) { return member_items(n, 1); }
 
-// Per member m: fixed-order sum of item partials [begin[m], begin[m+1]) times inv_p[m].
-cudaError_t launch_batch_ke_finalize(const double* items, const long long* begin, const double* inv_p, double* out,
+// Per member m: fixed-order sum of partials [range[2m], range[2m+1]) times inv_p[m].
+cudaError_t launch_batch_ke_finalize(const double* items, const long long* range, const double* inv_p, double* out,
                                      int count, cudaStream_t s);
 
 }  // namespace sbli

@@ -1381,9 +1381,22 @@ __device__ __forceinline__ void block_reduce_pair(double (&red)[2][32], double k
   __syncthreads();
 }
 
-// Single grid: one CTA per (tile, z chunk).  ZT: x2-neighbour records in TMEM.
-template <typename T, typename TIN, typename TOUT, int TY, bool RHS_ONLY, bool WITH_KE, bool DF = false,
-          bool ZT = false>
+// How the work is split over CTAs.  Chunks: one CTA a (tile, z chunk).  Even
+// split: every CTA takes a contiguous run of the planes of all tiles, numbered
+// tile by tile (a run that crosses into the next tile starts a new march
+// there), one CTA per SM, so that no SM idles in a last wave and a grid with
+// fewer chunks than SMs still fills them.  The binary64-register kernels (one
+// CTA per SM, bound by arithmetic) choose by the longest CTA (plan_split); the
+// binary32 kernels, bound by memory and its latency, keep the chunks:
+// concurrent CTAs then march through the same planes and share their halos in
+// L2.
+template <typename T>
+constexpr bool even_split() {
+  return is_f64_class<T>();
+}
+
+// Single grid.  ZT: x2-neighbour records in TMEM.
+template <typename T, typename TIN, typename TOUT, int TY, bool RHS_ONLY, bool WITH_KE, bool DF, bool ZT, bool EVEN>
 __global__ void __launch_bounds__(TX* TY, fused_min_blocks<T, TY, ZT>())
     fused_stage_kernel(const StageArgs a, const Coef<T> c) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
@@ -1393,9 +1406,23 @@ __global__ void __launch_bounds__(TX* TY, fused_min_blocks<T, TY, ZT>())
   uint32_t tbase = 0, tbase2 = 0;
   if (ZT) tmem_acquire<NCOL, NCOL2>(sm.tmem_base, tbase, tbase2);
   double ke = 0.0, ens = 0.0;
-  const int zbeg = blockIdx.z * a.zc;
-  fused_march<T, TIN, TOUT, TY, RHS_ONLY, WITH_KE, DF, ZT>(a, c, blockIdx.x, blockIdx.y, zbeg, zbeg + a.zc, sm, ke,
-                                                          ens, tbase, tbase2);
+  if constexpr (EVEN) {
+    const int tiles_x = (a.g.n0 + tile_width<T>() - 1) / tile_width<T>(), tiles_y = (a.g.n1 + TY - 1) / TY;
+    const long long units = (long long)tiles_x * tiles_y * a.g.n2;
+    long long u = units * blockIdx.x / gridDim.x;
+    const long long end = units * (blockIdx.x + 1) / gridDim.x;
+    while (u < end) {
+      const int tile = (int)(u / a.g.n2), z = (int)(u - (long long)tile * a.g.n2);
+      const int len = (int)min((long long)(a.g.n2 - z), end - u);
+      fused_march<T, TIN, TOUT, TY, RHS_ONLY, WITH_KE, DF, ZT>(a, c, tile % tiles_x, tile / tiles_x, z, z + len, sm,
+                                                              ke, ens, tbase, tbase2);
+      u += len;
+    }
+  } else {
+    const int zbeg = blockIdx.z * a.zc;
+    fused_march<T, TIN, TOUT, TY, RHS_ONLY, WITH_KE, DF, ZT>(a, c, blockIdx.x, blockIdx.y, zbeg, zbeg + a.zc, sm, ke,
+                                                            ens, tbase, tbase2);
+  }
   if (WITH_KE) {
     const long long b = blockIdx.x + (long long)gridDim.x * (blockIdx.y + (long long)gridDim.y * blockIdx.z);
     block_reduce_pair<TX * TY>(sm.red, ke, ens, a.ke_partials + 2 * b);
@@ -1423,15 +1450,24 @@ cudaError_t ensure_smem_limit(K kernel, size_t bytes, std::atomic<unsigned long 
   return e;
 }
 
-template <typename T, typename TIN, typename TOUT, int TY, bool RHS_ONLY, bool WITH_KE, bool DF = false,
-          bool ZT = false>
-cudaError_t launch_fused_t(const StageArgs& a, const Coef<T>& c, cudaStream_t s) {
-  auto k = fused_stage_kernel<T, TIN, TOUT, TY, RHS_ONLY, WITH_KE, DF, ZT>;
+template <typename T, typename TIN, typename TOUT, int TY, bool RHS_ONLY, bool WITH_KE, bool DF, bool ZT, bool EVEN>
+cudaError_t launch_fused_k(const StageArgs& a, const Coef<T>& c, cudaStream_t s) {
+  auto k = fused_stage_kernel<T, TIN, TOUT, TY, RHS_ONLY, WITH_KE, DF, ZT, EVEN>;
   const size_t smem = sizeof(FusedSmem<T, TY, ZT>);
   static std::atomic<unsigned long long> done{0};  // devices this instantiation is configured on
   if (cudaError_t e = ensure_smem_limit(k, smem, done)) return e;
-  k<<<fused_grid<TY, tile_width<T>()>(a.g, a.zc), TX * TY, smem, s>>>(a, c);
+  const dim3 grid = EVEN ? dim3(a.ctas) : fused_grid<TY, tile_width<T>()>(a.g, a.zc);
+  k<<<grid, TX * TY, smem, s>>>(a, c);
   return cudaGetLastError();
+}
+
+template <typename T, typename TIN, typename TOUT, int TY, bool RHS_ONLY, bool WITH_KE, bool DF = false,
+          bool ZT = false>
+cudaError_t launch_fused_t(const StageArgs& a, const Coef<T>& c, cudaStream_t s) {
+  if constexpr (even_split<T>()) {
+    if (a.even) return launch_fused_k<T, TIN, TOUT, TY, RHS_ONLY, WITH_KE, DF, ZT, true>(a, c, s);
+  }
+  return launch_fused_k<T, TIN, TOUT, TY, RHS_ONLY, WITH_KE, DF, ZT, false>(a, c, s);
 }
 
 }  // namespace sbli

@@ -65,6 +65,7 @@ struct Geom {
 struct StageArgs {
   Geom g;
   int zc;                  // planes per CTA along x2
+  int ctas;                // CTAs of the even split
   const void* q_in;        // stage input (stencil reads)
   const double* acc_in;    // accumulator in (binary64; on stage 0 the state itself)
   double* acc_out;         // accumulator out (binary64), may alias acc_in
@@ -79,6 +80,7 @@ struct StageArgs {
   const float* dacc_in;
   float* dacc_out;
   int df_normalize;  // double-float accumulator: renormalise (hi, lo) in this stage (the last of a step)
+  int even;          // binary64-register kernels: the CTAs split the planes evenly (else chunks of zc)
 };
 
 // Launch configuration chosen for one grid (the autotuner's output).
@@ -114,6 +116,11 @@ cudaError_t launch_fused_fp32_pair(const StageArgs& a, const Coef<float>& c, con
 cudaError_t launch_fused_fp32_tmem(const StageArgs& a, const Coef<float>& c, const FusedConfig& cfg, bool in_fp64,
                                    bool df, bool rhs_only, cudaStream_t s);
 int fused_num_ctas(const Geom& g, const FusedConfig& cfg);
+// CTAs of a binary64-register stage and whether they split the planes evenly (else chunks of zc planes)
+struct Split {
+  int ctas, even;
+};
+Split plan_split(const Geom& g, int zc, int sms, bool double_float);
 
 // Diagnostics and state conversion (diag.cu).
 cudaError_t launch_init_tgv(const Geom& g, const sbli_params& p, double amplitude, double* q, cudaStream_t s);

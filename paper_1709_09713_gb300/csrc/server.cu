@@ -246,7 +246,7 @@ cudaError_t launch_group(sbli_server* s, int k, int precision, const std::vector
       p.item_begin[m] = acc;
       p.tiles_x[m] = (n[0] + 31) / 32;
       p.tiles_y[m] = (n[1] + 7) / 8;
-      acc += member_items(n);
+      acc += req_f64_registers(precision) ? member_planes(n) : member_items(n);
       p.a[m] = req_stage(s, q, k, &in64);
       p.c[m] = make_coef<T>(n, q.r.params);
     }
@@ -371,8 +371,8 @@ int sbli_server_create(sbli_server** out, void* arena, size_t arena_bytes, int m
   int dev = 0, sms = 152;
   cudaGetDevice(&dev);
   cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-  s->grid64 = sms * batch_ctas_per_sm(SBLI_FP64, batch_default_zq(SBLI_FP64));
-  s->grid32 = sms * batch_ctas_per_sm(SBLI_FP32, batch_default_zq(SBLI_FP32));
+  s->grid64 = batch_grid_ctas(sms, SBLI_FP64, batch_default_zq(SBLI_FP64));
+  s->grid32 = batch_grid_ctas(sms, SBLI_FP32, batch_default_zq(SBLI_FP32));
   s->lane[0].st = s->s64;
   s->lane[1].st = s->s32;
   for (Lane& l : s->lane) {
@@ -496,12 +496,18 @@ int sbli_server_tick(sbli_server* s, int* completed) {
       int K = 1;
       if (L.ms_per_step > 0) K = (int)std::max(1.0, std::floor(LANE_BATCH_MS / L.ms_per_step));
       K = std::min(K, kmin);
+      // the even split of a binary64-register stage ends on every SM at once,
+      // so binary32 requests would wait a whole stage for each of theirs:
+      // while there are any, an eighth of the SMs is left to them
+      bool other = false;
+      for (const Req& q : s->active) other |= lane_of(q.r.precision) != li && q.remaining > 0;
+      const int grid64 = other ? s->grid64 - s->grid64 / 8 : s->grid64;
       SBLI_STRY(cudaEventRecord(L.ev0, L.st), "cudaEventRecord");
       for (int step = 0; step < K; ++step) {
         for (int k = 0; k < 3; ++k) {
-          if (has[SBLI_FP64]) SBLI_STRY(launch_group<double>(s, k, SBLI_FP64, run, L.st, s->grid64), "fp64 stage");
+          if (has[SBLI_FP64]) SBLI_STRY(launch_group<double>(s, k, SBLI_FP64, run, L.st, grid64), "fp64 stage");
           if (has[SBLI_DF64])
-            SBLI_STRY(launch_group<dfloat>(s, k, SBLI_DF64, run, L.st, s->grid64), "double-float stage");
+            SBLI_STRY(launch_group<dfloat>(s, k, SBLI_DF64, run, L.st, grid64), "double-float stage");
           if (has[SBLI_FP32]) SBLI_STRY(launch_group<float>(s, k, SBLI_FP32, run, L.st, s->grid32), "fp32 stage");
           if (has[SBLI_FP32_DF])
             SBLI_STRY(launch_group<float>(s, k, SBLI_FP32_DF, run, L.st, s->grid32), "fp32 double-float stage");
