@@ -495,25 +495,22 @@ int sbli_set_state(sbli_grid* g, const double* q, int q_is_host) {
   if (int rc = check_grid(g)) return rc;
   if (!q) return fail(SBLI_EINVAL, "q is null");
   if (g->next_stage != 0) return fail(SBLI_EINVAL, "set_state between stages of a step (next stage %d)", g->next_stage);
-  const size_t bytes = 5 * (size_t)g->geom.P * sizeof(double);
-  // stage through a free register, then convert to deviation form
-  const int dst = g->state;
-  double* tmp = free64(g);
-  if (q_is_host) {
-    SBLI_TRY(cudaMemcpyAsync(tmp, q, bytes, cudaMemcpyHostToDevice, g->stream), "cudaMemcpyAsync H2D");
-  } else {
-    SBLI_TRY(cudaMemcpyAsync(tmp, q, bytes, cudaMemcpyDeviceToDevice, g->stream), "cudaMemcpyAsync D2D");
+  const double* src = q;
+  if (q_is_host || !direct_device_access(q)) {  // stage through a free register
+    double* tmp = free64(g);
+    SBLI_TRY(cudaMemcpyAsync(tmp, q, 5 * (size_t)g->geom.P * sizeof(double),
+                             q_is_host ? cudaMemcpyHostToDevice : cudaMemcpyDeviceToDevice, g->stream),
+             "cudaMemcpyAsync of the state");
+    src = tmp;
   }
-  if (g->precision == SBLI_FP32_DF) {
-    SBLI_TRY(launch_df_split(g->geom.P, g->ref, tmp, reinterpret_cast<float*>(g->reg64[dst]), g->stream), "df_split");
-  } else {
-    SBLI_TRY(launch_to_offset(g->geom, g->ref, tmp, state64(g), g->stream), "to_offset launch");
-    if (g->precision == SBLI_FP32)
-      SBLI_TRY(launch_narrow(5 * g->geom.P, g->reg64[dst], g->reg32[dst], g->stream), "narrow launch");
-    if (g->precision == SBLI_DF64)
-      SBLI_TRY(launch_pair_split(5 * g->geom.P, state64(g), reinterpret_cast<float*>(g->reg64[dst]), g->stream),
-               "pair_split launch");
-  }
+  StateForm to{};
+  if (g->precision == SBLI_FP32_DF)
+    to.df = reinterpret_cast<float*>(g->reg64[g->state]);
+  else
+    to.f64 = state64(g);
+  if (g->precision == SBLI_FP32) to.copy32 = g->reg32[g->state];
+  if (g->precision == SBLI_DF64) to.pairs = reinterpret_cast<float*>(g->reg64[g->state]);
+  SBLI_TRY(launch_import_state(g->geom.P, g->ref, src, to, g->stream), "import_state launch");
   if (q_is_host) SBLI_TRY(cudaStreamSynchronize(g->stream), "cudaStreamSynchronize");
   g->stages_done = 0;
   return SBLI_OK;
@@ -523,19 +520,19 @@ int sbli_get_state(sbli_grid* g, double* q, int q_is_host) {
   if (int rc = check_grid(g)) return rc;
   if (!q) return fail(SBLI_EINVAL, "q is null");
   if (g->next_stage != 0) return fail(SBLI_EINVAL, "get_state between stages of a step (next stage %d)", g->next_stage);
-  const size_t bytes = 5 * (size_t)g->geom.P * sizeof(double);
-  double* tmp = free64(g);
+  const bool staged = q_is_host || !direct_device_access(q);
+  double* dst = staged ? free64(g) : q;
   if (g->precision == SBLI_FP32_DF) {
-    SBLI_TRY(launch_df_join(g->geom.P, g->ref, reinterpret_cast<const float*>(g->reg64[g->state]), tmp, g->stream),
+    SBLI_TRY(launch_df_join(g->geom.P, g->ref, reinterpret_cast<const float*>(g->reg64[g->state]), dst, g->stream),
              "df_join");
   } else {
-    SBLI_TRY(launch_from_offset(g->geom, g->ref, state64(g), tmp, g->stream), "from_offset launch");
+    SBLI_TRY(launch_from_offset(g->geom, g->ref, state64(g), dst, g->stream), "from_offset launch");
   }
-  if (q_is_host) {
-    SBLI_TRY(cudaMemcpyAsync(q, tmp, bytes, cudaMemcpyDeviceToHost, g->stream), "cudaMemcpyAsync D2H");
-    SBLI_TRY(cudaStreamSynchronize(g->stream), "cudaStreamSynchronize");
-  } else {
-    SBLI_TRY(cudaMemcpyAsync(q, tmp, bytes, cudaMemcpyDeviceToDevice, g->stream), "cudaMemcpyAsync D2D");
+  if (staged) {
+    SBLI_TRY(cudaMemcpyAsync(q, dst, 5 * (size_t)g->geom.P * sizeof(double),
+                             q_is_host ? cudaMemcpyDeviceToHost : cudaMemcpyDeviceToDevice, g->stream),
+             "cudaMemcpyAsync of the state");
+    if (q_is_host) SBLI_TRY(cudaStreamSynchronize(g->stream), "cudaStreamSynchronize");
   }
   return SBLI_OK;
 }

@@ -572,23 +572,23 @@ int sbli_batch_set_state(sbli_batch* b, int member, const double* q, int q_is_ho
   if (int rc = check_batch(b, member)) return rc;
   if (!q) return bfail(SBLI_EINVAL, "q is null");
   const MemberLayout& M = b->L.m[member];
-  double* dst = reinterpret_cast<double*>(b->reg64[state_reg(b)] + M.off64);
-  double* tmp = reinterpret_cast<double*>(b->reg64[free_reg(b)] + M.off64);
-  SBLI_BTRY(cudaMemcpyAsync(tmp, q, 5 * M.P * sizeof(double), q_is_host ? cudaMemcpyHostToDevice : cudaMemcpyDeviceToDevice,
-                            b->stream),
-            "cudaMemcpyAsync");
-  if (b->precision == SBLI_FP32_DF) {
-    SBLI_BTRY(launch_df_split(M.P, make_ref(b->params[member]), tmp, reinterpret_cast<float*>(dst), b->stream),
-              "df_split");
-  } else {
-    SBLI_BTRY(launch_to_offset(member_geom(M), make_ref(b->params[member]), tmp, dst, b->stream), "to_offset");
-    if (b->precision == SBLI_DF64)
-      SBLI_BTRY(launch_pair_split(5 * M.P, dst, reinterpret_cast<float*>(b->reg64[b->state] + M.off64), b->stream),
-                "pair_split");
-    if (b->precision == SBLI_FP32)
-      SBLI_BTRY(launch_narrow(5 * M.P, dst, reinterpret_cast<float*>(b->reg32[b->state] + M.off32), b->stream),
-                "narrow");
+  const double* src = q;
+  if (q_is_host || !direct_device_access(q)) {  // stage through a free register
+    double* tmp = reinterpret_cast<double*>(b->reg64[free_reg(b)] + M.off64);
+    SBLI_BTRY(cudaMemcpyAsync(tmp, q, 5 * M.P * sizeof(double),
+                              q_is_host ? cudaMemcpyHostToDevice : cudaMemcpyDeviceToDevice, b->stream),
+              "cudaMemcpyAsync");
+    src = tmp;
   }
+  double* dst = reinterpret_cast<double*>(b->reg64[state_reg(b)] + M.off64);
+  StateForm to{};
+  if (b->precision == SBLI_FP32_DF)
+    to.df = reinterpret_cast<float*>(dst);
+  else
+    to.f64 = dst;
+  if (b->precision == SBLI_FP32) to.copy32 = reinterpret_cast<float*>(b->reg32[b->state] + M.off32);
+  if (b->precision == SBLI_DF64) to.pairs = reinterpret_cast<float*>(b->reg64[b->state] + M.off64);
+  SBLI_BTRY(launch_import_state(M.P, make_ref(b->params[member]), src, to, b->stream), "import_state");
   if (q_is_host) SBLI_BTRY(cudaStreamSynchronize(b->stream), "cudaStreamSynchronize");
   return SBLI_OK;
 }
@@ -598,16 +598,18 @@ int sbli_batch_get_state(sbli_batch* b, int member, double* q, int q_is_host) {
   if (!q) return bfail(SBLI_EINVAL, "q is null");
   const MemberLayout& M = b->L.m[member];
   const double* src = reinterpret_cast<double*>(b->reg64[state_reg(b)] + M.off64);
-  double* tmp = reinterpret_cast<double*>(b->reg64[free_reg(b)] + M.off64);
+  const bool staged = q_is_host || !direct_device_access(q);
+  double* dst = staged ? reinterpret_cast<double*>(b->reg64[free_reg(b)] + M.off64) : q;
   if (b->precision == SBLI_FP32_DF) {
-    SBLI_BTRY(launch_df_join(M.P, make_ref(b->params[member]), reinterpret_cast<const float*>(src), tmp, b->stream),
+    SBLI_BTRY(launch_df_join(M.P, make_ref(b->params[member]), reinterpret_cast<const float*>(src), dst, b->stream),
               "df_join");
   } else {
-    SBLI_BTRY(launch_from_offset(member_geom(M), make_ref(b->params[member]), src, tmp, b->stream), "from_offset");
+    SBLI_BTRY(launch_from_offset(member_geom(M), make_ref(b->params[member]), src, dst, b->stream), "from_offset");
   }
-  SBLI_BTRY(cudaMemcpyAsync(q, tmp, 5 * M.P * sizeof(double), q_is_host ? cudaMemcpyDeviceToHost : cudaMemcpyDeviceToDevice,
-                            b->stream),
-            "cudaMemcpyAsync");
+  if (staged)
+    SBLI_BTRY(cudaMemcpyAsync(q, dst, 5 * M.P * sizeof(double),
+                              q_is_host ? cudaMemcpyDeviceToHost : cudaMemcpyDeviceToDevice, b->stream),
+              "cudaMemcpyAsync");
   if (q_is_host) SBLI_BTRY(cudaStreamSynchronize(b->stream), "cudaStreamSynchronize");
   return SBLI_OK;
 }

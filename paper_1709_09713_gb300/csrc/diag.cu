@@ -3,6 +3,7 @@
 #include <math.h>
 
 #include "fpconv.cuh"
+#include "ke_march.cuh"
 #include "sbli_internal.cuh"
 
 namespace sbli {
@@ -55,29 +56,41 @@ RefState make_ref(const sbli_params& p) {
 // §4, Eqs. 9-12 with amplitude A; T = 1 so rho = gamma M^2 p (Eq. 5), rho E
 // from Eq. 4.  Written as deviations from the reference state:
 //   rho - 1 = gamma M^2 (p - p_ref),  rho E - E_ref = (p - p_ref)/(gamma-1) + rho |u|^2/2.
-__global__ void init_tgv_kernel(Geom g, double h0, double h1, double h2, double L, double A, double gM2,
-                                double inv_gm1, double* __restrict__ q) {
-  const long long P = g.P;
-  for (long long n = blockIdx.x * (long long)blockDim.x + threadIdx.x; n < P; n += (long long)gridDim.x * blockDim.x) {
-    const int i = (int)(n % g.n0);
-    const int j = (int)((n / g.n0) % g.n1);
-    const int k = (int)(n / ((long long)g.n0 * g.n1));
-    const double x = i * h0, y = j * h1, z = k * h2;
-    double sx, cx, sy, cy, sz, cz;
+// The field is made of functions of one coordinate each, so a thread evaluates
+// those of its column once for INIT_Z planes and a block those of x2 once for
+// its planes: the binary64 pipe, which bounds this kernel, spends itself on
+// the products and not on six trigonometric functions a point.
+constexpr int INIT_Z = 32;
+__global__ void __launch_bounds__(256) init_tgv_kernel(Geom g, double h0, double h1, double h2, double L, double A,
+                                                       double gM2, double inv_gm1, double* __restrict__ q) {
+  __shared__ double cz[INIT_Z], c2z[INIT_Z];
+  const int z0 = blockIdx.z * INIT_Z, nz = min(INIT_Z, g.n2 - z0);
+  if ((int)threadIdx.x < nz) {
+    const double z = (z0 + (int)threadIdx.x) * h2;
+    cz[threadIdx.x] = cos(z / L);
+    c2z[threadIdx.x] = cos(2.0 * z / L);
+  }
+  __syncthreads();
+  const long long P = g.P, plane = (long long)g.n0 * g.n1;
+  for (long long n = blockIdx.x * 256LL + threadIdx.x; n < plane; n += gridDim.x * 256LL) {
+    const double x = (int)(n % g.n0) * h0, y = (int)(n / g.n0) * h1;
+    double sx, cx, sy, cy;
     sincos(x / L, &sx, &cx);
     sincos(y / L, &sy, &cy);
-    sincos(z / L, &sz, &cz);
-    (void)sz;
-    const double u0 = A * sx * cy * cz;
-    const double u1 = -A * cx * sy * cz;
-    const double dp = A * A / 16.0 * (cos(2.0 * x / L) + cos(2.0 * y / L)) * (2.0 + cos(2.0 * z / L));
-    const double rho_p = gM2 * dp;
-    const double rho = 1.0 + rho_p;
-    q[n] = rho_p;
-    q[P + n] = rho * u0;
-    q[2 * P + n] = rho * u1;
-    q[3 * P + n] = 0.0;
-    q[4 * P + n] = dp * inv_gm1 + 0.5 * rho * (u0 * u0 + u1 * u1);
+    const double cxy = cos(2.0 * x / L) + cos(2.0 * y / L);
+    double* o = q + n + plane * z0;
+    for (int k = 0; k < nz; ++k, o += plane) {
+      const double u0 = A * sx * cy * cz[k];
+      const double u1 = -A * cx * sy * cz[k];
+      const double dp = A * A / 16.0 * cxy * (2.0 + c2z[k]);
+      const double rho_p = gM2 * dp;
+      const double rho = 1.0 + rho_p;
+      o[0] = rho_p;
+      o[P] = rho * u0;
+      o[2 * P] = rho * u1;
+      o[3 * P] = 0.0;
+      o[4 * P] = dp * inv_gm1 + 0.5 * rho * (u0 * u0 + u1 * u1);
+    }
   }
 }
 
@@ -88,34 +101,99 @@ static unsigned grid_for(long long n, int block) {
 
 cudaError_t launch_init_tgv(const Geom& g, const sbli_params& p, double amplitude, double* q, cudaStream_t s) {
   const double h0 = 2.0 * M_PI * p.L / g.n0, h1 = 2.0 * M_PI * p.L / g.n1, h2 = 2.0 * M_PI * p.L / g.n2;
-  init_tgv_kernel<<<grid_for(g.P, 256), 256, 0, s>>>(g, h0, h1, h2, p.L, amplitude, p.gamma * p.Mach * p.Mach,
+  const long long plane = (long long)g.n0 * g.n1;
+  const dim3 grid(grid_for(plane, 256), 1, (g.n2 + INIT_Z - 1) / INIT_Z);
+  init_tgv_kernel<<<grid, 256, 0, s>>>(g, h0, h1, h2, p.L, amplitude, p.gamma * p.Mach * p.Mach,
                                                      1.0 / (p.gamma - 1.0), q);
   return cudaGetLastError();
 }
 
-// sign = -1: plain -> deviation; +1: deviation -> plain.  Fields 0 and 4 only
-// differ; momenta are copied.
-__global__ void offset_kernel(long long P, double rho0, double E0, double sign, const double* __restrict__ src,
-                              double* __restrict__ dst) {
-  for (long long n = blockIdx.x * (long long)blockDim.x + threadIdx.x; n < 5 * P;
-       n += (long long)gridDim.x * blockDim.x) {
-    const long long f = n / P;
-    double v = src[n];
-    if (f == 0) v += sign * rho0;
-    if (f == 4) v += sign * E0;
-    dst[n] = v;
+// Conversions between a caller's plain conserved variables and the library's
+// own form of a state, one pass over memory each: a thread moves STATE_ITEMS
+// values of one field (blockIdx.y), 256 apart, all loads issued before the
+// stores, so every access is a coalesced row whatever the field's size and
+// alignment.
+constexpr int STATE_ITEMS = 4;
+static dim3 state_grid(long long P) {
+  const long long b = (P + 256 * STATE_ITEMS - 1) / (256 * STATE_ITEMS);
+  return dim3((unsigned)(b < (1 << 20) ? b : (1 << 20)), 5);
+}
+template <typename L, typename F>
+__device__ __forceinline__ void for_field(long long P, L&& load, F&& put) {
+  const long long f = blockIdx.y;
+  for (long long b = blockIdx.x; b * (256 * STATE_ITEMS) < P; b += gridDim.x) {
+    const long long n0 = b * (256 * STATE_ITEMS) + threadIdx.x;
+    double v[STATE_ITEMS];
+#pragma unroll
+    for (int k = 0; k < STATE_ITEMS; ++k)
+      if (n0 + 256 * k < P) v[k] = load(f * P + n0 + 256 * k);
+#pragma unroll
+    for (int k = 0; k < STATE_ITEMS; ++k)
+      if (n0 + 256 * k < P) put(f * P + n0 + 256 * k, v[k]);
   }
 }
+__device__ __forceinline__ double field_reference(double rho0, double E0) {
+  return blockIdx.y == 0 ? rho0 : (blockIdx.y == 4 ? E0 : 0.0);
+}
 
-cudaError_t launch_to_offset(const Geom& g, const RefState& r, const double* q_plain, double* q_off, cudaStream_t s) {
-  offset_kernel<<<grid_for(5 * g.P, 256), 256, 0, s>>>(g.P, r.rho0, r.E0, -1.0, q_plain, q_off);
+// plain -> own form: binary64 deviations with (copy32) the binary32 copy the
+// binary32 stages read or (pairs) the (hi, lo) pairs the double-float stages
+// read, or (dst64 null) the double-float register alone.
+__global__ void __launch_bounds__(256) import_state_kernel(long long P, double rho0, double E0,
+                                                           const double* __restrict__ src, double* __restrict__ dst64,
+                                                           float* __restrict__ copy32, float2* __restrict__ pairs,
+                                                           float* __restrict__ df) {
+  const double ref = field_reference(rho0, E0);
+  for_field(
+      P, [&](long long i) { return src[i]; },
+      [&](long long i, double x) {
+        const double v = blockIdx.y % 4 == 0 ? x - ref : x;
+        if (df) {
+          const float hi = __double2float_rn(v);
+          df[i] = hi;
+          df[i + 5 * P] = __double2float_rn(v - (double)hi);
+          return;
+        }
+        dst64[i] = v;
+        if (copy32) copy32[i] = narrow_f64_rna(v);
+        if (pairs) {
+          float hi, lo;
+          split_f64(v, hi, lo);
+          pairs[i] = make_float2(hi, lo);
+        }
+      });
+}
+
+cudaError_t launch_import_state(long long P, const RefState& r, const double* src, const StateForm& to,
+                                cudaStream_t s) {
+  import_state_kernel<<<state_grid(P), 256, 0, s>>>(P, r.rho0, r.E0, src, to.f64, to.copy32,
+                                                    reinterpret_cast<float2*>(to.pairs), to.df);
   return cudaGetLastError();
+}
+
+// deviation -> plain.  Fields 0 and 4 only differ; momenta are copied.
+__global__ void __launch_bounds__(256) from_offset_kernel(long long P, double rho0, double E0, const double* src,
+                                                          double* dst) {
+  const double ref = field_reference(rho0, E0);
+  for_field(
+      P, [&](long long i) { return src[i]; },
+      [&](long long i, double x) { dst[i] = blockIdx.y % 4 == 0 ? x + ref : x; });
 }
 
 cudaError_t launch_from_offset(const Geom& g, const RefState& r, const double* q_off, double* q_plain,
                                cudaStream_t s) {
-  offset_kernel<<<grid_for(5 * g.P, 256), 256, 0, s>>>(g.P, r.rho0, r.E0, 1.0, q_off, q_plain);
+  from_offset_kernel<<<state_grid(g.P), 256, 0, s>>>(g.P, r.rho0, r.E0, q_off, q_plain);
   return cudaGetLastError();
+}
+
+bool direct_device_access(const void* p) {
+  cudaPointerAttributes a;
+  int dev = 0;
+  if (cudaGetDevice(&dev) != cudaSuccess || cudaPointerGetAttributes(&a, p) != cudaSuccess) {
+    cudaGetLastError();
+    return false;
+  }
+  return a.type == cudaMemoryTypeDevice && a.device == dev && (uintptr_t)p % sizeof(double) == 0;
 }
 
 __global__ void widen_kernel(long long n, const float* __restrict__ src, double* __restrict__ dst) {
@@ -151,12 +229,12 @@ __global__ void df_split_kernel(long long n5, long long P, double rho0, double E
   }
 }
 
-__global__ void df_join_kernel(long long n5, long long P, double rho0, double E0, const float* __restrict__ src,
-                               double* __restrict__ dst) {
-  for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < n5; i += (long long)gridDim.x * blockDim.x) {
-    const long long f = i / P;
-    dst[i] = ((double)src[i] + (double)src[i + 5 * P]) + (f == 0 ? rho0 : (f == 4 ? E0 : 0.0));
-  }
+__global__ void __launch_bounds__(256) df_join_kernel(long long P, double rho0, double E0,
+                                                      const float* __restrict__ src, double* __restrict__ dst) {
+  const double ref = field_reference(rho0, E0);
+  for_field(
+      P, [&](long long i) { return (double)src[i] + (double)src[i + 5 * P]; },
+      [&](long long i, double x) { dst[i] = x + ref; });
 }
 
 cudaError_t launch_df_split(long long P, const RefState& r, const double* src, float* dst, cudaStream_t s) {
@@ -165,7 +243,7 @@ cudaError_t launch_df_split(long long P, const RefState& r, const double* src, f
 }
 
 cudaError_t launch_df_join(long long P, const RefState& r, const float* src, double* dst, cudaStream_t s) {
-  df_join_kernel<<<grid_for(5 * P, 256), 256, 0, s>>>(5 * P, P, r.rho0, r.E0, src, dst);
+  df_join_kernel<<<state_grid(P), 256, 0, s>>>(P, r.rho0, r.E0, src, dst);
   return cudaGetLastError();
 }
 
@@ -236,70 +314,9 @@ cudaError_t launch_sample_state(long long P, const RefState& r, const double* q6
 }
 
 // ------------------------------------------------------------------ KE
-constexpr int KE_BLOCK = 256;
-constexpr int KE_MAX_BLOCKS = 1024;
+constexpr int KE_MAX_BLOCKS = 1024;  // partial sums the callers' scratch holds
 
-int ke_num_partials(const Geom& g) {
-  long long b = (g.P + KE_BLOCK - 1) / KE_BLOCK;
-  return (int)(b < KE_MAX_BLOCKS ? (b < 1 ? 1 : b) : KE_MAX_BLOCKS);
-}
-
-__device__ __forceinline__ double vel(const double* __restrict__ q, long long P, long long n, int i) {
-  return q[(1 + i) * P + n] / (1.0 + q[n]);
-}
-
-// Per point: ke = rho |u|^2 / 2, enstrophy = rho |curl u|^2 / 2 with Eq. 6
-// derivatives of u (u recomputed at the stencil points).  Each thread sums
-// its points in a fixed order; blocks reduce in a fixed order.
-__global__ void __launch_bounds__(KE_BLOCK) ke_kernel(Geom g, Coef<double> c, const double* __restrict__ q,
-                                                      double* __restrict__ partials) {
-  const long long P = g.P;
-  const int n0 = g.n0, n1 = g.n1, n2 = g.n2;
-  double ke = 0.0, en = 0.0;
-  for (long long n = blockIdx.x * (long long)KE_BLOCK + threadIdx.x; n < P; n += (long long)gridDim.x * KE_BLOCK) {
-    const int i = (int)(n % n0);
-    const int j = (int)((n / n0) % n1);
-    const int k = (int)(n / ((long long)n0 * n1));
-    auto idx = [&](int ii, int jj, int kk) {
-      return (long long)wrapi(ii, n0) + (long long)n0 * (wrapi(jj, n1) + (long long)n1 * wrapi(kk, n2));
-    };
-    auto d1 = [&](int comp, int axis) {
-      const int o[4] = {-2, -1, 1, 2};
-      double f[4];
-      for (int m = 0; m < 4; ++m) {
-        const long long nn = axis == 0 ? idx(i + o[m], j, k) : axis == 1 ? idx(i, j + o[m], k) : idx(i, j, k + o[m]);
-        f[m] = vel(q, P, nn, comp);
-      }
-      return c.c1[axis] * (f[2] - f[1]) - c.c2[axis] * (f[3] - f[0]);
-    };
-    const double rho = 1.0 + q[n];
-    const double u0 = vel(q, P, n, 0), u1 = vel(q, P, n, 1), u2 = vel(q, P, n, 2);
-    const double w0 = d1(2, 1) - d1(1, 2);
-    const double w1 = d1(0, 2) - d1(2, 0);
-    const double w2 = d1(1, 0) - d1(0, 1);
-    ke += 0.5 * rho * (u0 * u0 + u1 * u1 + u2 * u2);
-    en += 0.5 * rho * (w0 * w0 + w1 * w1 + w2 * w2);
-  }
-  __shared__ double red[2][KE_BLOCK / 32];
-  for (int o = 16; o > 0; o >>= 1) {
-    ke += __shfl_down_sync(0xffffffffu, ke, o);
-    en += __shfl_down_sync(0xffffffffu, en, o);
-  }
-  if ((threadIdx.x & 31) == 0) {
-    red[0][threadIdx.x >> 5] = ke;
-    red[1][threadIdx.x >> 5] = en;
-  }
-  __syncthreads();
-  if (threadIdx.x == 0) {
-    double a = 0.0, b = 0.0;
-    for (int w = 0; w < KE_BLOCK / 32; ++w) {
-      a += red[0][w];
-      b += red[1][w];
-    }
-    partials[2 * blockIdx.x] = a;
-    partials[2 * blockIdx.x + 1] = b;
-  }
-}
+int ke_num_partials(const Geom& g) { return ke_blocks(g, KE_MAX_BLOCKS); }
 
 // One block: thread t sums pairs t, t+256, ... in order, then a fixed tree.
 __global__ void __launch_bounds__(256) finalize_ke_kernel(const double* __restrict__ partials, int n, double inv_p,
@@ -335,7 +352,7 @@ cudaError_t launch_ke(const Geom& g, const Coef<double>& c, const RefState& r, c
                       double* partials, double* out, cudaStream_t s) {
   (void)r;
   const int nb = ke_num_partials(g);
-  ke_kernel<<<nb, KE_BLOCK, 0, s>>>(g, c, q_off, partials);
+  ke_march_kernel<false><<<nb, KE_THREADS, 0, s>>>(g, c, q_off, partials);
   cudaError_t e = cudaGetLastError();
   if (e != cudaSuccess) return e;
   return launch_finalize_ke(partials, nb, 1.0 / (double)g.P, out, s);

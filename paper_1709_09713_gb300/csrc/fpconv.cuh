@@ -95,6 +95,20 @@ __device__ __forceinline__ float narrow_f64_rna(double d) {
   return __uint_as_float(bits);
 }
 
+// 1/x in binary64: the hardware approximation (rcp.approx.ftz.f64) refined by
+// two Newton-Raphson steps y <- y + y (1 - x y), each a pair of fused
+// multiply-adds that squares the relative error (within one unit in the last
+// place of 1/x; tests/test_gpu_recip.py compares it with CUDA's correctly
+// rounded reciprocal)
+__device__ __forceinline__ double rcp_newton_f64(double x) {
+  double y;
+  asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(x));
+  double e = fma(-x, y, 1.0);
+  y = fma(y, e, y);
+  e = fma(-x, y, 1.0);
+  return fma(y, e, y);
+}
+
 // binary64 -> double-float pair: hi = RN32(v), lo = RN32(v - hi); the
 // narrowings and the widening of hi are integer re-packings, the remainder one
 // DADD (exact: v - hi has at most 29 significant bits).  The stage kernels

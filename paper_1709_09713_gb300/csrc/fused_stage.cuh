@@ -138,19 +138,9 @@ __device__ __forceinline__ float rcp_approx_f32(float x) {
 }
 template <typename T>
 __device__ __forceinline__ T recip(T x);
-// binary64: the hardware approximation (rcp.approx.ftz.f64) refined by two
-// Newton-Raphson steps y <- y + y (1 - x y), each a pair of fused
-// multiply-adds that squares the relative error (within one unit in the
-// last place of 1/x; tests/test_gpu_recip.py compares it with CUDA's
-// correctly rounded reciprocal)
 template <>
 __device__ __forceinline__ double recip<double>(double x) {
-  double y;
-  asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(x));
-  double e = fma(-x, y, 1.0);
-  y = fma(y, e, y);
-  e = fma(-x, y, 1.0);
-  return fma(y, e, y);
+  return rcp_newton_f64(x);
 }
 template <>
 __device__ __forceinline__ float recip<float>(float x) { return rcp_approx_f32(x); }

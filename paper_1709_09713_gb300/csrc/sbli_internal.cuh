@@ -124,7 +124,20 @@ Split plan_split(const Geom& g, int zc, int sms, bool double_float);
 
 // Diagnostics and state conversion (diag.cu).
 cudaError_t launch_init_tgv(const Geom& g, const sbli_params& p, double amplitude, double* q, cudaStream_t s);
-cudaError_t launch_to_offset(const Geom& g, const RefState& r, const double* q_plain, double* q_off, cudaStream_t s);
+// Plain conserved variables -> a state in the library's form, in one pass:
+// binary64 deviations (f64) with the binary32 copy or the (hi, lo) pair copy
+// that the precision's first stage reads, or the double-float register (df).
+struct StateForm {
+  double* f64;
+  float* copy32;
+  float* pairs;
+  float* df;
+};
+cudaError_t launch_import_state(long long P, const RefState& r, const double* src, const StateForm& to,
+                                cudaStream_t s);
+// Whether a kernel of the current device may read or write p itself: its own
+// memory, aligned.  (Other memory that the copy engines reach is staged.)
+bool direct_device_access(const void* p);
 cudaError_t launch_from_offset(const Geom& g, const RefState& r, const double* q_off, double* q_plain,
                                cudaStream_t s);
 // dst[i] = (double)src[i], i < n

@@ -322,16 +322,19 @@ int retire(sbli_server* s, Req& q) {
   double h[2];
   SBLI_STRY(cudaMemcpyAsync(h, s->ke_dev, sizeof h, cudaMemcpyDeviceToHost, st), "D2H");
   if (q.r.result) {
-    double* tmp = r64(s, q, req_free_reg(q));  // a register the finished state does not occupy
+    const bool staged = q.r.result_is_host || !direct_device_access(q.r.result);
+    // staged through a register the finished state does not occupy
+    double* dst = staged ? r64(s, q, req_free_reg(q)) : q.r.result;
     if (q.r.precision == SBLI_FP32_DF) {
-      SBLI_STRY(launch_df_join(q.P, make_ref(q.r.params), reinterpret_cast<const float*>(r64(s, q, q.state)), tmp, st),
+      SBLI_STRY(launch_df_join(q.P, make_ref(q.r.params), reinterpret_cast<const float*>(r64(s, q, q.state)), dst, st),
                 "df_join");
     } else {
-      SBLI_STRY(launch_from_offset(g, make_ref(q.r.params), state, tmp, st), "from_offset");
+      SBLI_STRY(launch_from_offset(g, make_ref(q.r.params), state, dst, st), "from_offset");
     }
-    SBLI_STRY(cudaMemcpyAsync(q.r.result, tmp, 5 * (size_t)q.P * sizeof(double),
-                              q.r.result_is_host ? cudaMemcpyDeviceToHost : cudaMemcpyDeviceToDevice, st),
-              "copy result");
+    if (staged)
+      SBLI_STRY(cudaMemcpyAsync(q.r.result, dst, 5 * (size_t)q.P * sizeof(double),
+                                q.r.result_is_host ? cudaMemcpyDeviceToHost : cudaMemcpyDeviceToDevice, st),
+                "copy result");
   }
   SBLI_STRY(cudaStreamSynchronize(st), "cudaStreamSynchronize");
   q.ke = h[0];
