@@ -83,16 +83,60 @@ __device__ __forceinline__ dfloat& operator+=(dfloat& x, dfloat y) { return x = 
 __device__ __forceinline__ dfloat& operator-=(dfloat& x, dfloat y) { return x = x - y; }
 __device__ __forceinline__ dfloat& operator*=(dfloat& x, dfloat y) { return x = x * y; }
 
-// 1 / x: t = RN(1/x.hi), residual e = 1 - x t (FMA for the high part, the low
-// part subtracted), result t + t e.
+// 1 / x: t close to 1/x.hi (the hardware approximation refined by one Newton
+// step in binary32, so within about half a unit in the last place, without
+// the rounding correction and its branch), residual e = 1 - x t (FMA for the
+// high part, the low part subtracted), result t + t e.
 __device__ __forceinline__ dfloat dw_reciprocal(dfloat xin) {
   const dfloat x = dw_normalise(xin);
-  const float t = __frcp_rn(x.hi);
+  float t;
+  asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(t) : "f"(x.hi));
+  t = __fmaf_rn(t, __fmaf_rn(-x.hi, t, 1.0f), t);
   float e = __fmaf_rn(-x.hi, t, 1.0f);
   e = __fmaf_rn(-x.lo, t, e);
   float zh, zl;
   dw::fast_two_sum(t, __fmul_rn(t, e), zh, zl);
   return dfloat(zh, zl);
+}
+
+// x times a power of two (exact)
+__device__ __forceinline__ dfloat dw_scale(dfloat x, float s) { return dfloat(__fmul_rn(x.hi, s), __fmul_rn(x.lo, s)); }
+
+// Two double-float values side by side: every operation is the one above on
+// each, issued as packed two-lane instructions (the same roundings; half the
+// instructions, negation is an operand modifier).
+struct dfloat2 {
+  float2 hi, lo;
+  dfloat2() = default;
+  __device__ __forceinline__ dfloat2(float2 h, float2 l) : hi(h), lo(l) {}
+  __device__ __forceinline__ dfloat2(dfloat x, dfloat y) : hi(make_float2(x.hi, y.hi)), lo(make_float2(x.lo, y.lo)) {}
+  __device__ __forceinline__ explicit dfloat2(dfloat x) : dfloat2(x, x) {}
+  __device__ __forceinline__ dfloat a() const { return dfloat(hi.x, lo.x); }
+  __device__ __forceinline__ dfloat b() const { return dfloat(hi.y, lo.y); }
+};
+namespace dw {
+__device__ __forceinline__ float2 neg2(float2 x) { return make_float2(-x.x, -x.y); }
+__device__ __forceinline__ float2 sub2(float2 x, float2 y) { return __fadd2_rn(x, neg2(y)); }
+}  // namespace dw
+__device__ __forceinline__ dfloat2 operator+(dfloat2 x, dfloat2 y) {
+  const float2 s = __fadd2_rn(x.hi, y.hi);
+  const float2 ap = dw::sub2(s, y.hi);
+  const float2 bp = dw::sub2(s, ap);
+  const float2 t = __fadd2_rn(dw::sub2(x.hi, ap), dw::sub2(y.hi, bp));
+  return dfloat2(s, __fadd2_rn(t, __fadd2_rn(x.lo, y.lo)));
+}
+__device__ __forceinline__ dfloat2 operator-(dfloat2 x) { return dfloat2(dw::neg2(x.hi), dw::neg2(x.lo)); }
+__device__ __forceinline__ dfloat2 operator-(dfloat2 x, dfloat2 y) { return x + (-y); }
+__device__ __forceinline__ dfloat2 operator*(dfloat2 x, dfloat2 y) {
+  const float2 p = __fmul2_rn(x.hi, y.hi);
+  float2 e = __ffma2_rn(x.hi, y.hi, dw::neg2(p));
+  e = __ffma2_rn(x.hi, y.lo, e);
+  e = __ffma2_rn(x.lo, y.hi, e);
+  return dfloat2(p, e);
+}
+__device__ __forceinline__ dfloat2 dw_scale(dfloat2 x, float s) {
+  const float2 v = make_float2(s, s);
+  return dfloat2(__fmul2_rn(x.hi, v), __fmul2_rn(x.lo, v));
 }
 
 }  // namespace sbli

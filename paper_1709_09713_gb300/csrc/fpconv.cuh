@@ -109,14 +109,30 @@ __device__ __forceinline__ double rcp_newton_f64(double x) {
   return fma(y, e, y);
 }
 
-// binary64 -> double-float pair: hi = RN32(v), lo = RN32(v - hi); the
-// narrowings and the widening of hi are integer re-packings, the remainder one
-// DADD (exact: v - hi has at most 29 significant bits).  The stage kernels
-// split binary64 stage inputs this way, and the double-float path stores its
-// stage fields already split this way.
+// binary64 -> double-float pair, hi = v rounded to nearest (ties away from
+// zero), lo = v - hi rounded to nearest, without the FP64 pipe: the low word
+// shifted left by 3 holds the 29 mantissa bits that hi drops at the top of a
+// signed integer, which is negative just when hi was rounded up -- the exact
+// remainder in units of 2^(e - 55); converted (one rounding, to 24 bits) and
+// scaled by that power of two with the sign of v.  Zero and results below the
+// binary32 normal range become signed zero (lo: below 2^-72 of v); magnitudes
+// of 2^128 and above and infinities give an infinite hi, NaNs a NaN, with lo 0.
+// The stage kernels split binary64 stage inputs this way, and the
+// double-float path stores its stage fields already split this way.
 __device__ __forceinline__ void split_f64(double v, float& hi, float& lo) {
-  hi = narrow_f64_fast(v);
-  lo = narrow_f64_fast(v - widen_f32_fast(hi));
+  const unsigned vh = (unsigned)__double2hiint(v), vl = (unsigned)__double2loint(v);
+  const unsigned sign = vh & 0x80000000u, eb = (vh >> 20) & 0x7FFu;
+  unsigned bits = (__funnelshift_l(vl, vh, 3) + 0x40000000u + ((vl >> 28) & 1u)) | sign;
+  unsigned scale = sign | ((eb - 951u) << 23);  // 2^(e - 55), biased: eb - 1023 + 127 - 55
+  const float rest = __int2float_rn((int)(vl << 3));
+  bits = eb < 897u ? sign : bits;
+  scale = eb < 952u ? 0u : scale;
+  if (eb > 1150u) {  // 2^128 and above, infinities, NaNs
+    bits = sign | 0x7F800000u | (eb == 0x7FFu && ((vh & 0xFFFFFu) | vl) != 0u ? 0x400000u : 0u);
+    scale = 0u;
+  }
+  hi = __uint_as_float(bits);
+  lo = __fmul_rn(rest, __uint_as_float(scale));
 }
 
 }  // namespace sbli

@@ -21,8 +21,8 @@
 //     derivative terms start, so HBM latency overlaps the arithmetic;
 //   * x0/x1 derivatives read the centre slot, x2 derivatives read the ring;
 //     each axis streams its four neighbour records through the accumulators
-//     one at a time (axis_terms_stream; the double-float type keeps the
-//     difference-first form, axis_terms);
+//     one at a time (axis_terms_stream; the double-float type takes differences
+//     first and two values at a time, axis_terms_dw);
 //   * ZT (the z queue): each thread keeps its own column's records of the
 //     five ring planes, and their in-plane gradients, in tensor memory
 //     (TMEM), so the x2 derivatives read TMEM and shared memory keeps full
@@ -75,11 +75,12 @@ constexpr int HALO = 2;
 constexpr int SX = TX + 2 * HALO;
 constexpr int NSLOT = 5;
 
-// primitive values of one point record in a ring slot; V_P holds 2 p' (the
+// primitive values of one point record in a ring slot; V_H is E' + 2 p' (see
+// StreamTerms), V_P holds 2 p' (the
 // pressure enters Eqs. 2-3 only as 2 D_i p and 2 D_j(p u_j) in the combined
 // skew form, so the factor 2 is applied once per point instead of once per
 // stencil neighbour; scaling by 2 is exact)
-enum { V_RHO, V_M0, V_M1, V_M2, V_H, V_E = V_H, V_U0, V_U1, V_U2, V_P, V_T, NV };
+enum { V_RHO, V_M0, V_M1, V_M2, V_H, V_U0, V_U1, V_U2, V_P, V_T, NV };
 static_assert(V_U2 == V_U1 + 1 && V_U1 % 2 == 0, "u1, u2 form one 8-byte pair of a binary32 record");
 
 // ZT (binary32 with the TMEM z queue): the x2 neighbours of a thread's own
@@ -87,9 +88,9 @@ static_assert(V_U2 == V_U1 + 1 && V_U1 % 2 == 0, "u1, u2 form one 8-byte pair of
 // for the planes that are still to become the centre (entering, middle,
 // centre: 3 slots), u_2 alone on the five ring planes (for D1_z u_2 on the
 // halo), and no D1_x u0 / D1_y u1 ring.
-template <int TY, bool ZT>
+template <typename T, int TY, bool ZT>
 constexpr int full_slots() {
-  return ZT ? (TY >= 16 ? 4 : 3) : NSLOT;
+  return ZT ? (TY >= 16 && sizeof(T) == 4 ? 4 : 3) : NSLOT;
 }
 // Binary32 arithmetic types group the mixed second derivatives so that the
 // x2 derivative is applied last (see fused_march): their helpers are
@@ -98,16 +99,10 @@ template <typename T>
 constexpr bool mixz() {
   return std::is_same<T, float>::value || std::is_same<T, f32x2>::value;
 }
-// The hardware FMA types keep H = E' + 2p' in the record (see StreamTerms),
-// double-float E' itself.
-template <typename T>
-constexpr bool hrec() {
-  return !std::is_same<T, dfloat>::value;
-}
 template <typename T, int TY, bool ZT = false>
 struct FusedSmem {
   static constexpr int SY = TY + 2 * HALO;
-  static constexpr int NFULL = full_slots<TY, ZT>();
+  static constexpr int NFULL = full_slots<T, TY, ZT>();
   static constexpr bool MIXZ = mixz<T>();
   static constexpr bool U2 = ZT && !MIXZ;      // u_2 ring (binary64 / double-float TMEM queue)
   static constexpr int NDV = MIXZ ? 4 : 2;     // per-plane gradients in the shared ring
@@ -195,20 +190,43 @@ __device__ __forceinline__ void store_rec(f32x2* p, const f32x2 (&r)[NV]) {
 #pragma unroll
   for (int i = 0; i < NV / 2; ++i) q[i] = make_float4(r[2 * i].x, r[2 * i].y, r[2 * i + 1].x, r[2 * i + 1].y);
 }
-// double-float records: 80 bytes, two values per 16-byte access
-__device__ __forceinline__ void load_rec(const dfloat* p, dfloat (&r)[NV]) {
+// Double-float records: 80 bytes, five pairs of values of 16 bytes each, (hi,
+// hi, lo, lo), so that a pair is one 16-byte access and comes as the operands
+// of the packed instructions (dfloat2): (m0, m1), (m2, H), (u0, u1), (u2, T'),
+// (rho', 2p').
+enum { W_M01, W_M2H, W_U01, W_U2T, W_RHOP, NW };
+constexpr int dw_slot(int v) {  // 2 * pair + lane of a value
+  return v == V_RHO ? 8 : v == V_P ? 9 : v == V_T ? 7 : v <= V_H ? v - V_M0 : v - V_U0 + 4;
+}
+__device__ __forceinline__ void load_pairs(const dfloat* p, dfloat2 (&r)[NW]) {
   const float4* q = reinterpret_cast<const float4*>(p);
 #pragma unroll
-  for (int i = 0; i < NV / 2; ++i) {
+  for (int i = 0; i < NW; ++i) {
     const float4 v = q[i];
-    r[2 * i] = dfloat(v.x, v.y);
-    r[2 * i + 1] = dfloat(v.z, v.w);
+    r[i] = dfloat2(make_float2(v.x, v.y), make_float2(v.z, v.w));
   }
 }
 __device__ __forceinline__ void store_rec(dfloat* p, const dfloat (&r)[NV]) {
   float4* q = reinterpret_cast<float4*>(p);
+  dfloat s[NV];
 #pragma unroll
-  for (int i = 0; i < NV / 2; ++i) q[i] = make_float4(r[2 * i].hi, r[2 * i].lo, r[2 * i + 1].hi, r[2 * i + 1].lo);
+  for (int v = 0; v < NV; ++v) s[dw_slot(v)] = r[v];
+#pragma unroll
+  for (int i = 0; i < NW; ++i) q[i] = make_float4(s[2 * i].hi, s[2 * i + 1].hi, s[2 * i].lo, s[2 * i + 1].lo);
+}
+// one value of a record
+template <typename T>
+__device__ __forceinline__ T rec_value(const T* r, int v) {
+  return r[v];
+}
+// (the 16-byte load of its pair: 4-byte loads at this stride conflict 4-way)
+__device__ __forceinline__ dfloat2 load_pair(const dfloat* r, int pair) {
+  const float4 v = reinterpret_cast<const float4*>(r)[pair];
+  return dfloat2(make_float2(v.x, v.y), make_float2(v.z, v.w));
+}
+__device__ __forceinline__ dfloat rec_value(const dfloat* r, int v) {
+  const dfloat2 x = load_pair(r, dw_slot(v) / 2);
+  return dw_slot(v) % 2 ? x.b() : x.a();
 }
 
 // ---- tensor memory (TMEM) as a per-thread queue of x2-neighbour records.
@@ -378,10 +396,26 @@ __device__ __forceinline__ void tmem_store_rec(uint32_t win, int slot, const dou
   tmem_store_rec8(win, slot, r);
 }
 __device__ __forceinline__ void tmem_load_rec(uint32_t win, int slot, double (&r)[NV]) { tmem_load_rec8(win, slot, r); }
+// double-float records go through TMEM in the pair order of the shared-memory
+// record, as ten 8-byte values (hi, hi), (lo, lo) a pair
 __device__ __forceinline__ void tmem_store_rec(uint32_t win, int slot, const dfloat (&r)[NV]) {
-  tmem_store_rec8(win, slot, r);
+  dfloat s[NV], w[NV];
+#pragma unroll
+  for (int v = 0; v < NV; ++v) s[dw_slot(v)] = r[v];
+#pragma unroll
+  for (int i = 0; i < NW; ++i) {
+    w[2 * i] = dfloat(s[2 * i].hi, s[2 * i + 1].hi);
+    w[2 * i + 1] = dfloat(s[2 * i].lo, s[2 * i + 1].lo);
+  }
+  tmem_store_rec8(win, slot, w);
 }
-__device__ __forceinline__ void tmem_load_rec(uint32_t win, int slot, dfloat (&r)[NV]) { tmem_load_rec8(win, slot, r); }
+__device__ __forceinline__ void tmem_load_pairs(uint32_t win, int slot, dfloat2 (&r)[NW]) {
+  dfloat w[NV];
+  tmem_load_rec8(win, slot, w);
+#pragma unroll
+  for (int i = 0; i < NW; ++i)
+    r[i] = dfloat2(make_float2(w[2 * i].hi, w[2 * i].lo), make_float2(w[2 * i + 1].hi, w[2 * i + 1].lo));
+}
 __device__ __forceinline__ void tmem_store_diag(uint32_t win, int slot, double d00, double d11) {
   tmem_store_diag8(win, slot, d00, d11);
 }
@@ -529,70 +563,6 @@ __device__ __forceinline__ double as_double(double x) { return x; }
 __device__ __forceinline__ double as_double(float x) { return widen_f32_fast(x); }
 __device__ __forceinline__ double as_double(dfloat x) { return widen_f32_fast(x.hi) + widen_f32_fast(x.lo); }
 
-// Accumulated terms of the residual at one point.  By linearity of D1 and
-// because the centre values u_j^c are constants over a stencil, the
-// convective and skew terms of Eqs. 1-3 combine into single derivatives:
-//   D_j(m_i u_j) + u_j^c D_j m_i       = D_j( m_i (u_j + u_j^c) )
-//   D_j m_j + u_j^c D_j rho'            = D_j( m_j + u_j^c rho' )
-//   D_j(E' u_j) + u_j^c D_j E'          = D_j( E' (u_j + u_j^c) )
-template <typename T>
-struct Terms {
-  T g[3][3];   // g[i][j] = D1_j u_i
-  T rrho;      // sum_j D_j(m_j + u_j^c rho')                     (Eq. 1 without rho div u)
-  T rM[3];     // sum_j D_j(m_i (u_j + u_j^c)) + 2 D_i p'          (Eq. 2 without m_i div u)
-  T rE;        // sum_j D_j(E' (u_j + u_j^c)) + 2 D_j(p' u_j)      (Eq. 3 without E' div u)
-  T lap[3];    // sum_j D2_j u_i, off-centre part
-  T lapT;      // sum_j D2_j T', off-centre part
-  T G[3];      // sum_j d2 u_j / dx_i dx_j (Eq. 7 on j = i, D1 o D1 otherwise)
-};
-
-// All derivatives along axis A at one point.  ldrec(k, r) loads the record of
-// the neighbour k = 0..3 (offsets -2, -1, +1, +2 along A); uc are the centre
-// velocities; sfun(k) gives the mixed-term helper s_A at neighbour k.
-template <int A, typename T, typename LD, typename SF>
-__device__ __forceinline__ void axis_terms(const LD& ldrec, const SF& sfun, const Coef<T>& c, const T (&uc)[3],
-                                           Terms<T>& t) {
-  const T c1 = c.c1[A], c2 = c.c2[A], e0 = c.e0[A], e1 = c.e1[A], e2 = c.e2[A];
-  const T nc2 = -c2;
-  auto d1 = [&](T fm2, T fm1, T fp1, T fp2) { return mad(c1, fp1 - fm1, nc2 * (fp2 - fm2)); };
-
-  T r[4][NV];
-#pragma unroll
-  for (int k = 0; k < 4; ++k) ldrec(k, r[k]);
-  T s[4];
-#pragma unroll
-  for (int k = 0; k < 4; ++k) s[k] = sfun(k);
-#define SBLI_D1(V) d1(r[0][V], r[1][V], r[2][V], r[3][V])
-  const T ua = uc[A];
-  // stencil weights times (u_A + u_A^c):  D1(f w) = f+1 W1 - f-1 V1 - f+2 W2 + f-2 V2
-  const T W1 = c1 * (r[2][V_U0 + A] + ua), V1 = c1 * (r[1][V_U0 + A] + ua);
-  const T W2 = c2 * (r[3][V_U0 + A] + ua), V2 = c2 * (r[0][V_U0 + A] + ua);
-  const T nV1 = -V1, nW2 = -W2;
-  auto d1w = [&](int V) { return mad(r[0][V], V2, mad(r[3][V], nW2, mad(r[1][V], nV1, r[2][V] * W1))); };
-  // stencil weights times u_A:  D1(f u_A)
-  const T X1 = c1 * r[2][V_U0 + A], Y1 = c1 * r[1][V_U0 + A];
-  const T X2 = c2 * r[3][V_U0 + A], Y2 = c2 * r[0][V_U0 + A];
-  const T mY1 = -Y1, mX2 = -X2;
-#pragma unroll
-  for (int i = 0; i < 3; ++i) t.rM[i] += d1w(V_M0 + i);
-  t.rM[A] = t.rM[A] + SBLI_D1(V_P);  // D_A (2 p')
-  t.rE += mad(r[0][V_P], Y2, mad(r[3][V_P], mX2, mad(r[1][V_P], mY1, r[2][V_P] * X1))) + d1w(V_E);
-  t.rrho += d1(fma(ua, r[0][V_RHO], r[0][V_M0 + A]), fma(ua, r[1][V_RHO], r[1][V_M0 + A]),
-               fma(ua, r[2][V_RHO], r[2][V_M0 + A]), fma(ua, r[3][V_RHO], r[3][V_M0 + A]));
-#pragma unroll
-  for (int i = 0; i < 3; ++i) {
-    const T off = mad(e1, r[2][V_U0 + i] + r[1][V_U0 + i], e2 * (r[3][V_U0 + i] + r[0][V_U0 + i]));
-    t.lap[i] += off;
-    if (i == A) {
-      t.G[A] = fma(e0, uc[A], off) + d1(s[0], s[1], s[2], s[3]);
-    } else {
-      t.g[i][A] = SBLI_D1(V_U0 + i);
-    }
-  }
-  t.lapT += mad(e1, r[2][V_T] + r[1][V_T], e2 * (r[3][V_T] + r[0][V_T]));
-#undef SBLI_D1
-}
-
 // a * b + c with one rounding in every scalar type (and lane): the streamed
 // terms below never leave a contraction to the compiler, so that every
 // instantiation of the kernel rounds alike.
@@ -736,29 +706,135 @@ __device__ __forceinline__ void assemble_streamed(const StreamTerms<T>& t, T rho
   R[4] = fmadd(c.kappa, t.lapT, fmadd(c.inv_re, q, fmadd(-c.H0, div, half(fmadd(Ec, hdiv, t.rE)))));
 }
 
-// Eqs. 1-3 at one point from the accumulated derivative terms and the
-// centre values (deviation form: rho' = rho - 1, E' = rho E - (rho E)_ref).
-template <typename T>
-__device__ __forceinline__ void assemble_residual(const Terms<T>& t, T rho_p, const T (&mc)[3], T Ec, const T (&uc)[3],
-                                                  T Tc, const Coef<T>& c, T (&R)[5]) {
-  const T e0sum = c.e0[0] + c.e0[1] + c.e0[2];  // centre coefficient of the Laplacian
-  const T div = t.g[0][0] + t.g[1][1] + t.g[2][2];
-  const T rho = T(1) + rho_p;
-  R[0] = T(-0.5) * mad(rho, div, t.rrho);
-  T uvisc = T(0);
-#pragma unroll
-  for (int i = 0; i < 3; ++i) {
-    const T lap = fma(e0sum, uc[i], t.lap[i]);
-    const T visc = mad(t.G[i], T(1.0 / 3.0), lap);  // Laplacian + G - (2/3) G
-    uvisc = mad(uc[i], visc, uvisc);
-    R[1 + i] = mad(c.inv_re, visc, T(-0.5) * mad(mc[i], div, t.rM[i]));
+// ---- double-float: the same terms in pairs.  A double-word sum costs 8
+// instructions and a product 4, so differences and sums of neighbours come
+// first, then one product with the common weight: with c1 = 8 c2 and
+// e1 = -16 e2 (Eqs. 6-7) a first derivative is c2 (8 (f+1 - f-1) - (f+2 - f-2)) and
+// the off-centre part of a second one e2 ((f+2 + f-2) - 16 (f+1 + f-1)), the scalings
+// exact; the weights u_j + u_j^c take the 8 themselves.  Two values at a time
+// go through packed two-lane instructions: the pairs of the record, and for
+// the cross gradients and (m_A, s_A) pairs put together in registers.  256^3,
+// 37 planes a CTA: 2.43 -> 2.20 ms a stage, 3727 -> about 2450 instructions a point;
+// bound by the latency of dependent instructions and of shared memory at the
+// two warps a sub-partition that 200 registers leave (issue 45 %, FMA pipe 47 %).
+struct DwTerms {
+  dfloat2 m01, m2e;  // -1/2 the convective sums of Eq. 2 (i = 0, 1), (i = 2 and Eq. 3)
+  dfloat2 v01, v2t;  // sum_j D2_j u_i + 1/3 sum_j d2 u_j / dx_i dx_j, and sum_j D2_j T'
+  dfloat rho;        // -1/2 sum_j D_j(m_j + u_j^c rho')
+  dfloat a01, a02, a12;  // D1_j u_i + D1_i u_j
+  dfloat w01, w02, w12;  // their differences D1_j u_i - D1_i u_j, i < j (diagnostics only)
+};
+__device__ __forceinline__ dfloat2 dw_first(dfloat2 m2, dfloat2 m1, dfloat2 p1, dfloat2 p2, dfloat2 k) {
+  return (dw_scale(p1 - m1, 8.0f) - (p2 - m2)) * k;
+}
+template <int A>
+__device__ __forceinline__ dfloat pair_u(const dfloat2 (&r)[NW]) {  // u_A of a record
+  return A == 0 ? r[W_U01].a() : A == 1 ? r[W_U01].b() : r[W_U2T].a();
+}
+template <int A>
+__device__ __forceinline__ dfloat pair_m(const dfloat2 (&r)[NW]) {  // m_A
+  return A == 0 ? r[W_M01].a() : A == 1 ? r[W_M01].b() : r[W_M2H].a();
+}
+
+// All terms along axis A; ldp(k, pairs) loads the record of neighbour k (offsets
+// -2, -1, +1, +2), sfun(k) the mixed-term helper s_A there.
+template <int A, bool WITH_KE, typename LD, typename SF>
+__device__ __forceinline__ void axis_terms_dw(const LD& ldp, const SF& sfun, const Coef<dfloat>& c, dfloat ua,
+                                              DwTerms& t) {
+  const dfloat2 kh(c.hc2[A]);
+  // the inner neighbours, then the outer ones: two records live at a time
+  dfloat2 cm01, cm2e, rp, dms, l01, l2t, g;
+  auto cross = [](const dfloat2(&r)[NW]) {  // (u_i, u_j), i, j != A
+    return A == 2 ? r[W_U01] : dfloat2(A == 0 ? r[W_U01].b() : r[W_U01].a(), r[W_U2T].a());
+  };
+  {
+    dfloat2 m[NW], p[NW];
+    ldp(1, m);
+    ldp(2, p);
+    const dfloat2 wm(dw_scale(pair_u<A>(m) + ua, -8.0f)), wp(dw_scale(pair_u<A>(p) + ua, 8.0f));
+    cm01 = wp * p[W_M01] + wm * m[W_M01];
+    cm2e = wp * p[W_M2H] + wm * m[W_M2H];
+    rp = dw_scale(p[W_RHOP] - m[W_RHOP], 8.0f);
+    dms = dw_scale(dfloat2(pair_m<A>(p), sfun(2)) - dfloat2(pair_m<A>(m), sfun(1)), 8.0f);
+    l01 = dw_scale(p[W_U01] + m[W_U01], 16.0f);
+    l2t = dw_scale(p[W_U2T] + m[W_U2T], 16.0f);
+    g = dw_scale(cross(p) - cross(m), 8.0f);
   }
-  // viscous dissipation du_i/dx_j (du_i/dx_j + du_j/dx_i - 2/3 div delta_ij)
-  const T a01 = t.g[0][1] + t.g[1][0], a02 = t.g[0][2] + t.g[2][0], a12 = t.g[1][2] + t.g[2][1];
-  const T sq = mad(t.g[2][2], t.g[2][2], mad(t.g[1][1], t.g[1][1], t.g[0][0] * t.g[0][0]));
-  const T diss = mad(T(2), sq, mad(a12, a12, mad(a02, a02, mad(a01, a01, T(-2.0 / 3.0) * div * div))));
-  const T lapT = fma(e0sum, Tc, t.lapT);
-  R[4] = mad(c.kappa, lapT, mad(c.inv_re, uvisc + diss, mad(-c.H0, div, T(-0.5) * mad(Ec, div, t.rE))));
+  {
+    dfloat2 m[NW], p[NW];
+    ldp(0, m);
+    ldp(3, p);
+    const dfloat2 wm(pair_u<A>(m) + ua), wp(-(pair_u<A>(p) + ua));
+    cm01 = (cm01 + (wp * p[W_M01] + wm * m[W_M01])) * kh;
+    cm2e = (cm2e + (wp * p[W_M2H] + wm * m[W_M2H])) * kh;
+    rp = (rp - (p[W_RHOP] - m[W_RHOP])) * kh;
+    dms = (dms - (dfloat2(pair_m<A>(p), sfun(3)) - dfloat2(pair_m<A>(m), sfun(0)))) * dfloat2(c.hc2[A], c.t2[A]);
+    // 4/3 e on u_A: Laplacian and one third of Eq. 7
+    const dfloat e = c.e2[A], f = c.f2[A];
+    l01 = ((p[W_U01] + m[W_U01]) - l01) * dfloat2(A == 0 ? f : e, A == 1 ? f : e);
+    l2t = ((p[W_U2T] + m[W_U2T]) - l2t) * dfloat2(A == 2 ? f : e, e);
+    g = (g - (cross(p) - cross(m))) * dfloat2(c.c2[A]);
+  }
+  t.m01 = t.m01 + cm01;
+  t.m2e = t.m2e + cm2e;
+  t.rho = t.rho + (dms.a() + ua * rp.a());
+  const dfloat up = ua * rp.b();
+  if (A == 0) t.m01 = dfloat2(t.m01.a() + rp.b(), t.m01.b());
+  if (A == 1) t.m01 = dfloat2(t.m01.a(), t.m01.b() + rp.b());
+  if (A == 2)
+    t.m2e = t.m2e + dfloat2(rp.b(), -up);
+  else
+    t.m2e = dfloat2(t.m2e.a(), t.m2e.b() - up);
+  t.v01 = t.v01 + l01;
+  t.v2t = t.v2t + l2t;
+  if (A == 0) t.v01 = dfloat2(t.v01.a() + dms.b(), t.v01.b());
+  if (A == 1) t.v01 = dfloat2(t.v01.a(), t.v01.b() + dms.b());
+  if (A == 2) t.v2t = dfloat2(t.v2t.a() + dms.b(), t.v2t.b());
+  if (A == 0) {  // D_x u1, D_x u2
+    t.a01 = g.a();
+    t.a02 = g.b();
+    if (WITH_KE) {
+      t.w01 = -g.a();
+      t.w02 = -g.b();
+    }
+  } else if (A == 1) {  // D_y u0, D_y u2
+    t.a01 = t.a01 + g.a();
+    t.a12 = g.b();
+    if (WITH_KE) {
+      t.w01 = t.w01 + g.a();
+      t.w12 = -g.b();
+    }
+  } else {  // D_z u0, D_z u1
+    t.a02 = t.a02 + g.a();
+    t.a12 = t.a12 + g.b();
+    if (WITH_KE) {
+      t.w02 = t.w02 + g.a();
+      t.w12 = t.w12 + g.b();
+    }
+  }
+}
+
+// Eqs. 1-3 from the terms, the centre record and the diagonal gradients
+// (d00, d11), d22 and d00 + d11.
+__device__ __forceinline__ void assemble_dw(const DwTerms& t, const dfloat2 (&cen)[NW], dfloat2 d01, dfloat d22,
+                                            dfloat d0p1, const Coef<dfloat>& c, dfloat (&R)[5]) {
+  const dfloat div = d0p1 + d22;
+  const dfloat hdiv = dw_scale(div, -0.5f);
+  R[0] = t.rho + (dfloat(1.0f, 0.0f) + cen[W_RHOP].a()) * hdiv;
+  const dfloat Ec = cen[W_M2H].b() - cen[W_RHOP].b();
+  const dfloat2 h2(hdiv);
+  const dfloat2 r01 = (t.m01 + cen[W_M01] * h2) + t.v01 * dfloat2(c.inv_re);
+  const dfloat2 r2e = (t.m2e + dfloat2(cen[W_M2H].a(), Ec) * h2) + t.v2t * dfloat2(c.inv_re, c.kappa);
+  R[1] = r01.a();
+  R[2] = r01.b();
+  R[3] = r2e.a();
+  // viscous dissipation and the work of the viscous force
+  const dfloat2 a0(t.a01, t.a02), dd(d22, t.a12);
+  const dfloat2 sq = (a0 * a0 + cen[W_U01] * t.v01) + dw_scale(d01 * d01, 2.0f);
+  const dfloat2 s2 = dd * dd;
+  dfloat q = (sq.a() + sq.b()) + (dw_scale(s2.a(), 2.0f) + s2.b());
+  q = q + (cen[W_U2T].a() * t.v2t.a() - dfloat(2.0 / 3.0) * div * div);
+  R[4] = r2e.b() + (c.inv_re * q - c.H0 * div);
 }
 
 // TIN: type of the stage input in HBM; TOUT: type of the stage output.
@@ -788,6 +864,7 @@ __device__ __forceinline__ void fused_march(const StageArgs& a, const Coef<T>& c
                                             uint32_t tmem_base = 0, uint32_t tmem_base2 = 0) {
   using S = FusedSmem<T, TY, ZT>;
   constexpr bool MIXZ = S::MIXZ;
+  constexpr bool DW = std::is_same<T, dfloat>::value;  // double-float: terms in pairs
   constexpr int SY = S::SY;
   constexpr int NT = TX * TY;
   constexpr int PTS = SX * SY;
@@ -969,7 +1046,7 @@ __device__ __forceinline__ void fused_march(const StageArgs& a, const Coef<T>& c
           rec[V_M0] = m0;
           rec[V_M1] = m1;
           rec[V_M2] = m2;
-          rec[V_H] = hrec<T>() ? E_p + p2 : E_p;
+          rec[V_H] = E_p + p2;
           rec[V_U0] = u0;
           rec[V_U1] = u1;
           rec[V_U2] = u2;
@@ -988,7 +1065,22 @@ __device__ __forceinline__ void fused_march(const StageArgs& a, const Coef<T>& c
     // --------------------------------------------------------------- phase 2a
     // in-plane diagonal gradients of the entering plane, kept for s_2 and
     // for the velocity gradient when the plane is the centre.
-    {
+    if constexpr (DW) {
+      const dfloat* r = &sm.ring[fe][ty + HALO][tx + HALO][0];
+      dfloat2 g[4];  // u0 of the x0 neighbours beside u1 of the x1 neighbours
+#pragma unroll
+      for (int k = 0; k < 4; ++k) {
+        const int o = k < 2 ? k - 2 : k - 1;
+        g[k] = dfloat2(rec_value(r + o * NV, V_U0), rec_value(r + o * SX * NV, V_U1));
+      }
+      const dfloat2 dg = dw_first(g[0], g[1], g[2], g[3], dfloat2(c.c2[0], c.c2[1]));
+      if constexpr (ZT) {
+        tmem_store_diag(twin, se, dg.a(), dg.b());  // this thread's column only
+      } else {
+        sm.dring[se][0][ty][tx] = dg.a();
+        sm.dring[se][1][ty][tx] = dg.b();
+      }
+    } else {
       const T(*R)[SX][NV] = sm.ring[fe];
       const int sy = ty + HALO, sx = tx + HALO;
       const T d00 = mad(c.c1[0], R[sy][sx + 1][V_U0] - R[sy][sx - 1][V_U0],
@@ -1094,13 +1186,46 @@ __device__ __forceinline__ void fused_march(const StageArgs& a, const Coef<T>& c
         g11c = sm.dring[scen][1][ty][tx];
       }
     } else {
-      const int sy = ty + HALO, sx = tx + HALO;
       auto u2at = [&](int slot, int yy, int xx) {
         if constexpr (ZT)
           return sm.u2ring[slot][yy][xx];
         else
-          return sm.ring[slot][yy][xx][V_U2];
+          return rec_value(&sm.ring[slot][yy][xx][0], V_U2);
       };
+      if constexpr (DW) {
+        const int sy = ty + HALO, sx = tx + HALO;
+        const int zs[4] = {sl[0], sl[1], sl[3], sl[4]};
+        if constexpr (ZT) {
+          tmem_load_diag(twin, scen, g00c, g11c);
+        } else {
+          g00c = sm.dring[scen][0][ty][tx];
+          g11c = sm.dring[scen][1][ty][tx];
+        }
+        d22 = (dw_scale(u2at(zs[2], sy, sx) - u2at(zs[1], sy, sx), 8.0f) - (u2at(zs[3], sy, sx) - u2at(zs[0], sy, sx))) *
+              c.c2[2];
+        const dfloat2 s = dfloat2(g11c, g00c) + dfloat2(d22);
+        sm.s0buf[0][ty][sx] = s.a();
+        sm.s1buf[0][sy][tx] = s.b();
+        const dfloat* R = &sm.ring[fc][0][0][0];
+#pragma unroll
+        for (int j = 0; j < HPT; ++j) {
+          if (hk[j] == 0) continue;
+          // kind 1: D1_y u1 (s_0), kind 2: D1_x u0 (s_1), beside D1_z u2
+          const int hy = hxy[j] >> 8, hx = hxy[j] & 0xFF;
+          const bool k1 = hk[j] == 1;
+          const dfloat* q = R + (hy * SX + hx) * NV;
+          const int st = NV * (k1 ? SX : 1);
+          dfloat2 g[4];
+#pragma unroll
+          for (int k = 0; k < 4; ++k) {
+            const dfloat2 v = load_pair(q + (k < 2 ? k - 2 : k - 1) * st, W_U01);
+            g[k] = dfloat2(k1 ? v.b() : v.a(), u2at(zs[k], hy, hx));
+          }
+          const dfloat2 dg = dw_first(g[0], g[1], g[2], g[3], dfloat2(k1 ? c.c2[1] : c.c2[0], c.c2[2]));
+          (k1 ? &sm.s0buf[0][0][0] : &sm.s1buf[0][0][0])[hdst[j]] = dg.a() + dg.b();
+        }
+      } else {
+      const int sy = ty + HALO, sx = tx + HALO;
       auto u2z = [&](int yy, int xx) {
         return mad(c.c1[2], u2at(sl[3], yy, xx) - u2at(sl[1], yy, xx),
                    -c.c2[2] * (u2at(sl[4], yy, xx) - u2at(sl[0], yy, xx)));
@@ -1128,6 +1253,7 @@ __device__ __forceinline__ void fused_march(const StageArgs& a, const Coef<T>& c
           (&sm.s1buf[0][0][0])[hdst[j]] = d00 + u2z(hy, hx);
         }
       }
+      }
       __syncthreads();
     }
     // ---------------------------------------------------------------- phase 3
@@ -1135,31 +1261,14 @@ __device__ __forceinline__ void fused_march(const StageArgs& a, const Coef<T>& c
       fetch_acc();
       const int sy = ty + HALO, sx = tx + HALO;
       const T(*C)[SX][NV] = sm.ring[fc];
-      T cen[NV];
-      if constexpr (ZT)
-        tmem_load_rec(twin, scen, cen);
-      else
-        load_rec(&C[sy][sx][0], cen);
-      const T rho_p = cen[V_RHO];
-      const T mc[3] = {cen[V_M0], cen[V_M1], cen[V_M2]};
-      const T Ec = hrec<T>() ? cen[V_H] - cen[V_P] : cen[V_E];
-      const T uc[3] = {cen[V_U0], cen[V_U1], cen[V_U2]};
-      const T Tc = cen[V_T];
+      T rho_p, mc[3], uc[3];  // centre values
 
       // neighbours k = 0..3 (offsets -2, -1, +1, +2): records and mixed-term helpers
       const int sbc = MIXZ ? rb[0] : 0;  // helper buffers of the centre plane
       const int off[4] = {-2, -1, 1, 2};
       const int zs[4] = {sl[0], sl[1], sl[3], sl[4]};
-      auto ld0 = [&](int k, T(&r)[NV]) { load_rec(&C[sy][sx + off[k]][0], r); };
       auto sf0 = [&](int k) { return sm.s0buf[sbc][ty][sx + off[k]]; };
-      auto ld1 = [&](int k, T(&r)[NV]) { load_rec(&C[sy + off[k]][sx][0], r); };
       auto sf1 = [&](int k) { return sm.s1buf[sbc][sy + off[k]][tx]; };
-      auto ld2 = [&](int k, T(&r)[NV]) {
-        if constexpr (ZT)
-          tmem_load_rec(twin, zs[k], r);
-        else
-          load_rec(&sm.ring[zs[k]][sy][sx][0], r);
-      };
       auto sf2 = [&](int k) {
         if constexpr (ZT) {
           T a, b;
@@ -1184,27 +1293,63 @@ __device__ __forceinline__ void fused_march(const StageArgs& a, const Coef<T>& c
       T R[5];
       T w0 = T(0), w1 = T(0), w2 = T(0);  // vorticity (WITH_KE)
       // x0 group first (SN2 ordering), then x1, x2
-      if constexpr (std::is_same<T, dfloat>::value) {
-        Terms<T> t;
-        t.rrho = t.rE = t.lapT = T(0);
-#pragma unroll
-        for (int i = 0; i < 3; ++i) {
-          t.rM[i] = T(0);
-          t.lap[i] = T(0);
-        }
-        t.g[0][0] = g00c;
-        t.g[1][1] = g11c;
-        t.g[2][2] = d22;
-        axis_terms<0>(ld0, sf0, c, uc, t);
-        axis_terms<1>(ld1, sf1, c, uc, t);
-        axis_terms<2>(ld2, sf2, c, uc, t);
-        assemble_residual(t, rho_p, mc, Ec, uc, Tc, c, R);
+      if constexpr (DW) {
+        auto lp0 = [&](int k, dfloat2(&r)[NW]) { load_pairs(&C[sy][sx + off[k]][0], r); };
+        auto lp1 = [&](int k, dfloat2(&r)[NW]) { load_pairs(&C[sy + off[k]][sx][0], r); };
+        auto lp2 = [&](int k, dfloat2(&r)[NW]) {
+          if constexpr (ZT)
+            tmem_load_pairs(twin, zs[k], r);
+          else
+            load_pairs(&sm.ring[zs[k]][sy][sx][0], r);
+        };
+        dfloat2 cen[NW];
+        if constexpr (ZT)
+          tmem_load_pairs(twin, scen, cen);
+        else
+          load_pairs(&C[sy][sx][0], cen);
+        const dfloat ua[3] = {cen[W_U01].a(), cen[W_U01].b(), cen[W_U2T].a()};
+        DwTerms t;
+        t.m01 = t.m2e = dfloat2(dfloat(0.0f, 0.0f));
+        t.rho = dfloat(0.0f, 0.0f);
+        t.v01 = dfloat2(c.v0[0], c.v0[1]) * cen[W_U01];
+        t.v2t = dfloat2(c.v0[2], c.e0s) * cen[W_U2T];
+        axis_terms_dw<0, WITH_KE>(lp0, sf0, c, ua[0], t);
+        axis_terms_dw<1, WITH_KE>(lp1, sf1, c, ua[1], t);
+        axis_terms_dw<2, WITH_KE>(lp2, sf2, c, ua[2], t);
+        assemble_dw(t, cen, dfloat2(g00c, g11c), d22, g00c + g11c, c, R);
         if (WITH_KE) {
-          w0 = t.g[2][1] - t.g[1][2];
-          w1 = t.g[0][2] - t.g[2][0];
-          w2 = t.g[1][0] - t.g[0][1];
+          rho_p = cen[W_RHOP].a();
+          mc[0] = cen[W_M01].a();
+          mc[1] = cen[W_M01].b();
+          mc[2] = cen[W_M2H].a();
+#pragma unroll
+          for (int i = 0; i < 3; ++i) uc[i] = ua[i];
+          w0 = t.w12;  // squared below: the sign does not matter
+          w1 = t.w02;
+          w2 = t.w01;
         }
       } else {
+        auto ld0 = [&](int k, T(&r)[NV]) { load_rec(&C[sy][sx + off[k]][0], r); };
+        auto ld1 = [&](int k, T(&r)[NV]) { load_rec(&C[sy + off[k]][sx][0], r); };
+        auto ld2 = [&](int k, T(&r)[NV]) {
+          if constexpr (ZT)
+            tmem_load_rec(twin, zs[k], r);
+          else
+            load_rec(&sm.ring[zs[k]][sy][sx][0], r);
+        };
+        T cen[NV];
+        if constexpr (ZT)
+          tmem_load_rec(twin, scen, cen);
+        else
+          load_rec(&C[sy][sx][0], cen);
+        rho_p = cen[V_RHO];
+        const T Ec = cen[V_H] - cen[V_P];
+        const T Tc = cen[V_T];
+#pragma unroll
+        for (int i = 0; i < 3; ++i) {
+          mc[i] = cen[V_M0 + i];
+          uc[i] = cen[V_U0 + i];
+        }
         StreamTerms<T> t;
         t.rrho = t.rE = T(0);
         t.lapT = c.e0s * Tc;
