@@ -570,6 +570,14 @@ __device__ __forceinline__ double fmadd(double a, double b, double c) { return :
 __device__ __forceinline__ float fmadd(float a, float b, float c) { return ::fmaf(a, b, c); }
 __device__ __forceinline__ f32x2 fmadd(f32x2 a, f32x2 b, f32x2 c) { return fma(a, b, c); }
 
+// a + b, never contracted with the product that formed b
+__device__ __forceinline__ double add_nc(double a, double b) { return __dadd_rn(a, b); }
+__device__ __forceinline__ float add_nc(float a, float b) { return __fadd_rn(a, b); }
+template <typename T>
+__device__ __forceinline__ T add_nc(T a, T b) {
+  return a + b;
+}
+
 // Accumulated terms of the residual at one point for the hardware FMA types.
 // The centre values u_j^c, m_i^c are constant over a stencil, so the
 // convective terms of Eqs. 2-3 share the weight w = c (u_j + u_j^c) and
@@ -983,9 +991,10 @@ __device__ __forceinline__ void fused_march(const StageArgs& a, const Coef<T>& c
   // binary32 helper-buffer slots of planes e-2, e-1, e
   int rb[3] = {1, 2, 0};
 
-  TIN pf[LPT][NF][PP];
+  using Loads = TIN[LPT][NF][PP];
+  Loads pf;
   int zl = wrapi(zbeg - HALO, n2);  // next plane to load (periodic), advanced one plane per load
-  auto issue_loads = [&]() {
+  auto issue_loads = [&](Loads& pf) {
     const unsigned zoff = (unsigned)zl * plane;
     zl = (zl + 1 == n2) ? 0 : zl + 1;
 #pragma unroll
@@ -1000,32 +1009,32 @@ __device__ __forceinline__ void fused_march(const StageArgs& a, const Coef<T>& c
       }
     }
   };
-  issue_loads();
 
-  for (int it = 0; it < nit; ++it) {
-    // ---------------------------------------------------------------- phase 1
-    // plane e = zbeg - 2 + it enters slot it % 5: derive primitives (Eqs. 4-5
-    // in deviation form) on the haloed tile from the prefetched Q'.
+  // A plane enters in three parts.  Its slots:
+  auto rotate = [&]() {
     {
       const int t0 = rs[0];
 #pragma unroll
       for (int k = 0; k < NSLOT - 1; ++k) rs[k] = rs[k + 1];
       rs[NSLOT - 1] = t0;
     }
-    const int se = rs[NSLOT - 1];
     if constexpr (ZT) {
       const int t0 = rf[0];
 #pragma unroll
       for (int k = 0; k < NFULL - 1; ++k) rf[k] = rf[k + 1];
       rf[NFULL - 1] = t0;
     }
-    const int fe = ZT ? rf[ZT ? NFULL - 1 : 0] : se;  // full-record slot of the entering plane
     if constexpr (MIXZ) {
       const int t0 = rb[0];
       rb[0] = rb[1];
       rb[1] = rb[2];
       rb[2] = t0;
     }
+  };
+  // ---------------------------------------------------------------- phase 1
+  // derive primitives (Eqs. 4-5 in deviation form) on the haloed tile from the
+  // loaded Q' into ring slot se (full-record slot fe).
+  auto convert = [&](const Loads& pf, int se, int fe) {
     {
       T* ring = &sm.ring[fe][0][0][0];
 #pragma unroll
@@ -1046,7 +1055,7 @@ __device__ __forceinline__ void fused_march(const StageArgs& a, const Coef<T>& c
           rec[V_M0] = m0;
           rec[V_M1] = m1;
           rec[V_M2] = m2;
-          rec[V_H] = E_p + p2;
+          rec[V_H] = add_nc(E_p, p2);
           rec[V_U0] = u0;
           rec[V_U1] = u1;
           rec[V_U2] = u2;
@@ -1060,11 +1069,11 @@ __device__ __forceinline__ void fused_march(const StageArgs& a, const Coef<T>& c
         }
       }
     }
-    if (it + 1 < nit) issue_loads();
-    __syncthreads();
-    // --------------------------------------------------------------- phase 2a
-    // in-plane diagonal gradients of the entering plane, kept for s_2 and
-    // for the velocity gradient when the plane is the centre.
+  };
+  // --------------------------------------------------------------- phase 2a
+  // in-plane diagonal gradients of the entering plane, kept for s_2 and
+  // for the velocity gradient when the plane is the centre.
+  auto gradients = [&](int se, int fe, int sbe) {
     if constexpr (DW) {
       const dfloat* r = &sm.ring[fe][ty + HALO][tx + HALO][0];
       dfloat2 g[4];  // u0 of the x0 neighbours beside u1 of the x1 neighbours
@@ -1123,7 +1132,6 @@ __device__ __forceinline__ void fused_march(const StageArgs& a, const Coef<T>& c
           sm.dring[se][2][ty][tx] = d02;
           sm.dring[se][3][ty][tx] = d12;
         }
-        const int sbe = rb[2];
         sm.s0buf[sbe][ty][sx] = d11;
         sm.s1buf[sbe][sy][tx] = d00;
 #pragma unroll
@@ -1139,6 +1147,46 @@ __device__ __forceinline__ void fused_march(const StageArgs& a, const Coef<T>& c
         }
       }
     }
+  };
+  auto full_slot = [&]() { return ZT ? rf[ZT ? NFULL - 1 : 0] : rs[NSLOT - 1]; };  // of the entering plane
+
+  // The first FILL planes enter together: their loads are in flight at the same
+  // time and two barriers serve them all, where one plane after another paid
+  // the latency of memory and of both phases for each.  Double-float 256^3 2.204
+  // -> 2.091 ms a stage, 64^3 44.6 -> 42.3 us (the same code shape schedules
+  // better in its full iterations too), binary64 and binary32 rings 1 to 4 % at
+  // 16^3 ... 40^3.  Two columns per thread have no registers for it, nor has
+  // the binary32 TMEM queue at 80 (spills in the batch kernel, 0.3 % on 256^3).
+  constexpr int FILL = PP == 2 || (sizeof(T) == 4 && ZT) ? 0 : (ZT ? 3 : 4);
+  if constexpr (FILL > 0) {
+    Loads pb[FILL > 0 ? FILL : 1];
+    int se[FILL > 0 ? FILL : 1], fe[FILL > 0 ? FILL : 1], sbe[FILL > 0 ? FILL : 1];
+#pragma unroll
+    for (int p = 0; p < FILL; ++p) issue_loads(pb[p]);
+#pragma unroll
+    for (int p = 0; p < FILL; ++p) {
+      rotate();
+      se[p] = rs[NSLOT - 1];
+      fe[p] = full_slot();
+      sbe[p] = rb[2];
+      convert(pb[p], se[p], fe[p]);
+    }
+    issue_loads(pf);
+    __syncthreads();
+#pragma unroll
+    for (int p = 0; p < FILL; ++p) gradients(se[p], fe[p], sbe[p]);
+    if constexpr (ZT) __syncthreads();  // the next plane's records replace the first one's
+  } else {
+    issue_loads(pf);
+  }
+
+  for (int it = FILL; it < nit; ++it) {
+    // plane e = zbeg - 2 + it enters
+    rotate();
+    convert(pf, rs[NSLOT - 1], full_slot());
+    if (it + 1 < nit) issue_loads(pf);
+    __syncthreads();
+    gradients(rs[NSLOT - 1], full_slot(), rb[2]);
     if (it < 4) continue;  // ring not yet full; slots written so far are not read again before the next sync
 
     const int zc = zbeg + it - 4;  // centre plane
