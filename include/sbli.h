@@ -212,7 +212,8 @@ SBLI_API int sbli_kinetic_energy_noalloc(const double* q_dev, int n0, int n1, in
  * is 32 x tile_y points per column a thread owns; binary64-register grids
  * (SBLI_FP64, SBLI_DF64) use 8, binary32 grids 8 or 16), planes per CTA
  * along x2 (>= 4; binary64-register grids split all planes evenly over the SMs
- * instead where that leaves the longest CTA fewer of them), where each thread keeps its column's records of the five
+ * instead where that leaves the longest CTA fewer of them, and 4 lets binary32
+ * grids too small to give every SM a CTA take fewer), where each thread keeps its column's records of the five
  * x2 planes (z_queue = 0: the shared-memory ring; 1: a per-thread queue in
  * Blackwell tensor memory, with only three full-record planes in shared
  * memory -- four for binary32 tile_y 16, which saves one barrier per plane)
@@ -265,7 +266,8 @@ SBLI_API int sbli_batch_work_items(const sbli_batch* b, long long* items);
  * and each member's planes per work item (planes_per_item[count]: the z chunk
  * a CTA marches through; >= 4, clamped to the member's n2).  A batch starts
  * with the TMEM queue for binary32 precisions and the ring otherwise, and
- * min(n2, 32) planes per item.  Every schedule gives bitwise the same
+ * min(n2, 32) planes per item, an upper bound as long as the schedule is not set:
+ * members too small to fill the GPU take fewer.  Every schedule gives bitwise the same
  * results.  Members of the binary64-register precisions are split evenly over
  * the CTAs whatever their planes per item.  set_schedule (between steps; SBLI_EINVAL for z_queue outside 0..1
  * or fewer than 4 planes) drops the captured step graphs; planes_per_item may
@@ -276,7 +278,7 @@ SBLI_API int sbli_batch_set_schedule(sbli_batch* b, int z_queue, const int* plan
  * the accumulator they write equals the state they read, so a state updated
  * in place keeps its value, and the stage field goes to a free register) of
  * every z_queue mode with one planes-per-item value for all
- * members (8, 16, 32, 64, 128, whole member), then refines the planes per
+ * members (4, 8, 16, 32, 64, 128, whole member), then refines the planes per
  * item of each size class (members with the same n2) in turn, and keeps the
  * fastest schedule (if a trial launch fails, the schedule in place before
  * the call is restored and SBLI_ECUDA returned).  The state is not

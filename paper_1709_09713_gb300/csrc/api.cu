@@ -60,10 +60,8 @@ bool valid_sizes(int n0, int n1, int n2) {
   return true;
 }
 
-FusedConfig default_config(const Geom& g, int precision);
+FusedConfig default_config(const Geom& g, int precision, int sms);
 
-// most CTAs (one per SM) the even split of a binary64-register grid may use
-constexpr int MAX_EVEN_CTAS = 512;
 
 // binary64 state, accumulator and stage registers (three-register rotation)
 bool f64_registers(int precision) { return precision == SBLI_FP64 || precision == SBLI_DF64; }
@@ -79,7 +77,7 @@ Layout layout_for(int n0, int n1, int n2, int precision, int variant) {
   // use (the smallest zc gives the most CTAs), or the KE kernel's blocks
   const long long tiles = (long long)((n0 + 31) / 32) * ((n1 + 3) / 4);
   const long long max_ctas = tiles * ((n2 + 3) / 4);
-  const long long np = std::max<long long>(std::max<long long>(max_ctas, ke_num_partials(g)), MAX_EVEN_CTAS);
+  const long long np = std::max<long long>(std::max<long long>(max_ctas, ke_num_partials(g)), MAX_SMALL_CTAS);
   L.partials = align_up((size_t)(2 * np + 2) * sizeof(double));
   L.storeall = variant == SBLI_STORE_ALL
                    ? align_up(storeall_scratch_doubles(g, precision == SBLI_FP64 ? 8 : 4) * sizeof(double))
@@ -113,6 +111,7 @@ struct sbli_grid {
   long long stages_done;
   FusedConfig cfg;
   int sms;      // SMs of the device
+  int zc;       // planes per CTA of a launch (cfg.zc, or fewer on small binary32 grids)
   Split split;  // binary64-register grids: the work split of cfg
   Coef<double> cd;
   Coef<float> cf;
@@ -182,10 +181,17 @@ void rank_zc(const Geom& g, int precision, int ty, int* best, int nbest, int px 
 
 void use_config(sbli_grid* g, const FusedConfig& cfg) {
   g->cfg = cfg;
-  if (f64_registers(g->precision)) g->split = plan_split(g->geom, cfg.zc, g->sms, g->precision == SBLI_DF64);
+  g->zc = cfg.zc;
+  if (f64_registers(g->precision))
+    g->split = plan_split(g->geom, cfg.zc, g->sms, g->precision == SBLI_DF64);
+  else
+    g->zc = binary32_launch_zc(g->geom, cfg, g->sms);
 }
 
-FusedConfig default_config(const Geom& g, int precision) {
+// Binary32 grids: z queue and planes per CTA by the model of their stage (us a
+// stage, shared ring with planes by waves -> this: 128^3 96.7 -> 70.4, 96^3 35.8 ->
+// 33.7, 40^3 9.3 -> 7.8, 32^3 9.2 -> 4.8).
+FusedConfig default_config(const Geom& g, int precision, int sms) {
   FusedConfig cfg;
   cfg.ty = 8;
   cfg.zq = 0;
@@ -193,6 +199,19 @@ FusedConfig default_config(const Geom& g, int precision) {
   int zc[1];
   rank_zc(g, precision, cfg.ty, zc, 1);
   cfg.zc = std::max(4, std::min(zc[0], g.n2));
+  if (f64_registers(precision)) return cfg;
+  double best = 0.0;
+  FusedConfig c = cfg;
+  for (c.zq = 0; c.zq < 2; ++c.zq)
+    for (c.zc = 4; c.zc <= std::max(4, g.n2); ++c.zc) {
+      FusedConfig launch = c;
+      launch.zc = binary32_launch_zc(g, c, sms);
+      const double us = binary32_stage_us(fused_num_ctas(g, launch), launch.zc, c.zq, sms);
+      if (best == 0.0 || us < best) {
+        best = us;
+        cfg = c;
+      }
+    }
   return cfg;
 }
 
@@ -294,7 +313,7 @@ cudaError_t enqueue_stage(sbli_grid* g, int k, int state, double dt, double* ke_
   if (g->variant == SBLI_FUSED) {
     StageArgs a{};
     a.g = g->geom;
-    a.zc = g->cfg.zc;
+    a.zc = g->zc;
     a.ctas = g->split.ctas;
     a.even = g->split.even;
     a.q_in = p.q_in;
@@ -444,8 +463,8 @@ int sbli_create_grid(sbli_grid** out, int n0, int n1, int n2, int precision, int
   g->stages_done = 0;
   int dev = 0, sms = 152;
   if (cudaGetDevice(&dev) == cudaSuccess) cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-  g->sms = std::min(sms, MAX_EVEN_CTAS);
-  use_config(g, default_config(g->geom, precision));
+  g->sms = std::min(sms, MAX_SMALL_CTAS);
+  use_config(g, default_config(g->geom, precision, g->sms));
   g->cd = make_coef<double>(g->n, p);
   g->cf = make_coef<float>(g->n, p);
   g->cw = make_coef<dfloat>(g->n, p);
@@ -608,7 +627,7 @@ int sbli_rhs(sbli_grid* g, double* r_dev) {
   if (g->variant == SBLI_FUSED) {
     StageArgs a{};
     a.g = g->geom;
-    a.zc = g->cfg.zc;
+    a.zc = g->zc;
     a.ctas = g->split.ctas;
     a.even = g->split.even;
     a.q_in = q;
@@ -678,7 +697,9 @@ int sbli_step_n_history(sbli_grid* g, int nsteps, double dt, double* ke_hist_dev
   if (!(dt > 0) || !isfinite(dt)) return fail(SBLI_EINVAL, "dt must be finite and > 0");
   if (g->next_stage != 0) return fail(SBLI_EINVAL, "step_n_history must start at a step boundary");
   if (g->variant != SBLI_FUSED) return fail(SBLI_EUNSUPPORTED, "history needs the fused variant");
-  const int nctas = f64_registers(g->precision) ? g->split.ctas : fused_num_ctas(g->geom, g->cfg);
+  FusedConfig launch = g->cfg;
+  launch.zc = g->zc;
+  const int nctas = f64_registers(g->precision) ? g->split.ctas : fused_num_ctas(g->geom, launch);
   for (int s = 0; s < nsteps; ++s) {
     SBLI_TRY(enqueue_stage(g, 0, g->state, dt, g->partials, g->stream), "stage launch");
     SBLI_TRY(launch_finalize_ke(g->partials, nctas, 1.0 / (double)g->geom.P, ke_hist_dev + 2 * s, g->stream),

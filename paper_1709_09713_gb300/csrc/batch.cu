@@ -181,6 +181,7 @@ size_t balign(size_t v) { return (v + BALIGN - 1) / BALIGN * BALIGN; }
 struct MemberLayout {
   int n[3];
   int zc;  // planes per work item (the schedule; batch_zc at creation)
+  int launch_zc;  // planes per item of a launch: zc, or under the default schedule at most batch_zc_cap
   long long P;
   size_t off64, off32;  // byte offsets inside the binary64 / binary32 register regions
 };
@@ -207,7 +208,7 @@ BatchLayout batch_layout(int count, const int* n, int precision) {
     MemberLayout& M = L.m[i];
     for (int a = 0; a < 3; ++a) M.n[a] = n[3 * i + a];
     M.P = (long long)M.n[0] * M.n[1] * M.n[2];
-    M.zc = batch_zc(M.n[2]);
+    M.zc = M.launch_zc = batch_zc(M.n[2]);
     M.off64 = o64;
     M.off32 = o32;
     o64 += balign((size_t)M.P * 5 * sizeof(double));
@@ -221,7 +222,7 @@ BatchLayout batch_layout(int count, const int* n, int precision) {
   // partials: one per work item, or (even split) one per CTA and member
   L.items_bytes = balign((size_t)(2 * std::max<long long>(L.total_items, BATCH_MAX_EVEN_CTAS + count) + 2) * sizeof(double));
   L.total_items = 0;
-  for (const MemberLayout& M : L.m) L.total_items += member_items(M.n, M.zc);
+  for (const MemberLayout& M : L.m) L.total_items += member_items(M.n, M.zc);  // set again with the ranges
   // per member: KE result pair, 1/P, range of partials; plus the KE kernel partials
   L.misc_bytes = balign((size_t)count * 2 * sizeof(double)) + balign((size_t)count * sizeof(double)) +
                  balign((size_t)(2 * count) * sizeof(long long)) + balign(2 * 1024 * sizeof(double));
@@ -274,7 +275,7 @@ StageArgs member_stage(const sbli_batch* b, int m, int k, int state, double dt, 
   const MemberLayout& M = b->L.m[m];
   StageArgs a{};
   a.g = member_geom(M);
-  a.zc = M.zc;
+  a.zc = M.launch_zc;
   a.a_dt = RK_A[k] * dt;
   a.b_dt = RK_B[k] * dt;
   a.amb_dt = (RK_A[k] - RK_B[k]) * dt;
@@ -339,7 +340,7 @@ cudaError_t enqueue_batch_stage_t(sbli_batch* b, int k, int state, double dt, do
     p.item_begin[m] = acc;
     p.tiles_x[m] = (M.n[0] + TX - 1) / TX;
     p.tiles_y[m] = (M.n[1] + 7) / 8;
-    acc += batch_f64_registers(b->precision) ? member_planes(M.n) : member_items(M.n, M.zc);
+    acc += batch_f64_registers(b->precision) ? member_planes(M.n) : member_items(M.n, M.launch_zc);
     p.a[m] = member_stage(b, m, k, state, dt, &in64);
     p.c[m] = make_coef<T>(M.n, b->params[m]);
   }
@@ -413,9 +414,9 @@ cudaError_t upload_ranges(sbli_batch* b) {
       range[2 * m + 1] = cta_of(at - 1) + m + 1;
     } else {
       range[2 * m] = items;
-      range[2 * m + 1] = items + member_items(M.n, M.zc);
+      range[2 * m + 1] = items + member_items(M.n, M.launch_zc);
     }
-    items += member_items(M.n, M.zc);
+    items += member_items(M.n, M.launch_zc);
   }
   b->L.total_items = items;
   cudaError_t e = cudaMemcpyAsync(b->range, range.data(), range.size() * sizeof(long long), cudaMemcpyHostToDevice,
@@ -431,7 +432,7 @@ cudaError_t apply_schedule(sbli_batch* b, int zq, const std::vector<int>& zc) {
   if (cudaGetDevice(&dev) == cudaSuccess) cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
   b->zq = zq;
   b->grid_ctas = batch_grid_ctas(sms, b->precision, zq);
-  for (int m = 0; m < b->count; ++m) b->L.m[m].zc = zc[m];
+  for (int m = 0; m < b->count; ++m) b->L.m[m].zc = b->L.m[m].launch_zc = zc[m];
   batch_drop_graphs(b);
   return upload_ranges(b);
 }
@@ -506,6 +507,11 @@ int sbli_batch_create(sbli_batch** out, int count, const int* n, const sbli_para
   cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
   b->zq = batch_default_zq(precision);
   b->grid_ctas = batch_grid_ctas(sms, precision, b->zq);
+  if (!batch_f64_registers(precision)) {
+    const int cap = batch_zc_cap(
+        count, [&](int m) { return b->L.m[m].n; }, b->zq, sms);
+    for (MemberLayout& M : b->L.m) M.launch_zc = std::min(M.zc, cap);
+  }
   // per-member constants for the KE finalisation
   std::vector<double> inv(count);
   for (int m = 0; m < count; ++m) inv[m] = 1.0 / (double)b->L.m[m].P;
@@ -733,7 +739,7 @@ int sbli_batch_autotune(sbli_batch* b, int reps, int* z_queue, float* best_stage
     for (int m = 0; m < b->count; ++m) zc[m] = std::max(4, std::min(Z, b->L.m[m].n[2]));
     return zc;
   };
-  const int Zs[6] = {8, 16, 32, 64, 128, 1 << 24};
+  const int Zs[7] = {4, 8, 16, 32, 64, 128, 1 << 24};
   // 1. one z-queue mode and one planes-per-item value for every member
   int best_zq = b->zq;
   std::vector<int> best_zc(b->count);

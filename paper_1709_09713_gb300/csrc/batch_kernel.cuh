@@ -60,9 +60,33 @@ inline int batch_zc(int n2) { return n2 < 32 ? n2 : 32; }
 inline long long member_items(const int n[3], int zc) {
   return (long long)((n[0] + 31) / 32) * ((n[1] + 7) / 8) * ((n[2] + zc - 1) / zc);
 }
-inline long long member_items(const int n[3]) { return member_items(n, batch_zc(n[2])); }
 // Planes of all tiles of one member: the units of the even split.
 inline long long member_planes(const int n[3]) { return member_items(n, 1); }
+
+// Binary32 members under the default schedule: the cap on the planes per item
+// (32, 16, 8 or 4; a member's own are batch_zc) that the model of a stage
+// (binary32_stage_us) ranks best, so that a few small members fill the GPU too.
+// edges(m) is member m's (n0, n1, n2).  Two 64^3 members are 64 items of 32
+// planes, one for every other of 152 SMs with room for three each, but 256 of 8.
+template <typename F>
+int batch_zc_cap(int count, const F& edges, int zq, int sms) {
+  int best = 32;
+  double cost = 0.0;
+  for (int cap = 32; cap >= 4; cap /= 2) {
+    long long items = 0;
+    for (int m = 0; m < count; ++m) {
+      const int* n = edges(m);
+      const int zc = batch_zc(n[2]);
+      items += member_items(n, zc < cap ? zc : cap);
+    }
+    const double us = binary32_stage_us(items, cap, zq, sms);
+    if (cap == 32 || us < cost) {
+      cost = us;
+      best = cap;
+    }
+  }
+  return best;
+}
 
 // Per member m: fixed-order sum of partials [range[2m], range[2m+1]) times inv_p[m].
 cudaError_t launch_batch_ke_finalize(const double* items, const long long* range, const double* inv_p, double* out,

@@ -58,11 +58,41 @@ int fused_num_ctas(const Geom& g, const FusedConfig& cfg) {
   return (int)(gx * gy * gz);
 }
 
-// The longest CTA decides, in planes, each march's four warm-up planes
-// counting WARM of a plane (their primitives) each.  A plane of the even split
-// costs double-float kernels up to 9 % more (its CTAs share no halos in L2): 256^3
-// 2.500 ms a stage against 2.456 in chunks of 64 planes, 129 x 97 x 66 179
-// against 176 us, but 32^3 11.0 against 26.4.  Binary64: 256^3 8.84 against 9.24
+// Measured at 16^3 ... 160^3 (binary64 accumulator; the double-float one ranks
+// alike): a plane takes 1.47 us with one CTA on an SM, 2.5 with two, 3.3 with
+// three (TMEM queue, which also pays 0.6 us for its allocation), the fill of a
+// march 1.5 planes, a launch 1 us; CTAs go to SMs one each first.  Within 8 % of
+// the measured time over both queues and 1 to 40 planes per CTA.
+double binary32_stage_us(long long ctas, int zc, int zq, int sms) {
+  const double plane[2][4] = {{0.0, 1.47, 2.5, 2.5}, {0.0, 1.5, 2.4, 3.3}};
+  const int most = zq ? 3 : 2;
+  const long long slots = (long long)sms * most;
+  const long long full = ctas / slots, rest = ctas % slots;
+  const int last = (int)((rest + sms - 1) / sms);
+  return (zq ? 1.6 : 1.0) + (zc + 1.5) * ((double)full * plane[zq][most] + plane[zq][last]);
+}
+
+int binary32_launch_zc(const Geom& g, const FusedConfig& cfg, int sms) {
+  if (cfg.zc != 4 || cfg.ty != 8 || cfg.px != 1) return cfg.zc;
+  FusedConfig c = cfg;
+  int best = 4;
+  double cost = binary32_stage_us(fused_num_ctas(g, cfg), 4, cfg.zq, sms);
+  for (c.zc = 3; c.zc >= 1; --c.zc) {
+    const int ctas = fused_num_ctas(g, c);
+    const double us = binary32_stage_us(ctas, c.zc, cfg.zq, sms);
+    if (ctas <= MAX_SMALL_CTAS && us < cost) {
+      cost = us;
+      best = c.zc;
+    }
+  }
+  return best;
+}
+
+// The longest CTA decides, in planes, each march's four fill planes counting
+// WARM of a plane (their primitives) each.  A plane of the even split costs
+// double-float kernels some percent more (its CTAs share no halos in L2): 64^3
+// 43.7 us a stage against 42.2 in chunks of 8 planes, 256^3 2.109 ms against
+// 2.116 in chunks of 64, 32^3 10.2 against 26.  Binary64: 256^3 8.84 against 9.24
 // ms, 128^3 1.130 against 1.202, 64^3 168 against 177 us, 32^3 33.7 against 94.9.
 Split plan_split(const Geom& g, int zc, int sms, bool double_float) {
   constexpr double WARM = 0.12;

@@ -83,6 +83,11 @@ struct StageArgs {
   int even;          // binary64-register kernels: the CTAs split the planes evenly (else chunks of zc)
 };
 
+// CTAs (partial sums of the diagnostics) a grid of any size has room for: the
+// even split of a binary64-register grid and binary32 launches of fewer than
+// four planes per CTA stay within it.
+constexpr int MAX_SMALL_CTAS = 512;
+
 // Launch configuration chosen for one grid (the autotuner's output).
 struct FusedConfig {
   int ty;  // in-plane tile height (tile is 32 x ty)
@@ -116,6 +121,13 @@ cudaError_t launch_fused_fp32_pair(const StageArgs& a, const Coef<float>& c, con
 cudaError_t launch_fused_fp32_tmem(const StageArgs& a, const Coef<float>& c, const FusedConfig& cfg, bool in_fp64,
                                    bool df, bool rhs_only, cudaStream_t s);
 int fused_num_ctas(const Geom& g, const FusedConfig& cfg);
+// Time in us of a binary32 stage of `ctas` CTAs of zc planes each (32 x 8 tiles,
+// one column per thread), from measured times of a plane at one, two and three
+// CTAs an SM.
+double binary32_stage_us(long long ctas, int zc, int zq, int sms);
+// Planes per CTA of a binary32 launch configured with zc: fewer than the
+// smallest configurable 4 on grids too small to give every SM a CTA otherwise.
+int binary32_launch_zc(const Geom& g, const FusedConfig& cfg, int sms);
 // CTAs of a binary64-register stage and whether they split the planes evenly (else chunks of zc planes)
 struct Split {
   int ctas, even;

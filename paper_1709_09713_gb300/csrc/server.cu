@@ -23,6 +23,7 @@
 #include <string.h>
 
 #include <algorithm>
+#include <array>
 #include <chrono>
 #include <deque>
 #include <map>
@@ -156,7 +157,7 @@ struct sbli_server {
   std::deque<Req> done;
   long long next_id = 0;
   long long ticks = 0;
-  int grid64, grid32;
+  int grid64, grid32, sms;
   Lane lane[2];  // 0: binary64-register precisions on s64; 1: binary32 precisions on s32
   std::chrono::steady_clock::time_point t0;
   double now() const { return std::chrono::duration<double>(std::chrono::steady_clock::now() - t0).count(); }
@@ -171,10 +172,10 @@ float* r32(const sbli_server* s, const Req& q, int r) {
   return reinterpret_cast<float*>(s->arena + q.off + 2 * q.reg64 + (size_t)r * q.reg32);
 }
 
-StageArgs req_stage(const sbli_server* s, const Req& q, int k, bool* in64) {
+StageArgs req_stage(const sbli_server* s, const Req& q, int k, int zc, bool* in64) {
   StageArgs a{};
   a.g = Geom{q.r.n0, q.r.n1, q.r.n2, q.P};
-  a.zc = batch_zc(q.r.n2);
+  a.zc = zc;
   a.a_dt = RK_A[k] * q.r.dt;
   a.b_dt = RK_B[k] * q.r.dt;
   a.amb_dt = (RK_A[k] - RK_B[k]) * q.r.dt;
@@ -240,14 +241,23 @@ cudaError_t launch_group(sbli_server* s, int k, int precision, const std::vector
     p.count = cnt;
     long long acc = 0;
     bool in64 = true;
+    const bool even = req_f64_registers(precision);
+    std::vector<std::array<int, 3>> edges(cnt);
+    for (int m = 0; m < cnt; ++m) {
+      const sbli_request& r = mem[base + m]->r;
+      edges[m] = {r.n0, r.n1, r.n2};
+    }
+    const int cap = even ? 32 : batch_zc_cap(
+        cnt, [&](int m) { return edges[m].data(); }, batch_default_zq(precision), s->sms);
     for (int m = 0; m < cnt; ++m) {
       const Req& q = *mem[base + m];
-      const int n[3] = {q.r.n0, q.r.n1, q.r.n2};
+      const int* n = edges[m].data();
+      const int zc = std::min(batch_zc(n[2]), cap);
       p.item_begin[m] = acc;
       p.tiles_x[m] = (n[0] + 31) / 32;
       p.tiles_y[m] = (n[1] + 7) / 8;
-      acc += req_f64_registers(precision) ? member_planes(n) : member_items(n);
-      p.a[m] = req_stage(s, q, k, &in64);
+      acc += even ? member_planes(n) : member_items(n, zc);
+      p.a[m] = req_stage(s, q, k, zc, &in64);
       p.c[m] = make_coef<T>(n, q.r.params);
     }
     p.item_begin[cnt] = acc;
@@ -374,6 +384,7 @@ int sbli_server_create(sbli_server** out, void* arena, size_t arena_bytes, int m
   int dev = 0, sms = 152;
   cudaGetDevice(&dev);
   cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+  s->sms = sms;
   s->grid64 = batch_grid_ctas(sms, SBLI_FP64, batch_default_zq(SBLI_FP64));
   s->grid32 = batch_grid_ctas(sms, SBLI_FP32, batch_default_zq(SBLI_FP32));
   s->lane[0].st = s->s64;
