@@ -7,15 +7,16 @@
 // thread keeping its own column's velocities of five planes in registers (the
 // x2 derivatives), the centre plane's going through shared memory (x0 and x1
 // derivatives; the halo's, 0.375 a point, are formed anew), with the
-// reciprocal of the density shared by the three components.  About 45
-// binary64 instructions a point where dividing at every stencil point took
-// about 260.  Blocks take contiguous runs of planes, one block per SM, so that all
+// reciprocal of the density shared by the three components, and the stencils
+// summed in integers.  About 30 binary64 instructions a point where dividing at
+// every stencil point took about 260.  Blocks take contiguous runs of planes, one block per SM, so that all
 // SMs end together.  160 x 200 x 120 points, both entry points with the state in and
-// out: 4.15 -> 0.85 ms.
+// out: 4.15 -> 0.67 ms (0.85 with the stencils on the binary64 pipe).
 #pragma once
 
 #include "fpconv.cuh"
 #include "sbli_internal.cuh"
+#include "stencil_int.cuh"
 
 namespace sbli {
 
@@ -135,13 +136,13 @@ __global__ void __launch_bounds__(KE_THREADS)
       const double(*s1)[KE_TX + 4] = su[buf][1] + ty + 2;
       const double(*s2)[KE_TX + 4] = su[buf][2] + ty + 2;
       const int i = tx + 2;
-      const double cx1 = c.c1[0], cx2 = c.c2[0], cy1 = c.c1[1], cy2 = c.c2[1], cz1 = c.c1[2], cz2 = c.c2[2];
-      auto d1 = [](double k1, double k2, double m2, double m1, double q1, double q2) {
-        return k1 * (q1 - m1) - k2 * (q2 - m2);
-      };
-      const double w0 = d1(cy1, cy2, s2[-2][i], s2[-1][i], s2[1][i], s2[2][i]) - d1(cz1, cz2, a1[0], a1[1], a1[3], a1[4]);
-      const double w1 = d1(cz1, cz2, a0[0], a0[1], a0[3], a0[4]) - d1(cx1, cx2, s2[0][i - 2], s2[0][i - 1], s2[0][i + 1], s2[0][i + 2]);
-      const double w2 = d1(cx1, cx2, s1[0][i - 2], s1[0][i - 1], s1[0][i + 1], s1[0][i + 2]) - d1(cy1, cy2, s0[-2][i], s0[-1][i], s0[1][i], s0[2][i]);
+      // Eq. 6 derivatives, their sums in integers
+      const double cx = c.c2[0], cy = c.c2[1], cz = c.c2[2];
+      const double w0 = cy * stencil_first(s2[-2][i], s2[-1][i], s2[1][i], s2[2][i]) - cz * stencil_first(a1[0], a1[1], a1[3], a1[4]);
+      const double w1 = cz * stencil_first(a0[0], a0[1], a0[3], a0[4]) -
+                        cx * stencil_first(s2[0][i - 2], s2[0][i - 1], s2[0][i + 1], s2[0][i + 2]);
+      const double w2 = cx * stencil_first(s1[0][i - 2], s1[0][i - 1], s1[0][i + 1], s1[0][i + 2]) -
+                        cy * stencil_first(s0[-2][i], s0[-1][i], s0[1][i], s0[2][i]);
       if (valid) {
         const double hrho = 0.5 * rr[0];
         ke += hrho * (a0[2] * a0[2] + a1[2] * a1[2] + a2[0] * a2[0]);

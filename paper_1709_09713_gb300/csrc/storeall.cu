@@ -9,7 +9,9 @@
 // (d) the Runge-Kutta update of Fig. 1 runs as its own kernel.
 //
 // Variables are deviations from the reference state, as in the fused path.
+#include "fpconv.cuh"
 #include "sbli_internal.cuh"
+#include "stencil_int.cuh"
 
 namespace sbli {
 
@@ -52,10 +54,22 @@ __global__ void bl_primitives(Geom g, Coef<T> c, const TIN* __restrict__ q, T* _
     const T m[3] = {T(q[P + n]), T(q[2 * P + n]), T(q[3 * P + n])};
     const T E_p = T(q[4 * P + n]);
     const T rho = T(1) + rho_p;
+    // one reciprocal for the four quotients, each corrected by its residual
+    // (Markstein), so that they round as divisions do
+    T rinv = T(0);
+    if constexpr (sizeof(T) == 8) rinv = rcp_newton_f64(rho);
+    auto quotient = [&](T x) -> T {
+      if constexpr (sizeof(T) == 8) {
+        const T q = x * rinv;
+        return fma(fma(-q, rho, x), rinv, q);
+      } else {
+        return x / rho;
+      }
+    };
     T u[3];
-    for (int i = 0; i < 3; ++i) u[i] = m[i] / rho;
+    for (int i = 0; i < 3; ++i) u[i] = quotient(m[i]);
     const T p_p = c.gm1 * (E_p - T(0.5) * rho * (u[0] * u[0] + u[1] * u[1] + u[2] * u[2]));  // Eq. 4
-    const T T_p = (c.gM2 * p_p - rho_p) / rho;                                              // Eq. 5
+    const T T_p = quotient(c.gM2 * p_p - rho_p);                                            // Eq. 5
     for (int i = 0; i < 3; ++i) s[(A_U + i) * P + n] = u[i];
     s[A_P * P + n] = p_p;
     s[A_T * P + n] = T_p;
@@ -69,24 +83,61 @@ __global__ void bl_primitives(Geom g, Coef<T> c, const TIN* __restrict__ q, T* _
 }
 
 // One derivative of one array along one axis (Listing 1): order 1 is Eq. 6,
-// order 2 is Eq. 7.
+// order 2 is Eq. 7.  A thread takes BL_Z points of one column: its wrapped
+// offsets are formed once (by comparisons), the values along x2 stay in
+// registers, and in binary64 the stencil is summed in integers, leaving one
+// binary64 product a point.  The modulo of every wrapped index had bounded it as
+// much as the binary64 pipe; integer instructions still do (15 us for 33.5 MB
+// moved at 128^3).  With the reciprocal and the shorter residual below, the
+// 128^3 store-all stage takes 1.37 instead of 1.80 ms.
+constexpr int BL_Z = 4;
+template <int ORDER, typename T>
+__device__ __forceinline__ T bl_stencil(T m2, T m1, T c, T p1, T p2, T k0, T k1, T k2) {
+  if constexpr (sizeof(T) == 8) {  // k2 = 1/(12 h) and -1/(12 h^2)
+    return ORDER == 1 ? k2 * stencil_first(m2, m1, p1, p2) : -k2 * stencil_second(m2, m1, c, p1, p2);
+  } else {
+    return ORDER == 1 ? k1 * (p1 - m1) - k2 * (p2 - m2) : k0 * c + k1 * (p1 + m1) + k2 * (p2 + m2);
+  }
+}
 template <typename T, typename TS, int AXIS, int ORDER>
 __global__ void __launch_bounds__(256) bl_derivative(Geom g, const TS* __restrict__ f, T* __restrict__ df, T k0, T k1,
                                                      T k2) {
-  const int i = blockIdx.x * 32 + threadIdx.x, j = blockIdx.y * 8 + threadIdx.y, k = blockIdx.z;
+  const int i = blockIdx.x * 32 + threadIdx.x, j = blockIdx.y * 8 + threadIdx.y, k0z = blockIdx.z * BL_Z;
   if (i >= g.n0 || j >= g.n1) return;
-  const long long n0 = g.n0, pl = (long long)g.n0 * g.n1;
-  auto at = [&](int s) -> T {
-    if (AXIS == 0) return T(f[wrapi(i + s, g.n0) + n0 * j + pl * k]);
-    if (AXIS == 1) return T(f[i + n0 * wrapi(j + s, g.n1) + pl * k]);
-    return T(f[i + n0 * j + pl * wrapi(k + s, g.n2)]);
-  };
-  T v;
-  if (ORDER == 1)
-    v = k1 * (at(1) - at(-1)) - k2 * (at(2) - at(-2));
-  else
-    v = k0 * at(0) + k1 * (at(1) + at(-1)) + k2 * (at(2) + at(-2));
-  df[i + n0 * j + pl * k] = v;
+  const long long pl = (long long)g.n0 * g.n1;
+  auto near = [](int v, int n) { return v < 0 ? v + n : (v >= n ? v - n : v); };  // |offset| <= 2 < n
+  const int own = i + g.n0 * j;
+  int o[5];
+#pragma unroll
+  for (int s = -2; s <= 2; ++s)
+    o[s + 2] = AXIS == 0 ? near(i + s, g.n0) + g.n0 * j : AXIS == 1 ? i + g.n0 * near(j + s, g.n1) : own;
+  T w[4];  // AXIS 2: planes k - 2 .. k + 1
+  if constexpr (AXIS == 2) {
+#pragma unroll
+    for (int s = -2; s <= 1; ++s) {
+      int z = k0z + s;
+      while (z >= g.n2) z -= g.n2;
+      w[s + 2] = T(f[own + pl * (z < 0 ? z + g.n2 : z)]);
+    }
+  }
+#pragma unroll
+  for (int q = 0; q < BL_Z; ++q) {
+    const int k = k0z + q;
+    if (k >= g.n2) break;
+    T v;
+    if constexpr (AXIS == 2) {
+      const T p2 = T(f[own + pl * near(k + 2, g.n2)]);
+      v = bl_stencil<ORDER>(w[0], w[1], w[2], w[3], p2, k0, k1, k2);
+      w[0] = w[1];
+      w[1] = w[2];
+      w[2] = w[3];
+      w[3] = p2;
+    } else {
+      const TS* p = f + pl * k;
+      v = bl_stencil<ORDER>(T(p[o[0]]), T(p[o[1]]), ORDER == 2 ? T(p[o[2]]) : T(0), T(p[o[3]]), T(p[o[4]]), k0, k1, k2);
+    }
+    df[own + pl * k] = v;
+  }
 }
 
 template <typename T>
@@ -108,41 +159,47 @@ __global__ void bl_residual(Geom g, Coef<T> c, const T* __restrict__ qrho, const
     auto dd = [&](int i, int j) { return i == j ? A(A_D2U + 3 * i + i) : A(A_DDU + offd(i, j)); };
     const T div = du[0][0] + du[1][1] + du[2][2];
     // Eq. 1
-    T conv = T(0);
-    for (int j = 0; j < 3; ++j) conv += A(A_DRHOU + 3 * j + j) + rho * du[j][j] + u[j] * A(A_DRHO + j);
+    T conv = rho * div;
+    for (int j = 0; j < 3; ++j) conv += A(A_DRHOU + 3 * j + j) + u[j] * A(A_DRHO + j);
     s[(A_R + 0) * P + n] = T(-0.5) * conv;
     // Eq. 2
-    T sd[3];
+    T vw = T(0);
     for (int i = 0; i < 3; ++i) {
-      conv = T(0);
-      for (int j = 0; j < 3; ++j) conv += A(A_DRHOUU + 3 * i + j) + m[i] * du[j][j] + u[j] * A(A_DRHOU + 3 * i + j);
+      conv = m[i] * div;
+      for (int j = 0; j < 3; ++j) conv += A(A_DRHOUU + 3 * i + j) + u[j] * A(A_DRHOU + 3 * i + j);
       T lap = T(0), cross = T(0);
       for (int j = 0; j < 3; ++j) {
         lap += A(A_D2U + 3 * i + j);
         cross += dd(i, j);
       }
-      sd[i] = lap + cross - T(2.0 / 3.0) * cross;
-      s[(A_R + 1 + i) * P + n] = T(-0.5) * conv - A(A_DP + i) + c.inv_re * sd[i];
+      const T sd = lap + T(1.0 / 3.0) * cross;  // Laplacian + G - 2/3 G
+      vw += u[i] * sd;
+      s[(A_R + 1 + i) * P + n] = (T(-0.5) * conv - A(A_DP + i)) + c.inv_re * sd;
     }
     // Eq. 3 (reference enthalpy carries the constant parts of rho E and p)
-    conv = T(0);
-    T pw = T(0), heat = T(0), vw = T(0), diss = T(0);
+    conv = E * div;
+    T pw = T(0), heat = T(0);
     for (int j = 0; j < 3; ++j) {
-      conv += A(A_DEU + j) + E * du[j][j] + u[j] * A(A_DE + j);
+      conv += A(A_DEU + j) + u[j] * A(A_DE + j);
       pw += A(A_DPU + j);
       heat += A(A_D2T + j);
     }
+    // du_i/dx_j (du_i/dx_j + du_j/dx_i - 2/3 div delta_ij)
+    T diag = T(0), off = T(0);
     for (int i = 0; i < 3; ++i) {
-      vw += u[i] * c.inv_re * sd[i];
-      for (int j = 0; j < 3; ++j) diss += du[i][j] * (du[i][j] + du[j][i] - (i == j ? T(2.0 / 3.0) * div : T(0)));
+      diag += du[i][i] * du[i][i];
+      const int j = (i + 1) % 3;
+      const T a = du[i][j] + du[j][i];
+      off += a * a;
     }
-    s[(A_R + 4) * P + n] = T(-0.5) * conv - c.H0 * div - pw + vw + c.inv_re * diss + c.kappa * heat;
+    const T diss = T(2) * diag + (off - T(2.0 / 3.0) * div * div);
+    s[(A_R + 4) * P + n] = ((T(-0.5) * conv - pw) - c.H0 * div) + (c.inv_re * (vw + diss) + c.kappa * heat);
   }
 }
 
 template <typename T, typename TS>
 cudaError_t launch_der(const Geom& g, const Coef<T>& c, const TS* f, T* df, int axis, int order, cudaStream_t s) {
-  dim3 blk(32, 8), grd((g.n0 + 31) / 32, (g.n1 + 7) / 8, g.n2);
+  dim3 blk(32, 8), grd((g.n0 + 31) / 32, (g.n1 + 7) / 8, (g.n2 + BL_Z - 1) / BL_Z);
   const T k0 = c.e0[axis];
   const T k1 = order == 1 ? c.c1[axis] : c.e1[axis];
   const T k2 = order == 1 ? c.c2[axis] : c.e2[axis];
