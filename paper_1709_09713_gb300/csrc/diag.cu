@@ -26,9 +26,7 @@ Coef<T> make_coef(const int n[3], const sbli_params& p) {
     c.e2[a] = T(-1.0 / (12.0 * h * h));
     c.hc1[a] = T(-1.0 / (3.0 * h));
     c.hc2[a] = T(-1.0 / (24.0 * h));
-    c.t1[a] = T(2.0 / (9.0 * h));
     c.t2[a] = T(1.0 / (36.0 * h));
-    c.f1[a] = T(16.0 / (9.0 * h * h));
     c.f2[a] = T(-1.0 / (9.0 * h * h));
     c.v0[a] = T(e0s - 5.0 / (6.0 * h * h));
   }

@@ -18,9 +18,7 @@ cudaError_t launch_fused_fp32_pair(const StageArgs& a, const Coef<float>& cf, co
     c.e2[i] = f32x2(cf.e2[i], cf.e2[i]);
     c.hc1[i] = f32x2(cf.hc1[i], cf.hc1[i]);
     c.hc2[i] = f32x2(cf.hc2[i], cf.hc2[i]);
-    c.t1[i] = f32x2(cf.t1[i], cf.t1[i]);
     c.t2[i] = f32x2(cf.t2[i], cf.t2[i]);
-    c.f1[i] = f32x2(cf.f1[i], cf.f1[i]);
     c.f2[i] = f32x2(cf.f2[i], cf.f2[i]);
     c.v0[i] = f32x2(cf.v0[i], cf.v0[i]);
   }

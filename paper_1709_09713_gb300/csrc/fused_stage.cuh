@@ -20,9 +20,10 @@
 //     plane is stored, and the centre plane's accumulator values as its
 //     derivative terms start, so HBM latency overlaps the arithmetic;
 //   * x0/x1 derivatives read the centre slot, x2 derivatives read the ring;
-//     each axis streams its four neighbour records through the accumulators
-//     one at a time (axis_terms_stream; the double-float type takes differences
-//     first and two values at a time, axis_terms_dw);
+//     each axis takes its four neighbour records (binary32 one at a time,
+//     axis_terms_stream; binary64 sums its linear stencils in integers,
+//     axis_terms_fixed; double-float takes differences first and two values at a
+//     time, axis_terms_dw);
 //   * ZT (the z queue): each thread keeps its own column's records of the
 //     five ring planes, and their in-plane gradients, in tensor memory
 //     (TMEM), so the x2 derivatives read TMEM and shared memory keeps full
@@ -67,6 +68,7 @@
 #include "f32x2.cuh"
 #include "fpconv.cuh"
 #include "sbli_internal.cuh"
+#include "stencil_int.cuh"
 
 namespace sbli {
 
@@ -588,15 +590,13 @@ __device__ __forceinline__ T add_nc(T a, T b) {
 // take the rounding of u_j = m_j / rho into the mass balance: 1.45 times its
 // error, so Eq. 1 keeps two.)  The viscous terms of Eq. 2 are accumulated as
 // their sum (Laplacian + G/3), the symmetric off-diagonal gradients as their
-// sum: 15 multiply-adds a neighbour instead of the 17 of one accumulator per
-// derivative.  The number of instructions is what bounds these kernels
-// (binary64: of binary64 ones, at 0.92 of the pipe's measured peak): a 256^3
-// stage of binary64 went from 10.25 to 9.25 ms, the 512^3 binary32 one (binary64
-// accumulator) from 3.73 to 3.63 ms.
-// Binary64 also takes the factors -1/2 (convective terms) and 1/3, 4/3
-// (viscous terms) in its weights, 1.5 % fewer instructions; in binary32 the
-// 24 constants of that are too many for the uniform registers (479 -> 504 us),
-// and the factors are applied to the sums of an axis.
+// sum: 15 multiply-adds a neighbour in binary32 instead of the 17 of one
+// accumulator per derivative (the number of instructions bounds these kernels:
+// 512^3, binary64 accumulator, 3.73 -> 3.63 ms a stage).  Binary64 takes the linear
+// stencils in integers (axis_terms_sums) and the factors -1/2 (convective terms)
+// and 1/3, 4/3 (viscous terms) in its weights; in binary32 the constants of that
+// are too many for the uniform registers (256^3: 479 -> 504 us), and the factors
+// are applied to the sums of an axis.
 template <typename T>
 constexpr bool scaled_weights() {
   return std::is_same<T, double>::value;
@@ -620,11 +620,11 @@ struct NoXTerms {
   __device__ void operator()(int, T&, T&) const {}
 };
 
-// All derivatives along axis A, the four neighbours streamed through
+// Binary32: all derivatives along axis A, the four neighbours streamed through
 // registers one at a time, so only one record is live.  ldrec(k, r) loads the
 // record of the neighbour k = 0..3 (offsets -2, -1, +1, +2 along A; Eq. 6
 // weights +c2, -c1, +c1, -c2, Eq. 7 e2, e1, e1, e2); sfun(k) gives the
-// mixed-term helper s_A there.  ZX (binary32, A = 2): the mixed derivatives
+// mixed-term helper s_A there.  ZX (A = 2): the mixed derivatives
 // that involve x2 are taken with the x2 derivative last, D1_z(D1_x u2) and
 // D1_z(D1_y u2) from xfun(k, ...) (the neighbours' in-plane gradients of u2);
 // the stream also forms D1_z u2 at the centre.  WITH_KE: also lo[].
@@ -632,31 +632,27 @@ template <int A, bool ZX, bool WITH_KE, typename T, typename LD, typename SF, ty
 __device__ __forceinline__ void axis_terms_stream(const LD& ldrec, const SF& sfun, const Coef<T>& c,
                                                   const T (&uc)[3], StreamTerms<T>& t, const XF& xfun = XF()) {
   static_assert(!ZX || A == 2, "x2-last mixed terms belong to the x2 axis");
-  constexpr bool SW = scaled_weights<T>();
   const T ua = uc[A];
-  T dp = T(0);                            // D1_A 2p' (times -1/2)
-  T lA = T(0), gA = T(0);                 // !SW: D2_A u_A off-centre, D1_A s_A
-  T gz0 = T(0), gz1 = T(0);               // !SW, ZX: the x2 parts of G_0, G_1
+  T dp = T(0);               // D1_A 2p'
+  T lA = T(0), gA = T(0);    // D2_A u_A off-centre, D1_A s_A
+  T gz0 = T(0), gz1 = T(0);  // ZX: the x2 parts of G_0, G_1
   auto sgn = [](int k, T inner, T outer) {  // the antisymmetric weight of neighbour k
     return k == 0 ? outer : k == 1 ? -inner : k == 2 ? inner : -outer;
   };
-  const T* w1 = SW ? c.hc1 : c.c1;
-  const T* w2 = SW ? c.hc2 : c.c2;
   // the per-axis products c u_A^c once, so that each neighbour's weight is one multiply-add
-  const T cu1 = w1[A] * ua, cu2 = w2[A] * ua;
+  const T cu1 = c.c1[A] * ua, cu2 = c.c2[A] * ua;
 #pragma unroll
   for (int k = 0; k < 4; ++k) {
     const T cd = sgn(k, c.c1[A], c.c2[A]);
-    const T hd = sgn(k, w1[A], w2[A]);
     const T ed = (k == 0 || k == 3) ? c.e2[A] : c.e1[A];
     T r[NV];
     ldrec(k, r);
-    const T w = fmadd(hd, r[V_U0 + A], sgn(k, cu1, cu2));
+    const T w = fmadd(cd, r[V_U0 + A], sgn(k, cu1, cu2));
 #pragma unroll
     for (int i = 0; i < 3; ++i) t.rM[i] = fmadd(w, r[V_M0 + i], t.rM[i]);
     t.rE = fmadd(w, r[V_H], t.rE);
-    t.rrho = fmadd(hd, fmadd(ua, r[V_RHO], r[V_M0 + A]), t.rrho);
-    dp = fmadd(hd, r[V_P], dp);
+    t.rrho = fmadd(cd, fmadd(ua, r[V_RHO], r[V_M0 + A]), t.rrho);
+    dp = fmadd(cd, r[V_P], dp);
 #pragma unroll
     for (int i = 0; i < 3; ++i) {
       if (i != A) {
@@ -667,16 +663,10 @@ __device__ __forceinline__ void axis_terms_stream(const LD& ldrec, const SF& sfu
       }
     }
     // the Laplacian and one third of Eq. 7 on j = A, one third of D1_A s_A
-    if constexpr (SW) {
-      t.v[A] = fmadd((k == 0 || k == 3) ? c.f2[A] : c.f1[A], r[V_U0 + A], t.v[A]);
-      t.v[A] = fmadd(sgn(k, c.t1[A], c.t2[A]), sfun(k), t.v[A]);
-    } else {
-      lA = fmadd(ed, r[V_U0 + A], lA);
-      gA = fmadd(cd, sfun(k), gA);
-    }
+    lA = fmadd(ed, r[V_U0 + A], lA);
+    gA = fmadd(cd, sfun(k), gA);
     t.lapT = fmadd(ed, r[V_T], t.lapT);
     if constexpr (ZX) {
-      static_assert(!SW, "binary32 only");
       T x02, x12;
       xfun(k, x02, x12);
       gz0 = fmadd(cd, x02, gz0);
@@ -686,11 +676,85 @@ __device__ __forceinline__ void axis_terms_stream(const LD& ldrec, const SF& sfu
   }
   t.rM[A] = t.rM[A] + dp;
   t.rE = fmadd(-ua, dp, t.rE);
-  if constexpr (!SW) t.v[A] = fmadd(T(4.0 / 3.0), lA, fmadd(T(1.0 / 3.0), gA, t.v[A]));
+  t.v[A] = fmadd(T(4.0 / 3.0), lA, fmadd(T(1.0 / 3.0), gA, t.v[A]));
   if constexpr (ZX) {
     t.v[0] = fmadd(T(1.0 / 3.0), gz0, t.v[0]);
     t.v[1] = fmadd(T(1.0 / 3.0), gz1, t.v[1]);
   }
+}
+
+// Binary64: the linear stencils of an axis (Laplacians of u and T', cross
+// gradients, D1_A of p', rho', m_A and s_A) in integers, the products with the
+// velocities on the binary64 pipe: 34 binary64 instructions an axis instead of
+// 62, beside some 800 integer ones that run while that pipe is busy (about 180
+// instead of 280 a point with the primitives and the update).  256^3 8.86 -> 6.39 ms a
+// stage, 64^3 168 -> 128 us, 32^3 33.4 -> 28.0; the pipe stays the bound, at 0.88 of
+// its measured peak.  Values too large to align, infinities and NaNs take the
+// sums in binary64 (FIXED false).
+template <int A, bool WITH_KE, bool FIXED>
+__device__ __forceinline__ void axis_terms_sums(const double (&r)[4][NV], const double (&sx)[4], const double (&sy)[4],
+                                                const uint32_t (&top)[NV], uint32_t stop, const Coef<double>& c,
+                                                const double (&uc)[3], StreamTerms<double>& t) {
+  const double ua = uc[A];
+  const double hu1 = c.hc1[A] * ua, hu2 = c.hc2[A] * ua;
+#pragma unroll
+  for (int k = 0; k < 4; ++k) {
+    const double hd = k == 0 ? c.hc2[A] : k == 1 ? -c.hc1[A] : k == 2 ? c.hc1[A] : -c.hc2[A];
+    const double hu = k == 0 ? hu2 : k == 1 ? -hu1 : k == 2 ? hu1 : -hu2;
+    const double w = fmadd(hd, r[k][V_U0 + A], hu);
+#pragma unroll
+    for (int i = 0; i < 3; ++i) t.rM[i] = fmadd(w, r[k][V_M0 + i], t.rM[i]);
+    t.rE = fmadd(w, r[k][V_H], t.rE);
+  }
+  auto first = [&](int v) { return first_sum<FIXED>(r[0][v], r[1][v], r[2][v], r[3][v], top[v]); };
+  auto second = [&](int v) { return second_sum<FIXED>(r[0][v], r[1][v], r[2][v], r[3][v], top[v]); };
+  const double dp = c.hc2[A] * first(V_P);
+  t.rM[A] = add_nc(t.rM[A], dp);
+  t.rE = fmadd(-ua, dp, t.rE);
+  t.rrho = fmadd(c.hc2[A], fmadd(ua, first(V_RHO), first(V_M0 + A)), t.rrho);
+#pragma unroll
+  for (int i = 0; i < 3; ++i) {
+    const int v = V_U0 + i;
+    if (i == A) {  // the Laplacian and one third of Eq. 7 on j = A
+      t.v[i] = fmadd(c.f2[A], second(v), t.v[i]);
+    } else {
+      double f, s;
+      both_sums<FIXED>(r[0][v], r[1][v], r[2][v], r[3][v], top[v], f, s);
+      t.v[i] = fmadd(c.e2[A], s, t.v[i]);
+      const int pair = i + A - 1;  // (0,1) -> 0, (0,2) -> 1, (1,2) -> 2
+      t.a[pair] = fmadd(c.c2[A], f, t.a[pair]);
+      if (WITH_KE && i < A) t.lo[pair] = fmadd(c.c2[A], f, t.lo[pair]);
+    }
+  }
+  t.lapT = fmadd(c.e2[A], second(V_T), t.lapT);
+  const double ds = A == 2 ? first_sum<FIXED>(sx, sy, stop) : first_sum<FIXED>(sx[0], sx[1], sx[2], sx[3], stop);
+  t.v[A] = fmadd(c.t2[A], ds, t.v[A]);
+}
+// ldrec(k, r) loads the record of neighbour k (offsets -2, -1, +1, +2); sfun(k, x,
+// y) the mixed-term helper s_A there (x; x + y along x2).
+template <int A, bool WITH_KE, typename LD, typename SF>
+__device__ __forceinline__ void axis_terms_fixed(const LD& ldrec, const SF& sfun, const Coef<double>& c,
+                                                 const double (&uc)[3], StreamTerms<double>& t) {
+  double r[4][NV], sx[4], sy[4];
+#pragma unroll
+  for (int k = 0; k < 4; ++k) {
+    ldrec(k, r[k]);
+    sfun(k, sx[k], sy[k]);
+  }
+  uint32_t top[NV], worst = 0;
+#pragma unroll
+  for (int v = 0; v < NV; ++v) {
+    if (v == V_H || (v >= V_M0 && v <= V_M2 && v != V_M0 + A)) continue;  // no linear stencil of these
+    top[v] = fixed::top_exponent(r[0][v], r[1][v], r[2][v], r[3][v]);
+    worst = max(worst, top[v]);
+  }
+  uint32_t stop = fixed::top_exponent(sx[0], sx[1], sx[2], sx[3]);
+  if (A == 2) stop = max(stop, fixed::top_exponent(sy[0], sy[1], sy[2], sy[3]));
+  worst = max(worst, stop);
+  if (fixed::alignable(worst))
+    axis_terms_sums<A, WITH_KE, true>(r, sx, sy, top, stop, c, uc, t);
+  else
+    axis_terms_sums<A, WITH_KE, false>(r, sx, sy, top, stop, c, uc, t);
 }
 
 // Eqs. 1-3 at one point from the streamed terms and the centre values.
@@ -872,7 +936,8 @@ __device__ __forceinline__ void fused_march(const StageArgs& a, const Coef<T>& c
                                             uint32_t tmem_base = 0, uint32_t tmem_base2 = 0) {
   using S = FusedSmem<T, TY, ZT>;
   constexpr bool MIXZ = S::MIXZ;
-  constexpr bool DW = std::is_same<T, dfloat>::value;  // double-float: terms in pairs
+  constexpr bool DW = std::is_same<T, dfloat>::value;     // double-float: terms in pairs
+  constexpr bool FIXED = std::is_same<T, double>::value;  // binary64: linear stencils in integers
   constexpr int SY = S::SY;
   constexpr int NT = TX * TY;
   constexpr int PTS = SX * SY;
@@ -1089,6 +1154,19 @@ __device__ __forceinline__ void fused_march(const StageArgs& a, const Coef<T>& c
         sm.dring[se][0][ty][tx] = dg.a();
         sm.dring[se][1][ty][tx] = dg.b();
       }
+    } else if constexpr (FIXED) {
+      const T(*R)[SX][NV] = sm.ring[fe];
+      const int sy = ty + HALO, sx = tx + HALO;
+      const T d00 = c.c2[0] * stencil_first(R[sy][sx - 2][V_U0], R[sy][sx - 1][V_U0], R[sy][sx + 1][V_U0],
+                                            R[sy][sx + 2][V_U0]);
+      const T d11 = c.c2[1] * stencil_first(R[sy - 2][sx][V_U1], R[sy - 1][sx][V_U1], R[sy + 1][sx][V_U1],
+                                            R[sy + 2][sx][V_U1]);
+      if constexpr (ZT) {
+        tmem_store_diag(twin, se, d00, d11);  // this thread's column only
+      } else {
+        sm.dring[se][0][ty][tx] = d00;
+        sm.dring[se][1][ty][tx] = d11;
+      }
     } else {
       const T(*R)[SX][NV] = sm.ring[fe];
       const int sy = ty + HALO, sx = tx + HALO;
@@ -1273,34 +1351,30 @@ __device__ __forceinline__ void fused_march(const StageArgs& a, const Coef<T>& c
           (k1 ? &sm.s0buf[0][0][0] : &sm.s1buf[0][0][0])[hdst[j]] = dg.a() + dg.b();
         }
       } else {
-      const int sy = ty + HALO, sx = tx + HALO;
-      auto u2z = [&](int yy, int xx) {
-        return mad(c.c1[2], u2at(sl[3], yy, xx) - u2at(sl[1], yy, xx),
-                   -c.c2[2] * (u2at(sl[4], yy, xx) - u2at(sl[0], yy, xx)));
-      };
-      d22 = u2z(sy, sx);
-      if constexpr (ZT) {
-        tmem_load_diag(twin, scen, g00c, g11c);
-      } else {
-        g00c = sm.dring[scen][0][ty][tx];
-        g11c = sm.dring[scen][1][ty][tx];
-      }
-      sm.s0buf[0][ty][sx] = g11c + d22;
-      sm.s1buf[0][sy][tx] = g00c + d22;
-      const T(*R)[SX][NV] = sm.ring[fc];
-#pragma unroll
-      for (int j = 0; j < HPT; ++j) {
-        const int hy = hxy[j] >> 8, hx = hxy[j] & 0xFF;
-        if (hk[j] == 1) {
-          const T d11 = mad(c.c1[1], R[hy + 1][hx][V_U1] - R[hy - 1][hx][V_U1],
-                            -c.c2[1] * (R[hy + 2][hx][V_U1] - R[hy - 2][hx][V_U1]));
-          (&sm.s0buf[0][0][0])[hdst[j]] = d11 + u2z(hy, hx);
-        } else if (hk[j] == 2) {
-          const T d00 = mad(c.c1[0], R[hy][hx + 1][V_U0] - R[hy][hx - 1][V_U0],
-                            -c.c2[0] * (R[hy][hx + 2][V_U0] - R[hy][hx - 2][V_U0]));
-          (&sm.s1buf[0][0][0])[hdst[j]] = d00 + u2z(hy, hx);
+        const int sy = ty + HALO, sx = tx + HALO;
+        auto u2z = [&](int yy, int xx) {
+          return c.c2[2] * stencil_first(u2at(sl[0], yy, xx), u2at(sl[1], yy, xx), u2at(sl[3], yy, xx), u2at(sl[4], yy, xx));
+        };
+        d22 = u2z(sy, sx);
+        if constexpr (ZT) {
+          tmem_load_diag(twin, scen, g00c, g11c);
+        } else {
+          g00c = sm.dring[scen][0][ty][tx];
+          g11c = sm.dring[scen][1][ty][tx];
         }
-      }
+        sm.s0buf[0][ty][sx] = add_nc(g11c, d22);
+        sm.s1buf[0][sy][tx] = add_nc(g00c, d22);
+#pragma unroll
+        for (int j = 0; j < HPT; ++j) {
+          if (hk[j] == 0) continue;
+          // kind 1: D1_y u1 (s_0), kind 2: D1_x u0 (s_1)
+          const int hy = hxy[j] >> 8, hx = hxy[j] & 0xFF;
+          const bool k1 = hk[j] == 1;
+          const T* q = &sm.ring[fc][hy][hx][k1 ? V_U1 : V_U0];
+          const int st = k1 ? SX * NV : NV;
+          const T dd = (k1 ? c.c2[1] : c.c2[0]) * stencil_first(q[-2 * st], q[-st], q[st], q[2 * st]);
+          (k1 ? &sm.s0buf[0][0][0] : &sm.s1buf[0][0][0])[hdst[j]] = add_nc(dd, u2z(hy, hx));
+        }
       }
       __syncthreads();
     }
@@ -1409,13 +1483,29 @@ __device__ __forceinline__ void fused_march(const StageArgs& a, const Coef<T>& c
         t.gd[0] = g00c;
         t.gd[1] = g11c;
         t.gd[2] = d22;
-        axis_terms_stream<0, false, WITH_KE>(ld0, sf0, c, uc, t);
-        // shared-memory loads of one axis at a time: hoisted over the axes they spill at the binary32 ring
-        // kernel's 128 registers (256^3: 674 us a stage without these two, 651 with)
-        if constexpr (!ZT && sizeof(T) == 4) asm volatile("" ::: "memory");
-        axis_terms_stream<1, false, WITH_KE>(ld1, sf1, c, uc, t);
-        if constexpr (!ZT && sizeof(T) == 4) asm volatile("" ::: "memory");
-        axis_terms_stream<2, MIXZ, WITH_KE>(ld2, sf2, c, uc, t, xf);
+        if constexpr (FIXED) {
+          auto at0 = [&](int k, T& x, T&) { x = sf0(k); };
+          auto at1 = [&](int k, T& x, T&) { x = sf1(k); };
+          auto at2 = [&](int k, T& x, T& y) {
+            if constexpr (ZT) {
+              tmem_load_diag(twin, zs[k], x, y);
+            } else {
+              x = sm.dring[zs[k]][0][ty][tx];
+              y = sm.dring[zs[k]][1][ty][tx];
+            }
+          };
+          axis_terms_fixed<0, WITH_KE>(ld0, at0, c, uc, t);
+          axis_terms_fixed<1, WITH_KE>(ld1, at1, c, uc, t);
+          axis_terms_fixed<2, WITH_KE>(ld2, at2, c, uc, t);
+        } else {
+          axis_terms_stream<0, false, WITH_KE>(ld0, sf0, c, uc, t);
+          // shared-memory loads of one axis at a time: hoisted over the axes they spill at the binary32 ring
+          // kernel's 128 registers (256^3: 674 us a stage without these two, 651 with)
+          if constexpr (!ZT && sizeof(T) == 4) asm volatile("" ::: "memory");
+          axis_terms_stream<1, false, WITH_KE>(ld1, sf1, c, uc, t);
+          if constexpr (!ZT && sizeof(T) == 4) asm volatile("" ::: "memory");
+          axis_terms_stream<2, MIXZ, WITH_KE>(ld2, sf2, c, uc, t, xf);
+        }
         assemble_streamed(t, rho_p, mc, Ec, uc, c, R);
         if (WITH_KE) {  // D1_j u_i - D1_i u_j = 2 D1_j u_i - (their sum), lo = D1_j u_i with i < j
           w2 = fmadd(T(-2), t.lo[0], t.a[0]);

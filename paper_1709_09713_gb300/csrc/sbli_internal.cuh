@@ -26,9 +26,9 @@ struct Coef {
   // Eq. 7: D2 f = e0 f[0] + e1 (f[+1] + f[-1]) + e2 (f[+2] + f[-2]),
   //   e0 = -5/(2h^2), e1 = 4/(3h^2), e2 = -1/(12h^2)
   T e0[3], e1[3], e2[3];
-  // derived weights of the streamed terms: -c/2, c/3, 4e/3, the centre weight
-  // of sum_j D2_j u_i + 1/3 D2_i u_i (e0s + e0/3) and the Laplacian's (e0s)
-  T hc1[3], hc2[3], t1[3], t2[3], f1[3], f2[3], v0[3], e0s;
+  // derived weights: -c/2, c2/3, 4/3 e2, the centre weight of
+  // sum_j D2_j u_i + 1/3 D2_i u_i (e0s + e0/3) and the Laplacian's (e0s)
+  T hc1[3], hc2[3], t2[3], f2[3], v0[3], e0s;
   T gm1;    // gamma - 1                    (Eq. 4)
   T gM2;    // gamma M^2                    (Eq. 5)
   T gm1x2;  // 2 (gamma - 1): the fused kernels keep 2 p' (both uses of p in Eqs. 2-3 carry a factor 2)
