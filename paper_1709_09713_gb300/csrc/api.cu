@@ -189,8 +189,8 @@ void use_config(sbli_grid* g, const FusedConfig& cfg) {
 }
 
 // Binary32 grids: z queue and planes per CTA by the model of their stage (us a
-// stage, shared ring with planes by waves -> this: 128^3 96.7 -> 70.4, 96^3 35.8 ->
-// 33.7, 40^3 9.3 -> 7.8, 32^3 9.2 -> 4.8).
+// stage, shared ring with planes by waves -> this: 128^3 96.7 -> 63.7, 96^3 35.8 ->
+// 30.3, 40^3 9.3 -> 7.6, 32^3 9.2 -> 4.4).
 FusedConfig default_config(const Geom& g, int precision, int sms) {
   FusedConfig cfg;
   cfg.ty = 8;

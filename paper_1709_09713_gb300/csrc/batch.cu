@@ -25,12 +25,13 @@ namespace sbli {
 // the CTA's TMEM columns held for all of its work items.  DF: binary32 stages
 // with the double-float accumulator (SBLI_FP32_DF members).
 template <typename T, typename TIN, typename TOUT, int TY, bool WITH_KE, bool ZT = false, bool DF = false>
-__global__ void __launch_bounds__(TX* TY, fused_min_blocks<T, TY, ZT>())
+__global__ void __launch_bounds__(TX* FusedSmem<T, TY, ZT>::NR, fused_min_blocks<T, TY, ZT>())
     batch_stage_kernel(const __grid_constant__ BatchParams<T> p) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
   FusedSmem<T, TY, ZT>& sm = *reinterpret_cast<FusedSmem<T, TY, ZT>*>(smem_raw);
-  constexpr int NCOL = tmem_columns<TY, T>();
-  constexpr int NCOL2 = tmem_columns2<TY, T>();
+  constexpr int NW = FusedSmem<T, TY, ZT>::NR;
+  constexpr int NCOL = tmem_columns<NW, T>();
+  constexpr int NCOL2 = tmem_columns2<NW, T>();
   uint32_t tbase = 0, tbase2 = 0;
   if (ZT) tmem_acquire<NCOL, NCOL2>(sm.tmem_base, tbase, tbase2);
   // member owning item or unit u (binary search over item_begin)
@@ -59,7 +60,7 @@ __global__ void __launch_bounds__(TX* TY, fused_min_blocks<T, TY, ZT>())
       u += len;
       // the CTA's part of this member ends: CTA + member numbers its partial sum
       if (WITH_KE && (u == end || u == p.item_begin[m + 1])) {
-        block_reduce_pair<TX * TY>(sm.red, ke, ens, p.ke_items + 2 * ((long long)blockIdx.x + m));
+        block_reduce_pair<TX * NW>(sm.red, ke, ens, p.ke_items + 2 * ((long long)blockIdx.x + m));
         ke = ens = 0.0;
       }
     }
@@ -76,7 +77,7 @@ __global__ void __launch_bounds__(TX* TY, fused_min_blocks<T, TY, ZT>())
       double ke = 0.0, ens = 0.0;
       fused_march<T, TIN, TOUT, TY, false, WITH_KE, DF, ZT>(a, p.c[lo], bx, by, zbeg, zbeg + a.zc, sm, ke, ens,
                                                             tbase, tbase2);
-      if (WITH_KE) block_reduce_pair<TX * TY>(sm.red, ke, ens, p.ke_items + 2 * item);
+      if (WITH_KE) block_reduce_pair<TX * NW>(sm.red, ke, ens, p.ke_items + 2 * item);
     }
   }
   if (ZT) tmem_release<NCOL, NCOL2>(tbase, tbase2);
@@ -109,7 +110,7 @@ static cudaError_t launch_batch_k(const BatchParams<T>& p, int grid, cudaStream_
   static std::atomic<unsigned long long> done{0};
   if (cudaError_t e = ensure_smem_limit(k, smem, done)) return e;
   if (even_split<T>()) grid = (int)std::min<long long>(grid, p.total_items);
-  k<<<grid, TX * 8, smem, s>>>(p);
+  k<<<grid, TX * FusedSmem<T, 8, ZT>::NR, smem, s>>>(p);
   return cudaGetLastError();
 }
 
@@ -123,12 +124,31 @@ static cudaError_t launch_batch_zq(const BatchParams<T>& p, int grid, cudaStream
 }
 
 // binary32 members (every stage input is binary32; the grid is sized by the
-// caller with batch_ctas_per_sm for the z-queue mode)
+// caller with batch_ctas_per_sm for the z-queue mode): the shared ring one point
+// per thread, the TMEM queue by row pairs, as single grids
+template <bool DF>
+static cudaError_t launch_batch_b32(const BatchParams<float>& p, int grid, cudaStream_t s, int zq) {
+  if (!zq)
+    return p.ke_items ? launch_batch_k<float, float, float, true, false, DF>(p, grid, s)
+                      : launch_batch_k<float, float, float, false, false, DF>(p, grid, s);
+  BatchParams<f32x2> r;
+  r.count = p.count;
+  r.total_items = p.total_items;
+  r.ke_items = p.ke_items;
+  for (int m = 0; m <= p.count; ++m) r.item_begin[m] = p.item_begin[m];
+  for (int m = 0; m < p.count; ++m) {
+    r.tiles_x[m] = p.tiles_x[m];
+    r.tiles_y[m] = p.tiles_y[m];
+    r.a[m] = p.a[m];
+    r.c[m] = both_lanes(p.c[m]);
+  }
+  return p.ke_items ? launch_batch_k<f32x2, float, float, true, true, DF>(r, grid, s)
+                    : launch_batch_k<f32x2, float, float, false, true, DF>(r, grid, s);
+}
 template <>
 cudaError_t launch_batch_t<float>(const BatchParams<float>& p, bool in64, int grid, cudaStream_t s, bool df, int zq) {
   if (in64) return cudaErrorInvalidValue;  // stages read the binary32 copy of the state
-  if (df) return launch_batch_zq<float, float, float, true>(p, grid, s, zq);
-  return launch_batch_zq<float, float, float, false>(p, grid, s, zq);
+  return df ? launch_batch_b32<true>(p, grid, s, zq) : launch_batch_b32<false>(p, grid, s, zq);
 }
 
 // double-float arithmetic members: every stage reads a field of (hi, lo)

@@ -37,7 +37,7 @@ cudaError_t launch_batch_t(const BatchParams<T>& p, bool in64, int grid, cudaStr
 inline int batch_default_zq(int precision) { return precision == SBLI_FP32 || precision == SBLI_FP32_DF ? 1 : 0; }
 
 // Resident CTAs per SM of the multi-member launch: binary32 members run the
-// TMEM-queue kernel (59 KiB shared, 80 registers: 3 per SM) or the shared
+// TMEM-queue kernel (59 KiB shared, four warps of at most 168 registers: 3 per SM) or the shared
 // ring (113 KiB: 2 per SM); binary64 and double-float-arithmetic members
 // the 194.5 KiB shared ring or the 124 KiB TMEM-queue kernel (1 per SM).
 inline int batch_ctas_per_sm(int precision, int zq) {

@@ -59,12 +59,12 @@ int fused_num_ctas(const Geom& g, const FusedConfig& cfg) {
 }
 
 // Measured at 16^3 ... 160^3 (binary64 accumulator; the double-float one ranks
-// alike): a plane takes 1.47 us with one CTA on an SM, 2.5 with two, 3.3 with
-// three (TMEM queue, which also pays 0.6 us for its allocation), the fill of a
-// march 1.5 planes, a launch 1 us; CTAs go to SMs one each first.  Within 8 % of
+// alike): a plane of the shared ring takes 1.47 us with one CTA on an SM, 2.5 with
+// two; one of the TMEM queue 1.69, 2.3 and with three 3.05, and 0.6 us for its
+// allocation; the fill of a march 1.5 planes, a launch 1 us; CTAs go to SMs one each first.  Within 8 % of
 // the measured time over both queues and 1 to 40 planes per CTA.
 double binary32_stage_us(long long ctas, int zc, int zq, int sms) {
-  const double plane[2][4] = {{0.0, 1.47, 2.5, 2.5}, {0.0, 1.5, 2.4, 3.3}};
+  const double plane[2][4] = {{0.0, 1.47, 2.5, 2.5}, {0.0, 1.69, 2.3, 3.05}};
   const int most = zq ? 3 : 2;
   const long long slots = (long long)sms * most;
   const long long full = ctas / slots, rest = ctas % slots;

@@ -36,7 +36,9 @@
 //     slot nobody reads any more, so the barrier that ends each plane is not
 //     needed;
 //   * the arithmetic type T is double, float, dfloat (double-float, binary64
-//     storage) or f32x2 (two columns per thread in packed FP32x2 instructions);
+//     storage) or f32x2: two points per thread in packed FP32x2 instructions,
+//     two columns x and x + 32 with the shared ring, or with the TMEM queue (the
+//     binary32 default) two neighbouring rows (row pairs, see FusedSmem);
 //   * the mixed second derivatives of the stress divergence (the D1_a o D1_b
 //     reading of the mixed term), for each i sum_{j != i} d2 u_j/dx_i dx_j:
 //     - binary64 and double-float, by linearity of D1_i,
@@ -101,9 +103,27 @@ template <typename T>
 constexpr bool mixz() {
   return std::is_same<T, float>::value || std::is_same<T, f32x2>::value;
 }
+// Row pairs (f32x2 with the TMEM queue): a thread owns two neighbouring rows
+// of its column, and a record holds both rows' values side by side, so the
+// rows of records are pairs: TY / 2 of them, with one pair of halo on each side.
+// One point per thread was bound by shared-memory wavefronts (67 % of the L1
+// pipe) and issue (62 %): a pair shares its x1 neighbours (four row loads for
+// eight), its packed instructions do two points (466 instructions a point for
+// 690), and 12 warps of 164 registers hold the points that 24 of 80 did.  Every
+// operation rounds as in the one-point kernel, so results are bitwise the same.
+// us a stage: 128^3 70.4 -> 63.7, 256^3 483 -> 450 (double-float accumulator 443 ->
+// 416), 512^3 3640 -> 3443 (3328 -> 3163), 64-member ensemble 12 %.  Now bound by
+// latency (issue 45 %; loads from memory, shared memory, barriers).
+template <typename T, bool ZT>
+constexpr bool row_pairs() {
+  return std::is_same<T, f32x2>::value && ZT;
+}
 template <typename T, int TY, bool ZT = false>
 struct FusedSmem {
-  static constexpr int SY = TY + 2 * HALO;
+  static constexpr bool RP = row_pairs<T, ZT>();
+  static constexpr int HR = RP ? HALO / 2 : HALO;  // rows of halo records on each side
+  static constexpr int NR = RP ? TY / 2 : TY;      // rows of records of the tile (warps of a CTA)
+  static constexpr int SY = NR + 2 * HR;
   static constexpr int NFULL = full_slots<T, TY, ZT>();
   static constexpr bool MIXZ = mixz<T>();
   static constexpr bool U2 = ZT && !MIXZ;      // u_2 ring (binary64 / double-float TMEM queue)
@@ -113,11 +133,11 @@ struct FusedSmem {
   T u2ring[U2 ? NSLOT : 1][U2 ? SY : 1][U2 ? SX : 1];  // u_2 per haloed point of the five ring planes
   // without the TMEM queue: D1_x u0, D1_y u1 (and, binary32, D1_x u2, D1_y u2)
   // per plane (tile only)
-  T dring[ZT ? 1 : NSLOT][ZT ? 1 : NDV][ZT ? 1 : TY][ZT ? 1 : TX];
+  T dring[ZT ? 1 : NSLOT][ZT ? 1 : NDV][ZT ? 1 : NR][ZT ? 1 : TX];
   // binary64 / double-float: s_0 = D1_y u1 + D1_z u2 and s_1 = D1_x u0 + D1_z u2
   // on the centre plane; binary32: D1_y u1 and D1_x u0 of the last three
   // planes to enter (x0-haloed rows, x1-haloed columns)
-  T s0buf[NSB][TY][SX];
+  T s0buf[NSB][NR][SX];
   T s1buf[NSB][SY][TX];
   double red[2][32];          // block reduction of (ke, enstrophy)
   uint32_t tmem_base[2];      // TMEM allocations (z queue variant)
@@ -260,11 +280,14 @@ constexpr int tmem_columns() {
 }
 // The binary32 queue's second window (a separate allocation): the pair
 // (D1_x u2, D1_y u2) of slot s in columns 2s, 2s + 1 of a 16-column window.
-constexpr int TM_XCOLS = 16;
+template <typename T>
+constexpr int tm_xcols() {
+  return 16 * (int)(sizeof(T) / 4);
+}
 template <int NW, typename T = float>
 constexpr int tmem_columns2() {
   if (!mixz<T>()) return 0;
-  constexpr int need = TM_XCOLS * ((NW + 3) / 4);
+  constexpr int need = tm_xcols<T>() * ((NW + 3) / 4);
   int c = 32;
   while (c < need) c *= 2;
   return c;
@@ -430,11 +453,24 @@ __device__ __forceinline__ void tmem_store_diag(uint32_t win, int slot, dfloat d
 __device__ __forceinline__ void tmem_load_diag(uint32_t win, int slot, dfloat& d00, dfloat& d11) {
   tmem_load_diag8(win, slot, d00, d11);
 }
-// two columns per thread keep the shared-memory ring (no TMEM queue)
-__device__ __forceinline__ void tmem_store_diag(uint32_t, int, f32x2, f32x2) {}
-__device__ __forceinline__ void tmem_load_diag(uint32_t, int, f32x2&, f32x2&) {}
-__device__ __forceinline__ void tmem_load_rec(uint32_t, int, f32x2 (&)[NV]) {}
-__device__ __forceinline__ void tmem_store_rec(uint32_t, int, const f32x2 (&)[NV]) {}
+// row pairs: a value is two words, one a row
+__device__ __forceinline__ void to_words(f32x2 x, uint32_t& a, uint32_t& b) {
+  a = __float_as_uint(x.x);
+  b = __float_as_uint(x.y);
+}
+__device__ __forceinline__ void from_words(uint32_t a, uint32_t b, f32x2& x) {
+  x = f32x2(__uint_as_float(a), __uint_as_float(b));
+}
+__device__ __forceinline__ void tmem_store_rec(uint32_t win, int slot, const f32x2 (&r)[NV]) {
+  tmem_store_rec8(win, slot, r);
+}
+__device__ __forceinline__ void tmem_load_rec(uint32_t win, int slot, f32x2 (&r)[NV]) { tmem_load_rec8(win, slot, r); }
+__device__ __forceinline__ void tmem_store_diag(uint32_t win, int slot, f32x2 d00, f32x2 d11) {
+  tmem_store_diag8(win, slot, d00, d11);
+}
+__device__ __forceinline__ void tmem_load_diag(uint32_t win, int slot, f32x2& d00, f32x2& d11) {
+  tmem_load_diag8(win, slot, d00, d11);
+}
 
 // Allocate / release the CTA's TMEM columns (warp 0): NCOL for the queue
 // and, binary32, NCOL2 for its second window, publishing the base addresses
@@ -479,9 +515,10 @@ __device__ __forceinline__ uint32_t tmem_window(uint32_t base) {
   const uint32_t w = threadIdx.x >> 5;
   return base + (((w & 3u) * 32u) << 16) + (w >> 2) * (uint32_t)TmLayout<T>::COLS;
 }
+template <typename T>
 __device__ __forceinline__ uint32_t tmem_window2(uint32_t base2) {
   const uint32_t w = threadIdx.x >> 5;
-  return base2 + (((w & 3u) * 32u) << 16) + (w >> 2) * (uint32_t)TM_XCOLS;
+  return base2 + (((w & 3u) * 32u) << 16) + (w >> 2) * (uint32_t)tm_xcols<T>();
 }
 // the pair (D1_x u2, D1_y u2) of this thread's column in slot `slot` of the
 // second window
@@ -502,6 +539,25 @@ __device__ __forceinline__ void tmem_load_xdiag(uint32_t win2, int slot, float& 
       : "memory");
   d02 = __uint_as_float(a);
   d12 = __uint_as_float(b);
+}
+
+__device__ __forceinline__ void tmem_store_xdiag(uint32_t win2, int slot, f32x2 d02, f32x2 d12) {
+  asm volatile(
+      "tcgen05.st.sync.aligned.32x32b.x4.b32 [%0], {%1, %2, %3, %4};\n\t"
+      "tcgen05.wait::st.sync.aligned;" ::"r"(win2 + (uint32_t)(4 * slot)),
+      "r"(__float_as_uint(d02.x)), "r"(__float_as_uint(d02.y)), "r"(__float_as_uint(d12.x)), "r"(__float_as_uint(d12.y))
+      : "memory");
+}
+__device__ __forceinline__ void tmem_load_xdiag(uint32_t win2, int slot, f32x2& d02, f32x2& d12) {
+  uint32_t w[4];
+  asm volatile(
+      "tcgen05.ld.sync.aligned.32x32b.x4.b32 {%0, %1, %2, %3}, [%4];\n\t"
+      "tcgen05.wait::ld.sync.aligned;"
+      : "=r"(w[0]), "=r"(w[1]), "=r"(w[2]), "=r"(w[3])
+      : "r"(win2 + (uint32_t)(4 * slot))
+      : "memory");
+  from_words(w[0], w[1], d02);
+  from_words(w[2], w[3], d12);
 }
 
 // Stage input value in the arithmetic type (binary64 inputs to a binary32
@@ -543,6 +599,9 @@ __device__ __forceinline__ T mad(T a, T b, T c) {
   return a * b + c;
 }
 __device__ __forceinline__ f32x2 mad(f32x2 a, f32x2 b, f32x2 c) { return fma(a, b, c); }
+__device__ __forceinline__ float mad(float a, float b, float c) { return ::fmaf(a, b, c); }
+// rows y + 1, y + 2 from the pairs of rows (y, y + 1) and (y + 2, y + 3)
+__device__ __forceinline__ f32x2 next_row(f32x2 a, f32x2 b) { return f32x2(a.y, b.x); }
 
 // A stage value built from the stage input of each column a thread owns.
 template <typename T, typename TIN>
@@ -628,7 +687,7 @@ struct NoXTerms {
 // that involve x2 are taken with the x2 derivative last, D1_z(D1_x u2) and
 // D1_z(D1_y u2) from xfun(k, ...) (the neighbours' in-plane gradients of u2);
 // the stream also forms D1_z u2 at the centre.  WITH_KE: also lo[].
-template <int A, bool ZX, bool WITH_KE, typename T, typename LD, typename SF, typename XF = NoXTerms>
+template <int A, bool ZX, bool WITH_KE, bool HALVES = false, typename T = float, typename LD, typename SF, typename XF = NoXTerms>
 __device__ __forceinline__ void axis_terms_stream(const LD& ldrec, const SF& sfun, const Coef<T>& c,
                                                   const T (&uc)[3], StreamTerms<T>& t, const XF& xfun = XF()) {
   static_assert(!ZX || A == 2, "x2-last mixed terms belong to the x2 axis");
@@ -645,33 +704,41 @@ __device__ __forceinline__ void axis_terms_stream(const LD& ldrec, const SF& sfu
   for (int k = 0; k < 4; ++k) {
     const T cd = sgn(k, c.c1[A], c.c2[A]);
     const T ed = (k == 0 || k == 3) ? c.e2[A] : c.e1[A];
+    // rows that straddle two pairs: lane by lane, which spares putting the
+    // values together in register pairs
+    auto fm = [k](T x, T y, T z) {
+      if constexpr (HALVES) {
+        if (k == 1 || k == 2) return T(__fmaf_rn(x.x, y.x, z.x), __fmaf_rn(x.y, y.y, z.y));
+      }
+      return fmadd(x, y, z);
+    };
     T r[NV];
     ldrec(k, r);
-    const T w = fmadd(cd, r[V_U0 + A], sgn(k, cu1, cu2));
+    const T w = fm(cd, r[V_U0 + A], sgn(k, cu1, cu2));
 #pragma unroll
-    for (int i = 0; i < 3; ++i) t.rM[i] = fmadd(w, r[V_M0 + i], t.rM[i]);
-    t.rE = fmadd(w, r[V_H], t.rE);
-    t.rrho = fmadd(cd, fmadd(ua, r[V_RHO], r[V_M0 + A]), t.rrho);
-    dp = fmadd(cd, r[V_P], dp);
+    for (int i = 0; i < 3; ++i) t.rM[i] = fm(w, r[V_M0 + i], t.rM[i]);
+    t.rE = fm(w, r[V_H], t.rE);
+    t.rrho = fm(cd, fm(ua, r[V_RHO], r[V_M0 + A]), t.rrho);
+    dp = fm(cd, r[V_P], dp);
 #pragma unroll
     for (int i = 0; i < 3; ++i) {
       if (i != A) {
-        t.v[i] = fmadd(ed, r[V_U0 + i], t.v[i]);
+        t.v[i] = fm(ed, r[V_U0 + i], t.v[i]);
         const int pair = i + A - 1;  // (0,1) -> 0, (0,2) -> 1, (1,2) -> 2
-        t.a[pair] = fmadd(cd, r[V_U0 + i], t.a[pair]);
-        if (WITH_KE && i < A) t.lo[pair] = fmadd(cd, r[V_U0 + i], t.lo[pair]);
+        t.a[pair] = fm(cd, r[V_U0 + i], t.a[pair]);
+        if (WITH_KE && i < A) t.lo[pair] = fm(cd, r[V_U0 + i], t.lo[pair]);
       }
     }
     // the Laplacian and one third of Eq. 7 on j = A, one third of D1_A s_A
-    lA = fmadd(ed, r[V_U0 + A], lA);
-    gA = fmadd(cd, sfun(k), gA);
-    t.lapT = fmadd(ed, r[V_T], t.lapT);
+    lA = fm(ed, r[V_U0 + A], lA);
+    gA = fm(cd, sfun(k), gA);
+    t.lapT = fm(ed, r[V_T], t.lapT);
     if constexpr (ZX) {
       T x02, x12;
       xfun(k, x02, x12);
-      gz0 = fmadd(cd, x02, gz0);
-      gz1 = fmadd(cd, x12, gz1);
-      t.gd[2] = fmadd(cd, r[V_U2], t.gd[2]);
+      gz0 = fm(cd, x02, gz0);
+      gz1 = fm(cd, x12, gz1);
+      t.gd[2] = fm(cd, r[V_U2], t.gd[2]);
     }
   }
   t.rM[A] = t.rM[A] + dp;
@@ -912,16 +979,16 @@ __device__ __forceinline__ void assemble_dw(const DwTerms& t, const dfloat2 (&ce
 // TIN: type of the stage input in HBM; TOUT: type of the stage output.
 // CTAs per SM the launch bounds plan for: shared memory allows two 32 x 8
 // binary32 CTAs per SM with the 5-slot ring (113 KiB each) and three with
-// the TMEM queue and 3-slot ring (59 KiB each, 80 registers); binary64 and
+// the TMEM queue and 3-slot ring (59 KiB each, row pairs: 168 registers); binary64 and
 // double-float (194.5 KiB) and 32 x 16 tiles take one.
 template <typename T, int TY, bool ZT = false>
 constexpr int fused_min_blocks() {
-  return (sizeof(T) == 4 && TY <= 8) ? (ZT ? 3 : 2) : 1;
+  return ((sizeof(T) == 4 && TY <= 8) || row_pairs<T, ZT>()) ? (ZT ? 3 : 2) : 1;
 }
 // tile width in points: 32 columns per warp row, times the columns per thread
-template <typename T>
+template <typename T, bool ZT>
 constexpr int tile_width() {
-  return TX * Lanes<T>::N;
+  return row_pairs<T, ZT>() ? TX : TX * Lanes<T>::N;
 }
 
 // The z march of one CTA over the 32 x TY column tile (bx, by), output
@@ -939,28 +1006,29 @@ __device__ __forceinline__ void fused_march(const StageArgs& a, const Coef<T>& c
   constexpr bool DW = std::is_same<T, dfloat>::value;     // double-float: terms in pairs
   constexpr bool FIXED = std::is_same<T, double>::value;  // binary64: linear stencils in integers
   constexpr int SY = S::SY;
-  constexpr int NT = TX * TY;
+  constexpr bool RP = S::RP;
+  constexpr int HR = S::HR, NR = S::NR;
+  constexpr int NT = TX * NR;
   constexpr int PTS = SX * SY;
   constexpr int NHALO = PTS - NT;                  // haloed points outside the tile
   constexpr int LPT = 1 + (NHALO + NT - 1) / NT;   // own point + halo points per thread
 
-  constexpr int PP = Lanes<T>::N;  // columns per thread: tx and tx + 32
+  constexpr int PP = Lanes<T>::N;  // points per thread: columns tx and tx + 32, or (RP) rows 2 ty and 2 ty + 1
   const int n0 = a.g.n0, n1 = a.g.n1, n2 = a.g.n2;
   const unsigned plane = (unsigned)n0 * (unsigned)n1;
   const int tid = threadIdx.x;
   const int tx = tid % TX, ty = tid / TX;
-  const int x0 = bx * (TX * PP), y0 = by * TY;
+  const int x0 = bx * tile_width<T, ZT>(), y0 = by * TY;
   const int zend = min(zend_req, n2);
-  const int gy = y0 + ty;
   bool valid[PP];
   unsigned own[PP];
 #pragma unroll
   for (int j = 0; j < PP; ++j) {
-    const int gx = x0 + tx + TX * j;
+    const int gx = x0 + tx + (RP ? 0 : TX * j);
+    const int gy = y0 + (RP ? 2 * ty + j : ty);
     valid[j] = (gx < n0) && (gy < n1);
     own[j] = valid[j] ? (unsigned)gx + (unsigned)n0 * (unsigned)gy : 0u;
   }
-  const bool valid_xy = valid[0];  // column tx (the second column is valid only if the first is)
   // per-field base pointers; offsets inside a field are 32-bit (P < 2^32)
   const TIN* qf[NF];
   const double* accf[NF];
@@ -979,25 +1047,26 @@ __device__ __forceinline__ void fused_march(const StageArgs& a, const Coef<T>& c
   for (int l = 0; l < LPT; ++l) {
     int sy = -1, sx = -1;
     if (l == 0) {
-      sy = ty + HALO;
+      sy = ty + HR;
       sx = tx + HALO;
     } else {
       const int h = tid + (l - 1) * NT;
-      if (h < 4 * SX) {
+      if (h < 2 * HR * SX) {
         const int r = h / SX;
-        sy = (r < 2) ? r : TY + r;
+        sy = (r < HR) ? r : NR + r;
         sx = h % SX;
       } else if (h < NHALO) {
-        const int h2 = h - 4 * SX;
+        const int h2 = h - 2 * HR * SX;
         const int k = h2 & 3;
-        sy = HALO + (h2 >> 2);
+        sy = HR + (h2 >> 2);
         sx = (k < 2) ? k : TX + k;
       }
     }
     if (sy >= 0) {
 #pragma unroll
       for (int j = 0; j < PP; ++j)
-        ld_off[l][j] = wrapi(x0 - HALO + sx + TX * j, n0) + n0 * wrapi(y0 - HALO + sy, n1);
+        ld_off[l][j] = wrapi(x0 - HALO + sx + (RP ? 0 : TX * j), n0) +
+                       n0 * wrapi(y0 - HALO + (RP ? 2 * sy + j : sy), n1);
       ld_s[l] = sy * SX + sx;
     } else {
 #pragma unroll
@@ -1011,28 +1080,28 @@ __device__ __forceinline__ void fused_march(const StageArgs& a, const Coef<T>& c
   // the window address is warp-uniform; broadcasting lane 0's copy lets the
   // compiler keep it in a uniform register for the tcgen05 operands
   const uint32_t twin = ZT ? __shfl_sync(0xffffffffu, tmem_window<T>(tmem_base), 0) : 0u;
-  const uint32_t twin2 = (ZT && MIXZ) ? __shfl_sync(0xffffffffu, tmem_window2(tmem_base2), 0) : 0u;
+  const uint32_t twin2 = (ZT && MIXZ) ? __shfl_sync(0xffffffffu, tmem_window2<T>(tmem_base2), 0) : 0u;
   T d22 = T(0);
   T g00c = T(0), g11c = T(0);  // D1_x u0, D1_y u1 at the centre point
 
   // halo tasks of phase 2b, fixed for the whole z march: s_0 on the x0-halo
   // columns (4*TY points) and s_1 on the x1-halo rows (4*TX points)
-  constexpr int NHT = 4 * (TX + TY);
+  constexpr int NHT = 4 * NR + 2 * HR * TX;
   constexpr int HPT = (NHT + NT - 1) / NT;  // tasks per thread
   int hk[HPT], hxy[HPT], hdst[HPT];         // kind (0 none, 1 s_0, 2 s_1), packed (hy, hx), buffer index
 #pragma unroll
   for (int j = 0; j < HPT; ++j) {
     const int h = tid + j * NT;
-    if (h < 4 * TY) {
+    if (h < 4 * NR) {
       const int r = h >> 2, k = h & 3;
       const int hx = (k < 2) ? k : TX + k;  // 0, 1, TX+2, TX+3
       hk[j] = 1;
-      hxy[j] = ((r + HALO) << 8) | hx;
+      hxy[j] = ((r + HR) << 8) | hx;
       hdst[j] = r * SX + hx;
     } else if (h < NHT) {
-      const int h2 = h - 4 * TY;
+      const int h2 = h - 4 * NR;
       const int col = h2 % TX, k = h2 / TX;
-      const int hy = (k < 2) ? k : TY + k;
+      const int hy = (k < HR) ? k : NR + k;
       hk[j] = 2;
       hxy[j] = (hy << 8) | (col + HALO);
       hdst[j] = hy * TX + col;
@@ -1169,13 +1238,23 @@ __device__ __forceinline__ void fused_march(const StageArgs& a, const Coef<T>& c
       }
     } else {
       const T(*R)[SX][NV] = sm.ring[fe];
-      const int sy = ty + HALO, sx = tx + HALO;
+      const int sy = ty + HR, sx = tx + HALO;
       const T d00 = mad(c.c1[0], R[sy][sx + 1][V_U0] - R[sy][sx - 1][V_U0],
                         -c.c2[0] * (R[sy][sx + 2][V_U0] - R[sy][sx - 2][V_U0]));
       // u1 and u2 of the x1 neighbours (adjacent fields: one 8-byte load each
       // in binary32, whose records sit at 8-byte multiples)
       T y1[4], y2[4];
-      {
+      if constexpr (RP) {
+        f32x2 u1[3], u2[3];
+#pragma unroll
+        for (int k = 0; k < 3; ++k) {
+          const float4 v = *reinterpret_cast<const float4*>(&R[sy + k - 1][sx][V_U1]);
+          u1[k] = f32x2(v.x, v.y);
+          u2[k] = f32x2(v.z, v.w);
+        }
+        y1[0] = u1[0], y1[1] = next_row(u1[0], u1[1]), y1[2] = next_row(u1[1], u1[2]), y1[3] = u1[2];
+        y2[0] = u2[0], y2[1] = next_row(u2[0], u2[1]), y2[2] = next_row(u2[1], u2[2]), y2[3] = u2[2];
+      } else {
         const int oy[4] = {-2, -1, 1, 2};
 #pragma unroll
         for (int k = 0; k < 4; ++k) {
@@ -1216,8 +1295,20 @@ __device__ __forceinline__ void fused_march(const StageArgs& a, const Coef<T>& c
         for (int j = 0; j < HPT; ++j) {
           const int hy = hxy[j] >> 8, hx = hxy[j] & 0xFF;
           if (hk[j] == 1) {
-            (&sm.s0buf[sbe][0][0])[hdst[j]] = mad(c.c1[1], R[hy + 1][hx][V_U1] - R[hy - 1][hx][V_U1],
-                                                  -c.c2[1] * (R[hy + 2][hx][V_U1] - R[hy - 2][hx][V_U1]));
+            T m2, m1, p1, p2;
+            if constexpr (RP) {
+              const T o = R[hy][hx][V_U1];
+              m2 = R[hy - 1][hx][V_U1];
+              p2 = R[hy + 1][hx][V_U1];
+              m1 = next_row(m2, o);
+              p1 = next_row(o, p2);
+            } else {
+              m2 = R[hy - 2][hx][V_U1];
+              m1 = R[hy - 1][hx][V_U1];
+              p1 = R[hy + 1][hx][V_U1];
+              p2 = R[hy + 2][hx][V_U1];
+            }
+            (&sm.s0buf[sbe][0][0])[hdst[j]] = mad(c.c1[1], p1 - m1, -c.c2[1] * (p2 - m2));
           } else if (hk[j] == 2) {
             (&sm.s1buf[sbe][0][0])[hdst[j]] = mad(c.c1[0], R[hy][hx + 1][V_U0] - R[hy][hx - 1][V_U0],
                                                   -c.c2[0] * (R[hy][hx + 2][V_U0] - R[hy][hx - 2][V_U0]));
@@ -1381,7 +1472,7 @@ __device__ __forceinline__ void fused_march(const StageArgs& a, const Coef<T>& c
     // ---------------------------------------------------------------- phase 3
     {
       fetch_acc();
-      const int sy = ty + HALO, sx = tx + HALO;
+      const int sy = ty + HR, sx = tx + HALO;
       const T(*C)[SX][NV] = sm.ring[fc];
       T rho_p, mc[3], uc[3];  // centre values
 
@@ -1390,7 +1481,16 @@ __device__ __forceinline__ void fused_march(const StageArgs& a, const Coef<T>& c
       const int off[4] = {-2, -1, 1, 2};
       const int zs[4] = {sl[0], sl[1], sl[3], sl[4]};
       auto sf0 = [&](int k) { return sm.s0buf[sbc][ty][sx + off[k]]; };
-      auto sf1 = [&](int k) { return sm.s1buf[sbc][sy + off[k]][tx]; };
+      auto sf1 = [&](int k) {
+        if constexpr (RP) {
+          const int q = k < 2 ? sy - 1 : sy;
+          if (k == 0) return sm.s1buf[sbc][sy - 1][tx];
+          if (k == 3) return sm.s1buf[sbc][sy + 1][tx];
+          return next_row(sm.s1buf[sbc][q][tx], sm.s1buf[sbc][q + 1][tx]);
+        } else {
+          return sm.s1buf[sbc][sy + off[k]][tx];
+        }
+      };
       auto sf2 = [&](int k) {
         if constexpr (ZT) {
           T a, b;
@@ -1452,14 +1552,25 @@ __device__ __forceinline__ void fused_march(const StageArgs& a, const Coef<T>& c
         }
       } else {
         auto ld0 = [&](int k, T(&r)[NV]) { load_rec(&C[sy][sx + off[k]][0], r); };
-        auto ld1 = [&](int k, T(&r)[NV]) { load_rec(&C[sy + off[k]][sx][0], r); };
+        T cen[NV];
+        T yp[RP ? NV : 1];  // row pairs: the pair above, then the one below
+        auto ld1 = [&](int k, T(&r)[NV]) {
+          if constexpr (RP) {  // rows y + off, y + 1 + off: a pair, or halves of two
+            if (k == 0) load_rec(&C[sy - 1][sx][0], yp);
+            if (k == 2) load_rec(&C[sy + 1][sx][0], yp);
+#pragma unroll
+            for (int v = 0; v < NV; ++v)
+              r[v] = k == 1 ? next_row(yp[v], cen[v]) : k == 2 ? next_row(cen[v], yp[v]) : yp[v];
+          } else {
+            load_rec(&C[sy + off[k]][sx][0], r);
+          }
+        };
         auto ld2 = [&](int k, T(&r)[NV]) {
           if constexpr (ZT)
             tmem_load_rec(twin, zs[k], r);
           else
             load_rec(&sm.ring[zs[k]][sy][sx][0], r);
         };
-        T cen[NV];
         if constexpr (ZT)
           tmem_load_rec(twin, scen, cen);
         else
@@ -1502,7 +1613,7 @@ __device__ __forceinline__ void fused_march(const StageArgs& a, const Coef<T>& c
           // shared-memory loads of one axis at a time: hoisted over the axes they spill at the binary32 ring
           // kernel's 128 registers (256^3: 674 us a stage without these two, 651 with)
           if constexpr (!ZT && sizeof(T) == 4) asm volatile("" ::: "memory");
-          axis_terms_stream<1, false, WITH_KE>(ld1, sf1, c, uc, t);
+          axis_terms_stream<1, false, WITH_KE, RP>(ld1, sf1, c, uc, t);
           if constexpr (!ZT && sizeof(T) == 4) asm volatile("" ::: "memory");
           axis_terms_stream<2, MIXZ, WITH_KE>(ld2, sf2, c, uc, t, xf);
         }
@@ -1614,8 +1725,8 @@ __device__ __forceinline__ void fused_march(const StageArgs& a, const Coef<T>& c
           }
         }
         if (WITH_KE) {
-          const T ke_t = T(0.5) * (mc[0] * uc[0] + mc[1] * uc[1] + mc[2] * uc[2]);
-          const T ens_t = T(0.5) * (T(1) + rho_p) * (w0 * w0 + w1 * w1 + w2 * w2);
+          const T ke_t = T(0.5) * mad(mc[2], uc[2], mad(mc[1], uc[1], mc[0] * uc[0]));
+          const T ens_t = T(0.5) * (T(1) + rho_p) * mad(w2, w2, mad(w1, w1, w0 * w0));
           ke_acc += double(lane(ke_t, j));
           ens_acc += double(lane(ens_t, j));
         }
@@ -1670,17 +1781,18 @@ constexpr bool even_split() {
 
 // Single grid.  ZT: x2-neighbour records in TMEM.
 template <typename T, typename TIN, typename TOUT, int TY, bool RHS_ONLY, bool WITH_KE, bool DF, bool ZT, bool EVEN>
-__global__ void __launch_bounds__(TX* TY, fused_min_blocks<T, TY, ZT>())
+__global__ void __launch_bounds__(TX* FusedSmem<T, TY, ZT>::NR, fused_min_blocks<T, TY, ZT>())
     fused_stage_kernel(const StageArgs a, const Coef<T> c) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
   FusedSmem<T, TY, ZT>& sm = *reinterpret_cast<FusedSmem<T, TY, ZT>*>(smem_raw);
-  constexpr int NCOL = tmem_columns<TY, T>();  // TX*TY/32 = TY warps
-  constexpr int NCOL2 = tmem_columns2<TY, T>();
+  constexpr int NW = FusedSmem<T, TY, ZT>::NR;  // warps, one a row of records
+  constexpr int NCOL = tmem_columns<NW, T>();
+  constexpr int NCOL2 = tmem_columns2<NW, T>();
   uint32_t tbase = 0, tbase2 = 0;
   if (ZT) tmem_acquire<NCOL, NCOL2>(sm.tmem_base, tbase, tbase2);
   double ke = 0.0, ens = 0.0;
   if constexpr (EVEN) {
-    const int tiles_x = (a.g.n0 + tile_width<T>() - 1) / tile_width<T>(), tiles_y = (a.g.n1 + TY - 1) / TY;
+    const int tiles_x = (a.g.n0 + tile_width<T, ZT>() - 1) / tile_width<T, ZT>(), tiles_y = (a.g.n1 + TY - 1) / TY;
     const long long units = (long long)tiles_x * tiles_y * a.g.n2;
     long long u = units * blockIdx.x / gridDim.x;
     const long long end = units * (blockIdx.x + 1) / gridDim.x;
@@ -1698,7 +1810,7 @@ __global__ void __launch_bounds__(TX* TY, fused_min_blocks<T, TY, ZT>())
   }
   if (WITH_KE) {
     const long long b = blockIdx.x + (long long)gridDim.x * (blockIdx.y + (long long)gridDim.y * blockIdx.z);
-    block_reduce_pair<TX * TY>(sm.red, ke, ens, a.ke_partials + 2 * b);
+    block_reduce_pair<TX * NW>(sm.red, ke, ens, a.ke_partials + 2 * b);
   }
   if (ZT) tmem_release<NCOL, NCOL2>(tbase, tbase2);
 }
@@ -1706,6 +1818,32 @@ __global__ void __launch_bounds__(TX* TY, fused_min_blocks<T, TY, ZT>())
 template <int TY, int W = TX>
 inline dim3 fused_grid(const Geom& g, int zc) {
   return dim3((g.n0 + W - 1) / W, (g.n1 + TY - 1) / TY, (g.n2 + zc - 1) / zc);
+}
+
+// binary32 constants for two-lane arithmetic
+inline Coef<f32x2> both_lanes(const Coef<float>& cf) {
+  Coef<f32x2> c;
+  for (int i = 0; i < 3; ++i) {
+    c.c1[i] = f32x2(cf.c1[i], cf.c1[i]);
+    c.c2[i] = f32x2(cf.c2[i], cf.c2[i]);
+    c.e0[i] = f32x2(cf.e0[i], cf.e0[i]);
+    c.e1[i] = f32x2(cf.e1[i], cf.e1[i]);
+    c.e2[i] = f32x2(cf.e2[i], cf.e2[i]);
+    c.hc1[i] = f32x2(cf.hc1[i], cf.hc1[i]);
+    c.hc2[i] = f32x2(cf.hc2[i], cf.hc2[i]);
+    c.t2[i] = f32x2(cf.t2[i], cf.t2[i]);
+    c.f2[i] = f32x2(cf.f2[i], cf.f2[i]);
+    c.v0[i] = f32x2(cf.v0[i], cf.v0[i]);
+  }
+  c.e0s = f32x2(cf.e0s, cf.e0s);
+  c.gm1 = f32x2(cf.gm1, cf.gm1);
+  c.gM2 = f32x2(cf.gM2, cf.gM2);
+  c.gm1x2 = f32x2(cf.gm1x2, cf.gm1x2);
+  c.hgM2 = f32x2(cf.hgM2, cf.hgM2);
+  c.inv_re = f32x2(cf.inv_re, cf.inv_re);
+  c.kappa = f32x2(cf.kappa, cf.kappa);
+  c.H0 = f32x2(cf.H0, cf.H0);
+  return c;
 }
 
 // The dynamic shared-memory limit is a per-device attribute of a kernel: set
@@ -1729,8 +1867,8 @@ cudaError_t launch_fused_k(const StageArgs& a, const Coef<T>& c, cudaStream_t s)
   const size_t smem = sizeof(FusedSmem<T, TY, ZT>);
   static std::atomic<unsigned long long> done{0};  // devices this instantiation is configured on
   if (cudaError_t e = ensure_smem_limit(k, smem, done)) return e;
-  const dim3 grid = EVEN ? dim3(a.ctas) : fused_grid<TY, tile_width<T>()>(a.g, a.zc);
-  k<<<grid, TX * TY, smem, s>>>(a, c);
+  const dim3 grid = EVEN ? dim3(a.ctas) : fused_grid<TY, tile_width<T, ZT>()>(a.g, a.zc);
+  k<<<grid, TX * FusedSmem<T, TY, ZT>::NR, smem, s>>>(a, c);
   return cudaGetLastError();
 }
 

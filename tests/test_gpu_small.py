@@ -20,9 +20,9 @@ def S():
     return sbli
 
 
-# one plane a CTA, two, three, the smallest configurable four, and more
+# one plane a CTA, two, three, the smallest configurable four, and more; odd row counts (row pairs with one valid row)
 @pytest.mark.parametrize("precision", [1, 2])
-@pytest.mark.parametrize("n", [(5, 5, 5), (32, 32, 32), (33, 40, 40), (64, 33, 41), (96, 70, 50)])
+@pytest.mark.parametrize("n", [(5, 5, 5), (31, 7, 20), (40, 9, 12), (32, 32, 32), (33, 40, 40), (64, 33, 41), (96, 70, 50)])
 def test_default_agrees_with_whole_tiles(S, n, precision):
     seen = []
     for cfg in (None, (8, 4, 0, 1), (8, 4, 1, 1), (8, max(4, n[2]), 0, 1)):
@@ -33,7 +33,7 @@ def test_default_agrees_with_whole_tiles(S, n, precision):
         g.init_tgv(0.9)
         hist = g.step_n_history(2, 1e-3).cpu().numpy()
         g.step_n(1, 1e-3)
-        seen.append((g.get_state().clone(), hist))
+        seen.append((torch.stack([g.get_state(), g.rhs()]), hist))
         g.close()
     for q, h in seen[:-1]:
         assert torch.equal(q, seen[-1][0])
