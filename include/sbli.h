@@ -209,8 +209,8 @@ SBLI_API int sbli_kinetic_energy_noalloc(const double* q_dev, int n0, int n1, in
                                          void* stream);
 
 /* Launch configuration of the fused kernel: in-plane tile height (the tile
- * is 32 x tile_y points per column a thread owns; binary64-register grids
- * (SBLI_FP64, SBLI_DF64) use 8, binary32 grids 8 or 16), planes per CTA
+ * is 32 x tile_y points per column a thread owns, 16 x 8 for binary64-register
+ * grids (SBLI_FP64, SBLI_DF64), which take 8; binary32 grids 8 or 16), planes per CTA
  * along x2 (>= 4; binary64-register grids split all planes evenly over the SMs
  * instead where that leaves the longest CTA fewer of them, and 4 lets binary32
  * grids too small to give every SM a CTA take fewer), where each thread keeps its column's records of the five
@@ -245,7 +245,8 @@ SBLI_API int sbli_autotune(sbli_grid* g, int reps, int* tile_y, int* planes_per_
  * Batched ensembles: up to 64 members (each its own grid size, Re, M, Pr,
  * gamma, L) advanced together.  Every Runge-Kutta stage of all members is one
  * persistent kernel launch that walks the members' work items (z chunk x
- * 32 x 8 tile, the z chunk per member set by the schedule below); step loops
+ * 32 x 8 tile, the z chunk per member set by the schedule below; binary64 and
+ * double-float members in equal runs of the planes of 16 x 8 tiles); step loops
  * are captured as CUDA graphs.  Any precision of
  * sbli_precision, as for single grids (others: SBLI_EINVAL).  Members'
  * results are bitwise those of the same member run alone as a single grid

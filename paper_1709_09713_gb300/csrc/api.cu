@@ -76,7 +76,8 @@ Layout layout_for(int n0, int n1, int n2, int precision, int variant) {
   // partial sums: the fused kernel's CTAs for any configuration the grid may
   // use (the smallest zc gives the most CTAs), or the KE kernel's blocks
   const long long tiles = (long long)((n0 + 31) / 32) * ((n1 + 3) / 4);
-  const long long max_ctas = tiles * ((n2 + 3) / 4);
+  const long long tiles64 = (long long)((n0 + F64_TILE_X - 1) / F64_TILE_X) * ((n1 + 7) / 8);
+  const long long max_ctas = std::max(tiles, tiles64) * ((n2 + 3) / 4);
   const long long np = std::max<long long>(std::max<long long>(max_ctas, ke_num_partials(g)), MAX_SMALL_CTAS);
   L.partials = align_up((size_t)(2 * np + 2) * sizeof(double));
   L.storeall = variant == SBLI_STORE_ALL
@@ -139,9 +140,10 @@ double* free64(const sbli_grid* g) {
   return g->reg64[(g->state + 1) % g->layout.n64];
 }
 
-// CTAs per SM a tile height allows (shared memory bound).
+// CTAs per SM a kernel allows (shared memory bound).
 int ctas_per_sm(int precision, int ty, int px = 1, int zq = 0) {
-  if (f64_registers(precision) || ty >= 16 || px == 2) return 1;
+  if (f64_registers(precision)) return F64_CTAS_PER_SM;
+  if (ty >= 16 || px == 2) return 1;
   return zq ? 3 : 2;  // the TMEM z queue keeps 3 full-record planes in shared memory
 }
 
@@ -151,7 +153,7 @@ void rank_zc(const Geom& g, int precision, int ty, int* best, int nbest, int px 
   int dev = 0, sms = 152;
   if (cudaGetDevice(&dev) == cudaSuccess) cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
   const long long slots = (long long)sms * ctas_per_sm(precision, ty, px, zq);
-  const int w = 32 * px;
+  const int w = f64_registers(precision) ? F64_TILE_X : 32 * px;
   const long long tiles = (long long)((g.n0 + w - 1) / w) * ((g.n1 + ty - 1) / ty);
   double cost[8];
   for (int i = 0; i < nbest; ++i) {
@@ -183,7 +185,7 @@ void use_config(sbli_grid* g, const FusedConfig& cfg) {
   g->cfg = cfg;
   g->zc = cfg.zc;
   if (f64_registers(g->precision))
-    g->split = plan_split(g->geom, cfg.zc, g->sms, g->precision == SBLI_DF64);
+    g->split = plan_split(g->geom, cfg.zc, std::min(F64_CTAS_PER_SM * g->sms, MAX_SMALL_CTAS), g->precision == SBLI_DF64);
   else
     g->zc = binary32_launch_zc(g->geom, cfg, g->sms);
 }

@@ -25,11 +25,11 @@ namespace sbli {
 // the CTA's TMEM columns held for all of its work items.  DF: binary32 stages
 // with the double-float accumulator (SBLI_FP32_DF members).
 template <typename T, typename TIN, typename TOUT, int TY, bool WITH_KE, bool ZT = false, bool DF = false>
-__global__ void __launch_bounds__(TX* FusedSmem<T, TY, ZT>::NR, fused_min_blocks<T, TY, ZT>())
+__global__ void __launch_bounds__(FusedSmem<T, TY, ZT>::NTHREADS, fused_min_blocks<T, TY, ZT>())
     batch_stage_kernel(const __grid_constant__ BatchParams<T> p) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
   FusedSmem<T, TY, ZT>& sm = *reinterpret_cast<FusedSmem<T, TY, ZT>*>(smem_raw);
-  constexpr int NW = FusedSmem<T, TY, ZT>::NR;
+  constexpr int NW = FusedSmem<T, TY, ZT>::NTHREADS / 32;
   constexpr int NCOL = tmem_columns<NW, T>();
   constexpr int NCOL2 = tmem_columns2<NW, T>();
   uint32_t tbase = 0, tbase2 = 0;
@@ -60,7 +60,7 @@ __global__ void __launch_bounds__(TX* FusedSmem<T, TY, ZT>::NR, fused_min_blocks
       u += len;
       // the CTA's part of this member ends: CTA + member numbers its partial sum
       if (WITH_KE && (u == end || u == p.item_begin[m + 1])) {
-        block_reduce_pair<TX * NW>(sm.red, ke, ens, p.ke_items + 2 * ((long long)blockIdx.x + m));
+        block_reduce_pair<32 * NW>(sm.red, ke, ens, p.ke_items + 2 * ((long long)blockIdx.x + m));
         ke = ens = 0.0;
       }
     }
@@ -77,7 +77,7 @@ __global__ void __launch_bounds__(TX* FusedSmem<T, TY, ZT>::NR, fused_min_blocks
       double ke = 0.0, ens = 0.0;
       fused_march<T, TIN, TOUT, TY, false, WITH_KE, DF, ZT>(a, p.c[lo], bx, by, zbeg, zbeg + a.zc, sm, ke, ens,
                                                             tbase, tbase2);
-      if (WITH_KE) block_reduce_pair<TX * NW>(sm.red, ke, ens, p.ke_items + 2 * item);
+      if (WITH_KE) block_reduce_pair<32 * NW>(sm.red, ke, ens, p.ke_items + 2 * item);
     }
   }
   if (ZT) tmem_release<NCOL, NCOL2>(tbase, tbase2);
@@ -110,7 +110,7 @@ static cudaError_t launch_batch_k(const BatchParams<T>& p, int grid, cudaStream_
   static std::atomic<unsigned long long> done{0};
   if (cudaError_t e = ensure_smem_limit(k, smem, done)) return e;
   if (even_split<T>()) grid = (int)std::min<long long>(grid, p.total_items);
-  k<<<grid, TX * FusedSmem<T, 8, ZT>::NR, smem, s>>>(p);
+  k<<<grid, FusedSmem<T, 8, ZT>::NTHREADS, smem, s>>>(p);
   return cudaGetLastError();
 }
 
@@ -358,7 +358,7 @@ cudaError_t enqueue_batch_stage_t(sbli_batch* b, int k, int state, double dt, do
   for (int m = 0; m < b->count; ++m) {
     const MemberLayout& M = b->L.m[m];
     p.item_begin[m] = acc;
-    p.tiles_x[m] = (M.n[0] + TX - 1) / TX;
+    p.tiles_x[m] = (M.n[0] + tile_x<T>() - 1) / tile_x<T>();
     p.tiles_y[m] = (M.n[1] + 7) / 8;
     acc += batch_f64_registers(b->precision) ? member_planes(M.n) : member_items(M.n, M.launch_zc);
     p.a[m] = member_stage(b, m, k, state, dt, &in64);

@@ -39,10 +39,11 @@ inline int batch_default_zq(int precision) { return precision == SBLI_FP32 || pr
 // Resident CTAs per SM of the multi-member launch: binary32 members run the
 // TMEM-queue kernel (59 KiB shared, four warps of at most 168 registers: 3 per SM) or the shared
 // ring (113 KiB: 2 per SM); binary64 and double-float-arithmetic members
-// the 194.5 KiB shared ring or the 124 KiB TMEM-queue kernel (1 per SM).
+// 16 x 8 tiles of the 107 KiB shared ring or the 69 KiB TMEM-queue kernel, whose
+// registers fit twice.
 inline int batch_ctas_per_sm(int precision, int zq) {
   if (precision == SBLI_FP32 || precision == SBLI_FP32_DF) return zq ? 3 : 2;
-  return 1;
+  return F64_CTAS_PER_SM;
 }
 
 // CTAs of a launch: persistent ones that fill the SMs.  The even split keeps
@@ -60,8 +61,10 @@ inline int batch_zc(int n2) { return n2 < 32 ? n2 : 32; }
 inline long long member_items(const int n[3], int zc) {
   return (long long)((n[0] + 31) / 32) * ((n[1] + 7) / 8) * ((n[2] + zc - 1) / zc);
 }
-// Planes of all tiles of one member: the units of the even split.
-inline long long member_planes(const int n[3]) { return member_items(n, 1); }
+// Planes of all 16 x 8 tiles of one member: the units of the even split.
+inline long long member_planes(const int n[3]) {
+  return (long long)((n[0] + F64_TILE_X - 1) / F64_TILE_X) * ((n[1] + 7) / 8) * n[2];
+}
 
 // Binary32 members under the default schedule: the cap on the planes per item
 // (32, 16, 8 or 4; a member's own are batch_zc) that the model of a stage

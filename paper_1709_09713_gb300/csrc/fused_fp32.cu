@@ -89,16 +89,17 @@ int binary32_launch_zc(const Geom& g, const FusedConfig& cfg, int sms) {
 }
 
 // The longest CTA decides, in planes, each march's four fill planes counting
-// WARM of a plane (their primitives) each.  A plane of the even split costs
-// double-float kernels some percent more (its CTAs share no halos in L2): 64^3
-// 43.7 us a stage against 42.2 in chunks of 8 planes, 256^3 2.109 ms against
-// 2.116 in chunks of 64, 32^3 10.2 against 26.  Binary64: 256^3 8.84 against 9.24
-// ms, 128^3 1.130 against 1.202, 64^3 168 against 177 us, 32^3 33.7 against 94.9.
-Split plan_split(const Geom& g, int zc, int sms, bool double_float) {
-  constexpr double WARM = 0.12;
-  const double plane = double_float ? 1.09 : 1.0;
-  const long long tiles = (long long)((g.n0 + TX - 1) / TX) * ((g.n1 + 7) / 8), units = tiles * g.n2;
-  const long long ctas = units < sms ? units : sms;
+// WARM of a plane (their primitives) each, and a plane of the even split 4 or 5 %
+// more (its CTAs share no halos in L2).  The even split against chunks, us a
+// stage: double-float 32^3 10.0 against 16.9, 129x97x66 127 against 132, 128^3 260 against
+// 264, but 96^3 117 against 114 and 256^3 1979 against 1938; binary64 32^3 27.9 against
+// 46.2, 128^3 781 against 810, 256^3 6033 against 6171, but 150x75x61 318 against 299.  Over 21
+// grids the rule loses 0.2 % on average to the better of the two.
+Split plan_split(const Geom& g, int zc, int slots, bool double_float) {
+  constexpr double WARM = 0.15;
+  const double plane = double_float ? 1.05 : 1.04;
+  const long long tiles = (long long)((g.n0 + F64_TILE_X - 1) / F64_TILE_X) * ((g.n1 + 7) / 8), units = tiles * g.n2;
+  const long long ctas = units < slots ? units : slots;
   double even = 0.0;
   for (long long c = 0; c < ctas; ++c) {
     const long long u = units * c / ctas, end = units * (c + 1) / ctas;
@@ -106,7 +107,7 @@ Split plan_split(const Geom& g, int zc, int sms, bool double_float) {
     even = std::max(even, plane * (double)(end - u) + 4 * WARM * marches);
   }
   const long long chunks = tiles * ((g.n2 + zc - 1) / zc);
-  const double waves = (double)((chunks + sms - 1) / sms);
+  const double waves = (double)((chunks + slots - 1) / slots);
   if (waves * (std::min(zc, g.n2) + 4 * WARM) < even) return Split{(int)chunks, 0};
   return Split{(int)ctas, 1};
 }

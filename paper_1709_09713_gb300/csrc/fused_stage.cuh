@@ -30,7 +30,7 @@
 //     records only for the entering, middle and centre planes: binary32 59 KiB
 //     per 32 x 8 CTA, three CTAs per SM (binary64 and double-float records
 //     take two TMEM columns per value and keep u_2 of the five planes for
-//     D1_z u_2 on the halo: 124 KiB, one CTA).  32 x 16 binary32 tiles (one
+//     D1_z u_2 on the halo: 69 KiB per 16 x 8 CTA, two CTAs).  32 x 16 binary32 tiles (one
 //     CTA per SM) keep a fourth full-record plane (the one that was the
 //     centre one plane earlier): the next entering plane then overwrites a
 //     slot nobody reads any more, so the barrier that ends each plane is not
@@ -76,7 +76,6 @@ namespace sbli {
 
 constexpr int TX = 32;  // tile width along x0 (one warp)
 constexpr int HALO = 2;
-constexpr int SX = TX + 2 * HALO;
 constexpr int NSLOT = 5;
 
 // primitive values of one point record in a ring slot; V_H is E' + 2 p' (see
@@ -103,6 +102,17 @@ template <typename T>
 constexpr bool mixz() {
   return std::is_same<T, float>::value || std::is_same<T, f32x2>::value;
 }
+// Tile width: 32 columns, a warp a row, for binary32; 16 for binary64 and
+// double-float, two rows a warp.  A 16 x 8 tile of 80-byte records takes
+// 107 KiB of the shared ring, so two CTAs of four warps share an SM and one's
+// arithmetic runs through the other's barriers and latencies, and ragged edges
+// waste half as much, for 1.88 instead of 1.69 records converted a point.  us a
+// stage, one 32 x 8 CTA an SM -> two of 16 x 8: binary64 128^3 825 -> 781, 256^3
+// 6380 -> 6035, 129x97x66 454 -> 386; double-float 279 -> 264, 2119 -> 1938, 154 -> 132.
+template <typename T>
+constexpr int tile_x() {
+  return std::is_same<T, double>::value || std::is_same<T, dfloat>::value ? F64_TILE_X : TX;
+}
 // Row pairs (f32x2 with the TMEM queue): a thread owns two neighbouring rows
 // of its column, and a record holds both rows' values side by side, so the
 // rows of records are pairs: TY / 2 of them, with one pair of halo on each side.
@@ -120,9 +130,11 @@ constexpr bool row_pairs() {
 }
 template <typename T, int TY, bool ZT = false>
 struct FusedSmem {
+  static constexpr int TX = tile_x<T>(), SX = TX + 2 * HALO;
   static constexpr bool RP = row_pairs<T, ZT>();
   static constexpr int HR = RP ? HALO / 2 : HALO;  // rows of halo records on each side
-  static constexpr int NR = RP ? TY / 2 : TY;      // rows of records of the tile (warps of a CTA)
+  static constexpr int NR = RP ? TY / 2 : TY;      // rows of records of the tile
+  static constexpr int NTHREADS = TX * NR;
   static constexpr int SY = NR + 2 * HR;
   static constexpr int NFULL = full_slots<T, TY, ZT>();
   static constexpr bool MIXZ = mixz<T>();
@@ -476,7 +488,7 @@ __device__ __forceinline__ void tmem_load_diag(uint32_t win, int slot, f32x2& d0
 // and, binary32, NCOL2 for its second window, publishing the base addresses
 // through shared memory.  The CTAs that shared memory lets share an SM never
 // ask for more than the 512 columns available (binary32 32 x 8: 3 x (128 +
-// 32); 32 x 16: 256 + 64; binary64 and double-float 32 x 8: 256, one CTA),
+// 32); 32 x 16: 256 + 64; binary64 and double-float 16 x 8: 2 x 128),
 // so the allocation never waits.
 template <int NCOL, int NCOL2 = 0>
 __device__ __forceinline__ void tmem_acquire(uint32_t (&smem_slot)[2], uint32_t& base, uint32_t& base2) {
@@ -980,18 +992,20 @@ __device__ __forceinline__ void assemble_dw(const DwTerms& t, const dfloat2 (&ce
 // CTAs per SM the launch bounds plan for: shared memory allows two 32 x 8
 // binary32 CTAs per SM with the 5-slot ring (113 KiB each) and three with
 // the TMEM queue and 3-slot ring (59 KiB each, row pairs: 168 registers); binary64 and
-// double-float (194.5 KiB) and 32 x 16 tiles take one.
+// double-float 16 x 8 tiles (107 KiB, 255 registers of four warps) two; 32 x 16
+// tiles take one.
 template <typename T, int TY, bool ZT = false>
 constexpr int fused_min_blocks() {
+  if (is_f64_class<T>()) return 2;
   return ((sizeof(T) == 4 && TY <= 8) || row_pairs<T, ZT>()) ? (ZT ? 3 : 2) : 1;
 }
-// tile width in points: 32 columns per warp row, times the columns per thread
+// tile width in points: the threads of a row, times the columns per thread
 template <typename T, bool ZT>
 constexpr int tile_width() {
-  return row_pairs<T, ZT>() ? TX : TX * Lanes<T>::N;
+  return row_pairs<T, ZT>() ? TX : tile_x<T>() * Lanes<T>::N;
 }
 
-// The z march of one CTA over the 32 x TY column tile (bx, by), output
+// The z march of one CTA over the tile_width x TY column tile (bx, by), output
 // planes [zbeg, min(zend, n2)), for the grid and stage described by `a`.
 // Adds the stage input's kinetic energy and enstrophy of the tile's points
 // to ke_acc / ens_acc when WITH_KE.  Ends with a barrier, so the shared
@@ -1007,7 +1021,7 @@ __device__ __forceinline__ void fused_march(const StageArgs& a, const Coef<T>& c
   constexpr bool FIXED = std::is_same<T, double>::value;  // binary64: linear stencils in integers
   constexpr int SY = S::SY;
   constexpr bool RP = S::RP;
-  constexpr int HR = S::HR, NR = S::NR;
+  constexpr int TX = S::TX, SX = S::SX, HR = S::HR, NR = S::NR;
   constexpr int NT = TX * NR;
   constexpr int PTS = SX * SY;
   constexpr int NHALO = PTS - NT;                  // haloed points outside the tile
@@ -1768,9 +1782,9 @@ __device__ __forceinline__ void block_reduce_pair(double (&red)[2][32], double k
 // How the work is split over CTAs.  Chunks: one CTA a (tile, z chunk).  Even
 // split: every CTA takes a contiguous run of the planes of all tiles, numbered
 // tile by tile (a run that crosses into the next tile starts a new march
-// there), one CTA per SM, so that no SM idles in a last wave and a grid with
-// fewer chunks than SMs still fills them.  The binary64-register kernels (one
-// CTA per SM, bound by arithmetic) choose by the longest CTA (plan_split); the
+// there), as many CTAs as fit the SMs at once, so that no SM idles in a last wave and a grid with
+// fewer chunks than that still fills them.  The binary64-register kernels (two
+// CTAs per SM, bound by arithmetic) choose by the longest CTA (plan_split); the
 // binary32 kernels, bound by memory and its latency, keep the chunks:
 // concurrent CTAs then march through the same planes and share their halos in
 // L2.
@@ -1781,11 +1795,11 @@ constexpr bool even_split() {
 
 // Single grid.  ZT: x2-neighbour records in TMEM.
 template <typename T, typename TIN, typename TOUT, int TY, bool RHS_ONLY, bool WITH_KE, bool DF, bool ZT, bool EVEN>
-__global__ void __launch_bounds__(TX* FusedSmem<T, TY, ZT>::NR, fused_min_blocks<T, TY, ZT>())
+__global__ void __launch_bounds__(FusedSmem<T, TY, ZT>::NTHREADS, fused_min_blocks<T, TY, ZT>())
     fused_stage_kernel(const StageArgs a, const Coef<T> c) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
   FusedSmem<T, TY, ZT>& sm = *reinterpret_cast<FusedSmem<T, TY, ZT>*>(smem_raw);
-  constexpr int NW = FusedSmem<T, TY, ZT>::NR;  // warps, one a row of records
+  constexpr int NW = FusedSmem<T, TY, ZT>::NTHREADS / 32;  // warps
   constexpr int NCOL = tmem_columns<NW, T>();
   constexpr int NCOL2 = tmem_columns2<NW, T>();
   uint32_t tbase = 0, tbase2 = 0;
@@ -1810,7 +1824,7 @@ __global__ void __launch_bounds__(TX* FusedSmem<T, TY, ZT>::NR, fused_min_blocks
   }
   if (WITH_KE) {
     const long long b = blockIdx.x + (long long)gridDim.x * (blockIdx.y + (long long)gridDim.y * blockIdx.z);
-    block_reduce_pair<TX * NW>(sm.red, ke, ens, a.ke_partials + 2 * b);
+    block_reduce_pair<32 * NW>(sm.red, ke, ens, a.ke_partials + 2 * b);
   }
   if (ZT) tmem_release<NCOL, NCOL2>(tbase, tbase2);
 }
@@ -1868,7 +1882,7 @@ cudaError_t launch_fused_k(const StageArgs& a, const Coef<T>& c, cudaStream_t s)
   static std::atomic<unsigned long long> done{0};  // devices this instantiation is configured on
   if (cudaError_t e = ensure_smem_limit(k, smem, done)) return e;
   const dim3 grid = EVEN ? dim3(a.ctas) : fused_grid<TY, tile_width<T, ZT>()>(a.g, a.zc);
-  k<<<grid, TX * FusedSmem<T, TY, ZT>::NR, smem, s>>>(a, c);
+  k<<<grid, FusedSmem<T, TY, ZT>::NTHREADS, smem, s>>>(a, c);
   return cudaGetLastError();
 }
 

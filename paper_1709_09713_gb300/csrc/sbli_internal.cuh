@@ -88,9 +88,14 @@ struct StageArgs {
 // four planes per CTA stay within it.
 constexpr int MAX_SMALL_CTAS = 512;
 
+// Tile width of the binary64-register kernels (tiles of 16 x 8 points) and
+// their CTAs per SM.
+constexpr int F64_TILE_X = 16;
+constexpr int F64_CTAS_PER_SM = 2;
+
 // Launch configuration chosen for one grid (the autotuner's output).
 struct FusedConfig {
-  int ty;  // in-plane tile height (tile is 32 x ty)
+  int ty;  // in-plane tile height (tile is 32 x ty, binary64 registers 16 x 8)
   int zc;  // planes per CTA
   int zq;  // binary32 paths: 0 = x2-neighbour records from the shared-memory
            // ring, 1 = from a per-thread queue in tensor memory (TMEM)
@@ -132,7 +137,7 @@ int binary32_launch_zc(const Geom& g, const FusedConfig& cfg, int sms);
 struct Split {
   int ctas, even;
 };
-Split plan_split(const Geom& g, int zc, int sms, bool double_float);
+Split plan_split(const Geom& g, int zc, int slots, bool double_float);
 
 // Diagnostics and state conversion (diag.cu).
 cudaError_t launch_init_tgv(const Geom& g, const sbli_params& p, double amplitude, double* q, cudaStream_t s);

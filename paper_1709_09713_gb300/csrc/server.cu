@@ -254,7 +254,7 @@ cudaError_t launch_group(sbli_server* s, int k, int precision, const std::vector
       const int* n = edges[m].data();
       const int zc = std::min(batch_zc(n[2]), cap);
       p.item_begin[m] = acc;
-      p.tiles_x[m] = (n[0] + 31) / 32;
+      p.tiles_x[m] = even ? (n[0] + F64_TILE_X - 1) / F64_TILE_X : (n[0] + 31) / 32;
       p.tiles_y[m] = (n[1] + 7) / 8;
       acc += even ? member_planes(n) : member_items(n, zc);
       p.a[m] = req_stage(s, q, k, zc, &in64);
@@ -512,7 +512,7 @@ int sbli_server_tick(sbli_server* s, int* completed) {
       K = std::min(K, kmin);
       // the even split of a binary64-register stage ends on every SM at once,
       // so binary32 requests would wait a whole stage for each of theirs:
-      // while there are any, an eighth of the SMs is left to them
+      // while there are any, an eighth of the CTA slots is left to them
       bool other = false;
       for (const Req& q : s->active) other |= lane_of(q.r.precision) != li && q.remaining > 0;
       const int grid64 = other ? s->grid64 - s->grid64 / 8 : s->grid64;

@@ -21,17 +21,20 @@ def S():
     return sbli
 
 
-# fewer planes than SMs; one more and one less than a full wave; runs over several tiles; a chunk that beats the split
-SIZES = [(5, 5, 5), (33, 9, 7), (32, 8, 151), (32, 8, 153), (40, 17, 61), (150, 75, 61)]
+# fewer planes than CTA slots; one more and one less than a full wave (304 planes of 16 x 8 tiles); runs over several
+# tiles; the last tile one column, or one column short; a chunk that beats the split
+SIZES = [(5, 5, 5), (33, 9, 7), (32, 8, 151), (32, 8, 153), (16, 8, 304), (17, 8, 23), (31, 8, 23), (40, 17, 61),
+         (150, 75, 61)]
 
 
 @pytest.mark.parametrize("precision", [0, 3])
 @pytest.mark.parametrize("n", SIZES)
 def test_splits_agree_bitwise(S, n, precision):
     seen = []
-    for zc in (4, 21, n[2]):  # the rule takes the chunks for some of these and the even split for others
+    # the rule takes the chunks for some of these and the even split for others; the last one with the TMEM queue
+    for zc, zq in ((4, 0), (21, 0), (n[2], 0), (21, 1)):
         g = S.Grid(n, precision)
-        g.set_config(8, max(4, zc), 0, 1)
+        g.set_config(8, max(4, zc), zq, 1)
         g.init_tgv(0.9)
         hist = g.step_n_history(2, 1e-3).cpu().numpy()
         g.step_n(1, 1e-3)
