@@ -24,7 +24,7 @@ def S():
 # fewer planes than CTA slots; one more and one less than a full wave (304 planes of 16 x 8 tiles); runs over several
 # tiles; the last tile one column, or one column short; a chunk that beats the split
 SIZES = [(5, 5, 5), (33, 9, 7), (32, 8, 151), (32, 8, 153), (16, 8, 304), (17, 8, 23), (31, 8, 23), (40, 17, 61),
-         (150, 75, 61)]
+         (48, 48, 24), (150, 75, 61)]
 
 
 @pytest.mark.parametrize("precision", [0, 3])
