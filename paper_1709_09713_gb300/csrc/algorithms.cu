@@ -4,9 +4,9 @@
 // fused kernel:
 //
 //   RS  Recompute Some: the 9 velocity gradients D_j u_i are stored to global
-//       arrays first (velocity arrays, then one derivative launch each, as BL
-//       does); every other derivative is a stencil written into the residual
-//       expressions, evaluated again at each place it occurs.
+//       arrays first (by BL's derivative kernel); every other derivative is a
+//       stencil written into the residual expressions, evaluated again at each
+//       place it occurs.
 //   SS  Store Some: the same 9 stored arrays; every other derivative is
 //       evaluated once into a thread-local variable and reused.
 //   RA  Recompute All: nothing stored; every derivative, velocity gradients
@@ -397,14 +397,10 @@ cudaError_t launch_algorithm_stage(int alg, const Geom& g, const Coef<double>& c
   cudaError_t e = cudaGetLastError();
   if (e != cudaSuccess) return e;
   if (algorithm_stores_gradients(alg)) {
-    // the 9 velocity-gradient arrays, one derivative launch each
-    const double* U = W;
+    // the 9 velocity-gradient arrays
     double* Gw = scratch + 5 * g.P;
-    for (int i = 0; i < 3; ++i)
-      for (int j = 0; j < 3; ++j) {
-        e = launch_derivative_fp64(g, c, U + i * g.P, Gw + (3 * i + j) * g.P, j, 1, s);
-        if (e != cudaSuccess) return e;
-      }
+    e = launch_gradients_fp64(g, c, W, Gw, s);
+    if (e != cudaSuccess) return e;
     G = Gw;
   }
   switch (alg) {

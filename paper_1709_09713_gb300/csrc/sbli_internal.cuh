@@ -194,10 +194,9 @@ cudaError_t launch_storeall_rhs_fp32(const Geom& g, const Coef<float>& c, const 
                                      float* scratch, float* r_out, cudaStream_t s);
 cudaError_t launch_rk_update(const Geom& g, const void* r, bool r_fp64, const double* acc_in, double* acc_out,
                              void* q_out, bool out_fp64, double a_dt, double b_dt, cudaStream_t s);
-// One derivative of one binary64 array (Eq. 6 for order 1, Eq. 7 for order 2)
-// along one axis into its own array, as the store-all variant computes them.
-cudaError_t launch_derivative_fp64(const Geom& g, const Coef<double>& c, const double* f, double* df, int axis,
-                                   int order, cudaStream_t s);
+// The nine velocity gradients D_j u_i (grad + (3 i + j) P) of the arrays
+// u + i P, as the store-all variant computes them.
+cudaError_t launch_gradients_fp64(const Geom& g, const Coef<double>& c, const double* u, double* grad, cudaStream_t s);
 
 // The paper's other evaluation strategies, binary64 (algorithms.cu): alg is
 // SBLI_RS, SBLI_SS, SBLI_RA, SBLI_SN or SBLI_SN2.  r_out != nullptr writes R

@@ -162,5 +162,21 @@ __host__ __device__ __forceinline__ double stencil_second(double m2, double m1, 
   const int64_t v = fixed::aligned(c, top);
   return fixed::rounded((int64_t)((uint64_t)a << 4) - b - (int64_t)(((uint64_t)v << 5) - ((uint64_t)v << 1)), top);
 }
+// both, the values aligned once where the centre does not raise the exponent that
+// the first derivative's values are aligned to (else each by itself)
+__host__ __device__ __forceinline__ void stencil_both(double m2, double m1, double c, double p1, double p2,
+                                                      double& first, double& second) {
+  const uint32_t top = fixed::top_exponent(m2, m1, p1, p2);
+  if (!fixed::alignable(top) || (fixed::high(c) & fixed::EXPONENT) > top) {
+    first = stencil_first(m2, m1, p1, p2);
+    second = stencil_second(m2, m1, c, p1, p2);
+    return;
+  }
+  const int64_t ap = fixed::aligned(p1, top), am = fixed::aligned(m1, top), v = fixed::aligned(c, top);
+  const int64_t bp = fixed::aligned(p2, top), bm = fixed::aligned(m2, top);
+  first = fixed::rounded((int64_t)((uint64_t)(ap - am) << 3) - (bp - bm), top);
+  second = fixed::rounded(
+      (int64_t)((uint64_t)(ap + am) << 4) - (bp + bm) - (int64_t)(((uint64_t)v << 5) - ((uint64_t)v << 1)), top);
+}
 
 }  // namespace sbli

@@ -2,13 +2,16 @@
 // the paper's memory-intensive comparison point.
 //
 // Exactly as the paper describes BL: (a) primitives and every product that
-// is differentiated go to full-grid temporary arrays; (b) one derivative
-// kernel per (field, direction, order) writes each of the 60 distinct
-// derivatives of Eqs. 1-3 to its own global array (Listing 1's derx, one
-// launch each); (c) a residual kernel reads the arrays and assembles Eqs. 1-3;
+// is differentiated go to full-grid temporary arrays; (b) derivative
+// kernels write each of the 60 distinct derivatives of Eqs. 1-3 to its own
+// global array (Listing 1's derx; one launch for those of the fields, one for the
+// mixed ones); (c) a residual kernel reads the arrays and assembles Eqs. 1-3;
 // (d) the Runge-Kutta update of Fig. 1 runs as its own kernel.
 //
 // Variables are deviations from the reference state, as in the fused path.
+#include <algorithm>
+#include <type_traits>
+
 #include "fpconv.cuh"
 #include "sbli_internal.cuh"
 #include "stencil_int.cuh"
@@ -82,28 +85,53 @@ __global__ void bl_primitives(Geom g, Coef<T> c, const TIN* __restrict__ q, T* _
   }
 }
 
-// One derivative of one array along one axis (Listing 1): order 1 is Eq. 6,
-// order 2 is Eq. 7.  A thread takes BL_Z points of one column: its wrapped
-// offsets are formed once (by comparisons), the values along x2 stay in
-// registers, and in binary64 the stencil is summed in integers, leaving one
-// binary64 product a point.  The modulo of every wrapped index had bounded it as
-// much as the binary64 pipe; integer instructions still do (15 us for 33.5 MB
-// moved at 128^3).  With the reciprocal and the shorter residual below, the
-// 128^3 store-all stage takes 1.37 instead of 1.80 ms.
-constexpr int BL_Z = 4;
-template <int ORDER, typename T>
-__device__ __forceinline__ T bl_stencil(T m2, T m1, T c, T p1, T p2, T k0, T k1, T k2) {
-  if constexpr (sizeof(T) == 8) {  // k2 = 1/(12 h) and -1/(12 h^2)
-    return ORDER == 1 ? k2 * stencil_first(m2, m1, p1, p2) : -k2 * stencil_second(m2, m1, c, p1, p2);
+// Derivatives along one axis of one array (Listing 1): Eq. 6 into d1, Eq. 7 into
+// d2, each to its own array (null: not wanted).
+template <typename T>
+struct Derivative {
+  const T* f;
+  T* d1;
+  T* d2;
+  int axis;
+};
+constexpr int BL_JOBS = 48;
+template <typename T>
+struct Derivatives {
+  Derivative<T> job[BL_JOBS];
+  int count;
+};
+
+// A thread takes BL_Z points of one column: its wrapped offsets are formed once
+// (by comparisons) and the values along x2 stay in registers.  The modulo of
+// every wrapped index had bounded it as much as the binary64 pipe.  In binary64
+// the stencil is summed in integers, leaving one binary64 product a derivative, but
+// every third first derivative alone in a binary64 sum beside them, which
+// balances the two pipes (half or a sixth of them: 1.06 and 1.10 ms a stage against
+// 1.04).  All derivatives that do not read another's result are blocks of one
+// launch: 128^3 points are little over a wave of blocks, so a launch per
+// derivative left the SMs half idle in its last wave and between launches.
+// With the bounds on registers here and of the residual kernel, the 128^3
+// store-all stage takes 1.04 instead of 1.36 ms, the 64^3 one 151 instead of 298 us.
+constexpr int BL_Z = 9;
+template <typename T>
+__device__ __forceinline__ T bl_first(T m2, T m1, T p1, T p2, T k1, T k2, bool integer) {
+  if constexpr (sizeof(T) == 8) {  // k2 = 1/(12 h)
+    return k2 * (integer ? stencil_first(m2, m1, p1, p2) : first_sum<false>(m2, m1, p1, p2, 0));
   } else {
-    return ORDER == 1 ? k1 * (p1 - m1) - k2 * (p2 - m2) : k0 * c + k1 * (p1 + m1) + k2 * (p2 + m2);
+    return k1 * (p1 - m1) - k2 * (p2 - m2);
   }
 }
-template <typename T, typename TS, int AXIS, int ORDER>
-__global__ void __launch_bounds__(256) bl_derivative(Geom g, const TS* __restrict__ f, T* __restrict__ df, T k0, T k1,
-                                                     T k2) {
-  const int i = blockIdx.x * 32 + threadIdx.x, j = blockIdx.y * 8 + threadIdx.y, k0z = blockIdx.z * BL_Z;
-  if (i >= g.n0 || j >= g.n1) return;
+template <typename T>
+__device__ __forceinline__ T bl_second(T m2, T m1, T c, T p1, T p2, T k0, T k1, T k2) {
+  if constexpr (sizeof(T) == 8) {  // k2 = -1/(12 h^2)
+    return -k2 * stencil_second(m2, m1, c, p1, p2);
+  } else {
+    return k0 * c + k1 * (p1 + m1) + k2 * (p2 + m2);
+  }
+}
+template <int AXIS, bool FIRST, bool SECOND, typename T>
+__device__ __forceinline__ void bl_column(const Geom& g, const Coef<T>& c, const T* __restrict__ f,
+                                          T* __restrict__ d1, T* __restrict__ d2, int i, int j, int k0) {
   const long long pl = (long long)g.n0 * g.n1;
   auto near = [](int v, int n) { return v < 0 ? v + n : (v >= n ? v - n : v); };  // |offset| <= 2 < n
   const int own = i + g.n0 * j;
@@ -111,37 +139,88 @@ __global__ void __launch_bounds__(256) bl_derivative(Geom g, const TS* __restric
 #pragma unroll
   for (int s = -2; s <= 2; ++s)
     o[s + 2] = AXIS == 0 ? near(i + s, g.n0) + g.n0 * j : AXIS == 1 ? i + g.n0 * near(j + s, g.n1) : own;
-  T w[4];  // AXIS 2: planes k - 2 .. k + 1
+  T w[5];  // the stencil's values; AXIS 2 keeps planes k - 2 .. k + 1
   if constexpr (AXIS == 2) {
 #pragma unroll
     for (int s = -2; s <= 1; ++s) {
-      int z = k0z + s;
+      int z = k0 + s;
       while (z >= g.n2) z -= g.n2;
-      w[s + 2] = T(f[own + pl * (z < 0 ? z + g.n2 : z)]);
+      w[s + 2] = f[own + pl * (z < 0 ? z + g.n2 : z)];
     }
   }
 #pragma unroll
   for (int q = 0; q < BL_Z; ++q) {
-    const int k = k0z + q;
+    const int k = k0 + q;
     if (k >= g.n2) break;
-    T v;
     if constexpr (AXIS == 2) {
-      const T p2 = T(f[own + pl * near(k + 2, g.n2)]);
-      v = bl_stencil<ORDER>(w[0], w[1], w[2], w[3], p2, k0, k1, k2);
-      w[0] = w[1];
-      w[1] = w[2];
-      w[2] = w[3];
-      w[3] = p2;
+      w[4] = f[own + pl * near(k + 2, g.n2)];
     } else {
-      const TS* p = f + pl * k;
-      v = bl_stencil<ORDER>(T(p[o[0]]), T(p[o[1]]), ORDER == 2 ? T(p[o[2]]) : T(0), T(p[o[3]]), T(p[o[4]]), k0, k1, k2);
+#pragma unroll
+      for (int s = 0; s < 5; ++s)
+        if (SECOND || s != 2) w[s] = f[o[s] + pl * k];
     }
-    df[own + pl * k] = v;
+    const long long at = own + pl * k;
+    if constexpr (FIRST && SECOND && sizeof(T) == 8) {
+      double a, b;
+      stencil_both(w[0], w[1], w[2], w[3], w[4], a, b);
+      d1[at] = c.c2[AXIS] * a;
+      d2[at] = -c.e2[AXIS] * b;
+    } else {
+      if constexpr (FIRST) d1[at] = bl_first(w[0], w[1], w[3], w[4], c.c1[AXIS], c.c2[AXIS], q % 3 != 1);
+      if constexpr (SECOND) d2[at] = bl_second(w[0], w[1], w[2], w[3], w[4], c.e0[AXIS], c.e1[AXIS], c.e2[AXIS]);
+    }
+    if constexpr (AXIS == 2) {
+#pragma unroll
+      for (int s = 0; s < 4; ++s) w[s] = w[s + 1];
+    }
   }
+}
+template <int AXIS, typename T>
+__device__ __forceinline__ void bl_axis(const Geom& g, const Coef<T>& c, const Derivative<T>& d, int i, int j, int k0) {
+  if (d.d1 && d.d2)
+    bl_column<AXIS, true, true>(g, c, d.f, d.d1, d.d2, i, j, k0);
+  else if (d.d1)
+    bl_column<AXIS, true, false>(g, c, d.f, d.d1, d.d2, i, j, k0);
+  else
+    bl_column<AXIS, false, true>(g, c, d.f, d.d1, d.d2, i, j, k0);
+}
+// blocks of 32 x 8 columns, BL_Z planes each, job by job
+template <typename T>
+__global__ void __launch_bounds__(256, 8) bl_derivatives(Geom g, const __grid_constant__ Coef<T> c,
+                                                      const __grid_constant__ Derivatives<T> jobs) {
+  const unsigned bx = (g.n0 + 31) / 32, by = (g.n1 + 7) / 8, bz = (g.n2 + BL_Z - 1) / BL_Z;
+  unsigned b = blockIdx.x;
+  const int i = b % bx * 32 + threadIdx.x;
+  b /= bx;
+  const int j = b % by * 8 + threadIdx.y;
+  b /= by;
+  const int k0 = b % bz * BL_Z;
+  if (i >= g.n0 || j >= g.n1) return;
+  const Derivative<T>& d = jobs.job[b / bz];
+  if (d.axis == 0) bl_axis<0>(g, c, d, i, j, k0);
+  else if (d.axis == 1) bl_axis<1>(g, c, d, i, j, k0);
+  else bl_axis<2>(g, c, d, i, j, k0);
 }
 
 template <typename T>
-__global__ void bl_residual(Geom g, Coef<T> c, const T* __restrict__ qrho, const T* __restrict__ qm,
+cudaError_t launch_derivatives(const Geom& g, const Coef<T>& c, const Derivatives<T>& jobs, cudaStream_t s) {
+  const long long blocks = (long long)((g.n0 + 31) / 32) * ((g.n1 + 7) / 8) * ((g.n2 + BL_Z - 1) / BL_Z);
+  // as many jobs a launch as the grid's limit of 2^31 - 1 blocks allows
+  const int most = (int)std::min<long long>(jobs.count, std::max<long long>(1, 0x7FFFFFFFll / blocks));
+  for (int at = 0; at < jobs.count; at += most) {
+    Derivatives<T> some;
+    some.count = std::min(most, jobs.count - at);
+    std::copy(jobs.job + at, jobs.job + at + some.count, some.job);
+    bl_derivatives<T><<<(unsigned)(blocks * some.count), dim3(32, 8), 0, s>>>(g, c, some);
+    if (cudaError_t e = cudaGetLastError()) return e;
+  }
+  return cudaSuccess;
+}
+
+// Bound by the binary64 pipe: sums start from their first term, and three blocks on
+// an SM instead of two (128^3 359 -> 300 us).
+template <typename T>
+__global__ void __launch_bounds__(256, 3) bl_residual(Geom g, Coef<T> c, const T* __restrict__ qrho, const T* __restrict__ qm,
                             const T* __restrict__ qE, long long qstride, T* __restrict__ s) {
   const long long P = g.P;
   for (long long n = blockIdx.x * (long long)blockDim.x + threadIdx.x; n < P; n += (long long)gridDim.x * blockDim.x) {
@@ -167,54 +246,28 @@ __global__ void bl_residual(Geom g, Coef<T> c, const T* __restrict__ qrho, const
     for (int i = 0; i < 3; ++i) {
       conv = m[i] * div;
       for (int j = 0; j < 3; ++j) conv += A(A_DRHOUU + 3 * i + j) + u[j] * A(A_DRHOU + 3 * i + j);
-      T lap = T(0), cross = T(0);
-      for (int j = 0; j < 3; ++j) {
-        lap += A(A_D2U + 3 * i + j);
-        cross += dd(i, j);
-      }
+      const T lap = A(A_D2U + 3 * i) + A(A_D2U + 3 * i + 1) + A(A_D2U + 3 * i + 2);
+      const T cross = dd(i, 0) + dd(i, 1) + dd(i, 2);
       const T sd = lap + T(1.0 / 3.0) * cross;  // Laplacian + G - 2/3 G
-      vw += u[i] * sd;
+      vw = i == 0 ? u[0] * sd : vw + u[i] * sd;
       s[(A_R + 1 + i) * P + n] = (T(-0.5) * conv - A(A_DP + i)) + c.inv_re * sd;
     }
     // Eq. 3 (reference enthalpy carries the constant parts of rho E and p)
     conv = E * div;
-    T pw = T(0), heat = T(0);
-    for (int j = 0; j < 3; ++j) {
-      conv += A(A_DEU + j) + u[j] * A(A_DE + j);
-      pw += A(A_DPU + j);
-      heat += A(A_D2T + j);
-    }
+    for (int j = 0; j < 3; ++j) conv += A(A_DEU + j) + u[j] * A(A_DE + j);
+    const T pw = A(A_DPU) + A(A_DPU + 1) + A(A_DPU + 2);
+    const T heat = A(A_D2T) + A(A_D2T + 1) + A(A_D2T + 2);
     // du_i/dx_j (du_i/dx_j + du_j/dx_i - 2/3 div delta_ij)
-    T diag = T(0), off = T(0);
+    T diag = du[0][0] * du[0][0], off = T(0);
     for (int i = 0; i < 3; ++i) {
-      diag += du[i][i] * du[i][i];
+      if (i > 0) diag += du[i][i] * du[i][i];
       const int j = (i + 1) % 3;
       const T a = du[i][j] + du[j][i];
-      off += a * a;
+      off = i == 0 ? a * a : off + a * a;
     }
     const T diss = T(2) * diag + (off - T(2.0 / 3.0) * div * div);
     s[(A_R + 4) * P + n] = ((T(-0.5) * conv - pw) - c.H0 * div) + (c.inv_re * (vw + diss) + c.kappa * heat);
   }
-}
-
-template <typename T, typename TS>
-cudaError_t launch_der(const Geom& g, const Coef<T>& c, const TS* f, T* df, int axis, int order, cudaStream_t s) {
-  dim3 blk(32, 8), grd((g.n0 + 31) / 32, (g.n1 + 7) / 8, (g.n2 + BL_Z - 1) / BL_Z);
-  const T k0 = c.e0[axis];
-  const T k1 = order == 1 ? c.c1[axis] : c.e1[axis];
-  const T k2 = order == 1 ? c.c2[axis] : c.e2[axis];
-#define SBLI_DER(A, O) bl_derivative<T, TS, A, O><<<grd, blk, 0, s>>>(g, f, df, k0, k1, k2)
-  if (order == 1) {
-    if (axis == 0) SBLI_DER(0, 1);
-    else if (axis == 1) SBLI_DER(1, 1);
-    else SBLI_DER(2, 1);
-  } else {
-    if (axis == 0) SBLI_DER(0, 2);
-    else if (axis == 1) SBLI_DER(1, 2);
-    else SBLI_DER(2, 2);
-  }
-#undef SBLI_DER
-  return cudaGetLastError();
 }
 
 unsigned pgrid(long long n) {
@@ -234,27 +287,33 @@ cudaError_t storeall_rhs(const Geom& g, const Coef<T>& c, const TIN* q, T* s, cu
   } while (0)
   bl_primitives<T, TIN><<<pgrid(P), 256, 0, st>>>(g, c, q, s);
   SBLI_CK(cudaGetLastError());
-  for (int i = 0; i < 3; ++i)
-    for (int j = 0; j < 3; ++j) {
-      SBLI_CK((launch_der<T, TIN>(g, c, q + (1 + i) * P, arr(A_DRHOU + 3 * i + j), j, 1, st)));
-      SBLI_CK((launch_der<T, T>(g, c, arr(A_U + i), arr(A_DU + 3 * i + j), j, 1, st)));
-      SBLI_CK((launch_der<T, T>(g, c, arr(A_MU + sym(i, j)), arr(A_DRHOUU + 3 * i + j), j, 1, st)));
-      SBLI_CK((launch_der<T, T>(g, c, arr(A_U + i), arr(A_D2U + 3 * i + j), j, 2, st)));
+  // field by field, so that the three axes find it in L2
+  static_assert(std::is_same<TIN, T>::value, "storeall_rhs differentiates conserved fields in the arithmetic type");
+  Derivatives<T> first{}, mixed{};
+  auto add = [](Derivatives<T>& d, const T* f, T* d1, T* d2, int axis) { d.job[d.count++] = {f, d1, d2, axis}; };
+  for (int i = 0; i < 3; ++i) {
+    for (int j = 0; j < 3; ++j) add(first, arr(A_U + i), arr(A_DU + 3 * i + j), arr(A_D2U + 3 * i + j), j);
+    for (int j = 0; j < 3; ++j) add(first, q + (1 + i) * P, arr(A_DRHOU + 3 * i + j), nullptr, j);
+    for (int j = i; j < 3; ++j) {
+      add(first, arr(A_MU + sym(i, j)), arr(A_DRHOUU + 3 * i + j), nullptr, j);
+      if (j != i) add(first, arr(A_MU + sym(i, j)), arr(A_DRHOUU + 3 * j + i), nullptr, i);
     }
+  }
+  for (int j = 0; j < 3; ++j) add(first, q, arr(A_DRHO + j), nullptr, j);
+  for (int j = 0; j < 3; ++j) add(first, arr(A_P), arr(A_DP + j), nullptr, j);
+  for (int j = 0; j < 3; ++j) add(first, q + 4 * P, arr(A_DE + j), nullptr, j);
+  for (int j = 0; j < 3; ++j) add(first, arr(A_T), nullptr, arr(A_D2T + j), j);
   for (int j = 0; j < 3; ++j) {
-    SBLI_CK((launch_der<T, TIN>(g, c, q, arr(A_DRHO + j), j, 1, st)));
-    SBLI_CK((launch_der<T, T>(g, c, arr(A_P), arr(A_DP + j), j, 1, st)));
-    SBLI_CK((launch_der<T, TIN>(g, c, q + 4 * P, arr(A_DE + j), j, 1, st)));
-    SBLI_CK((launch_der<T, T>(g, c, arr(A_EU + j), arr(A_DEU + j), j, 1, st)));
-    SBLI_CK((launch_der<T, T>(g, c, arr(A_PU + j), arr(A_DPU + j), j, 1, st)));
-    SBLI_CK((launch_der<T, T>(g, c, arr(A_T), arr(A_D2T + j), j, 2, st)));
+    add(first, arr(A_EU + j), arr(A_DEU + j), nullptr, j);
+    add(first, arr(A_PU + j), arr(A_DPU + j), nullptr, j);
   }
   // mixed derivatives D_i (D_j u_j), i != j, from the stored diagonal gradients
-  for (int i = 0; i < 3; ++i)
-    for (int j = 0; j < 3; ++j)
-      if (i != j) SBLI_CK((launch_der<T, T>(g, c, arr(A_DU + 3 * j + j), arr(A_DDU + offd(i, j)), i, 1, st)));
+  for (int j = 0; j < 3; ++j)
+    for (int i = 0; i < 3; ++i)
+      if (i != j) add(mixed, arr(A_DU + 3 * j + j), arr(A_DDU + offd(i, j)), nullptr, i);
+  SBLI_CK(launch_derivatives(g, c, first, st));
+  SBLI_CK(launch_derivatives(g, c, mixed, st));
   // conserved variables in the arithmetic type (callers pass T == TIN)
-  static_assert(sizeof(TIN) == sizeof(T), "storeall_rhs reads conserved fields in the arithmetic type");
   const T* qrho = reinterpret_cast<const T*>(q);
   const T* qm = qrho + P;
   const T* qE = qrho + 4 * P;
@@ -284,9 +343,11 @@ __global__ void rk_update_kernel(long long n, const TR* __restrict__ r, const do
 
 }  // namespace
 
-cudaError_t launch_derivative_fp64(const Geom& g, const Coef<double>& c, const double* f, double* df, int axis,
-                                   int order, cudaStream_t s) {
-  return launch_der<double, double>(g, c, f, df, axis, order, s);
+cudaError_t launch_gradients_fp64(const Geom& g, const Coef<double>& c, const double* u, double* grad, cudaStream_t s) {
+  Derivatives<double> d{};
+  for (int i = 0; i < 3; ++i)
+    for (int j = 0; j < 3; ++j) d.job[d.count++] = {u + i * g.P, grad + (3 * i + j) * g.P, nullptr, j};
+  return launch_derivatives(g, c, d, s);
 }
 
 size_t storeall_scratch_doubles(const Geom& g, int elem_bytes) {

@@ -1,6 +1,6 @@
 // Compiled by tests/test_stencil_int.py.  Seeded values -2, -1, 0, +1, +2 of
 // narrow and wide ranges of exponents, zeros and special values; prints one
-// line a case: the five values and the three sums of stencil_int.cuh as bit
+// line a case: the five values and the sums of stencil_int.cuh as bit
 // patterns.  With the argument "gpu" also evaluates them on the GPU and compares
 // bit for bit.
 #include <cmath>
@@ -12,7 +12,7 @@
 #include "stencil_int.cuh"
 
 struct Case {
-  double v[5], r[4];
+  double v[5], r[6];
 };
 
 __host__ __device__ void evaluate(Case& c) {
@@ -26,6 +26,7 @@ __host__ __device__ void evaluate(Case& c) {
   else
     sbli::both_sums<false>(v[0], v[1], v[3], v[4], top, f, c.r[2]);
   c.r[3] = f;
+  sbli::stencil_both(v[0], v[1], v[2], v[3], v[4], c.r[4], c.r[5]);
 }
 __global__ void run(Case* c, int n) {
   const int i = blockIdx.x * blockDim.x + threadIdx.x;
@@ -66,6 +67,9 @@ int main(int argc, char** argv) {
     }
   std::vector<Case> host = cases;
   for (Case& c : host) evaluate(c);
+  for (const Case& c : host)  // both at once: the bits of each by itself
+    for (int k = 0; k < 2; ++k)
+      if (!(std::isnan(c.r[k]) && std::isnan(c.r[4 + k])) && memcmp(&c.r[k], &c.r[4 + k], 8)) return 3;
   if (argc > 1 && !strcmp(argv[1], "gpu")) {
     const int n = (int)cases.size();
     Case* d;
@@ -75,11 +79,11 @@ int main(int argc, char** argv) {
     if (cudaMemcpy(cases.data(), d, n * sizeof(Case), cudaMemcpyDeviceToHost) != cudaSuccess) return 2;
     int bad = 0;
     for (int i = 0; i < n; ++i)
-      for (int k = 0; k < 4; ++k) {
+      for (int k = 0; k < 6; ++k) {
         const double a = cases[i].r[k], b = host[i].r[k];
         if (!(std::isnan(a) && std::isnan(b)) && memcmp(&a, &b, 8)) ++bad;
       }
-    std::printf("%d of %d sums differ\n", bad, 4 * n);
+    std::printf("%d of %d sums differ\n", bad, 6 * n);
     return bad ? 1 : 0;
   }
   for (const Case& c : host) {
