@@ -95,18 +95,16 @@ __device__ __forceinline__ float narrow_f64_rna(double d) {
   return __uint_as_float(bits);
 }
 
-// 1/x in binary64: the hardware approximation (rcp.approx.ftz.f64) refined by
-// two Newton-Raphson steps y <- y + y (1 - x y), each a pair of fused
-// multiply-adds that squares the relative error (within one unit in the last
-// place of 1/x; tests/test_gpu_recip.py compares it with CUDA's correctly
-// rounded reciprocal)
+// 1/x in binary64: the hardware approximation y (rcp.approx.ftz.f64, 20 bits)
+// refined in one step of third order, y (1 + e + e^2) with e = 1 - x y, whose relative
+// error e^3 is below 2^-59: three fused multiply-adds where two Newton-Raphson
+// steps take four (within one unit in the last place of 1/x;
+// tests/test_gpu_recip.py compares it with CUDA's correctly rounded reciprocal)
 __device__ __forceinline__ double rcp_newton_f64(double x) {
   double y;
   asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(x));
-  double e = fma(-x, y, 1.0);
-  y = fma(y, e, y);
-  e = fma(-x, y, 1.0);
-  return fma(y, e, y);
+  const double e = fma(-x, y, 1.0);
+  return fma(y, fma(e, e, e), y);
 }
 
 // binary64 -> double-float pair, hi = v rounded to nearest (ties away from

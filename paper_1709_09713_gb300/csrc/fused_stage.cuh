@@ -155,7 +155,7 @@ struct FusedSmem {
   uint32_t tmem_base[2];      // TMEM allocations (z queue variant)
 };
 
-// 1/rho for the primitives (Eqs. 4-5): a Newton-refined approximation in
+// 1/rho for the primitives (Eqs. 4-5): a refined hardware approximation in
 // binary64, a double-word reciprocal in double-float; binary32 takes the
 // hardware approximation (rcp.approx, within one unit in the last place),
 // far inside the binary32 tolerance and one instruction instead of the
@@ -764,11 +764,13 @@ __device__ __forceinline__ void axis_terms_stream(const LD& ldrec, const SF& sfu
 
 // Binary64: the linear stencils of an axis (Laplacians of u and T', cross
 // gradients, D1_A of p', rho', m_A and s_A) in integers, the products with the
-// velocities on the binary64 pipe: 34 binary64 instructions an axis instead of
-// 62, beside some 800 integer ones that run while that pipe is busy (about 180
-// instead of 280 a point with the primitives and the update).  256^3 8.86 -> 6.39 ms a
-// stage, 64^3 168 -> 128 us, 32^3 33.4 -> 28.0; the pipe stays the bound, at 0.88 of
-// its measured peak.  Values too large to align, infinities and NaNs take the
+// velocities on the binary64 pipe: 33 binary64 instructions an axis instead of
+// 62, beside some 800 integer ones that run while that pipe is busy (about 155
+// instead of 280 a point with the primitives and the update).  32 x 8 tiles: 256^3 8.86
+// -> 6.39 ms a stage, 64^3 168 -> 128 us; the pipe stays the bound, 81 % busy with two
+// CTAs of 16 x 8 (the other CTA does not always have binary64 work when one waits).
+// The pressure sum folded into two multiply-adds and the reciprocal's third-order step
+// (fpconv.cuh): 6.05 -> 5.89 ms, 64^3 122.9 -> 119.1 us.  Values too large to align, infinities and NaNs take the
 // sums in binary64 (FIXED false).
 template <int A, bool WITH_KE, bool FIXED>
 __device__ __forceinline__ void axis_terms_sums(const double (&r)[4][NV], const double (&sx)[4], const double (&sy)[4],
@@ -787,9 +789,9 @@ __device__ __forceinline__ void axis_terms_sums(const double (&r)[4][NV], const 
   }
   auto first = [&](int v) { return first_sum<FIXED>(r[0][v], r[1][v], r[2][v], r[3][v], top[v]); };
   auto second = [&](int v) { return second_sum<FIXED>(r[0][v], r[1][v], r[2][v], r[3][v], top[v]); };
-  const double dp = c.hc2[A] * first(V_P);
-  t.rM[A] = add_nc(t.rM[A], dp);
-  t.rE = fmadd(-ua, dp, t.rE);
+  const double dp = first(V_P);
+  t.rM[A] = fmadd(c.hc2[A], dp, t.rM[A]);
+  t.rE = fmadd(-hu2, dp, t.rE);
   t.rrho = fmadd(c.hc2[A], fmadd(ua, first(V_RHO), first(V_M0 + A)), t.rrho);
 #pragma unroll
   for (int i = 0; i < 3; ++i) {

@@ -1,5 +1,5 @@
 // Compiled by tests/test_gpu_recip.py: the stage kernels' binary64 reciprocal
-// (sbli::recip<double>, a Newton-refined hardware approximation) against
+// (sbli::recip<double>, a refined hardware approximation) against
 // CUDA's correctly rounded reciprocal, as the largest difference in units in
 // the last place over seeded inputs.
 #include <cstdint>

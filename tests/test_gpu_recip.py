@@ -1,5 +1,5 @@
 """The binary64 reciprocal of the stage kernels (a hardware approximation
-refined by two Newton-Raphson steps) against CUDA's correctly rounded
+refined by one step of third order) against CUDA's correctly rounded
 reciprocal: within one unit in the last place on seeded inputs spanning the
 density range of the kernels and a wide exponent range."""
 import os
