@@ -32,6 +32,7 @@
 // Variables are deviations from the reference state, as in the other paths.
 #include <utility>
 
+#include "fpconv.cuh"
 #include "sbli_internal.cuh"
 
 namespace sbli {
@@ -236,13 +237,19 @@ static_assert(sn2_is_permutation(), "SN2 order lists each derivative once");
 template <class DP>
 __device__ __forceinline__ void assemble(const DP& d, double rho, const double (&m)[3], const double (&u)[3],
                                          double E, const Coef<double>& c, double (&R)[5]) {
+  // sums start from their first term: 0 + x costs an instruction of the binary64 pipe,
+  // which bounds these kernels (with the quotients of primitives_kernel from one
+  // reciprocal, 128^3: SS 1.79 -> 1.68 ms a stage, SN 2.23 -> 2.11).  Stencils in
+  // integers, as in the store-all kernels, cost more registers than they save here
+  // (SS 1.73, SN 2.14 with the second derivatives alone)
+  auto sum = [](auto J, double& s, double x) { s = decltype(J)::value == 0 ? x : s + x; };
   auto div = [&]() { return d.template get<D_U + 0>() + d.template get<D_U + 4>() + d.template get<D_U + 8>(); };
   // Eq. 1
   double conv = 0.0;
   static_for<0, 3>([&](auto J) {
     constexpr int j = J;
-    conv += d.template get<D_RHOU + 3 * j + j>() + rho * d.template get<D_U + 3 * j + j>() +
-            u[j] * d.template get<D_RHO + j>();
+    sum(J, conv, d.template get<D_RHOU + 3 * j + j>() + rho * d.template get<D_U + 3 * j + j>() +
+                     u[j] * d.template get<D_RHO + j>());
   });
   R[0] = -0.5 * conv;
   // Eq. 2: viscous part sd_i = sum_j D2_j u_i + (1/3) sum_j D_i D_j u_j
@@ -251,11 +258,11 @@ __device__ __forceinline__ void assemble(const DP& d, double rho, const double (
     double lap = 0.0, cross = 0.0;
     static_for<0, 3>([&](auto J) {
       constexpr int j = J;
-      lap += d.template get<D2_U + 3 * i + j>();
+      sum(J, lap, d.template get<D2_U + 3 * i + j>());
       if constexpr (j == i)
-        cross += d.template get<D2_U + 3 * i + i>();
+        sum(J, cross, d.template get<D2_U + 3 * i + i>());
       else
-        cross += d.template get<DD_U + offd_c(i, j)>();
+        sum(J, cross, d.template get<DD_U + offd_c(i, j)>());
     });
     return lap + cross - (2.0 / 3.0) * cross;
   };
@@ -264,8 +271,8 @@ __device__ __forceinline__ void assemble(const DP& d, double rho, const double (
     double cv = 0.0;
     static_for<0, 3>([&](auto J) {
       constexpr int j = J;
-      cv += d.template get<D_RHOUU + 3 * i + j>() + m[i] * d.template get<D_U + 3 * j + j>() +
-            u[j] * d.template get<D_RHOU + 3 * i + j>();
+      sum(J, cv, d.template get<D_RHOUU + 3 * i + j>() + m[i] * d.template get<D_U + 3 * j + j>() +
+                     u[j] * d.template get<D_RHOU + 3 * i + j>());
     });
     R[1 + i] = -0.5 * cv - d.template get<D_P + i>() + c.inv_re * sd(I);
   });
@@ -274,17 +281,20 @@ __device__ __forceinline__ void assemble(const DP& d, double rho, const double (
   double pw = 0.0, heat = 0.0, vw = 0.0, diss = 0.0;
   static_for<0, 3>([&](auto J) {
     constexpr int j = J;
-    conv += d.template get<D_EU + j>() + E * d.template get<D_U + 3 * j + j>() + u[j] * d.template get<D_E + j>();
-    pw += d.template get<D_PU + j>();
-    heat += d.template get<D2_T + j>();
+    sum(J, conv,
+        d.template get<D_EU + j>() + E * d.template get<D_U + 3 * j + j>() + u[j] * d.template get<D_E + j>());
+    sum(J, pw, d.template get<D_PU + j>());
+    sum(J, heat, d.template get<D2_T + j>());
   });
   static_for<0, 3>([&](auto I) {
     constexpr int i = I;
-    vw += u[i] * c.inv_re * sd(I);
+    sum(I, vw, u[i] * c.inv_re * sd(I));
     static_for<0, 3>([&](auto J) {
       constexpr int j = J;
       const double g = d.template get<D_U + 3 * i + j>();
-      diss += g * (g + d.template get<D_U + 3 * j + i>() - (i == j ? (2.0 / 3.0) * div() : 0.0));
+      double s = g + d.template get<D_U + 3 * j + i>();
+      if constexpr (i == j) s -= (2.0 / 3.0) * div();
+      sum(std::integral_constant<int, 3 * i + j>{}, diss, g * s);
     });
   });
   R[4] = -0.5 * conv - c.H0 * div() - pw + vw + c.inv_re * diss + c.kappa * heat;
@@ -358,13 +368,13 @@ __global__ void __launch_bounds__(256) algorithm_stage_kernel(Geom g, const __gr
 __global__ void primitives_kernel(long long P, const __grid_constant__ Coef<double> c, const double* __restrict__ q,
                                   double* __restrict__ w) {
   for (long long n = blockIdx.x * (long long)blockDim.x + threadIdx.x; n < P; n += (long long)gridDim.x * blockDim.x) {
-    const double rho_p = q[n], rho = 1.0 + rho_p;
+    const double rho_p = q[n], rho = 1.0 + rho_p, rinv = rcp_newton_f64(rho);
     double u[3];
-    for (int i = 0; i < 3; ++i) u[i] = q[(1 + i) * P + n] / rho;
+    for (int i = 0; i < 3; ++i) u[i] = corrected_quotient(q[(1 + i) * P + n], rho, rinv);
     const double p_p = c.gm1 * (q[4 * P + n] - 0.5 * rho * (u[0] * u[0] + u[1] * u[1] + u[2] * u[2]));  // Eq. 4
     for (int i = 0; i < 3; ++i) w[i * P + n] = u[i];
     w[3 * P + n] = p_p;
-    w[4 * P + n] = (c.gM2 * p_p - rho_p) / rho;  // Eq. 5
+    w[4 * P + n] = corrected_quotient(c.gM2 * p_p - rho_p, rho, rinv);  // Eq. 5
   }
 }
 

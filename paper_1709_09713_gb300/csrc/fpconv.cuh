@@ -107,6 +107,13 @@ __device__ __forceinline__ double rcp_newton_f64(double x) {
   return fma(y, fma(e, e, e), y);
 }
 
+// x / y, given 1/y: the product corrected by its residual (Markstein), so that it
+// rounds as the division does
+__device__ __forceinline__ double corrected_quotient(double x, double y, double yinv) {
+  const double q = x * yinv;
+  return fma(fma(-q, y, x), yinv, q);
+}
+
 // binary64 -> double-float pair, hi = v rounded to nearest (ties away from
 // zero), lo = v - hi rounded to nearest, without the FP64 pipe: the low word
 // shifted left by 3 holds the 29 mantissa bits that hi drops at the top of a

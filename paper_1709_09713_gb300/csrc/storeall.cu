@@ -62,12 +62,8 @@ __global__ void bl_primitives(Geom g, Coef<T> c, const TIN* __restrict__ q, T* _
     T rinv = T(0);
     if constexpr (sizeof(T) == 8) rinv = rcp_newton_f64(rho);
     auto quotient = [&](T x) -> T {
-      if constexpr (sizeof(T) == 8) {
-        const T q = x * rinv;
-        return fma(fma(-q, rho, x), rinv, q);
-      } else {
-        return x / rho;
-      }
+      if constexpr (sizeof(T) == 8) return corrected_quotient(x, rho, rinv);
+      else return x / rho;
     };
     T u[3];
     for (int i = 0; i < 3; ++i) u[i] = quotient(m[i]);
