@@ -64,7 +64,7 @@ ALG_BYTES = {"fp64": 400.0 / 3.0, "fp32": 320.0 / 3.0, "fp32df": 320.0 / 3.0, "d
 #   df64 inst_per_pt: thread instructions (smsp__inst_executed x 32 / points),
 #        mean of the three stages of a 256^3 step, per z-queue mode.
 KERNEL_SOURCES = ["fused_stage.cuh", "fused_fp64.cu", "fused_df64.cu", "dfloat.cuh", "fpconv.cuh", "f32x2.cuh",
-                  "sbli_internal.cuh"]
+                  "sbli_internal.cuh", "stencil_int.cuh"]
 KERNEL_COUNTS = {
     "fp64": {"flop_per_pt": 568.44, "traffic_per_pt": 2.2499e9 / 256**3, "sources": "651ecf03b0a6",
              "profile": "profiles/fused_stage_fp64_256.md"},

@@ -770,8 +770,8 @@ __device__ __forceinline__ void axis_terms_stream(const LD& ldrec, const SF& sfu
 // -> 6.39 ms a stage, 64^3 168 -> 128 us; the pipe stays the bound, 81 % busy with two
 // CTAs of 16 x 8 (the other CTA does not always have binary64 work when one waits).
 // The pressure sum folded into two multiply-adds and the reciprocal's third-order step
-// (fpconv.cuh): 6.05 -> 5.89 ms, 64^3 122.9 -> 119.1 us.  Values too large to align, infinities and NaNs take the
-// sums in binary64 (FIXED false).
+// (fpconv.cuh): 6.05 -> 5.89 ms, 64^3 122.9 -> 119.1 us.  Values too large to align,
+// infinities and NaNs take the sums in binary64 (FIXED false).
 template <int A, bool WITH_KE, bool FIXED>
 __device__ __forceinline__ void axis_terms_sums(const double (&r)[4][NV], const double (&sx)[4], const double (&sy)[4],
                                                 const uint32_t (&top)[NV], uint32_t stop, const Coef<double>& c,
@@ -869,7 +869,8 @@ __device__ __forceinline__ void assemble_streamed(const StreamTerms<T>& t, T rho
 // the cross gradients and (m_A, s_A) pairs put together in registers.  256^3,
 // 37 planes a CTA: 2.43 -> 2.20 ms a stage, 3727 -> about 2450 instructions a point;
 // bound by the latency of dependent instructions and of shared memory at the
-// two warps a sub-partition that 200 registers leave (issue 45 %, FMA pipe 47 %).
+// two warps a sub-partition that the registers leave (16 x 8 tiles, two CTAs an SM:
+// issue 50 %, 1.94 ms; three CTAs of the TMEM queue at 168 registers spill, 2.10).
 struct DwTerms {
   dfloat2 m01, m2e;  // -1/2 the convective sums of Eq. 2 (i = 0, 1), (i = 2 and Eq. 3)
   dfloat2 v01, v2t;  // sum_j D2_j u_i + 1/3 sum_j d2 u_j / dx_i dx_j, and sum_j D2_j T'
@@ -1341,7 +1342,7 @@ __device__ __forceinline__ void fused_march(const StageArgs& a, const Coef<T>& c
   // -> 2.091 ms a stage, 64^3 44.6 -> 42.3 us (the same code shape schedules
   // better in its full iterations too), binary64 and binary32 rings 1 to 4 % at
   // 16^3 ... 40^3.  Two columns per thread have no registers for it, nor has
-  // the binary32 TMEM queue at 80 (spills in the batch kernel, 0.3 % on 256^3).
+  // the binary32 TMEM queue (the batch kernel spills, 1 % slower; 0.5 % faster alone).
   constexpr int FILL = PP == 2 || (sizeof(T) == 4 && ZT) ? 0 : (ZT ? 3 : 4);
   if constexpr (FILL > 0) {
     Loads pb[FILL > 0 ? FILL : 1];
