@@ -148,7 +148,8 @@ int ctas_per_sm(int precision, int ty, int px = 1, int zq = 0) {
 }
 
 // Planes per CTA ranked by a wave-balance model: cost = waves * (zc + 1.5),
-// the 4 warm-up planes of a z segment costing about 1.5 full planes.
+// the 4 warm-up planes of a z segment costing about 1.5 full planes (0.6 for
+// binary64 registers would rank chunks of 16 first at 256^3: 1.89 ms, of 64 1.86).
 void rank_zc(const Geom& g, int precision, int ty, int* best, int nbest, int px = 1, int zq = 0) {
   int dev = 0, sms = 152;
   if (cudaGetDevice(&dev) == cudaSuccess) cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
@@ -185,11 +186,18 @@ void use_config(sbli_grid* g, const FusedConfig& cfg) {
   g->cfg = cfg;
   g->zc = cfg.zc;
   if (f64_registers(g->precision))
-    g->split = plan_split(g->geom, cfg.zc, std::min(F64_CTAS_PER_SM * g->sms, MAX_SMALL_CTAS), g->precision == SBLI_DF64);
+    g->split = plan_split(g->geom, cfg, std::min(F64_CTAS_PER_SM * g->sms, MAX_SMALL_CTAS),
+                          g->precision == SBLI_DF64);
   else
     g->zc = binary32_launch_zc(g->geom, cfg, g->sms);
 }
 
+// Binary64-register grids: the TMEM queue where a CTA slot has 24 planes and more,
+// whose shared-memory traffic it takes; with fewer, its allocation and its fill
+// (three planes at once instead of four) cost more than that.  us a stage, shared ring against TMEM queue:
+// double-float 256^3 1902 against 1828, 160^3 483 against 461, 128^3 259 against 249,
+// 129x97x66 (25 planes a slot) 127.7 against 126.0; 96^3 (23) 113.6 against 114.3, 40^3 15.3
+// against 16.7; binary64 256^3 5887 against 5859, 128^3 760 against 755.
 // Binary32 grids: z queue and planes per CTA by the model of their stage (us a
 // stage, shared ring with planes by waves -> this: 128^3 96.7 -> 63.7, 96^3 35.8 ->
 // 30.3, 40^3 9.3 -> 7.6, 32^3 9.2 -> 4.4).
@@ -201,7 +209,11 @@ FusedConfig default_config(const Geom& g, int precision, int sms) {
   int zc[1];
   rank_zc(g, precision, cfg.ty, zc, 1);
   cfg.zc = std::max(4, std::min(zc[0], g.n2));
-  if (f64_registers(precision)) return cfg;
+  if (f64_registers(precision)) {
+    const long long tiles = (long long)((g.n0 + F64_TILE_X - 1) / F64_TILE_X) * ((g.n1 + 7) / 8);
+    cfg.zq = tiles * g.n2 >= 24LL * F64_CTAS_PER_SM * sms;
+    return cfg;
+  }
   double best = 0.0;
   FusedConfig c = cfg;
   for (c.zq = 0; c.zq < 2; ++c.zq)

@@ -88,33 +88,33 @@ int binary32_launch_zc(const Geom& g, const FusedConfig& cfg, int sms) {
   return best;
 }
 
-// The longest CTA decides, in planes, each march's four fill planes counting
-// WARM of a plane (their primitives) each, and a plane of the even split 4 or 5 %
-// more (its CTAs share no halos in L2).  The even split against chunks, us a
-// stage: double-float 32^3 10.0 against 16.9, 129x97x66 127 against 132, 128^3 260 against
-// 264, but 96^3 117 against 114 and 256^3 1979 against 1938; binary64 32^3 27.9 against
-// 46.2, 128^3 781 against 810, 256^3 6033 against 6171, but 150x75x61 318 against 299.  Over 21
-// grids the rule loses 0.2 % on average to the better of the two.
+// The longest CTA decides, in planes, each march's fill counting F64_FILL, and a
+// plane of the even split 4 to 8 % more (its CTAs share no halos in L2; 8 % for
+// double-float with the TMEM queue).  The even split against chunks, us a
+// stage: double-float 32^3 10.0 against 16.9, shared ring 129x97x66 128 against 132, 128^3
+// 259 against 264, but with the TMEM queue 128 against 126 and 255 against 249, and 96^3
+// 117 against 114; binary64 32^3 27.9 against 46.2, 128^3 760 against 795, 256^3 5887 against 5959.
+// Over 21 grids (shared ring) the rule loses 0.2 % on average to the better of the two.
 //
 // Two counts of even runs are ranked: as many as there are slots, and the most
 // that cut every tile into equally many, so that no run crosses into a second
 // tile and fills twice: on 304 slots 48^3 takes 288 runs of 3 planes (binary64 56.0 us
 // a stage, double-float 19.7; 304 runs of up to 3 over two tiles 67.3 and 22.9), 40^3
 // 300 of 2 (42.1 and 14.9; 49.7 and 17.9).
-Split plan_split(const Geom& g, int zc, int slots, bool double_float) {
-  constexpr double WARM = 0.15;
-  const double plane = double_float ? 1.05 : 1.04;
+Split plan_split(const Geom& g, const FusedConfig& cfg, int slots, bool double_float) {
+  const int zc = cfg.zc;
+  const double plane = !double_float ? 1.04 : cfg.zq ? 1.08 : 1.05;
   const long long tiles = (long long)((g.n0 + F64_TILE_X - 1) / F64_TILE_X) * ((g.n1 + 7) / 8), units = tiles * g.n2;
   const long long chunks = tiles * ((g.n2 + zc - 1) / zc);
   const double waves = (double)((chunks + slots - 1) / slots);
-  double best = waves * (std::min(zc, g.n2) + 4 * WARM);
+  double best = waves * (std::min(zc, g.n2) + F64_FILL);
   Split split{(int)chunks, 0};
   const auto even = [&](long long ctas) {
     double longest = 0.0;
     for (long long c = 0; c < ctas; ++c) {
       const long long u = units * c / ctas, end = units * (c + 1) / ctas;
       const long long marches = (end - 1) / g.n2 - u / g.n2 + 1;
-      longest = std::max(longest, plane * (double)(end - u) + 4 * WARM * marches);
+      longest = std::max(longest, plane * (double)(end - u) + F64_FILL * marches);
     }
     if (longest <= best) {
       best = longest;

@@ -92,6 +92,9 @@ constexpr int MAX_SMALL_CTAS = 512;
 // their CTAs per SM.
 constexpr int F64_TILE_X = 16;
 constexpr int F64_CTAS_PER_SM = 2;
+// The four planes that fill the ring of a march, in planes' time (their
+// primitives; binary64-register kernels enter them together).
+constexpr double F64_FILL = 0.6;
 
 // Launch configuration chosen for one grid (the autotuner's output).
 struct FusedConfig {
@@ -137,7 +140,7 @@ int binary32_launch_zc(const Geom& g, const FusedConfig& cfg, int sms);
 struct Split {
   int ctas, even;
 };
-Split plan_split(const Geom& g, int zc, int slots, bool double_float);
+Split plan_split(const Geom& g, const FusedConfig& cfg, int slots, bool double_float);
 
 // Diagnostics and state conversion (diag.cu).
 cudaError_t launch_init_tgv(const Geom& g, const sbli_params& p, double amplitude, double* q, cudaStream_t s);
