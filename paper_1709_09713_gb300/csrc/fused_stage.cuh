@@ -765,10 +765,10 @@ __device__ __forceinline__ void axis_terms_stream(const LD& ldrec, const SF& sfu
 // Binary64: the linear stencils of an axis (Laplacians of u and T', cross
 // gradients, D1_A of p', rho', m_A and s_A) in integers, the products with the
 // velocities on the binary64 pipe: 33 binary64 instructions an axis instead of
-// 62, beside some 800 integer ones that run while that pipe is busy (about 155
-// instead of 280 a point with the primitives and the update).  32 x 8 tiles: 256^3 8.86
-// -> 6.39 ms a stage, 64^3 168 -> 128 us; the pipe stays the bound, 81 % busy with two
-// CTAs of 16 x 8 (the other CTA does not always have binary64 work when one waits).
+// 62, beside some 800 integer ones that run while that pipe is busy.  32 x 8
+// tiles: 256^3 8.86 -> 6.39 ms a stage, 64^3 168 -> 128 us; the pipe stays the
+// bound: two CTAs of 16 x 8 keep it at 0.95 of its measured rate (512^3 0.97) with
+// 175 instructions a point, the primitives of the halo included.
 // The pressure sum folded into two multiply-adds and the reciprocal's third-order step
 // (fpconv.cuh): 6.05 -> 5.89 ms, 64^3 122.9 -> 119.1 us.  Values too large to align,
 // infinities and NaNs take the sums in binary64 (FIXED false).

@@ -213,8 +213,8 @@ cudaError_t launch_derivatives(const Geom& g, const Coef<T>& c, const Derivative
   return cudaSuccess;
 }
 
-// Bound by the binary64 pipe: sums start from their first term, and three blocks on
-// an SM instead of two (128^3 359 -> 300 us).
+// Bound by the binary64 pipe (at its measured rate): sums start from their first term, and three blocks on
+// an SM instead of two (128^3 359 -> 314 us).
 template <typename T>
 __global__ void __launch_bounds__(256, 3) bl_residual(Geom g, Coef<T> c, const T* __restrict__ qrho, const T* __restrict__ qm,
                             const T* __restrict__ qE, long long qstride, T* __restrict__ s) {
