@@ -3,16 +3,22 @@
 // workspace and the allocation-free entry points.
 //
 // Bound by the binary64 pipe, so every velocity is formed once where that is
-// possible: a block marches along x2 over the columns of a 32 x 16 tile, each
+// possible: a block marches along x2 over the columns of a 32 x 8 tile, each
 // thread keeping its own column's velocities of five planes in registers (the
 // x2 derivatives), the centre plane's going through shared memory (x0 and x1
-// derivatives; the halo's, 0.375 a point, are formed anew), with the
+// derivatives; the halo's, 0.625 a point, are formed anew), with the
 // reciprocal of the density shared by the three components, and the stencils
-// summed in integers.  About 30 binary64 instructions a point where dividing at
-// every stencil point took about 260.  Blocks take contiguous runs of planes, one block per SM, so that all
-// SMs end together.  160 x 200 x 120 points, both entry points with the state in and
-// out: 4.15 -> 0.67 ms (0.85 with the stencils on the binary64 pipe).
+// summed in integers.  About 26 binary64 instructions a point where dividing at
+// every stencil point took about 260.  Blocks take contiguous runs of planes, two
+// blocks per SM, so that all SMs end together and one block's binary64 work runs
+// beside the other's integer sums and barriers (one block of 32 x 16: 160 x 200 x 120
+// points 285 us instead of 232, 256^3 1113 instead of 926, 32^3 21 instead of 15; three or
+// four blocks of fewer registers 238, 236).  160 x 200 x 120 points, both entry points
+// with the state in and out, against dividing at every stencil point: 4.15 ->
+// 0.54 ms.
 #pragma once
+
+#include <algorithm>
 
 #include "fpconv.cuh"
 #include "sbli_internal.cuh"
@@ -20,18 +26,19 @@
 
 namespace sbli {
 
-constexpr int KE_TX = 32, KE_TY = 16;
+constexpr int KE_TX = 32, KE_TY = 8;
 constexpr int KE_THREADS = KE_TX * KE_TY;
+constexpr int KE_PER_SM = 2;  // blocks
 
 inline long long ke_units(const Geom& g) {
   return (long long)((g.n0 + KE_TX - 1) / KE_TX) * ((g.n1 + KE_TY - 1) / KE_TY) * g.n2;
 }
-// blocks of a launch (and partial sums it writes): one per SM, at most `most`
+// blocks of a launch (and partial sums it writes): KE_PER_SM per SM, at most `most`
 inline int ke_blocks(const Geom& g, int most) {
   int dev = 0, sms = 152;
   if (cudaGetDevice(&dev) == cudaSuccess) cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
   const long long units = ke_units(g);
-  const int b = sms < most ? sms : most;
+  const int b = std::min(KE_PER_SM * sms, most);
   return (int)(units < b ? units : b);
 }
 
@@ -39,7 +46,7 @@ inline int ke_blocks(const Geom& g, int most) {
 // Partial sums of block b in partials[2b], partials[2b + 1]: each thread's
 // points in a fixed order, warps by shuffles, then the warps in order.
 template <bool PLAIN>
-__global__ void __launch_bounds__(KE_THREADS)
+__global__ void __launch_bounds__(KE_THREADS, KE_PER_SM)
     ke_march_kernel(Geom g, const __grid_constant__ Coef<double> c, const double* __restrict__ q,
                     double* __restrict__ partials) {
   __shared__ double su[2][3][KE_TY + 4][KE_TX + 4];

@@ -29,7 +29,7 @@ namespace {
 // Capacity of the static scratch in (ke, enstrophy) pairs (one per block),
 // and the points it stands for; together they bound the grid to
 // NOALLOC_MAX_PARTIALS * NOALLOC_POINTS_PER_PARTIAL = 512^3 points, the
-// documented limit (a launch has one block per SM, far below it).
+// documented limit (a launch has two blocks per SM, far below it).
 constexpr int NOALLOC_MAX_PARTIALS = 8192;
 constexpr long long NOALLOC_POINTS_PER_PARTIAL = 16384;
 

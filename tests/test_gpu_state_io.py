@@ -57,8 +57,8 @@ def test_device_host_and_offset_buffers_agree(S, n, precision):
         g.close()
 
 
-# tile edges of the 32 x 16 tiles, runs of one plane, more planes than SMs
-@pytest.mark.parametrize("n", [(5, 5, 5), (32, 16, 8), (33, 17, 6), (31, 15, 160), (70, 40, 12)])
+# edges of the 32 x 8 tiles, runs of one plane, more planes than SMs
+@pytest.mark.parametrize("n", [(5, 5, 5), (32, 16, 8), (33, 17, 6), (31, 15, 160), (64, 24, 51), (70, 40, 12)])
 def test_kinetic_energy_and_enstrophy(S, orc, n):
     q = _state(n, 11)
     ke, ens = orc.ke_enstrophy(orc.params(n), q)
