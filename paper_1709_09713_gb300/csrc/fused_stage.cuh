@@ -305,6 +305,15 @@ constexpr int tmem_columns2() {
   return c;
 }
 
+// The tensor-memory accesses below are warp-aligned (.sync.aligned): all lanes
+// execute one together.  After code whose branches the lanes of a warp may take
+// differently (halo points, the columns of a ragged tile, values that the integer
+// sums cannot align) the march calls this first.
+template <bool ZT>
+__device__ __forceinline__ void tmem_converge() {
+  if constexpr (ZT) __syncwarp();
+}
+
 // win: this thread's window address (lane and window column), slot: ring slot
 __device__ __forceinline__ void tmem_store_rec(uint32_t win, int slot, const float (&r)[NV]) {
   using L = TmLayout<float>;
@@ -1215,7 +1224,10 @@ __device__ __forceinline__ void fused_march(const StageArgs& a, const Coef<T>& c
           store_rec(ring + ld_s[l] * NV, rec);
           if constexpr (S::U2) (&sm.u2ring[se][0][0])[ld_s[l]] = u2;
           if constexpr (ZT) {
-            if (l == 0) tmem_store_rec(twin, se, rec);  // l == 0: every thread
+            if (l == 0) {  // every thread
+              tmem_converge<ZT>();
+              tmem_store_rec(twin, se, rec);
+            }
           }
         }
       }
@@ -1247,6 +1259,7 @@ __device__ __forceinline__ void fused_march(const StageArgs& a, const Coef<T>& c
                                             R[sy][sx + 2][V_U0]);
       const T d11 = c.c2[1] * stencil_first(R[sy - 2][sx][V_U1], R[sy - 1][sx][V_U1], R[sy + 1][sx][V_U1],
                                             R[sy + 2][sx][V_U1]);
+      tmem_converge<ZT>();
       if constexpr (ZT) {
         tmem_store_diag(twin, se, d00, d11);  // this thread's column only
       } else {
@@ -1413,6 +1426,7 @@ __device__ __forceinline__ void fused_march(const StageArgs& a, const Coef<T>& c
     // and needs only the centre's in-plane gradients.
     if constexpr (MIXZ) {
       d22 = T(0);
+      tmem_converge<ZT>();
       if constexpr (ZT) {
         tmem_load_diag(twin, scen, g00c, g11c);
       } else {
@@ -1464,6 +1478,7 @@ __device__ __forceinline__ void fused_march(const StageArgs& a, const Coef<T>& c
           return c.c2[2] * stencil_first(u2at(sl[0], yy, xx), u2at(sl[1], yy, xx), u2at(sl[3], yy, xx), u2at(sl[4], yy, xx));
         };
         d22 = u2z(sy, sx);
+        tmem_converge<ZT>();
         if constexpr (ZT) {
           tmem_load_diag(twin, scen, g00c, g11c);
         } else {
@@ -1489,6 +1504,7 @@ __device__ __forceinline__ void fused_march(const StageArgs& a, const Coef<T>& c
     // ---------------------------------------------------------------- phase 3
     {
       fetch_acc();
+      tmem_converge<ZT>();
       const int sy = ty + HR, sx = tx + HALO;
       const T(*C)[SX][NV] = sm.ring[fc];
       T rho_p, mc[3], uc[3];  // centre values
@@ -1624,6 +1640,7 @@ __device__ __forceinline__ void fused_march(const StageArgs& a, const Coef<T>& c
           };
           axis_terms_fixed<0, WITH_KE>(ld0, at0, c, uc, t);
           axis_terms_fixed<1, WITH_KE>(ld1, at1, c, uc, t);
+          tmem_converge<ZT>();
           axis_terms_fixed<2, WITH_KE>(ld2, at2, c, uc, t);
         } else {
           axis_terms_stream<0, false, WITH_KE>(ld0, sf0, c, uc, t);
