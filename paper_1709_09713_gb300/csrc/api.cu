@@ -29,6 +29,7 @@ int fail(int code, const char* fmt, ...) {
 }
 
 int cuda_fail(cudaError_t e, const char* what) {
+  cudaGetLastError();  // reported here, not again by the next launch
   return fail(SBLI_ECUDA, "%s: %s (%s)", what, cudaGetErrorName(e), cudaGetErrorString(e));
 }
 
@@ -529,9 +530,10 @@ int sbli_set_state(sbli_grid* g, const double* q, int q_is_host) {
   if (!q) return fail(SBLI_EINVAL, "q is null");
   if (g->next_stage != 0) return fail(SBLI_EINVAL, "set_state between stages of a step (next stage %d)", g->next_stage);
   const double* src = q;
-  if (q_is_host || !direct_device_access(q)) {  // stage through a free register
+  const size_t bytes = 5 * (size_t)g->geom.P * sizeof(double);
+  if (q_is_host || !direct_device_access(q, bytes)) {  // stage through a free register
     double* tmp = free64(g);
-    SBLI_TRY(cudaMemcpyAsync(tmp, q, 5 * (size_t)g->geom.P * sizeof(double),
+    SBLI_TRY(cudaMemcpyAsync(tmp, q, bytes,
                              q_is_host ? cudaMemcpyHostToDevice : cudaMemcpyDeviceToDevice, g->stream),
              "cudaMemcpyAsync of the state");
     src = tmp;
@@ -553,7 +555,8 @@ int sbli_get_state(sbli_grid* g, double* q, int q_is_host) {
   if (int rc = check_grid(g)) return rc;
   if (!q) return fail(SBLI_EINVAL, "q is null");
   if (g->next_stage != 0) return fail(SBLI_EINVAL, "get_state between stages of a step (next stage %d)", g->next_stage);
-  const bool staged = q_is_host || !direct_device_access(q);
+  const size_t bytes = 5 * (size_t)g->geom.P * sizeof(double);
+  const bool staged = q_is_host || !direct_device_access(q, bytes);
   double* dst = staged ? free64(g) : q;
   if (g->precision == SBLI_FP32_DF) {
     SBLI_TRY(launch_df_join(g->geom.P, g->ref, reinterpret_cast<const float*>(g->reg64[g->state]), dst, g->stream),
@@ -562,7 +565,7 @@ int sbli_get_state(sbli_grid* g, double* q, int q_is_host) {
     SBLI_TRY(launch_from_offset(g->geom, g->ref, state64(g), dst, g->stream), "from_offset launch");
   }
   if (staged) {
-    SBLI_TRY(cudaMemcpyAsync(q, dst, 5 * (size_t)g->geom.P * sizeof(double),
+    SBLI_TRY(cudaMemcpyAsync(q, dst, bytes,
                              q_is_host ? cudaMemcpyDeviceToHost : cudaMemcpyDeviceToDevice, g->stream),
              "cudaMemcpyAsync of the state");
     if (q_is_host) SBLI_TRY(cudaStreamSynchronize(g->stream), "cudaStreamSynchronize");

@@ -186,6 +186,7 @@ int bfail(int code, const char* fmt, ...) {
 }
 
 int bcuda(cudaError_t e, const char* what) {
+  cudaGetLastError();  // reported here, not again by the next launch
   return bfail(SBLI_ECUDA, "%s: %s (%s)", what, cudaGetErrorName(e), cudaGetErrorString(e));
 }
 
@@ -599,9 +600,10 @@ int sbli_batch_set_state(sbli_batch* b, int member, const double* q, int q_is_ho
   if (!q) return bfail(SBLI_EINVAL, "q is null");
   const MemberLayout& M = b->L.m[member];
   const double* src = q;
-  if (q_is_host || !direct_device_access(q)) {  // stage through a free register
+  const size_t bytes = 5 * (size_t)M.P * sizeof(double);
+  if (q_is_host || !direct_device_access(q, bytes)) {  // stage through a free register
     double* tmp = reinterpret_cast<double*>(b->reg64[free_reg(b)] + M.off64);
-    SBLI_BTRY(cudaMemcpyAsync(tmp, q, 5 * M.P * sizeof(double),
+    SBLI_BTRY(cudaMemcpyAsync(tmp, q, bytes,
                               q_is_host ? cudaMemcpyHostToDevice : cudaMemcpyDeviceToDevice, b->stream),
               "cudaMemcpyAsync");
     src = tmp;
@@ -624,7 +626,8 @@ int sbli_batch_get_state(sbli_batch* b, int member, double* q, int q_is_host) {
   if (!q) return bfail(SBLI_EINVAL, "q is null");
   const MemberLayout& M = b->L.m[member];
   const double* src = reinterpret_cast<double*>(b->reg64[state_reg(b)] + M.off64);
-  const bool staged = q_is_host || !direct_device_access(q);
+  const size_t bytes = 5 * (size_t)M.P * sizeof(double);
+  const bool staged = q_is_host || !direct_device_access(q, bytes);
   double* dst = staged ? reinterpret_cast<double*>(b->reg64[free_reg(b)] + M.off64) : q;
   if (b->precision == SBLI_FP32_DF) {
     SBLI_BTRY(launch_df_join(M.P, make_ref(b->params[member]), reinterpret_cast<const float*>(src), dst, b->stream),
@@ -633,7 +636,7 @@ int sbli_batch_get_state(sbli_batch* b, int member, double* q, int q_is_host) {
     SBLI_BTRY(launch_from_offset(member_geom(M), make_ref(b->params[member]), src, dst, b->stream), "from_offset");
   }
   if (staged)
-    SBLI_BTRY(cudaMemcpyAsync(q, dst, 5 * M.P * sizeof(double),
+    SBLI_BTRY(cudaMemcpyAsync(q, dst, bytes,
                               q_is_host ? cudaMemcpyDeviceToHost : cudaMemcpyDeviceToDevice, b->stream),
               "cudaMemcpyAsync");
   if (q_is_host) SBLI_BTRY(cudaStreamSynchronize(b->stream), "cudaStreamSynchronize");

@@ -1,5 +1,6 @@
 // diag.cu -- Taylor-Green initial field, reference-state conversion and the
 // binary64 kinetic-energy / enstrophy reduction.
+#include <cuda.h>
 #include <math.h>
 
 #include "fpconv.cuh"
@@ -184,14 +185,30 @@ cudaError_t launch_from_offset(const Geom& g, const RefState& r, const double* q
   return cudaGetLastError();
 }
 
-bool direct_device_access(const void* p) {
+bool direct_device_access(const void* p, size_t bytes) {
   cudaPointerAttributes a;
   int dev = 0;
   if (cudaGetDevice(&dev) != cudaSuccess || cudaPointerGetAttributes(&a, p) != cudaSuccess) {
     cudaGetLastError();
     return false;
   }
-  return a.type == cudaMemoryTypeDevice && a.device == dev && (uintptr_t)p % sizeof(double) == 0;
+  if (a.type != cudaMemoryTypeDevice || a.device != dev || (uintptr_t)p % sizeof(double) != 0) return false;
+  // the allocation that p lies in, from the driver (found once, for all threads)
+  static const auto range_of = [] {
+    void* f = nullptr;
+    cudaDriverEntryPointQueryResult found;
+    if (cudaGetDriverEntryPointByVersion("cuMemGetAddressRange", &f, 12000, cudaEnableDefault, &found) != cudaSuccess ||
+        found != cudaDriverEntryPointSuccess) {
+      cudaGetLastError();
+      f = nullptr;
+    }
+    return reinterpret_cast<decltype(&cuMemGetAddressRange)>(f);
+  }();
+  CUdeviceptr base = 0;
+  size_t size = 0;
+  if (!range_of || range_of(&base, &size, (CUdeviceptr)(uintptr_t)p) != CUDA_SUCCESS) return false;
+  const size_t offset = (uintptr_t)p - (uintptr_t)base;
+  return offset <= size && bytes <= size - offset;
 }
 
 __global__ void widen_kernel(long long n, const float* __restrict__ src, double* __restrict__ dst) {

@@ -155,9 +155,10 @@ struct StateForm {
 };
 cudaError_t launch_import_state(long long P, const RefState& r, const double* src, const StateForm& to,
                                 cudaStream_t s);
-// Whether a kernel of the current device may read or write p itself: its own
-// memory, aligned.  (Other memory that the copy engines reach is staged.)
-bool direct_device_access(const void* p);
+// Whether a kernel of the current device may read or write p[0 .. bytes) itself:
+// its own memory, aligned, inside one allocation.  (Other memory is staged: the copy
+// reaches more than a kernel may, and refuses a range past its allocation.)
+bool direct_device_access(const void* p, size_t bytes);
 cudaError_t launch_from_offset(const Geom& g, const RefState& r, const double* q_off, double* q_plain,
                                cudaStream_t s);
 // dst[i] = (double)src[i], i < n

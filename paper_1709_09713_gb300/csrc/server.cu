@@ -46,6 +46,7 @@ int sfail(int code, const char* fmt, ...) {
 }
 
 int scuda(cudaError_t e, const char* what) {
+  cudaGetLastError();  // reported here, not again by the next launch
   return sfail(SBLI_ECUDA, "%s: %s (%s)", what, cudaGetErrorName(e), cudaGetErrorString(e));
 }
 
@@ -332,7 +333,8 @@ int retire(sbli_server* s, Req& q) {
   double h[2];
   SBLI_STRY(cudaMemcpyAsync(h, s->ke_dev, sizeof h, cudaMemcpyDeviceToHost, st), "D2H");
   if (q.r.result) {
-    const bool staged = q.r.result_is_host || !direct_device_access(q.r.result);
+    const size_t bytes = 5 * (size_t)q.P * sizeof(double);
+    const bool staged = q.r.result_is_host || !direct_device_access(q.r.result, bytes);
     // staged through a register the finished state does not occupy
     double* dst = staged ? r64(s, q, req_free_reg(q)) : q.r.result;
     if (q.r.precision == SBLI_FP32_DF) {
@@ -342,7 +344,7 @@ int retire(sbli_server* s, Req& q) {
       SBLI_STRY(launch_from_offset(g, make_ref(q.r.params), state, dst, st), "from_offset");
     }
     if (staged)
-      SBLI_STRY(cudaMemcpyAsync(q.r.result, dst, 5 * (size_t)q.P * sizeof(double),
+      SBLI_STRY(cudaMemcpyAsync(q.r.result, dst, bytes,
                                 q.r.result_is_host ? cudaMemcpyDeviceToHost : cudaMemcpyDeviceToDevice, st),
                 "copy result");
   }
