@@ -1,5 +1,5 @@
 """The double-float split of a binary64 value used by the stages: hi + lo is
-the value to 48 bits over the binary32 range, and zeros, overflow, infinities
+the value to 48 bits, or to 2^-126, over the binary32 range, and zeros, overflow, infinities
 and NaNs keep their meaning."""
 import os
 import subprocess
