@@ -690,7 +690,7 @@ struct StreamTerms {
   T v[3];     // sum_j D2_j u_i + 1/3 sum_j d2 u_j / dx_i dx_j
   T lapT;     // sum_j D2_j T'
   T a[3];     // D1_j u_i + D1_i u_j for (i, j) = (0, 1), (0, 2), (1, 2)
-  T lo[3];    // the first of the two alone (vorticity; diagnostics only)
+  T lo[3];    // the first of the two alone, D1_j u_i (vorticity; diagnostics only)
   T gd[3];    // D1_j u_j
 };
 
@@ -1627,6 +1627,12 @@ __device__ __forceinline__ void fused_march(const StageArgs& a, const Coef<T>& c
         t.gd[0] = g00c;
         t.gd[1] = g11c;
         t.gd[2] = d22;
+        // D1_i u_j, i < j, which axis i alone has put into the sum a when axis j starts (diagnostics)
+        T hi[3];
+        auto first_gradients = [&](int axis) {
+          if (WITH_KE && axis == 0) hi[0] = t.a[0], hi[1] = t.a[1];
+          if (WITH_KE && axis == 1) hi[2] = t.a[2];
+        };
         if constexpr (FIXED) {
           auto at0 = [&](int k, T& x, T&) { x = sf0(k); };
           auto at1 = [&](int k, T& x, T&) { x = sf1(k); };
@@ -1639,23 +1645,27 @@ __device__ __forceinline__ void fused_march(const StageArgs& a, const Coef<T>& c
             }
           };
           axis_terms_fixed<0, WITH_KE>(ld0, at0, c, uc, t);
+          first_gradients(0);
           axis_terms_fixed<1, WITH_KE>(ld1, at1, c, uc, t);
+          first_gradients(1);
           tmem_converge<ZT>();
           axis_terms_fixed<2, WITH_KE>(ld2, at2, c, uc, t);
         } else {
           axis_terms_stream<0, false, WITH_KE>(ld0, sf0, c, uc, t);
+          first_gradients(0);
           // shared-memory loads of one axis at a time: hoisted over the axes they spill at the binary32 ring
           // kernel's 128 registers (256^3: 674 us a stage without these two, 651 with)
           if constexpr (!ZT && sizeof(T) == 4) asm volatile("" ::: "memory");
           axis_terms_stream<1, false, WITH_KE, RP>(ld1, sf1, c, uc, t);
+          first_gradients(1);
           if constexpr (!ZT && sizeof(T) == 4) asm volatile("" ::: "memory");
           axis_terms_stream<2, MIXZ, WITH_KE>(ld2, sf2, c, uc, t, xf);
         }
         assemble_streamed(t, rho_p, mc, Ec, uc, c, R);
-        if (WITH_KE) {  // D1_j u_i - D1_i u_j = 2 D1_j u_i - (their sum), lo = D1_j u_i with i < j
-          w2 = fmadd(T(-2), t.lo[0], t.a[0]);
-          w1 = fmadd(T(2), t.lo[1], -t.a[1]);
-          w0 = fmadd(T(-2), t.lo[2], t.a[2]);
+        if (WITH_KE) {  // differences of two derivatives: D1_i u_j, i < j, and lo = D1_j u_i
+          w2 = hi[0] - t.lo[0];
+          w1 = t.lo[1] - hi[1];
+          w0 = hi[2] - t.lo[2];
         }
       }
 
