@@ -9,7 +9,6 @@
 // (d) the Runge-Kutta update of Fig. 1 runs as its own kernel.
 //
 // Variables are deviations from the reference state, as in the fused path.
-#include <algorithm>
 #include <type_traits>
 
 #include "fpconv.cuh"
@@ -81,38 +80,42 @@ __global__ void bl_primitives(Geom g, Coef<T> c, const TIN* __restrict__ q, T* _
   }
 }
 
-// Derivatives along one axis of one array (Listing 1): Eq. 6 into d1, Eq. 7 into
-// d2, each to its own array (null: not wanted).
+// Derivatives along one axis (Listing 1), each to its own array: Eq. 7 of one
+// array into d2, with Eq. 6 into d1[0] (null: not wanted); or, without a d2, Eq. 6
+// of up to BL_SET arrays (null: fewer).
+constexpr int BL_SET = 3, BL_JOBS = 24;
 template <typename T>
 struct Derivative {
-  const T* f;
-  T* d1;
+  const T* f[BL_SET];
+  T* d1[BL_SET];
   T* d2;
   int axis;
 };
-constexpr int BL_JOBS = 48;
 template <typename T>
 struct Derivatives {
-  Derivative<T> job[BL_JOBS];
-  int count;
+  Derivative<T> job[BL_JOBS];  // those with a d2 first
+  int with_second, count;
 };
 
-// A thread takes BL_Z points of one column: its wrapped offsets are formed once
-// (by comparisons) and the values along x2 stay in registers.  The modulo of
-// every wrapped index had bounded it as much as the binary64 pipe.  In binary64
-// the stencil is summed in integers, leaving one binary64 product a derivative, but
-// every third first derivative alone in a binary64 sum beside them, which
-// balances the two pipes (half or a sixth of them: 1.06 and 1.10 ms a stage against
-// 1.04).  All derivatives that do not read another's result are blocks of one
+// A thread takes BL_Z derivatives of one column: BL_Z planes of one array, or
+// BL_Z / BL_SET planes of a set.  Its wrapped offsets are formed once (by
+// comparisons); the modulo of every wrapped index had bounded it as much as the
+// binary64 pipe.  In binary64 the stencil is summed in integers, leaving one
+// binary64 product a derivative, but the second array of a set in a binary64 sum
+// beside the others, which balances the two pipes inside each thread.  (The array
+// decides, not the plane, so that a shifted state has the shifted derivatives, bit
+// for bit; every third plane in a binary64 sum took 1.036 ms a 128^3 stage, sets take
+// 1.047, all in integers 1.123, and sums of one kind a block, the kinds in turn, 1.148.)
+// All derivatives that do not read another's result are blocks of one
 // launch: 128^3 points are little over a wave of blocks, so a launch per
 // derivative left the SMs half idle in its last wave and between launches.
 // With the bounds on registers here and of the residual kernel, the 128^3
-// store-all stage takes 1.04 instead of 1.36 ms, the 64^3 one 151 instead of 298 us.
+// store-all stage takes 1.05 instead of 1.36 ms, the 64^3 one 151 instead of 298 us.
 constexpr int BL_Z = 9;
-template <typename T>
-__device__ __forceinline__ T bl_first(T m2, T m1, T p1, T p2, T k1, T k2, bool integer) {
+template <bool INTEGER, typename T>
+__device__ __forceinline__ T bl_first(T m2, T m1, T p1, T p2, T k1, T k2) {
   if constexpr (sizeof(T) == 8) {  // k2 = 1/(12 h)
-    return k2 * (integer ? stencil_first(m2, m1, p1, p2) : first_sum<false>(m2, m1, p1, p2, 0));
+    return k2 * (INTEGER ? stencil_first(m2, m1, p1, p2) : first_sum<false>(m2, m1, p1, p2, 0));
   } else {
     return k1 * (p1 - m1) - k2 * (p2 - m2);
   }
@@ -125,45 +128,47 @@ __device__ __forceinline__ T bl_second(T m2, T m1, T c, T p1, T p2, T k0, T k1, 
     return k0 * c + k1 * (p1 + m1) + k2 * (p2 + m2);
   }
 }
-template <int AXIS, bool FIRST, bool SECOND, typename T>
+__device__ __forceinline__ int bl_near(int v, int n) { return v < 0 ? v + n : (v >= n ? v - n : v); }  // |offset| <= 2 < n
+// in-plane offsets of the stencil's points, -2 .. +2 along AXIS
+template <int AXIS>
+__device__ __forceinline__ void bl_offsets(const Geom& g, int i, int j, int (&o)[5]) {
+#pragma unroll
+  for (int s = -2; s <= 2; ++s)
+    o[s + 2] = (AXIS == 0 ? bl_near(i + s, g.n0) : i) + g.n0 * (AXIS == 1 ? bl_near(j + s, g.n1) : j);
+}
+// the second derivative of one array and (FIRST) its first; along x2 the
+// values stay in registers
+template <int AXIS, bool FIRST, typename T>
 __device__ __forceinline__ void bl_column(const Geom& g, const Coef<T>& c, const T* __restrict__ f,
                                           T* __restrict__ d1, T* __restrict__ d2, int i, int j, int k0) {
   const long long pl = (long long)g.n0 * g.n1;
-  auto near = [](int v, int n) { return v < 0 ? v + n : (v >= n ? v - n : v); };  // |offset| <= 2 < n
-  const int own = i + g.n0 * j;
   int o[5];
-#pragma unroll
-  for (int s = -2; s <= 2; ++s)
-    o[s + 2] = AXIS == 0 ? near(i + s, g.n0) + g.n0 * j : AXIS == 1 ? i + g.n0 * near(j + s, g.n1) : own;
+  bl_offsets<AXIS>(g, i, j, o);
+  const int own = o[2];
   T w[5];  // the stencil's values; AXIS 2 keeps planes k - 2 .. k + 1
   if constexpr (AXIS == 2) {
 #pragma unroll
-    for (int s = -2; s <= 1; ++s) {
-      int z = k0 + s;
-      while (z >= g.n2) z -= g.n2;
-      w[s + 2] = f[own + pl * (z < 0 ? z + g.n2 : z)];
-    }
+    for (int s = -2; s <= 1; ++s) w[s + 2] = f[own + pl * bl_near(k0 + s, g.n2)];
   }
 #pragma unroll
   for (int q = 0; q < BL_Z; ++q) {
     const int k = k0 + q;
     if (k >= g.n2) break;
     if constexpr (AXIS == 2) {
-      w[4] = f[own + pl * near(k + 2, g.n2)];
+      w[4] = f[own + pl * bl_near(k + 2, g.n2)];
     } else {
 #pragma unroll
-      for (int s = 0; s < 5; ++s)
-        if (SECOND || s != 2) w[s] = f[o[s] + pl * k];
+      for (int s = 0; s < 5; ++s) w[s] = f[o[s] + pl * k];
     }
     const long long at = own + pl * k;
-    if constexpr (FIRST && SECOND && sizeof(T) == 8) {
+    if constexpr (FIRST && sizeof(T) == 8) {
       double a, b;
       stencil_both(w[0], w[1], w[2], w[3], w[4], a, b);
       d1[at] = c.c2[AXIS] * a;
       d2[at] = -c.e2[AXIS] * b;
     } else {
-      if constexpr (FIRST) d1[at] = bl_first(w[0], w[1], w[3], w[4], c.c1[AXIS], c.c2[AXIS], q % 3 != 1);
-      if constexpr (SECOND) d2[at] = bl_second(w[0], w[1], w[2], w[3], w[4], c.e0[AXIS], c.e1[AXIS], c.e2[AXIS]);
+      if constexpr (FIRST) d1[at] = bl_first<true>(w[0], w[1], w[3], w[4], c.c1[AXIS], c.c2[AXIS]);
+      d2[at] = bl_second(w[0], w[1], w[2], w[3], w[4], c.e0[AXIS], c.e1[AXIS], c.e2[AXIS]);
     }
     if constexpr (AXIS == 2) {
 #pragma unroll
@@ -171,46 +176,71 @@ __device__ __forceinline__ void bl_column(const Geom& g, const Coef<T>& c, const
     }
   }
 }
+// first derivatives of a set of arrays
 template <int AXIS, typename T>
-__device__ __forceinline__ void bl_axis(const Geom& g, const Coef<T>& c, const Derivative<T>& d, int i, int j, int k0) {
-  if (d.d1 && d.d2)
-    bl_column<AXIS, true, true>(g, c, d.f, d.d1, d.d2, i, j, k0);
-  else if (d.d1)
-    bl_column<AXIS, true, false>(g, c, d.f, d.d1, d.d2, i, j, k0);
-  else
-    bl_column<AXIS, false, true>(g, c, d.f, d.d1, d.d2, i, j, k0);
+__device__ __forceinline__ void bl_set(const Geom& g, const Coef<T>& c, const Derivative<T>& d, int i, int j, int k0) {
+  const long long pl = (long long)g.n0 * g.n1;
+  int o[5];
+  bl_offsets<AXIS>(g, i, j, o);
+#pragma unroll
+  for (int q = 0; q < BL_Z / BL_SET; ++q) {
+    const int k = k0 + q;
+    if (k >= g.n2) break;
+    auto at = [&](int s) { return o[s + 2] + pl * (AXIS == 2 ? bl_near(k + s, g.n2) : k); };
+    const long long m2 = at(-2), m1 = at(-1), p1 = at(1), p2 = at(2), own = o[2] + pl * k;
+    auto first = [&](auto integer, int m) {
+      const T* __restrict__ f = d.f[m];
+      d.d1[m][own] = bl_first<decltype(integer)::value>(f[m2], f[m1], f[p1], f[p2], c.c1[AXIS], c.c2[AXIS]);
+    };
+    first(std::true_type{}, 0);
+    first(std::false_type{}, 1);
+    if (d.f[2]) first(std::true_type{}, 2);
+  }
 }
-// blocks of 32 x 8 columns, BL_Z planes each, job by job
+// blocks of 32 x 8 columns, job by job
 template <typename T>
 __global__ void __launch_bounds__(256, 8) bl_derivatives(Geom g, const __grid_constant__ Coef<T> c,
                                                       const __grid_constant__ Derivatives<T> jobs) {
   const unsigned bx = (g.n0 + 31) / 32, by = (g.n1 + 7) / 8, bz = (g.n2 + BL_Z - 1) / BL_Z;
+  constexpr int ZS = BL_Z / BL_SET;
   unsigned b = blockIdx.x;
   const int i = b % bx * 32 + threadIdx.x;
   b /= bx;
   const int j = b % by * 8 + threadIdx.y;
   b /= by;
-  const int k0 = b % bz * BL_Z;
   if (i >= g.n0 || j >= g.n1) return;
-  const Derivative<T>& d = jobs.job[b / bz];
-  if (d.axis == 0) bl_axis<0>(g, c, d, i, j, k0);
-  else if (d.axis == 1) bl_axis<1>(g, c, d, i, j, k0);
-  else bl_axis<2>(g, c, d, i, j, k0);
+  if (b < jobs.with_second * bz) {
+    const Derivative<T>& d = jobs.job[b / bz];
+    const int k0 = b % bz * BL_Z;
+    auto column = [&](auto axis) {
+      constexpr int A = decltype(axis)::value;
+      if (d.d1[0]) bl_column<A, true>(g, c, d.f[0], d.d1[0], d.d2, i, j, k0);
+      else bl_column<A, false>(g, c, d.f[0], d.d1[0], d.d2, i, j, k0);
+    };
+    if (d.axis == 0) column(std::integral_constant<int, 0>{});
+    else if (d.axis == 1) column(std::integral_constant<int, 1>{});
+    else column(std::integral_constant<int, 2>{});
+  } else {
+    b -= jobs.with_second * bz;
+    const unsigned bs = (g.n2 + ZS - 1) / ZS;
+    const Derivative<T>& d = jobs.job[jobs.with_second + b / bs];
+    const int k0 = b % bs * ZS;
+    if (d.axis == 0) bl_set<0>(g, c, d, i, j, k0);
+    else if (d.axis == 1) bl_set<1>(g, c, d, i, j, k0);
+    else bl_set<2>(g, c, d, i, j, k0);
+  }
 }
 
+// (The blocks of a launch stay below the grid's limit of 2^31 - 1: fewer than 2^32 points,
+// 6.4 times as many with the padding of the narrowest tiles, 256 columns a block and
+// at most 5.4 blocks a column and plane are 5.8e8.)
 template <typename T>
 cudaError_t launch_derivatives(const Geom& g, const Coef<T>& c, const Derivatives<T>& jobs, cudaStream_t s) {
-  const long long blocks = (long long)((g.n0 + 31) / 32) * ((g.n1 + 7) / 8) * ((g.n2 + BL_Z - 1) / BL_Z);
-  // as many jobs a launch as the grid's limit of 2^31 - 1 blocks allows
-  const int most = (int)std::min<long long>(jobs.count, std::max<long long>(1, 0x7FFFFFFFll / blocks));
-  for (int at = 0; at < jobs.count; at += most) {
-    Derivatives<T> some;
-    some.count = std::min(most, jobs.count - at);
-    std::copy(jobs.job + at, jobs.job + at + some.count, some.job);
-    bl_derivatives<T><<<(unsigned)(blocks * some.count), dim3(32, 8), 0, s>>>(g, c, some);
-    if (cudaError_t e = cudaGetLastError()) return e;
-  }
-  return cudaSuccess;
+  const long long tiles = (long long)((g.n0 + 31) / 32) * ((g.n1 + 7) / 8);
+  const long long bz = (g.n2 + BL_Z - 1) / BL_Z, bs = (g.n2 + BL_Z / BL_SET - 1) / (BL_Z / BL_SET);
+  const long long blocks = tiles * (jobs.with_second * bz + (jobs.count - jobs.with_second) * bs);
+  bl_derivatives<T><<<(unsigned)blocks, dim3(32, 8), 0, s>>>(g, c, jobs);
+  return cudaGetLastError();
 }
 
 // Bound by the binary64 pipe (at its measured rate): sums start from their first term, and three blocks on
@@ -283,30 +313,30 @@ cudaError_t storeall_rhs(const Geom& g, const Coef<T>& c, const TIN* q, T* s, cu
   } while (0)
   bl_primitives<T, TIN><<<pgrid(P), 256, 0, st>>>(g, c, q, s);
   SBLI_CK(cudaGetLastError());
-  // field by field, so that the three axes find it in L2
   static_assert(std::is_same<TIN, T>::value, "storeall_rhs differentiates conserved fields in the arithmetic type");
   Derivatives<T> first{}, mixed{};
-  auto add = [](Derivatives<T>& d, const T* f, T* d1, T* d2, int axis) { d.job[d.count++] = {f, d1, d2, axis}; };
-  for (int i = 0; i < 3; ++i) {
-    for (int j = 0; j < 3; ++j) add(first, arr(A_U + i), arr(A_DU + 3 * i + j), arr(A_D2U + 3 * i + j), j);
-    for (int j = 0; j < 3; ++j) add(first, q + (1 + i) * P, arr(A_DRHOU + 3 * i + j), nullptr, j);
-    for (int j = i; j < 3; ++j) {
-      add(first, arr(A_MU + sym(i, j)), arr(A_DRHOUU + 3 * i + j), nullptr, j);
-      if (j != i) add(first, arr(A_MU + sym(i, j)), arr(A_DRHOUU + 3 * j + i), nullptr, i);
-    }
-  }
-  for (int j = 0; j < 3; ++j) add(first, q, arr(A_DRHO + j), nullptr, j);
-  for (int j = 0; j < 3; ++j) add(first, arr(A_P), arr(A_DP + j), nullptr, j);
-  for (int j = 0; j < 3; ++j) add(first, q + 4 * P, arr(A_DE + j), nullptr, j);
-  for (int j = 0; j < 3; ++j) add(first, arr(A_T), nullptr, arr(A_D2T + j), j);
-  for (int j = 0; j < 3; ++j) {
-    add(first, arr(A_EU + j), arr(A_DEU + j), nullptr, j);
-    add(first, arr(A_PU + j), arr(A_DPU + j), nullptr, j);
-  }
-  // mixed derivatives D_i (D_j u_j), i != j, from the stored diagonal gradients
+  // field by field, so that the three axes find it in L2
+  for (int i = 0; i < 3; ++i)
+    for (int j = 0; j < 3; ++j)
+      first.job[first.count++] = {{arr(A_U + i)}, {arr(A_DU + 3 * i + j)}, arr(A_D2U + 3 * i + j), j};
+  for (int j = 0; j < 3; ++j) first.job[first.count++] = {{arr(A_T)}, {}, arr(A_D2T + j), j};
+  first.with_second = first.count;
   for (int j = 0; j < 3; ++j)
-    for (int i = 0; i < 3; ++i)
-      if (i != j) add(mixed, arr(A_DU + 3 * j + j), arr(A_DDU + offd(i, j)), nullptr, i);
+    first.job[first.count++] = {{q + P, q + 2 * P, q + 3 * P},
+                                {arr(A_DRHOU + j), arr(A_DRHOU + 3 + j), arr(A_DRHOU + 6 + j)}, nullptr, j};
+  for (int j = 0; j < 3; ++j)
+    first.job[first.count++] = {{arr(A_MU + sym(0, j)), arr(A_MU + sym(1, j)), arr(A_MU + sym(2, j))},
+                                {arr(A_DRHOUU + j), arr(A_DRHOUU + 3 + j), arr(A_DRHOUU + 6 + j)}, nullptr, j};
+  for (int j = 0; j < 3; ++j)
+    first.job[first.count++] = {{q, arr(A_P), q + 4 * P}, {arr(A_DRHO + j), arr(A_DP + j), arr(A_DE + j)}, nullptr, j};
+  for (int j = 0; j < 3; ++j)
+    first.job[first.count++] = {{arr(A_EU + j), arr(A_PU + j)}, {arr(A_DEU + j), arr(A_DPU + j)}, nullptr, j};
+  // mixed derivatives D_i (D_j u_j), i != j, from the stored diagonal gradients
+  for (int i = 0; i < 3; ++i) {
+    const int j = (i + 1) % 3, k = (i + 2) % 3;
+    mixed.job[mixed.count++] = {{arr(A_DU + 4 * j), arr(A_DU + 4 * k)}, {arr(A_DDU + offd(i, j)), arr(A_DDU + offd(i, k))},
+                                nullptr, i};
+  }
   SBLI_CK(launch_derivatives(g, c, first, st));
   SBLI_CK(launch_derivatives(g, c, mixed, st));
   // conserved variables in the arithmetic type (callers pass T == TIN)
@@ -341,8 +371,8 @@ __global__ void rk_update_kernel(long long n, const TR* __restrict__ r, const do
 
 cudaError_t launch_gradients_fp64(const Geom& g, const Coef<double>& c, const double* u, double* grad, cudaStream_t s) {
   Derivatives<double> d{};
-  for (int i = 0; i < 3; ++i)
-    for (int j = 0; j < 3; ++j) d.job[d.count++] = {u + i * g.P, grad + (3 * i + j) * g.P, nullptr, j};
+  for (int j = 0; j < 3; ++j)
+    d.job[d.count++] = {{u, u + g.P, u + 2 * g.P}, {grad + j * g.P, grad + (3 + j) * g.P, grad + (6 + j) * g.P}, nullptr, j};
   return launch_derivatives(g, c, d, s);
 }
 
