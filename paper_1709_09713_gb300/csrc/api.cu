@@ -61,9 +61,6 @@ bool valid_sizes(int n0, int n1, int n2) {
   return true;
 }
 
-FusedConfig default_config(const Geom& g, int precision, int sms);
-
-
 // binary64 state, accumulator and stage registers (three-register rotation)
 bool f64_registers(int precision) { return precision == SBLI_FP64 || precision == SBLI_DF64; }
 
@@ -202,7 +199,9 @@ void use_config(sbli_grid* g, const FusedConfig& cfg) {
 // Binary32 grids: z queue and planes per CTA by the model of their stage (us a
 // stage, shared ring with planes by waves -> this: 128^3 96.7 -> 63.7, 96^3 35.8 ->
 // 30.3, 40^3 9.3 -> 7.6, 32^3 9.2 -> 4.4).
-FusedConfig default_config(const Geom& g, int precision, int sms) {
+// The other variants launch none of the fused kernels, and set_config takes no
+// TMEM queue for them, so their defaults have none either.
+FusedConfig default_config(const Geom& g, int precision, int variant, int sms) {
   FusedConfig cfg;
   cfg.ty = 8;
   cfg.zq = 0;
@@ -210,6 +209,7 @@ FusedConfig default_config(const Geom& g, int precision, int sms) {
   int zc[1];
   rank_zc(g, precision, cfg.ty, zc, 1);
   cfg.zc = std::max(4, std::min(zc[0], g.n2));
+  if (variant != SBLI_FUSED) return cfg;
   if (f64_registers(precision)) {
     const long long tiles = (long long)((g.n0 + F64_TILE_X - 1) / F64_TILE_X) * ((g.n1 + 7) / 8);
     cfg.zq = tiles * g.n2 >= 24LL * F64_CTAS_PER_SM * sms;
@@ -479,7 +479,7 @@ int sbli_create_grid(sbli_grid** out, int n0, int n1, int n2, int precision, int
   int dev = 0, sms = 152;
   if (cudaGetDevice(&dev) == cudaSuccess) cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
   g->sms = std::min(sms, MAX_SMALL_CTAS);
-  use_config(g, default_config(g->geom, precision, g->sms));
+  use_config(g, default_config(g->geom, precision, variant, g->sms));
   g->cd = make_coef<double>(g->n, p);
   g->cf = make_coef<float>(g->n, p);
   g->cw = make_coef<dfloat>(g->n, p);
