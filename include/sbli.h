@@ -212,8 +212,7 @@ SBLI_API int sbli_kinetic_energy_noalloc(const double* q_dev, int n0, int n1, in
  * is 32 x tile_y points per column a thread owns, 16 x 8 for binary64-register
  * grids (SBLI_FP64, SBLI_DF64), which take 8; binary32 grids 8 or 16), planes per CTA
  * along x2 (>= 4; binary64-register grids split all planes evenly over the SMs
- * instead where that leaves the longest CTA fewer of them, and 4 lets binary32
- * grids too small to give every SM a CTA take fewer), where each thread keeps its column's records of the five
+ * instead where that leaves the longest CTA fewer of them), where each thread keeps its column's records of the five
  * x2 planes (z_queue = 0: the shared-memory ring; 1: a per-thread queue in
  * Blackwell tensor memory, with only three full-record planes in shared
  * memory -- four for binary32 tile_y 16, which saves one barrier per plane)
@@ -225,6 +224,9 @@ SBLI_API int sbli_kinetic_energy_noalloc(const double* q_dev, int n0, int n1, in
  * fuse multiply-adds differently (bitwise equal among themselves, within the
  * binary32 tolerance of one column).  set_config validates and applies it
  * (cached step graphs are rebuilt); must be called at a step boundary.
+ * A binary32 grid too small to give every SM a CTA of 4 planes takes fewer under the
+ * configuration it starts with (and where the autotuner keeps that); get_config
+ * reports 4 then, and set_config with 4 launches 4.
  * z_queue and columns_per_thread may be NULL in get_config. */
 SBLI_API int sbli_get_config(const sbli_grid* g, int* tile_y, int* planes_per_cta, int* z_queue,
                              int* columns_per_thread);
@@ -232,7 +234,7 @@ SBLI_API int sbli_set_config(sbli_grid* g, int tile_y, int planes_per_cta, int z
 
 /* Autotuner: times candidate configurations (each allowed tile height, z
  * queue and columns per thread with the six planes-per-CTA values a
- * wave-balance model ranks best) on this grid with `reps` timed stage-0 launches each,
+ * wave-balance model ranks best, and the one the grid starts with) on this grid with `reps` timed stage-0 launches each,
  * at dt = 0 (the accumulator they write equals the state they read, so a
  * double-float grid's state, updated in place, keeps its value; the stage
  * field goes to a free register), keeps the

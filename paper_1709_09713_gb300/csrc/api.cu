@@ -110,7 +110,8 @@ struct sbli_grid {
   long long stages_done;
   FusedConfig cfg;
   int sms;      // SMs of the device
-  int zc;       // planes per CTA of a launch (cfg.zc, or fewer on small binary32 grids)
+  bool fewer;   // cfg is the grid's own choice, whose 4 planes per CTA may stand for fewer
+  int zc;       // planes per CTA of a launch: cfg.zc, or (fewer) binary32_launch_zc
   Split split;  // binary64-register grids: the work split of cfg
   Coef<double> cd;
   Coef<float> cf;
@@ -180,13 +181,16 @@ void rank_zc(const Geom& g, int precision, int ty, int* best, int nbest, int px 
     if (best[i] == 0) best[i] = best[0] ? best[0] : std::min(4, g.n2);
 }
 
-void use_config(sbli_grid* g, const FusedConfig& cfg) {
+// fewer: the grid's own choice (its default, or that of the autotuner); a
+// configuration that the caller sets is launched as it is.
+void use_config(sbli_grid* g, const FusedConfig& cfg, bool fewer) {
   g->cfg = cfg;
+  g->fewer = fewer;
   g->zc = cfg.zc;
   if (f64_registers(g->precision))
     g->split = plan_split(g->geom, cfg, std::min(F64_CTAS_PER_SM * g->sms, MAX_SMALL_CTAS),
                           g->precision == SBLI_DF64);
-  else
+  else if (fewer)
     g->zc = binary32_launch_zc(g->geom, cfg, g->sms);
 }
 
@@ -479,7 +483,7 @@ int sbli_create_grid(sbli_grid** out, int n0, int n1, int n2, int precision, int
   int dev = 0, sms = 152;
   if (cudaGetDevice(&dev) == cudaSuccess) cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
   g->sms = std::min(sms, MAX_SMALL_CTAS);
-  use_config(g, default_config(g->geom, precision, variant, g->sms));
+  use_config(g, default_config(g->geom, precision, variant, g->sms), true);
   g->cd = make_coef<double>(g->n, p);
   g->cf = make_coef<float>(g->n, p);
   g->cw = make_coef<dfloat>(g->n, p);
@@ -778,10 +782,8 @@ int sbli_set_config(sbli_grid* g, int tile_y, int planes_per_cta, int z_queue, i
   cfg.zc = std::min(planes_per_cta, g->geom.n2);
   cfg.zq = z_queue;
   cfg.px = columns_per_thread;
-  if (cfg.ty != g->cfg.ty || cfg.zc != g->cfg.zc || cfg.zq != g->cfg.zq || cfg.px != g->cfg.px) {
-    use_config(g, cfg);
-    drop_graphs(g);
-  }
+  if (cfg.ty != g->cfg.ty || cfg.zc != g->zc || cfg.zq != g->cfg.zq || cfg.px != g->cfg.px) drop_graphs(g);
+  use_config(g, cfg, false);
   return SBLI_OK;
 }
 
@@ -792,7 +794,7 @@ int sbli_autotune(sbli_grid* g, int reps, int* tile_y, int* planes_per_cta, int*
   if (g->variant != SBLI_FUSED) return fail(SBLI_EUNSUPPORTED, "autotune needs the fused variant");
   if (reps < 1) return fail(SBLI_EINVAL, "reps must be >= 1");
   constexpr int ZC_CANDIDATES = 6;  // planes-per-CTA values per kernel shape, best first by the wave model
-  FusedConfig cand[8 * ZC_CANDIDATES];
+  FusedConfig cand[8 * ZC_CANDIDATES + 1];
   int nc = 0;
   const int tys[2] = {8, 16};
   for (int px = 1; px <= 2; ++px)
@@ -809,6 +811,9 @@ int sbli_autotune(sbli_grid* g, int reps, int* tile_y, int* planes_per_cta, int*
           if (!dup && nc < 8 * ZC_CANDIDATES) cand[nc++] = FusedConfig{tys[t], z, zq, px};
         }
       }
+  // and the grid's default, which alone may launch fewer planes per CTA than 4
+  const int own = nc;
+  cand[nc++] = default_config(g->geom, g->precision, g->variant, g->sms);
   cudaEvent_t e0, e1;
   SBLI_TRY(cudaEventCreate(&e0), "cudaEventCreate");
   cudaError_t ce = cudaEventCreate(&e1);
@@ -817,11 +822,13 @@ int sbli_autotune(sbli_grid* g, int reps, int* tile_y, int* planes_per_cta, int*
     return cuda_fail(ce, "cudaEventCreate");
   }
   const FusedConfig saved = g->cfg;
+  const bool saved_fewer = g->fewer;
+  const int saved_zc = g->zc;
   int best = -1;
   float best_ms = 1e30f;
   cudaError_t err = cudaSuccess;
   for (int i = 0; i < nc && err == cudaSuccess; ++i) {
-    use_config(g, cand[i]);
+    use_config(g, cand[i], i == own);
     // stage 0 with dt = 0: the accumulator it writes equals the state it
     // reads (acc + 0 * R), so a double-float grid's state, updated in place,
     // keeps its value; the stage field goes to a free register
@@ -841,11 +848,11 @@ int sbli_autotune(sbli_grid* g, int reps, int* tile_y, int* planes_per_cta, int*
   cudaEventDestroy(e0);
   cudaEventDestroy(e1);
   if (err != cudaSuccess) {
-    use_config(g, saved);
+    use_config(g, saved, saved_fewer);
     return cuda_fail(err, "autotune launch");
   }
-  use_config(g, cand[best]);
-  if (g->cfg.ty != saved.ty || g->cfg.zc != saved.zc || g->cfg.zq != saved.zq || g->cfg.px != saved.px)
+  use_config(g, cand[best], best == own);
+  if (g->cfg.ty != saved.ty || g->zc != saved_zc || g->cfg.zq != saved.zq || g->cfg.px != saved.px)
     drop_graphs(g);
   if (tile_y) *tile_y = g->cfg.ty;
   if (planes_per_cta) *planes_per_cta = g->cfg.zc;

@@ -133,8 +133,8 @@ int fused_num_ctas(const Geom& g, const FusedConfig& cfg);
 // one column per thread), from measured times of a plane at one, two and three
 // CTAs an SM.
 double binary32_stage_us(long long ctas, int zc, int zq, int sms);
-// Planes per CTA of a binary32 launch configured with zc: fewer than the
-// smallest configurable 4 on grids too small to give every SM a CTA otherwise.
+// Planes per CTA that a binary32 grid's own configuration launches: cfg.zc, or fewer than
+// the smallest configurable 4 on grids too small to give every SM a CTA otherwise.
 int binary32_launch_zc(const Geom& g, const FusedConfig& cfg, int sms);
 // CTAs of a binary64-register stage and whether they split the planes evenly (else chunks of zc planes)
 struct Split {

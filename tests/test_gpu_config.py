@@ -30,3 +30,22 @@ def test_reported_config_can_be_set(S, variant, precision, n):
     g.set_config(*cfg)
     assert g.config() == cfg
     g.close()
+
+
+def test_configured_planes_are_launched(S):
+    """The kinetic energy shows which planes a CTA sums: 2 at x2 = 0 and 2^-53 at
+    x2 = 4, 5, 6 of one column.  CTAs of four planes form 3 x 2^-53 first, which moves
+    the total by a unit in the last place; singly each would be lost."""
+    n = (32, 32, 32)
+    q = torch.zeros((5, n[2], n[1], n[0]), dtype=torch.float64)
+    q[0], q[4] = 1.0, 200.0
+    q[1, 0, 0, 0] = 2.0
+    q[1, 4:7, 0, 0] = 2.0**-26
+    for precision in (S.SBLI_FP32, S.SBLI_FP32_DF):
+        g = S.Grid(n, precision)
+        start = g.config()
+        for cfg in ((8, 4, 0, 1), (8, 4, 1, 1)):  # one of them the grid's own default, of fewer planes
+            g.set_config(*cfg)
+            g.set_state(q)
+            assert g.step_n_history(1, 1e-6)[0, 0].item() == (2.0 + 2.0**-51) / 32**3, (start, cfg)
+        g.close()
