@@ -274,7 +274,8 @@ SBLI_API int sbli_batch_work_items(const sbli_batch* b, long long* items);
  * results.  Members of the binary64-register precisions are split evenly over
  * the CTAs whatever their planes per item.  set_schedule (between steps; SBLI_EINVAL for z_queue outside 0..1
  * or fewer than 4 planes) drops the captured step graphs; planes_per_item may
- * be NULL in both calls (keep, or do not return, the per-member values). */
+ * be NULL in both calls (keep, or do not return, the per-member values; a batch
+ * whose planes were never set keeps its own). */
 SBLI_API int sbli_batch_get_schedule(const sbli_batch* b, int* z_queue, int* planes_per_item);
 SBLI_API int sbli_batch_set_schedule(sbli_batch* b, int z_queue, const int* planes_per_item);
 /* Autotuner of the schedule: times stage-0 launches with dt = 0 (reps each;
@@ -283,8 +284,8 @@ SBLI_API int sbli_batch_set_schedule(sbli_batch* b, int z_queue, const int* plan
  * every z_queue mode with one planes-per-item value for all
  * members (4, 8, 16, 32, 64, 128, whole member), then refines the planes per
  * item of each size class (members with the same n2) in turn, and keeps the
- * fastest schedule (if a trial launch fails, the schedule in place before
- * the call is restored and SBLI_ECUDA returned).  The state is not
+ * fastest schedule, or the one in place if that is faster (if a trial launch
+ * fails, it is restored and SBLI_ECUDA returned).  The state is not
  * changed.  Synchronises the batch's
  * stream.  *z_queue and *best_stage_ms (may be NULL) return the choice and
  * its stage time; sbli_batch_get_schedule returns the planes per item. */

@@ -202,7 +202,7 @@ size_t balign(size_t v) { return (v + BALIGN - 1) / BALIGN * BALIGN; }
 struct MemberLayout {
   int n[3];
   int zc;  // planes per work item (the schedule; batch_zc at creation)
-  int launch_zc;  // planes per item of a launch: zc, or under the default schedule at most batch_zc_cap
+  int launch_zc;  // planes per item of a launch: zc, or under the batch's own schedule at most batch_zc_cap
   long long P;
   size_t off64, off32;  // byte offsets inside the binary64 / binary32 register regions
 };
@@ -242,8 +242,7 @@ BatchLayout batch_layout(int count, const int* n, int precision) {
   L.n32 = batch_f64_registers(precision) ? 0 : 2;
   // partials: one per work item, or (even split) one per CTA and member
   L.items_bytes = balign((size_t)(2 * std::max<long long>(L.total_items, BATCH_MAX_EVEN_CTAS + count) + 2) * sizeof(double));
-  L.total_items = 0;
-  for (const MemberLayout& M : L.m) L.total_items += member_items(M.n, M.zc);  // set again with the ranges
+  L.total_items = 0;  // set with the ranges
   // per member: KE result pair, 1/P, range of partials; plus the KE kernel partials
   L.misc_bytes = balign((size_t)count * 2 * sizeof(double)) + balign((size_t)count * sizeof(double)) +
                  balign((size_t)(2 * count) * sizeof(long long)) + balign(2 * 1024 * sizeof(double));
@@ -255,6 +254,7 @@ BatchLayout batch_layout(int count, const int* n, int precision) {
 
 struct sbli_batch {
   int count, precision;
+  bool planes_set;  // the caller or the autotuner has set the planes per item
   std::vector<sbli_params> params;
   BatchLayout L;
   cudaStream_t stream, cap_stream;
@@ -446,14 +446,37 @@ cudaError_t upload_ranges(sbli_batch* b) {
   return e;
 }
 
-// Apply a schedule (z-queue mode, planes per item of each member); the
-// captured step graphs are rebuilt on the next step.
-cudaError_t apply_schedule(sbli_batch* b, int zq, const std::vector<int>& zc) {
+// A schedule: z-queue mode and planes per item of each member, or (zc empty) the
+// batch's own planes, batch_zc of each member and in binary32 launches at most what
+// the model of a stage ranks best.
+struct Schedule {
+  int zq;
+  std::vector<int> zc;
+};
+
+Schedule current_schedule(const sbli_batch* b) {
+  Schedule s{b->zq, {}};
+  if (b->planes_set)
+    for (const MemberLayout& M : b->L.m) s.zc.push_back(M.zc);
+  return s;
+}
+
+// Apply it; the captured step graphs are rebuilt on the next step.
+cudaError_t apply_schedule(sbli_batch* b, const Schedule& s) {
   int dev = 0, sms = 152;
   if (cudaGetDevice(&dev) == cudaSuccess) cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-  b->zq = zq;
-  b->grid_ctas = batch_grid_ctas(sms, b->precision, zq);
-  for (int m = 0; m < b->count; ++m) b->L.m[m].zc = b->L.m[m].launch_zc = zc[m];
+  b->zq = s.zq;
+  b->grid_ctas = batch_grid_ctas(sms, b->precision, s.zq);
+  b->planes_set = !s.zc.empty();
+  for (int m = 0; m < b->count; ++m) {
+    MemberLayout& M = b->L.m[m];
+    M.zc = M.launch_zc = b->planes_set ? s.zc[m] : batch_zc(M.n[2]);
+  }
+  if (!b->planes_set && !batch_f64_registers(b->precision)) {
+    const int cap = batch_zc_cap(
+        b->count, [&](int m) { return b->L.m[m].n; }, b->zq, sms);
+    for (MemberLayout& M : b->L.m) M.launch_zc = std::min(M.zc, cap);
+  }
   batch_drop_graphs(b);
   return upload_ranges(b);
 }
@@ -523,22 +546,12 @@ int sbli_batch_create(sbli_batch** out, int count, const int* n, const sbli_para
   b->ke_scratch = reinterpret_cast<double*>(w);
   b->state = batch_initial_state(b->precision);
   b->steps_done = 0;
-  int dev = 0, sms = 152;
-  cudaGetDevice(&dev);
-  cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-  b->zq = batch_default_zq(precision);
-  b->grid_ctas = batch_grid_ctas(sms, precision, b->zq);
-  if (!batch_f64_registers(precision)) {
-    const int cap = batch_zc_cap(
-        count, [&](int m) { return b->L.m[m].n; }, b->zq, sms);
-    for (MemberLayout& M : b->L.m) M.launch_zc = std::min(M.zc, cap);
-  }
   // per-member constants for the KE finalisation
   std::vector<double> inv(count);
   for (int m = 0; m < count; ++m) inv[m] = 1.0 / (double)b->L.m[m].P;
   cudaError_t e = cudaStreamCreateWithFlags(&b->cap_stream, cudaStreamNonBlocking);
   if (e == cudaSuccess) e = cudaMemcpyAsync(b->inv_p, inv.data(), count * sizeof(double), cudaMemcpyHostToDevice, b->stream);
-  if (e == cudaSuccess) e = upload_ranges(b);
+  if (e == cudaSuccess) e = apply_schedule(b, Schedule{batch_default_zq(precision), {}});
   if (e == cudaSuccess) e = cudaStreamSynchronize(b->stream);
   if (e != cudaSuccess) {
     delete b;
@@ -722,13 +735,14 @@ int sbli_batch_get_schedule(const sbli_batch* b, int* z_queue, int* planes_per_i
 int sbli_batch_set_schedule(sbli_batch* b, int z_queue, const int* planes_per_item) {
   if (int rc = check_batch(b, 0)) return rc;
   if (z_queue < 0 || z_queue > 1) return bfail(SBLI_EINVAL, "z_queue %d not 0 or 1", z_queue);
-  std::vector<int> zc(b->count);
-  for (int m = 0; m < b->count; ++m) {
-    zc[m] = planes_per_item ? planes_per_item[m] : b->L.m[m].zc;
-    if (zc[m] < 4) return bfail(SBLI_EINVAL, "member %d: planes per item %d < 4", m, zc[m]);
-    zc[m] = std::min(zc[m], b->L.m[m].n[2]);
+  Schedule next = current_schedule(b);
+  next.zq = z_queue;
+  if (planes_per_item) next.zc.assign(planes_per_item, planes_per_item + b->count);
+  for (int m = 0; m < (int)next.zc.size(); ++m) {
+    if (next.zc[m] < 4) return bfail(SBLI_EINVAL, "member %d: planes per item %d < 4", m, next.zc[m]);
+    next.zc[m] = std::min(next.zc[m], b->L.m[m].n[2]);
   }
-  SBLI_BTRY(apply_schedule(b, z_queue, zc), "schedule");
+  SBLI_BTRY(apply_schedule(b, next), "schedule");
   return SBLI_OK;
 }
 
@@ -746,8 +760,8 @@ int sbli_batch_autotune(sbli_batch* b, int reps, int* z_queue, float* best_stage
   // double-float members update theirs in place) and a stage field into a
   // free register
   cudaError_t err = cudaSuccess;
-  auto time_schedule = [&](int zq, const std::vector<int>& zc) -> float {
-    if (err == cudaSuccess) err = apply_schedule(b, zq, zc);
+  auto time_schedule = [&](const Schedule& s) -> float {
+    if (err == cudaSuccess) err = apply_schedule(b, s);
     if (err == cudaSuccess) err = enqueue_batch_stage(b, 0, b->state, 0.0, nullptr, b->stream);
     if (err == cudaSuccess) err = cudaEventRecord(e0, b->stream);
     for (int r = 0; r < reps && err == cudaSuccess; ++r) err = enqueue_batch_stage(b, 0, b->state, 0.0, nullptr, b->stream);
@@ -757,6 +771,18 @@ int sbli_batch_autotune(sbli_batch* b, int reps, int* z_queue, float* best_stage
     if (err == cudaSuccess) err = cudaEventElapsedTime(&ms, e0, e1);
     return err == cudaSuccess ? ms / (float)reps : 1e30f;
   };
+  const Schedule start = current_schedule(b);  // restored if a trial launch fails
+  Schedule choice = start;
+  float best = time_schedule(start);
+  std::vector<int> start_planes;  // that it launches
+  for (const MemberLayout& M : b->L.m) start_planes.push_back(M.launch_zc);
+  auto trial = [&](const Schedule& s) {
+    const float ms = time_schedule(s);
+    if (ms < best) {
+      best = ms;
+      choice = s;
+    }
+  };
   auto uniform = [&](int Z) {
     std::vector<int> zc(b->count);
     for (int m = 0; m < b->count; ++m) zc[m] = std::max(4, std::min(Z, b->L.m[m].n[2]));
@@ -764,47 +790,28 @@ int sbli_batch_autotune(sbli_batch* b, int reps, int* z_queue, float* best_stage
   };
   const int Zs[7] = {4, 8, 16, 32, 64, 128, 1 << 24};
   // 1. one z-queue mode and one planes-per-item value for every member
-  int best_zq = b->zq;
-  std::vector<int> best_zc(b->count);
-  for (int m = 0; m < b->count; ++m) best_zc[m] = b->L.m[m].zc;
-  const int start_zq = best_zq;
-  const std::vector<int> start_zc = best_zc;  // restored if a trial launch fails
-  float best = time_schedule(best_zq, best_zc);
   for (int zq = 0; zq <= 1; ++zq)
-    for (int Z : Zs) {
-      const std::vector<int> zc = uniform(Z);
-      const float ms = time_schedule(zq, zc);
-      if (ms < best) {
-        best = ms;
-        best_zq = zq;
-        best_zc = zc;
-      }
-    }
+    for (int Z : Zs) trial(Schedule{zq, uniform(Z)});
   // 2. each size class (members with the same x2 extent) refined in turn
   std::vector<int> classes;
-  for (int m = 0; m < b->count; ++m)
-    if (std::find(classes.begin(), classes.end(), b->L.m[m].n[2]) == classes.end()) classes.push_back(b->L.m[m].n[2]);
-  for (int n2 : classes) {
+  for (const MemberLayout& M : b->L.m)
+    if (std::find(classes.begin(), classes.end(), M.n[2]) == classes.end()) classes.push_back(M.n[2]);
+  for (int n2 : classes)
     for (int Z : Zs) {
-      std::vector<int> zc = best_zc;
+      const std::vector<int> now = choice.zc.empty() ? start_planes : choice.zc;
+      Schedule s{choice.zq, now};
       for (int m = 0; m < b->count; ++m)
-        if (b->L.m[m].n[2] == n2) zc[m] = std::max(4, std::min(Z, n2));
-      if (zc == best_zc) continue;
-      const float ms = time_schedule(best_zq, zc);
-      if (ms < best) {
-        best = ms;
-        best_zc = zc;
-      }
+        if (b->L.m[m].n[2] == n2) s.zc[m] = std::max(4, std::min(Z, n2));
+      if (s.zc != now) trial(s);
     }
-  }
   cudaEventDestroy(e0);
   cudaEventDestroy(e1);
   if (err != cudaSuccess) {
-    apply_schedule(b, start_zq, start_zc);
+    apply_schedule(b, start);
     return bcuda(err, "autotune launch");
   }
-  SBLI_BTRY(apply_schedule(b, best_zq, best_zc), "schedule");
-  if (z_queue) *z_queue = best_zq;
+  SBLI_BTRY(apply_schedule(b, choice), "schedule");
+  if (z_queue) *z_queue = choice.zq;
   if (best_stage_ms) *best_stage_ms = best;
   return SBLI_OK;
 }

@@ -49,3 +49,25 @@ def test_configured_planes_are_launched(S):
             g.set_state(q)
             assert g.step_n_history(1, 1e-6)[0, 0].item() == (2.0 + 2.0**-51) / 32**3, (start, cfg)
         g.close()
+
+
+@pytest.mark.parametrize("precision", [1, 2])
+def test_batch_keeps_its_own_planes(S, precision):
+    """A batch too small for 32 planes an item: setting the z-queue mode alone, and
+    a tuned batch set back to what it reported, launch what they did."""
+    sizes = [(64, 64, 64), (48, 40, 64)]
+    b = S.Batch(sizes, precision)
+    own = b.work_items()
+    assert own > sum(-(-n[0] // 32) * -(-n[1] // 8) * 2 for n in sizes)  # more than items of 32 planes
+    zq, planes = b.schedule()
+    b.set_schedule(zq)
+    assert b.work_items() == own and b.schedule() == (zq, planes)
+    b.set_schedule(1 - zq)
+    b.set_schedule(zq)
+    assert b.work_items() == own
+    b.set_schedule(zq, [32, 32])  # set: 32 planes are 32 planes
+    items = b.work_items()
+    assert items < own
+    b.set_schedule(zq)
+    assert b.work_items() == items
+    b.close()
