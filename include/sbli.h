@@ -262,7 +262,8 @@ SBLI_API int sbli_batch_create(sbli_batch** out, int count, const int* n, const 
                                void* workspace, size_t workspace_bytes, void* stream);
 SBLI_API int sbli_batch_destroy(sbli_batch* b);
 SBLI_API int sbli_batch_count(const sbli_batch* b, int* count);
-/* Total work items of one stage (for scheduling diagnostics). */
+/* Total work items of one stage (for scheduling diagnostics); of binary64 and
+ * double-float members the planes of their tiles, which the CTAs share evenly. */
 SBLI_API int sbli_batch_work_items(const sbli_batch* b, long long* items);
 /* The batch's schedule: z_queue (0 = x2-neighbour records from the
  * shared-memory ring, 1 = from the per-thread TMEM queue, as for single grids)
@@ -285,7 +286,8 @@ SBLI_API int sbli_batch_set_schedule(sbli_batch* b, int z_queue, const int* plan
  * members (4, 8, 16, 32, 64, 128, whole member), then refines the planes per
  * item of each size class (members with the same n2) in turn, and keeps the
  * fastest schedule, or the one in place if that is faster (if a trial launch
- * fails, it is restored and SBLI_ECUDA returned).  The state is not
+ * fails, it is restored and SBLI_ECUDA returned).  Binary64 and double-float
+ * members: both z_queue modes alone.  The state is not
  * changed.  Synchronises the batch's
  * stream.  *z_queue and *best_stage_ms (may be NULL) return the choice and
  * its stage time; sbli_batch_get_schedule returns the planes per item. */

@@ -439,7 +439,7 @@ cudaError_t upload_ranges(sbli_batch* b) {
     }
     items += member_items(M.n, M.launch_zc);
   }
-  b->L.total_items = items;
+  b->L.total_items = batch_f64_registers(b->precision) ? units : items;
   cudaError_t e = cudaMemcpyAsync(b->range, range.data(), range.size() * sizeof(long long), cudaMemcpyHostToDevice,
                                   b->stream);
   if (e == cudaSuccess) e = cudaStreamSynchronize(b->stream);  // range is a host temporary
@@ -783,27 +783,32 @@ int sbli_batch_autotune(sbli_batch* b, int reps, int* z_queue, float* best_stage
       choice = s;
     }
   };
-  auto uniform = [&](int Z) {
-    std::vector<int> zc(b->count);
-    for (int m = 0; m < b->count; ++m) zc[m] = std::max(4, std::min(Z, b->L.m[m].n[2]));
-    return zc;
-  };
-  const int Zs[7] = {4, 8, 16, 32, 64, 128, 1 << 24};
-  // 1. one z-queue mode and one planes-per-item value for every member
-  for (int zq = 0; zq <= 1; ++zq)
-    for (int Z : Zs) trial(Schedule{zq, uniform(Z)});
-  // 2. each size class (members with the same x2 extent) refined in turn
-  std::vector<int> classes;
-  for (const MemberLayout& M : b->L.m)
-    if (std::find(classes.begin(), classes.end(), M.n[2]) == classes.end()) classes.push_back(M.n[2]);
-  for (int n2 : classes)
-    for (int Z : Zs) {
-      const std::vector<int> now = choice.zc.empty() ? start_planes : choice.zc;
-      Schedule s{choice.zq, now};
-      for (int m = 0; m < b->count; ++m)
-        if (b->L.m[m].n[2] == n2) s.zc[m] = std::max(4, std::min(Z, n2));
-      if (s.zc != now) trial(s);
-    }
+  if (batch_f64_registers(b->precision)) {
+    // split evenly whatever the planes per item: only the other z-queue mode differs
+    trial(Schedule{1 - start.zq, start.zc});
+  } else {
+    auto uniform = [&](int Z) {
+      std::vector<int> zc(b->count);
+      for (int m = 0; m < b->count; ++m) zc[m] = std::max(4, std::min(Z, b->L.m[m].n[2]));
+      return zc;
+    };
+    const int Zs[7] = {4, 8, 16, 32, 64, 128, 1 << 24};
+    // 1. one z-queue mode and one planes-per-item value for every member
+    for (int zq = 0; zq <= 1; ++zq)
+      for (int Z : Zs) trial(Schedule{zq, uniform(Z)});
+    // 2. each size class (members with the same x2 extent) refined in turn
+    std::vector<int> classes;
+    for (const MemberLayout& M : b->L.m)
+      if (std::find(classes.begin(), classes.end(), M.n[2]) == classes.end()) classes.push_back(M.n[2]);
+    for (int n2 : classes)
+      for (int Z : Zs) {
+        const std::vector<int> now = choice.zc.empty() ? start_planes : choice.zc;
+        Schedule s{choice.zq, now};
+        for (int m = 0; m < b->count; ++m)
+          if (b->L.m[m].n[2] == n2) s.zc[m] = std::max(4, std::min(Z, n2));
+        if (s.zc != now) trial(s);
+      }
+  }
   cudaEventDestroy(e0);
   cudaEventDestroy(e1);
   if (err != cudaSuccess) {

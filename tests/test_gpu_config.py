@@ -71,3 +71,17 @@ def test_batch_keeps_its_own_planes(S, precision):
     b.set_schedule(zq)
     assert b.work_items() == items
     b.close()
+
+
+@pytest.mark.parametrize("precision", [0, 3])
+def test_even_batch_reports_what_it_launches(S, precision):
+    """Binary64-register members: work items are planes of 16 x 8 tiles, and the
+    planes per item, which nothing launches, stay as they are through a tuning."""
+    sizes = [(40, 17, 61), (33, 9, 7), (64, 64, 64)]
+    b = S.Batch(sizes, precision)
+    assert b.work_items() == sum(-(-n[0] // 16) * -(-n[1] // 8) * n[2] for n in sizes)
+    planes = b.schedule()[1]
+    b.init_tgv()
+    zq, ms = b.autotune(1)
+    assert b.schedule() == (zq, planes) and ms > 0
+    b.close()
