@@ -58,12 +58,15 @@ RefState make_ref(const sbli_params& p) {
 // The field is made of functions of one coordinate each, so a thread evaluates
 // those of its column once for INIT_Z planes and a block those of x2 once for
 // its planes: the binary64 pipe, which bounds this kernel, spends itself on
-// the products and not on six trigonometric functions a point.
+// the products and not on six trigonometric functions a point.  Block b takes part
+// b % parts of the columns and planes INIT_Z (b / parts) ...: one grid dimension, as
+// the others' limit of 65,535 is 2^21 planes.
 constexpr int INIT_Z = 32;
-__global__ void __launch_bounds__(256) init_tgv_kernel(Geom g, double h0, double h1, double h2, double L, double A,
-                                                       double gM2, double inv_gm1, double* __restrict__ q) {
+__global__ void __launch_bounds__(256) init_tgv_kernel(Geom g, unsigned parts, double h0, double h1, double h2,
+                                                       double L, double A, double gM2, double inv_gm1,
+                                                       double* __restrict__ q) {
   __shared__ double cz[INIT_Z], c2z[INIT_Z];
-  const int z0 = blockIdx.z * INIT_Z, nz = min(INIT_Z, g.n2 - z0);
+  const int z0 = (int)(blockIdx.x / parts) * INIT_Z, nz = min(INIT_Z, g.n2 - z0);
   if ((int)threadIdx.x < nz) {
     const double z = (z0 + (int)threadIdx.x) * h2;
     cz[threadIdx.x] = cos(z / L);
@@ -71,7 +74,7 @@ __global__ void __launch_bounds__(256) init_tgv_kernel(Geom g, double h0, double
   }
   __syncthreads();
   const long long P = g.P, plane = (long long)g.n0 * g.n1;
-  for (long long n = blockIdx.x * 256LL + threadIdx.x; n < plane; n += gridDim.x * 256LL) {
+  for (long long n = blockIdx.x % parts * 256LL + threadIdx.x; n < plane; n += parts * 256LL) {
     const double x = (int)(n % g.n0) * h0, y = (int)(n / g.n0) * h1;
     double sx, cx, sy, cy;
     sincos(x / L, &sx, &cx);
@@ -101,9 +104,9 @@ static unsigned grid_for(long long n, int block) {
 cudaError_t launch_init_tgv(const Geom& g, const sbli_params& p, double amplitude, double* q, cudaStream_t s) {
   const double h0 = 2.0 * M_PI * p.L / g.n0, h1 = 2.0 * M_PI * p.L / g.n1, h2 = 2.0 * M_PI * p.L / g.n2;
   const long long plane = (long long)g.n0 * g.n1;
-  const dim3 grid(grid_for(plane, 256), 1, (g.n2 + INIT_Z - 1) / INIT_Z);
-  init_tgv_kernel<<<grid, 256, 0, s>>>(g, h0, h1, h2, p.L, amplitude, p.gamma * p.Mach * p.Mach,
-                                                     1.0 / (p.gamma - 1.0), q);
+  const unsigned parts = grid_for(plane, 256);
+  init_tgv_kernel<<<parts * ((g.n2 + INIT_Z - 1) / INIT_Z), 256, 0, s>>>(
+      g, parts, h0, h1, h2, p.L, amplitude, p.gamma * p.Mach * p.Mach, 1.0 / (p.gamma - 1.0), q);
   return cudaGetLastError();
 }
 
