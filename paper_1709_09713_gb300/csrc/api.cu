@@ -222,7 +222,7 @@ FusedConfig default_config(const Geom& g, int precision, int variant, int sms) {
   double best = 0.0;
   FusedConfig c = cfg;
   for (c.zq = 0; c.zq < 2; ++c.zq)
-    for (c.zc = 4; c.zc <= std::max(4, g.n2); ++c.zc) {
+    for (c.zc = 4; c.zc <= std::max(4, g.n2); c.zc = fewer_chunks(g.n2, c.zc)) {
       FusedConfig launch = c;
       launch.zc = binary32_launch_zc(g, c, sms);
       const double us = binary32_stage_us(fused_num_ctas(g, launch), launch.zc, c.zq, sms);

@@ -106,6 +106,13 @@ struct FusedConfig {
            // of a 64 x ty tile computed together)
 };
 
+// The next larger planes per CTA that make fewer CTAs of n2 planes (n2 + 1 after n2):
+// the values in between only make them longer.  About 2 sqrt(n2) of them lie in 4 .. n2.
+inline int fewer_chunks(int n2, int zc) {
+  const int chunks = (n2 + zc - 1) / zc;
+  return chunks < 2 ? (n2 > zc ? n2 : zc) + 1 : (n2 + chunks - 2) / (chunks - 1);
+}
+
 // Host launchers (defined in fused_fp64.cu / fused_fp32.cu).
 // in_fp64: stage input is binary64 (FP64 path, or FP32 path at stage 0).
 // out_fp64: stage output is binary64.
