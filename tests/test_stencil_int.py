@@ -53,6 +53,26 @@ def test_sums_against_exact_arithmetic(exe):
     assert checked > 25000
 
 
+def test_sums_of_eight_values(exe):
+    """The binary64 x2 helper sums: weights 18 on each of two values a neighbour."""
+    text = subprocess.run([exe, "eight"], capture_output=True, text=True, check=True, timeout=120).stdout
+    checked = 0
+    for line in text.splitlines():
+        x = [struct.unpack("<d", struct.pack("<Q", int(w, 16)))[0] for w in line.split()]
+        v, r = x[:8], x[8]
+        if not all(map(math.isfinite, v)) or max(map(abs, v)) > 1e300:  # the plain sums
+            continue
+        m2, m1, p1, p2 = (Fraction(v[k]) + Fraction(v[4 + k]) for k in range(4))
+        want = 8 * (p1 - m1) - (p2 - m2)
+        tops = [math.frexp(a)[1] - 1 if a else -1100 for a in v]
+        unit = Fraction(2) ** (max(max(tops), 66 - 1023) - 56)
+        spread = max(tops) - min(t for t, a in zip(tops, v) if a) if any(v) else 0
+        lost = 0 if spread <= 4 and max(tops) > -900 else 36 * unit
+        assert abs(Fraction(r) - want) <= abs(want) / 2**53 * (1 + Fraction(1, 2**50)) + lost * (1 + Fraction(1, 2**52)), (v, r)
+        checked += 1
+    assert checked > 25000
+
+
 @pytest.mark.gpu
 def test_gpu_equals_host(exe):
     r = subprocess.run([exe, "gpu"], capture_output=True, text=True, timeout=120)
