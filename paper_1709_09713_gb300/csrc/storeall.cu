@@ -105,7 +105,9 @@ struct Derivatives {
 // beside the others, which balances the two pipes inside each thread.  (The array
 // decides, not the plane, so that a shifted state has the shifted derivatives, bit
 // for bit; every third plane in a binary64 sum took 1.036 ms a 128^3 stage, sets take
-// 1.047, all in integers 1.123, and sums of one kind a block, the kinds in turn, 1.148.)
+// 1.049, all in integers 1.123, all in binary64 1.312, and sums of one kind a block, the
+// kinds in turn, 1.148.)  The binary64 sums take each its own weight, so that
+// the large one rounds once less than times a common factor.
 // All derivatives that do not read another's result are blocks of one
 // launch: 128^3 points are little over a wave of blocks, so a launch per
 // derivative left the SMs half idle in its last wave and between launches.
@@ -114,11 +116,8 @@ struct Derivatives {
 constexpr int BL_Z = 9;
 template <bool INTEGER, typename T>
 __device__ __forceinline__ T bl_first(T m2, T m1, T p1, T p2, T k1, T k2) {
-  if constexpr (sizeof(T) == 8) {  // k2 = 1/(12 h)
-    return k2 * (INTEGER ? stencil_first(m2, m1, p1, p2) : first_sum<false>(m2, m1, p1, p2, 0));
-  } else {
-    return k1 * (p1 - m1) - k2 * (p2 - m2);
-  }
+  if constexpr (sizeof(T) == 8 && INTEGER) return k2 * stencil_first(m2, m1, p1, p2);  // k2 = 1/(12 h)
+  return k1 * (p1 - m1) - k2 * (p2 - m2);
 }
 template <typename T>
 __device__ __forceinline__ T bl_second(T m2, T m1, T c, T p1, T p2, T k0, T k1, T k2) {
