@@ -3,10 +3,11 @@
 // captured as CUDA graphs, and the C ABI of sbli_batch_* (include/sbli.h).
 //
 // A member is one Taylor-Green problem (own n0 x n1 x n2, Re, M, Pr, gamma,
-// L, amplitude).  Its work is split into items (z chunk, 32 x TY tile); items
+// L, amplitude).  Binary32 work is split into items (z chunk, 32 x 8 tile); items
 // of all members are numbered consecutively, chunk-major inside a member so
 // that CTAs running at the same time work on neighbouring tiles of the same
-// planes.  The member table travels in the kernel's parameter space, so a
+// planes.  Binary64 and double-float CTAs take equal runs of the planes of all
+// members' 16 x 8 tiles.  The member table travels in the kernel's parameter space, so a
 // captured graph needs no device-side table.
 #include <math.h>
 #include <stdarg.h>

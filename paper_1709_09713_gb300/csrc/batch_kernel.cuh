@@ -32,8 +32,10 @@ template <typename T>
 cudaError_t launch_batch_t(const BatchParams<T>& p, bool in64, int grid, cudaStream_t s, bool df, int zq);
 
 // The z-queue mode a batch of this precision starts with: binary32 members
-// (either accumulator) the TMEM queue, binary64 and double-float arithmetic
-// the shared-memory ring (their measured faster choices on single grids).
+// (either accumulator) the TMEM queue, the faster one on single grids; binary64 and
+// double-float arithmetic the shared-memory ring, the faster one of marches below 24
+// planes a CTA (single grids of longer ones take the TMEM queue, see default_config;
+// the batch tuner times both).
 inline int batch_default_zq(int precision) { return precision == SBLI_FP32 || precision == SBLI_FP32_DF ? 1 : 0; }
 
 // Resident CTAs per SM of the multi-member launch: binary32 members run the

@@ -311,7 +311,7 @@ __global__ void sample_state_kernel(long long P, double rho0, double E0, const d
       double v = __longlong_as_double(0x7ff8000000000000LL);  // quiet NaN
       if (inside) {
         const long long m = (long long)f * P + n;
-        if (q64) {  // as offset_kernel
+        if (q64) {  // as from_offset_kernel
           v = q64[m];
           if (f == 0) v += rho0;
           if (f == 4) v += E0;

@@ -2,42 +2,13 @@
 //
 // GB300 executes F2F.F64.F32 / F2F.F32.F64 on its (narrow) FP64 pipe at the
 // DFMA rate, about 2 per clock per SM.  The binary32-storage stage converts
-// every stage value and accumulator increment, so these re-pack the IEEE bit
-// patterns with integer operations instead.  Both are exact (the widening is
-// exact by nature; the narrowing rounds to nearest, ties to even, as
-// __double2float_rn does); operands whose result is zero, subnormal, infinite
-// or NaN take the hardware conversion.
+// every stage value and accumulator increment, and the double-float one splits
+// every stage field, so these re-pack the IEEE bit patterns with integer operations
+// instead; each states how it rounds and what becomes of subnormals, infinities and
+// NaNs.
 #pragma once
 
 #include <cuda_runtime.h>
-
-namespace sbli {
-
-__device__ __forceinline__ double widen_f32(float x) {
-  const unsigned u = __float_as_uint(x);
-  const unsigned e = u & 0x7F800000u;
-  if (e == 0u || e == 0x7F800000u) return (double)x;
-  // exponent bias 127 -> 1023 (+896 at bit 20), mantissa 23 -> 52 bits
-  const unsigned hi = (((u & 0x7FFFFFFFu) >> 3) + 0x38000000u) | (u & 0x80000000u);
-  const unsigned lo = u << 29;
-  return __hiloint2double((int)hi, (int)lo);
-}
-
-__device__ __forceinline__ float narrow_f64(double d) {
-  const unsigned hi = (unsigned)__double2hiint(d);
-  const unsigned lo = (unsigned)__double2loint(d);
-  const unsigned eb = (hi >> 20) & 0x7FFu;
-  // binary32-normal results: biased exponent 897..1150
-  if (eb - 897u >= 254u) return __double2float_rn(d);
-  const unsigned mant = ((hi & 0xFFFFFu) << 3) | (lo >> 29);
-  unsigned bits = (hi & 0x80000000u) | ((eb - 896u) << 23) | mant;
-  const unsigned rest = lo & 0x1FFFFFFFu;  // the 29 bits dropped
-  const unsigned half = 0x10000000u;
-  bits += (rest > half || (rest == half && (bits & 1u))) ? 1u : 0u;  // carry may bump the exponent
-  return __uint_as_float(bits);
-}
-
-}  // namespace sbli
 
 namespace sbli {
 

@@ -6,9 +6,11 @@
 // writes the Runge-Kutta stage of §2.2 / Fig. 1 in the same pass.
 //
 // Work decomposition (2.5D streaming):
-//   * a CTA owns a 32 x TY tile of (x0, x1) columns and marches along x2
-//     over zc planes; one thread per column, a warp is one x0 row, so every
-//     global access is a coalesced row segment;
+//   * a CTA owns a tile of (x0, x1) columns and marches along x2 over a run of
+//     planes: 32 x TY columns, a warp a row of them, in binary32 (one thread per
+//     column, or two rows or two columns a thread, see below), 16 x 8, two rows a
+//     warp, in binary64 and double-float (tile_x); every global access is a
+//     coalesced row segment;
 //   * a ring of 5 shared-memory slots holds the primitives of planes
 //     z-2..z+2 on the tile plus a 2-point halo in x0 and x1 (corners
 //     included), one 10-value record per point (array of structures, read
@@ -591,9 +593,8 @@ template <>
 __device__ __forceinline__ float to_compute<float, double>(double v) {
   return narrow_f64_fast(v);
 }
-// binary64 -> double-float: hi = RN32(v), lo = RN32(v - hi); the narrowings
-// and the widening of hi are integer re-packings, the remainder one DADD
-// (exact: v - hi has at most 29 significant bits)
+// binary64 -> double-float: hi = v rounded to nearest, ties away from zero, and the
+// remainder (29 bits) rounded to 24, in integer and binary32 operations
 template <>
 __device__ __forceinline__ dfloat to_compute<dfloat, double>(double v) {
   float hi, lo;
@@ -670,9 +671,14 @@ __device__ __forceinline__ T add_nc(T a, T b) {
 // take the rounding of u_j = m_j / rho into the mass balance: 1.45 times its
 // error, so Eq. 1 keeps two.)  The viscous terms of Eq. 2 are accumulated as
 // their sum (Laplacian + G/3), the symmetric off-diagonal gradients as their
-// sum: 15 multiply-adds a neighbour in binary32 instead of the 17 of one
-// accumulator per derivative (the number of instructions bounds these kernels:
-// 512^3, binary64 accumulator, 3.73 -> 3.63 ms a stage).  Binary64 takes the linear
+// sum.  H carries one rounding that E' in its place would not (the centre's E' is
+// H - 2p'), for one product fewer a neighbour.  Errors of the energy's residual
+// against quadruple precision on 40 grids of 14 to 48 points an edge, with E' before
+// and with H: binary64 6.70e-14, 6.66e-14, double-float 4.47e-12, 4.19e-12, binary32
+// 5.05e-5 both (the rounding of its input).
+// All that is 15 multiply-adds a neighbour in binary32 instead of the 17 of one
+// accumulator per derivative (one point a thread, where the number of instructions
+// counted most: 512^3, binary64 accumulator, 3.73 -> 3.63 ms a stage).  Binary64 takes the linear
 // stencils in integers (axis_terms_sums) and the factors -1/2 (convective terms)
 // and 1/3, 4/3 (viscous terms) in its weights; in binary32 the constants of that
 // are too many for the uniform registers (256^3: 479 -> 504 us), and the factors
