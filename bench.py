@@ -66,9 +66,9 @@ ALG_BYTES = {"fp64": 400.0 / 3.0, "fp32": 320.0 / 3.0, "fp32df": 320.0 / 3.0, "d
 KERNEL_SOURCES = ["fused_stage.cuh", "fused_fp64.cu", "fused_df64.cu", "dfloat.cuh", "fpconv.cuh", "f32x2.cuh",
                   "sbli_internal.cuh", "stencil_int.cuh"]
 KERNEL_COUNTS = {
-    "fp64": {"flop_per_pt": 310.2, "traffic_per_pt": 4.609e9 / 256**3, "sources": "05e5aee57ddc",
+    "fp64": {"flop_per_pt": 310.2, "traffic_per_pt": 4.609e9 / 256**3, "sources": "1879af04f0d0",
              "profile": "profiles/fused_stage_fp64_256.md"},
-    "df64": {"inst_per_pt": {0: 2303.8, 1: 2369.2}, "sources": "05e5aee57ddc",
+    "df64": {"inst_per_pt": {0: 2295.8, 1: 2374.1}, "sources": "1879af04f0d0",
              "profile": "profiles/fused_stage_df64_256.md"},
 }
 

@@ -1,5 +1,5 @@
-"""The store-all derivative launches (blocks of 32 x 8 columns and nine planes,
-several arrays a launch) where a block's columns and planes end."""
+"""The store-all derivative launches (blocks of 32 x 8 columns, nine planes of one
+array or three of a set of arrays) where a block's columns and planes end."""
 import numpy as np
 import pytest
 
