@@ -32,7 +32,7 @@
 // Variables are deviations from the reference state, as in the other paths.
 #include <utility>
 
-#include "fpconv.cuh"
+#include "primitives.cuh"
 #include "sbli_internal.cuh"
 
 namespace sbli {
@@ -368,13 +368,10 @@ __global__ void __launch_bounds__(256) algorithm_stage_kernel(Geom g, const __gr
 __global__ void primitives_kernel(long long P, const __grid_constant__ Coef<double> c, const double* __restrict__ q,
                                   double* __restrict__ w) {
   for (long long n = blockIdx.x * (long long)blockDim.x + threadIdx.x; n < P; n += (long long)gridDim.x * blockDim.x) {
-    const double rho_p = q[n], rho = 1.0 + rho_p, rinv = rcp_newton_f64(rho);
-    double u[3];
-    for (int i = 0; i < 3; ++i) u[i] = corrected_quotient(q[(1 + i) * P + n], rho, rinv);
-    const double p_p = c.gm1 * (q[4 * P + n] - 0.5 * rho * (u[0] * u[0] + u[1] * u[1] + u[2] * u[2]));  // Eq. 4
-    for (int i = 0; i < 3; ++i) w[i * P + n] = u[i];
-    w[3 * P + n] = p_p;
-    w[4 * P + n] = corrected_quotient(c.gM2 * p_p - rho_p, rho, rinv);  // Eq. 5
+    const Primitives r = primitives_f64(q[n], q[P + n], q[2 * P + n], q[3 * P + n], q[4 * P + n], c.gm1, c.gM2);
+    for (int i = 0; i < 3; ++i) w[i * P + n] = r.u[i];
+    w[3 * P + n] = r.p;
+    w[4 * P + n] = r.t;
   }
 }
 

@@ -11,7 +11,7 @@
 // Variables are deviations from the reference state, as in the fused path.
 #include <type_traits>
 
-#include "fpconv.cuh"
+#include "primitives.cuh"
 #include "sbli_internal.cuh"
 #include "stencil_int.cuh"
 
@@ -55,19 +55,18 @@ __global__ void bl_primitives(Geom g, Coef<T> c, const TIN* __restrict__ q, T* _
     const T rho_p = T(q[n]);
     const T m[3] = {T(q[P + n]), T(q[2 * P + n]), T(q[3 * P + n])};
     const T E_p = T(q[4 * P + n]);
-    const T rho = T(1) + rho_p;
-    // one reciprocal for the four quotients, each corrected by its residual
-    // (Markstein), so that they round as divisions do
-    T rinv = T(0);
-    if constexpr (sizeof(T) == 8) rinv = rcp_newton_f64(rho);
-    auto quotient = [&](T x) -> T {
-      if constexpr (sizeof(T) == 8) return corrected_quotient(x, rho, rinv);
-      else return x / rho;
-    };
-    T u[3];
-    for (int i = 0; i < 3; ++i) u[i] = quotient(m[i]);
-    const T p_p = c.gm1 * (E_p - T(0.5) * rho * (u[0] * u[0] + u[1] * u[1] + u[2] * u[2]));  // Eq. 4
-    const T T_p = quotient(c.gM2 * p_p - rho_p);                                            // Eq. 5
+    [[maybe_unused]] const T rho = T(1) + rho_p;
+    T u[3], p_p, T_p;
+    if constexpr (sizeof(T) == 8) {
+      const Primitives r = primitives_f64(rho_p, m[0], m[1], m[2], E_p, c.gm1, c.gM2);
+      for (int i = 0; i < 3; ++i) u[i] = r.u[i];
+      p_p = r.p;
+      T_p = r.t;
+    } else {
+      for (int i = 0; i < 3; ++i) u[i] = m[i] / rho;
+      p_p = c.gm1 * (E_p - T(0.5) * rho * (u[0] * u[0] + u[1] * u[1] + u[2] * u[2]));  // Eq. 4
+      T_p = (c.gM2 * p_p - rho_p) / rho;                                              // Eq. 5
+    }
     for (int i = 0; i < 3; ++i) s[(A_U + i) * P + n] = u[i];
     s[A_P * P + n] = p_p;
     s[A_T * P + n] = T_p;

@@ -66,3 +66,41 @@ def test_bad_point_stays_local_and_queues_agree(S, precision, configs):
                 assert not np.isfinite(out[1][field][BAD]), (field, value)
                 assert np.array_equal(out[0][:, rhs_away], want[0][:, rhs_away]), (field, value)
                 assert np.array_equal(out[1][:, step_away], want[1][:, step_away]), (field, value)
+
+
+def _finite_residual(q, n):
+    """Where Eqs. 1-3 on binary64 values give a number: m / rho is a division (0 of an infinite density)."""
+    gm1, gm2 = 0.4, 1.4 * 0.01
+    at = lambda f, a, s: np.roll(f, -s, 2 - a)  # noqa: E731
+    d1 = lambda f, a: 8.0 * (at(f, a, 1) - at(f, a, -1)) - (at(f, a, 2) - at(f, a, -2))  # noqa: E731
+    d2 = lambda f, a: 16.0 * (at(f, a, 1) + at(f, a, -1)) - (at(f, a, 2) + at(f, a, -2)) - 30.0 * f  # noqa: E731
+    with np.errstate(all="ignore"):
+        rho_p, E = q[0] - 1.0, q[4] - E0
+        rho = 1.0 + rho_p
+        u = [q[1 + i] / rho for i in range(3)]
+        p = gm1 * (E - 0.5 * rho * (u[0] * u[0] + u[1] * u[1] + u[2] * u[2]))
+        t = (gm2 * p - rho_p) / rho
+        du = [[d1(u[i], j) for j in range(3)] for i in range(3)]
+        div = du[0][0] + du[1][1] + du[2][2]
+        skew = lambda f: f * div + sum(d1(f * u[j], j) + u[j] * d1(f, j) for j in range(3))  # noqa: E731
+        visc = [sum(d2(u[i], j) + (0.0 if i == j else d1(du[j][j], i)) for j in range(3)) for i in range(3)]
+        r = [rho * div + sum(d1(q[1 + j], j) + u[j] * d1(rho_p, j) for j in range(3))]
+        r += [skew(q[1 + i]) + d1(p, i) + visc[i] for i in range(3)]
+        r.append(skew(E) + sum(d1(p * u[j], j) + d2(t, j) + u[j] * visc[j] for j in range(3)) +
+                 sum(du[i][j] * (du[i][j] + du[j][i]) for i in range(3) for j in range(3)))
+    return np.isfinite(np.stack(r))
+
+
+@pytest.mark.parametrize("variant", ["SBLI_STORE_ALL", "SBLI_RS", "SBLI_SS", "SBLI_RA", "SBLI_SN", "SBLI_SN2"])
+def test_classes_divide_as_binary64_does(S, variant):
+    """An infinite density or momentum takes the residual from the points where it
+    takes it by the rules of division, and from no others."""
+    clean = workloads.smooth_state(N, 23, offsets=(1.0, 0.0, 0.0, 0.0, E0 + 0.5))
+    for field, value in ((0, np.inf), (1, -np.inf), (0, np.nan), (4, np.inf)):
+        q = clean.copy()
+        q[(field,) + BAD] = value
+        g = S.Grid(N, S.SBLI_FP64, getattr(S, variant))
+        g.set_state(torch.from_numpy(q))
+        got = np.isfinite(g.rhs().cpu().numpy())
+        g.close()
+        assert np.array_equal(got, _finite_residual(q, N)), (field, value, got.sum(), _finite_residual(q, N).sum())
